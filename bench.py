@@ -234,6 +234,16 @@ class Runner:
         return hQ, hK, hV, hOm, hY
 
 
+def measured_peaks():
+    peaks = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_burst": 1590.0, "source": "fallback", "sm_max_mhz": 1965.0}
+    pk = os.path.join(ROOT, "MEASURED_PEAKS.json")
+    if os.path.exists(pk):
+        j = json.load(open(pk))
+        peaks = {"hbm_gbs": j["hbm_gbs"], "bf16_tflops": j["bf16_tflops_sustained"], "bf16_tflops_burst": j["bf16_tflops"],
+                 "source": "measured (sustained bf16: the kernels are timed inside a long step)", "sm_max_mhz": j.get("sm_max_mhz", 1965.0)}
+    return peaks
+
+
 def backward_flops(w):
     """Multiply-adds x 2 of the backward pass as the kernels issue them (Section 2.2 differentiated; the header of
     csrc/backward.cu lists the products): features of both sides, the two key- / query-side sums, numerators and
@@ -342,19 +352,19 @@ def run_pairs(args):
     sampler.stop_flag = True
     sampler.join(timeout=2)
     nv = len(pw.variants)
-    sm_count = torch.cuda.get_device_properties(dev).multi_processor_count
     flops = nv * pw.R * pw.npairs * 2 * (2 * pw.M * pw.d)            # both sides' w^T B x per pair, draw and variant
-    peak = 128 * 2 * sm_count * 1965e6 / 1e12                           # fp32: 128 multiply-adds per clock and SM
-    t_k = kern["pairs_kernel"][0] / kern["pairs_kernel"][1] * 1e-3
+    peaks = measured_peaks()
+    peak = peaks["bf16_tflops"] / 6                                     # six bf16 part products per fp32 product
+    t_k = kern["tc_pairs_kernel"][0] / kern["tc_pairs_kernel"][1] * 1e-3
     out = {"metric": "kernel estimates for (x, y) pairs with empirical and closed-form variance", "value": pw.npairs / (ms * 1e-3),
            "unit": "pairs/s", "n_gpus": 1, "steps": steps, "warmup": warm, "ms_per_step": ms, "higher_is_better": True,
            "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
            "config": {"workload": f"{pw.name}: {pw.npairs} pairs, d {pw.d}, M {pw.M} orthogonal features, R {pw.R} draws, "
                                   f"parameterisations {', '.join(pw.variants)} (a step covers all of them)"},
            "clocks": sampler.result(), "gpu_launches": launches,
-           "roofline": {"kernel": "pairs_kernel", "bound": "alu", "achieved": flops / nv / t_k / 1e12, "peak": peak, "unit": "TFLOP/s",
+           "roofline": {"kernel": "tc_pairs_kernel", "bound": "tensor", "achieved": flops / nv / t_k / 1e12, "peak": peak, "unit": "TFLOP/s",
                         "frac": flops / nv / t_k / 1e12 / peak, "traffic": None,
-                        "peak_source": "128 fp32 multiply-adds per clock and SM x SMs x 1965 MHz"},
+                        "peak_source": peaks["source"] + ", bf16 / 6 (three-part fp32 operands)"},
            "kernels": {k: {"ms_per_launch": v[0] / v[1], "launches_per_step": v[1]} for k, v in kern.items()},
            "pooled_relative_variance": {v: {"empirical": float(pooled[v][0]), "closed_form": float(pooled[v][1])} for v in pw.variants}}
     if not args.no_cpu_baseline:
@@ -538,12 +548,7 @@ def main():
 
     tokens_per_step = world * sum(w.B * w.L for w in ws)
     value = tokens_per_step * args.steps / (ms * 1e-3)
-    peaks = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_burst": 1590.0, "source": "fallback", "sm_max_mhz": 1965.0}
-    pk = os.path.join(ROOT, "MEASURED_PEAKS.json")
-    if os.path.exists(pk):
-        j = json.load(open(pk))
-        peaks = {"hbm_gbs": j["hbm_gbs"], "bf16_tflops": j["bf16_tflops_sustained"], "bf16_tflops_burst": j["bf16_tflops"],
-                 "source": "measured (sustained bf16: the kernels are timed inside a long step)", "sm_max_mhz": j.get("sm_max_mhz", 1965.0)}
+    peaks = measured_peaks()
     sm_count = torch.cuda.get_device_properties(dev).multi_processor_count
 
     per_workload, attend_ms_total, roof_ms_total, roof_nominal_total, exp_ms_total = {}, 0.0, 0.0, 0.0, 0.0
