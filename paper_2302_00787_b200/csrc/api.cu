@@ -2,6 +2,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "feat3.cuh"
 #include "tc_layout.cuh"
 
 // tensor-core path (tc_*.cu)
@@ -114,7 +115,7 @@ int fsharp_featurize(fsharp_ctx* ctx, const void* X, const float* Omega, const d
     return fs_tc_featurize(ctx, X, dims, side, stab, prep_t, images, flags, phi, logscale, &wst);
   }
   const size_t need = ws_round(prep_f * 4) + ws_round((size_t)dims->B * dims->H * L * 4) +
-                      ws_round((size_t)dims->B * dims->H * 4);
+                      ws_round((size_t)dims->B * dims->H * 4) + feat3::image_bytes(G, dims->d, dims->M, 1);
   FS_TRY(fs_ws_reserve(ctx, need));
   WsAlloc ws{ctx->ws, 0};
   float* prep = ws.take<float>(prep_f);
@@ -123,7 +124,8 @@ int fsharp_featurize(fsharp_ctx* ctx, const void* X, const float* Omega, const d
   FS_TRY(fs_run_prep(ctx, Omega, dims->omega_head_stride, params, (int64_t)ParamsLayout{dims->d}.total(), G,
                      dims->H, dims->pool, dims->d, dims->M, prep));
   return fs_simt_featurize(ctx, X, dtype, fs_addr(st, dims->H, L, dims->d), dims->B, dims->H, L, dims->d, dims->M,
-                           dims->pool, prep, side, qk_scale, stab, rowc, gmax, phi, logscale);
+                           dims->pool, prep, side, qk_scale, stab, rowc, gmax, phi, logscale,
+                           ws.take<uint8_t>(feat3::image_bytes(G, dims->d, dims->M, 1)));
 }
 
 int fsharp_attend(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const float* Omega,

@@ -1,6 +1,6 @@
 // Backward pass of featurize + attend (Section 5.3 trains Transformers through the attention of
 // Section 2.2): given dY, the gradients with respect to Q, K and V, the random features Omega and
-// the fitted parameters being constants.  fp32 CUDA-core kernels.
+// the fitted parameters being constants.  Every product is a block product at fp32 precision on the tensor cores (mma3.cuh).
 //
 // With P = phi(Q) (L x M), S = phi(K), [num | den] = P KV_i, KV_i = sum_{j <= i} S_j [V_j | 1]^T
 // (all j when bidirectional), Y = num / den:
@@ -13,176 +13,146 @@
 // chunk, R_j = (sum over later chunks) + the masked part, with tril(P_c S_c^T) and tril(G_c [V_c | 1]^T)
 // formed per chunk.  The feature kernels' shifts (per query row, per (batch, head) for the keys)
 // cancel in every product above exactly as they do in Y.
-#include "common.cuh"
-#include "simt_tile.cuh"
+#include "f32_parts.cuh"
+#include "feat3.cuh"
 
 namespace {
 
+using mma3::Piece;
+using mma3::ROWS;
+
 struct BwdDims {
-  int H, Lq, Lk, d, dv, M, N, causal, C, nch;
+  int H, Lq, Lk, d, dv, M, NP, causal, C, nch;      // NP = dv + 16: [V | 1] rows, G rows and sums are padded to it
 };
 
-// ---- out[z][m][n] (+)= sum_{j in slice} F[j][m] * R[j][n] --------------------------------------
-// FROM_G = false: F = phi(K), R = [V | 1] (typed);  true: F = phi(Q), R = G (fp32, row stride N).
-template <typename T, bool FROM_G>
-__global__ void __launch_bounds__(NTH)
-bwd_state_kernel(const float* __restrict__ F, const T* __restrict__ V, TensorAddr av, const float* __restrict__ G,
-                 BwdDims q, int L, int slice_len, int nslices, int per_slice_out, float* __restrict__ out) {
-  __shared__ Tiles sm;
-  const int bh = blockIdx.z / nslices, sl = blockIdx.z % nslices;
-  const int b = bh / q.H, h = bh % q.H;
-  const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
-  const int j0 = sl * slice_len, j1 = min(L, j0 + slice_len);
-  if (j0 >= j1) return;
-  const int M = q.M, N = q.N, dv = q.dv;
-  const float* Fb = F + (int64_t)bh * L * M;
-  const T* Vb = V + b * av.sb + h * av.sh;
-  const float* Gb = G + (int64_t)bh * L * N;
-  float acc[4][4] = {};
-  tile_gemm<false, false>(
-      acc, j1 - j0, [&](int r, int k) { return (m0 + r < M) ? Fb[(int64_t)(j0 + k) * M + m0 + r] : 0.f; },
-      [&](int k, int c) {
-        const int n = n0 + c;
-        if (FROM_G) return n < N ? Gb[(int64_t)(j0 + k) * N + n] : 0.f;
-        return n < dv ? fs_load(Vb + (int64_t)(j0 + k) * av.sl + n) : (n == dv ? 1.f : 0.f);
-      },
-      sm);
-  float* O = out + (int64_t)(per_slice_out ? blockIdx.z : bh) * M * N;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-#pragma unroll
-  for (int i = 0; i < 4; i++) {
-    const int m = m0 + ty + 16 * i;
-    if (m >= M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-      const int n = n0 + tx + 16 * j;
-      if (n < N) {
-        if (per_slice_out) O[(int64_t)m * N + n] = acc[i][j];
-        else atomicAdd(&O[(int64_t)m * N + n], acc[i][j]);
-      }
-    }
-  }
+__device__ __forceinline__ float4 load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
+  const uint2 u = *reinterpret_cast<const uint2*>(p);
+  return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
 }
 
-// ---- exclusive running sum over the chunks, forwards (earlier chunks) or backwards (later chunks) ----
-__global__ void __launch_bounds__(NTH)
-bwd_scan_kernel(float* __restrict__ st, int nchunks, int64_t elems, int reverse) {
-  const int bh = blockIdx.y;
-  float* base = st + (int64_t)bh * nchunks * elems;
-  for (int64_t e = blockIdx.x * (int64_t)NTH + threadIdx.x; e < elems; e += (int64_t)gridDim.x * NTH) {
-    float run = 0.f;
-    for (int c0 = 0; c0 < nchunks; c0 += 8) {
-      float v[8];
-#pragma unroll
-      for (int u = 0; u < 8; u++) {
-        const int c = reverse ? nchunks - 1 - (c0 + u) : c0 + u;
-        v[u] = c0 + u < nchunks ? base[c * elems + e] : 0.f;
-      }
-#pragma unroll
-      for (int u = 0; u < 8; u++) {
-        const int c = reverse ? nchunks - 1 - (c0 + u) : c0 + u;
-        if (c0 + u < nchunks) base[c * elems + e] = run;
-        run += v[u];
-      }
-    }
-  }
-}
-
-// ---- masked blocks of a chunk: MODE 0  tril(phiQ_c phiK_c^T);  MODE 1  tril(G_c [V_c | 1]^T) --------
-template <typename T, int MODE>
-__global__ void __launch_bounds__(NTH)
-bwd_tri_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK, const float* __restrict__ G,
-               const T* __restrict__ V, TensorAddr av, BwdDims q, float* __restrict__ out) {
-  __shared__ Tiles sm;
-  const int bh = blockIdx.z / q.nch, c = blockIdx.z % q.nch;
-  const int b = bh / q.H, h = bh % q.H;
-  const int i0 = blockIdx.x * TM, j0 = blockIdx.y * TN;
-  const int C = q.C, M = q.M, N = q.N, dv = q.dv, L = q.Lq;
-  const int64_t row0 = (int64_t)c * C;
-  float* S = out + (int64_t)blockIdx.z * C * C;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  float acc[4][4] = {};
-  if (j0 <= i0) {
-    if (MODE == 0) {
-      const float* PQ = phiQ + ((int64_t)bh * L + row0) * M;
-      const float* PK = phiK + ((int64_t)bh * L + row0) * M;
-      tile_gemm<true, true>(
-          acc, M, [&](int r, int k) { return PQ[(int64_t)(i0 + r) * M + k]; },
-          [&](int k, int cc) { return PK[(int64_t)(j0 + cc) * M + k]; }, sm);
-    } else {
-      const float* Gc = G + ((int64_t)bh * L + row0) * N;
-      const T* Vb = V + b * av.sb + h * av.sh + row0 * av.sl;
-      tile_gemm<true, true>(
-          acc, N, [&](int r, int k) { return Gc[(int64_t)(i0 + r) * N + k]; },
-          [&](int k, int cc) { return k < dv ? fs_load(Vb + (int64_t)(j0 + cc) * av.sl + k) : 1.f; }, sm);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 4; i++)
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-      const int r = i0 + ty + 16 * i, cc = j0 + tx + 16 * j;
-      S[(int64_t)r * C + cc] = (cc <= r) ? acc[i][j] : 0.f;
-    }
-}
-
-// ---- [num | den] = phiQ KV (+ masked scores times [V_c | 1]) ------------------------------------
+// ---- masked blocks tril(G_c [V_c | 1]^T) of a chunk ----------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(NTH)
-bwd_numden_kernel(const float* __restrict__ phiQ, const float* __restrict__ KV, const float* __restrict__ sc,
-                  const T* __restrict__ V, TensorAddr av, BwdDims q, float* __restrict__ ND) {
-  __shared__ Tiles sm;
-  const int bh = blockIdx.z, b = bh / q.H, h = bh % q.H;
-  const int i0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
-  const int C = q.C, M = q.M, N = q.N, dv = q.dv, L = q.Lq;
-  const int chunk = q.causal ? i0 / C : 0, ic = q.causal ? i0 - chunk * C : 0;
-  const float* PQ = phiQ + (int64_t)bh * L * M;
-  const float* S = KV + ((int64_t)bh * q.nch + chunk) * M * N;
-  float acc[4][4] = {};
-  tile_gemm<true, false>(
-      acc, M, [&](int r, int k) { return (i0 + r < L) ? PQ[(int64_t)(i0 + r) * M + k] : 0.f; },
-      [&](int k, int c) { return (n0 + c < N) ? S[(int64_t)k * N + n0 + c] : 0.f; }, sm);
-  if (q.causal) {
-    const float* SC = sc + ((int64_t)bh * q.nch + chunk) * C * C;
-    const T* Vb = V + b * av.sb + h * av.sh + (int64_t)chunk * C * av.sl;
-    tile_gemm<true, false>(
-        acc, min(C, ic + TM), [&](int r, int k) { return SC[(int64_t)(ic + r) * C + k]; },
-        [&](int k, int c) {
-          const int n = n0 + c;
-          return n < dv ? fs_load(Vb + (int64_t)k * av.sl + n) : (n == dv ? 1.f : 0.f);
-        },
-        sm);
-  }
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-#pragma unroll
-  for (int i = 0; i < 4; i++) {
-    const int r = i0 + ty + 16 * i;
-    if (r >= L) continue;
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-      const int n = n0 + tx + 16 * j;
-      if (n < N) ND[((int64_t)bh * L + r) * N + n] = acc[i][j];
-    }
-  }
+__global__ void __launch_bounds__(mma3::THREADS, 2)
+bwd_tri_kernel(const float* __restrict__ G, const T* __restrict__ V, TensorAddr av, BwdDims q, float* __restrict__ out,
+               int* __restrict__ status) {
+  extern __shared__ uint8_t smem[];
+  const int bh = blockIdx.z / q.nch, c = blockIdx.z % q.nch, b = bh / q.H, h = bh % q.H;
+  const int i0 = blockIdx.x * ROWS, j0 = blockIdx.y * ROWS, C = q.C, dv = q.dv;
+  if (j0 > i0) return;
+  mma3::Block blk;
+  blk.begin(smem, ROWS, status);
+  const int rows = min(C, q.Lq - c * C);
+  const float* Gc = G + ((int64_t)bh * q.Lq + (int64_t)c * C + i0) * q.NP;
+  const T* Vc = V + b * av.sb + h * av.sh + ((int64_t)c * C + j0) * av.sl;
+  constexpr int VP = mma3::PartsOf<T>::N;
+  blk.template segment<true, 3, true, VP>(
+      q.NP, [&](int r, int k, Piece<3>& p) { if (i0 + r < rows) p.load(Gc + (int64_t)r * q.NP + k); else p.zero(); },
+      [&](int n, int k, Piece<VP>& p) {
+        if (j0 + n >= rows || k > dv) p.zero();
+        else if (k < dv) p.load(Vc + (int64_t)n * av.sl + k);
+        else p.unit();
+      });
+  blk.finish();
+  float* S = out + (int64_t)blockIdx.z * C * C;
+  blk.rows([&](int r, int n, float4 v) {
+    const int i = i0 + r, j = j0 + n;
+    if (j > i) v.x = 0.f;
+    if (j + 1 > i) v.y = 0.f;
+    if (j + 2 > i) v.z = 0.f;
+    if (j + 3 > i) v.w = 0.f;
+    *reinterpret_cast<float4*>(S + (int64_t)i * C + j) = v;
+  });
+  blk.end();
 }
 
-// ---- G_i = [dY_i / den_i | -(dY_i . Y_i) / den_i], in place over [num | den]; one warp per row -----
+// ---- [num | den] = phiQ KV (+ masked scores times [V_c | 1]), and from it G = [dY / den | -(dY . Y) / den] -----------
+// dv <= 64: one column tile holds the whole row and G is written; dv = 128 (two tiles): [num | den] is, for bwd_g_kernel.
+template <typename T>
+__global__ void __launch_bounds__(mma3::THREADS, 2)
+bwd_numden_kernel(const float* __restrict__ phiQ, const float* __restrict__ KV, const float* __restrict__ sc,
+                  const T* __restrict__ V, TensorAddr av, const T* __restrict__ dY, TensorAddr ay, BwdDims q, float* __restrict__ G,
+                  int* __restrict__ status) {
+  extern __shared__ uint8_t smem[];
+  __shared__ float inv_s[ROWS], dot_s[ROWS];
+  const int bh = blockIdx.z, b = bh / q.H, h = bh % q.H, i0 = blockIdx.x * ROWS;
+  const int C = q.C, M = q.M, NP = q.NP, dv = q.dv, L = q.Lq;
+  const ColTile ct(dv, blockIdx.y);
+  mma3::Block blk;
+  blk.begin(smem, ct.nt(), status);
+  const int chunk = q.causal ? i0 / C : 0;
+  const float* PQ = phiQ + ((int64_t)bh * L + i0) * M;
+  const float* S = KV + ((int64_t)bh * q.nch + chunk) * M * NP;
+  blk.template segment<true, 3, false, 3>(
+      M, [&](int r, int k, Piece<3>& p) { if (i0 + r < L) p.load(PQ + (int64_t)r * M + k); else p.zero(); },
+      [&](int c, int k, Piece<3>& p) { p.load(S + (int64_t)k * NP + ct.at(dv, c)); });
+  if (q.causal) {
+    const int ic = i0 - chunk * C, keys = min(ic + ROWS, L - chunk * C);
+    const float* SC = sc + (((int64_t)bh * q.nch + chunk) * C + ic) * C;
+    const T* Vc = V + b * av.sb + h * av.sh + (int64_t)chunk * C * av.sl;
+    constexpr int VP = mma3::PartsOf<T>::N;
+    blk.template segment<true, 3, false, VP>(
+        (keys + 7) & ~7, [&](int r, int k, Piece<3>& p) { p.load(SC + (int64_t)r * C + k); },
+        [&](int c, int k, Piece<VP>& p) {
+          if (k >= keys) p.zero();
+          else if (c < ct.wt) p.load(Vc + (int64_t)k * av.sl + ct.v0 + c);
+          else if (c == ct.wt) p.unit();
+          else p.zero();
+        });
+  }
+  blk.finish();
+  float* Gb = G + ((int64_t)bh * L + i0) * NP;
+  if (gridDim.y > 1) {
+    blk.rows([&](int r, int c, float4 v) {
+      if (i0 + r < L && (c < ct.wt || blockIdx.y == 0)) *reinterpret_cast<float4*>(Gb + (int64_t)r * NP + ct.at(dv, c)) = v;
+    });
+    blk.end();
+    return;
+  }
+  if (threadIdx.x < ROWS) {
+    const float den = blk.column(ct.wt);
+    if (i0 + (int)threadIdx.x < L && (!(den > 0.f) || !isfinite(den))) atomicExch(status, FSHARP_E_NONFINITE);
+    inv_s[threadIdx.x] = 1.f / den;
+    dot_s[threadIdx.x] = 0.f;
+  }
+  __syncthreads();
+  const T* dYb = dY + b * ay.sb + h * ay.sh + (int64_t)i0 * ay.sl;
+  blk.rows([&](int r, int c, float4 v) {
+    float s = 0.f;
+    if (i0 + r < L && c < dv) {
+      const float inv = inv_s[r];
+      const float4 y = load4(dYb + (int64_t)r * ay.sl + c);
+      s = fmaf(y.x, v.x * inv, fmaf(y.y, v.y * inv, fmaf(y.z, v.z * inv, y.w * (v.w * inv))));
+      *reinterpret_cast<float4*>(Gb + (int64_t)r * NP + c) = make_float4(y.x * inv, y.y * inv, y.z * inv, y.w * inv);
+    }
+    // the lanes of a row are neighbours: eight of them (32 columns at a time) or four
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    if ((threadIdx.x & 3) == 0) atomicAdd(&dot_s[r], s);
+  });
+  __syncthreads();
+  for (int e = threadIdx.x; e < ROWS * 4; e += mma3::THREADS) {
+    const int r = e >> 2, part = e & 3;
+    if (i0 + r < L) *reinterpret_cast<float4*>(Gb + (int64_t)r * NP + dv + 4 * part) = make_float4(part ? 0.f : -dot_s[r] * inv_s[r], 0.f, 0.f, 0.f);
+  }
+  blk.end();
+}
+
+// ---- G from [num | den], in place; one warp per row (dv = 128) --------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(NTH)
 bwd_g_kernel(float* __restrict__ ND, const T* __restrict__ dY, TensorAddr ay, BwdDims q, int* __restrict__ status) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int bh = blockIdx.y, b = bh / q.H, h = bh % q.H;
-  const int dv = q.dv, N = q.N, L = q.Lq;
+  const int bh = blockIdx.y, b = bh / q.H, h = bh % q.H, dv = q.dv;
   const T* dYb = dY + b * ay.sb + h * ay.sh;
-  for (int i = blockIdx.x * 8 + warp; i < L; i += gridDim.x * 8) {
-    float* row = ND + ((int64_t)bh * L + i) * N;
-    const float den = row[dv];
-    const float inv = 1.f / den;
+  for (int i = blockIdx.x * 8 + warp; i < q.Lq; i += gridDim.x * 8) {
+    float* row = ND + ((int64_t)bh * q.Lq + i) * q.NP;
+    const float den = row[dv], inv = 1.f / den;
     float s = 0.f;
-    for (int c = lane; c < dv; c += 32) {
-      const float dy = fs_load(dYb + (int64_t)i * ay.sl + c);
-      s = fmaf(dy, row[c] * inv, s);
-      row[c] = dy * inv;
+    for (int c = 4 * lane; c < dv; c += 128) {
+      const float4 y = load4(dYb + (int64_t)i * ay.sl + c), n = *reinterpret_cast<const float4*>(row + c);
+      s = fmaf(y.x, n.x * inv, fmaf(y.y, n.y * inv, fmaf(y.z, n.z * inv, fmaf(y.w, n.w * inv, s))));
+      *reinterpret_cast<float4*>(row + c) = make_float4(y.x * inv, y.y * inv, y.z * inv, y.w * inv);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -193,163 +163,171 @@ bwd_g_kernel(float* __restrict__ ND, const T* __restrict__ dY, TensorAddr ay, Bw
   }
 }
 
-// ---- E = dphi * phi (the gradient with respect to the exponents) --------------------------------
+// ---- E = dphi * phi (the gradient with respect to the exponents), and its row sums per feature tile ----------------
 // SIDE 1: dphiQ_c = G_c KV_c^T + tril(G_c [V_c | 1]^T) phiK_c;   SIDE 2: dphiK_c = [V_c | 1] R_c^T + tril(...)^T phiQ_c
+// rs [feature tile][BH][L]
 template <typename T, int SIDE>
-__global__ void __launch_bounds__(NTH)
+__global__ void __launch_bounds__(mma3::THREADS, 2)
 bwd_dfeat_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK, const float* __restrict__ G,
                  const float* __restrict__ St, const float* __restrict__ gv, const T* __restrict__ V, TensorAddr av,
-                 BwdDims q, float* __restrict__ E) {
-  __shared__ Tiles sm;
+                 BwdDims q, float* __restrict__ E, float* __restrict__ rs, int* __restrict__ status) {
+  extern __shared__ uint8_t smem[];
+  __shared__ float rs_s[ROWS];
   const int bh = blockIdx.z, b = bh / q.H, h = bh % q.H;
-  const int i0 = blockIdx.x * TM, m0 = blockIdx.y * TN;
-  const int C = q.C, M = q.M, N = q.N, dv = q.dv;
-  const int L = SIDE == 1 ? q.Lq : q.Lk;
+  const int m0 = blockIdx.x * ROWS, i0 = blockIdx.y * ROWS;
+  const int C = q.C, M = q.M, NP = q.NP, dv = q.dv, L = SIDE == 1 ? q.Lq : q.Lk;
   const int chunk = q.causal ? i0 / C : 0, ic = q.causal ? i0 - chunk * C : 0;
-  const float* S = St + ((int64_t)bh * q.nch + chunk) * M * N;
+  mma3::Block blk;
+  blk.begin(smem, min(ROWS, M - m0), status);
+  const float* S = St + ((int64_t)bh * q.nch + chunk) * M * NP + (int64_t)m0 * NP;
   const float* GV = q.causal ? gv + ((int64_t)bh * q.nch + chunk) * C * C : nullptr;
-  float acc[4][4] = {};
   if (SIDE == 1) {
-    const float* Gb = G + (int64_t)bh * L * N;
-    tile_gemm<true, true>(
-        acc, N, [&](int r, int k) { return (i0 + r < L) ? Gb[(int64_t)(i0 + r) * N + k] : 0.f; },
-        [&](int k, int c) { return (m0 + c < M) ? S[(int64_t)(m0 + c) * N + k] : 0.f; }, sm);
+    const float* Gb = G + ((int64_t)bh * L + i0) * NP;
+    blk.template segment<true, 3, true, 3>(
+        NP, [&](int r, int k, Piece<3>& p) { if (i0 + r < L) p.load(Gb + (int64_t)r * NP + k); else p.zero(); },
+        [&](int n, int k, Piece<3>& p) { p.load(S + (int64_t)n * NP + k); });
     if (q.causal) {
-      const float* PK = phiK + ((int64_t)bh * L + (int64_t)chunk * C) * M;
-      tile_gemm<true, false>(
-          acc, min(C, ic + TM), [&](int r, int k) { return GV[(int64_t)(ic + r) * C + k]; },
-          [&](int k, int c) { return (m0 + c < M) ? PK[(int64_t)k * M + m0 + c] : 0.f; }, sm);
+      const int keys = min(ic + ROWS, L - chunk * C);
+      const float* PK = phiK + ((int64_t)bh * L + (int64_t)chunk * C) * M + m0;
+      blk.template segment<true, 3, false, 3>(
+          (keys + 7) & ~7, [&](int r, int k, Piece<3>& p) { p.load(GV + (int64_t)(ic + r) * C + k); },
+          [&](int c, int k, Piece<3>& p) { if (k < keys) p.load(PK + (int64_t)k * M + c); else p.zero(); });
     }
   } else {
-    const T* Vb = V + b * av.sb + h * av.sh;
-    tile_gemm<true, true>(
-        acc, N,
-        [&](int r, int k) {
-          if (i0 + r >= L) return 0.f;
-          return k < dv ? fs_load(Vb + (int64_t)(i0 + r) * av.sl + k) : 1.f;
+    const T* Vb = V + b * av.sb + h * av.sh + (int64_t)i0 * av.sl;
+    constexpr int VP = mma3::PartsOf<T>::N;
+    blk.template segment<true, VP, true, 3>(
+        NP,
+        [&](int r, int k, Piece<VP>& p) {
+          if (i0 + r >= L || k > dv) p.zero();
+          else if (k < dv) p.load(Vb + (int64_t)r * av.sl + k);
+          else p.unit();
         },
-        [&](int k, int c) { return (m0 + c < M) ? S[(int64_t)(m0 + c) * N + k] : 0.f; }, sm);
+        [&](int n, int k, Piece<3>& p) { p.load(S + (int64_t)n * NP + k); });
     if (q.causal) {
       // rows ic + k of the masked block, k >= 0: the queries of this chunk at or after this tile's first key
-      const float* PQ = phiQ + ((int64_t)bh * L + (int64_t)chunk * C + ic) * M;
-      tile_gemm<false, false>(
-          acc, C - ic, [&](int r, int k) { return GV[(int64_t)(ic + k) * C + ic + r]; },
-          [&](int k, int c) { return (m0 + c < M) ? PQ[(int64_t)k * M + m0 + c] : 0.f; }, sm);
+      const float* PQ = phiQ + ((int64_t)bh * L + (int64_t)chunk * C + ic) * M + m0;
+      blk.template segment<false, 3, false, 3>(
+          min(C, L - chunk * C) - ic, [&](int r, int k, Piece<3>& p) { p.load(GV + (int64_t)(ic + k) * C + ic + r); },
+          [&](int c, int k, Piece<3>& p) { p.load(PQ + (int64_t)k * M + c); });
     }
   }
-  const float* Ph = (SIDE == 1 ? phiQ : phiK) + (int64_t)bh * L * M;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-#pragma unroll
-  for (int i = 0; i < 4; i++) {
-    const int r = i0 + ty + 16 * i;
-    if (r >= L) continue;
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-      const int m = m0 + tx + 16 * j;
-      if (m < M) E[((int64_t)bh * L + r) * M + m] = acc[i][j] * Ph[(int64_t)r * M + m];
+  blk.finish();
+  if (threadIdx.x < ROWS) rs_s[threadIdx.x] = 0.f;
+  __syncthreads();
+  const int64_t base = ((int64_t)bh * L + i0) * M + m0;
+  const float* Ph = (SIDE == 1 ? phiQ : phiK) + base;
+  blk.rows([&](int r, int c, float4 v) {
+    float s = 0.f;
+    if (i0 + r < L) {
+      const float4 f = *reinterpret_cast<const float4*>(Ph + (int64_t)r * M + c);
+      v.x *= f.x; v.y *= f.y; v.z *= f.z; v.w *= f.w;
+      *reinterpret_cast<float4*>(E + base + (int64_t)r * M + c) = v;
+      s = (v.x + v.y) + (v.z + v.w);
     }
-  }
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    if ((threadIdx.x & 3) == 0) atomicAdd(&rs_s[r], s);
+  });
+  __syncthreads();
+  if (threadIdx.x < ROWS && i0 + (int)threadIdx.x < L)
+    rs[((int64_t)blockIdx.x * gridDim.z + bh) * L + i0 + threadIdx.x] = rs_s[threadIdx.x];
+  blk.end();
 }
 
 // ---- dV_c = phiK_c R_c[:, :dv] + tril(phiQ_c phiK_c^T)^T G_c[:, :dv] ------------------------------
 template <typename T>
-__global__ void __launch_bounds__(NTH)
+__global__ void __launch_bounds__(mma3::THREADS, 2)
 bwd_dv_kernel(const float* __restrict__ phiK, const float* __restrict__ Rt, const float* __restrict__ sc,
-              const float* __restrict__ G, BwdDims q, T* __restrict__ dV, TensorAddr av) {
-  __shared__ Tiles sm;
-  const int bh = blockIdx.z, b = bh / q.H, h = bh % q.H;
-  const int j0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
-  const int C = q.C, M = q.M, N = q.N, dv = q.dv, L = q.Lk;
+              const float* __restrict__ G, BwdDims q, T* __restrict__ dV, TensorAddr av, int* __restrict__ status) {
+  extern __shared__ uint8_t smem[];
+  const int bh = blockIdx.z, b = bh / q.H, h = bh % q.H, j0 = blockIdx.x * ROWS;
+  const int C = q.C, M = q.M, NP = q.NP, dv = q.dv, L = q.Lk;
   const int chunk = q.causal ? j0 / C : 0, jc = q.causal ? j0 - chunk * C : 0;
-  const float* PK = phiK + (int64_t)bh * L * M;
-  const float* R = Rt + ((int64_t)bh * q.nch + chunk) * M * N;
-  float acc[4][4] = {};
-  tile_gemm<true, false>(
-      acc, M, [&](int r, int k) { return (j0 + r < L) ? PK[(int64_t)(j0 + r) * M + k] : 0.f; },
-      [&](int k, int c) { return (n0 + c < dv) ? R[(int64_t)k * N + n0 + c] : 0.f; }, sm);
+  mma3::Block blk;
+  blk.begin(smem, dv, status);
+  const float* PK = phiK + ((int64_t)bh * L + j0) * M;
+  const float* R = Rt + ((int64_t)bh * q.nch + chunk) * M * NP;
+  blk.template segment<true, 3, false, 3>(
+      M, [&](int r, int k, Piece<3>& p) { if (j0 + r < L) p.load(PK + (int64_t)r * M + k); else p.zero(); },
+      [&](int c, int k, Piece<3>& p) { p.load(R + (int64_t)k * NP + c); });
   if (q.causal) {
     const float* SC = sc + ((int64_t)bh * q.nch + chunk) * C * C;
-    const float* Gc = G + ((int64_t)bh * L + (int64_t)chunk * C + jc) * N;
-    tile_gemm<false, false>(
-        acc, C - jc, [&](int r, int k) { return SC[(int64_t)(jc + k) * C + jc + r]; },
-        [&](int k, int c) { return (n0 + c < dv) ? Gc[(int64_t)k * N + n0 + c] : 0.f; }, sm);
+    const float* Gc = G + ((int64_t)bh * L + (int64_t)chunk * C + jc) * NP;
+    blk.template segment<false, 3, false, 3>(
+        min(C, L - chunk * C) - jc, [&](int r, int k, Piece<3>& p) { p.load(SC + (int64_t)(jc + k) * C + jc + r); },
+        [&](int c, int k, Piece<3>& p) { p.load(Gc + (int64_t)k * NP + c); });
   }
-  T* Ob = dV + b * av.sb + h * av.sh;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-#pragma unroll
-  for (int i = 0; i < 4; i++) {
-    const int r = j0 + ty + 16 * i;
-    if (r >= L) continue;
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-      const int n = n0 + tx + 16 * j;
-      if (n < dv) fs_store(Ob + (int64_t)r * av.sl + n, acc[i][j]);
-    }
-  }
+  blk.finish();
+  T* Ob = dV + b * av.sb + h * av.sh + (int64_t)j0 * av.sl;
+  blk.rows([&](int r, int c, float4 v) { if (j0 + r < L) store4(Ob + (int64_t)r * av.sl + c, v); });
+  blk.end();
 }
 
 // ---- dX = qk_scale (E W + rowsum(E) x^T (C + C^T)),  x = qk_scale X ------------------------------
 template <typename T>
-__global__ void __launch_bounds__(NTH)
-bwd_dx_kernel(const float* __restrict__ E, const T* __restrict__ X, TensorAddr ax, int H, int L, int d, int M, int pool,
-              int side, const float* __restrict__ prep, float qk_scale, T* __restrict__ dX, int* __restrict__ status) {
-  __shared__ Tiles sm;
-  __shared__ float rs[TM];
-  const int bh = blockIdx.z, b = bh / H, h = bh % H;
-  const int i0 = blockIdx.x * TM, c0 = blockIdx.y * TN;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+__global__ void __launch_bounds__(mma3::THREADS, 2)
+bwd_dx_kernel(const float* __restrict__ E, const float* __restrict__ rs, int mtiles, const T* __restrict__ X, TensorAddr ax, int H, int L,
+              int d, int M, int pool, int side, const float* __restrict__ prep, float qk_scale, T* __restrict__ dX,
+              int* __restrict__ status) {
+  extern __shared__ uint8_t smem[];
+  __shared__ float rs_s[ROWS];
+  const int bh = blockIdx.z, b = bh / H, h = bh % H, i0 = blockIdx.x * ROWS;
   PrepLayout pr{d, M};
   const float* pp = prep + ((size_t)(pool == FSHARP_POOL_PER_BH ? bh : h) * 2 + (side - 1)) * pr.total();
   const float* W = pp + pr.W();
   const float* Cm = pp + pr.Cmat();
-  const float* Eb = E + (int64_t)bh * L * M;
-  const T* Xb = X + b * ax.sb + h * ax.sh;
-  {
-    const int r = tid >> 2, part = tid & 3;
+  const bool cscalar = pp[pr.scal() + PS_CSCALAR] != 0.f;
+  const float gamma = pp[pr.scal() + PS_CGAMMA];
+  mma3::Block blk;
+  blk.begin(smem, d, status);
+  if (threadIdx.x < ROWS) {
     float s = 0.f;
-    if (i0 + r < L)
-      for (int m = part; m < M; m += 4) s += Eb[(int64_t)(i0 + r) * M + m];
-    s += __shfl_xor_sync(0xffffffffu, s, 1);
-    s += __shfl_xor_sync(0xffffffffu, s, 2);
-    if (part == 0) rs[r] = s;
+    if (i0 + (int)threadIdx.x < L)
+      for (int t = 0; t < mtiles; t++) s += rs[((int64_t)t * gridDim.z + bh) * L + i0 + threadIdx.x];
+    rs_s[threadIdx.x] = qk_scale * s;
   }
   __syncthreads();
-  float acc[4][4] = {}, quad[4][4] = {};
-  tile_gemm<true, false>(
-      acc, M, [&](int r, int k) { return (i0 + r < L) ? Eb[(int64_t)(i0 + r) * M + k] : 0.f; },
-      [&](int k, int c) { return (c0 + c < d) ? W[(size_t)k * d + c0 + c] : 0.f; }, sm);
-  tile_gemm<true, false>(
-      quad, d, [&](int r, int k) { return (i0 + r < L) ? qk_scale * fs_load(Xb + (int64_t)(i0 + r) * ax.sl + k) : 0.f; },
-      [&](int k, int c) { return (c0 + c < d) ? Cm[(size_t)k * d + c0 + c] + Cm[(size_t)(c0 + c) * d + k] : 0.f; }, sm);
-  T* Ob = dX + b * ax.sb + h * ax.sh;
+  const float* Eb = E + ((int64_t)bh * L + i0) * M;
+  const T* Xb = X + b * ax.sb + h * ax.sh + (int64_t)i0 * ax.sl;
+  blk.template segment<true, 3, false, 3>(
+      M, [&](int r, int k, Piece<3>& p) { if (i0 + r < L) p.load(Eb + (int64_t)r * M + k); else p.zero(); },
+      [&](int c, int k, Piece<3>& p) { p.load(W + (size_t)k * d + c); });
+  if (!cscalar)
+    blk.template segment<true, 3, false, 3>(
+        d,
+        [&](int r, int k, Piece<3>& p) {
+          if (i0 + r >= L) { p.zero(); return; }
+          const float4 a = load4(Xb + (int64_t)r * ax.sl + k), c = load4(Xb + (int64_t)r * ax.sl + k + 4);
+          const float s = rs_s[r];
+          p.v[0] = s * a.x; p.v[1] = s * a.y; p.v[2] = s * a.z; p.v[3] = s * a.w;
+          p.v[4] = s * c.x; p.v[5] = s * c.y; p.v[6] = s * c.z; p.v[7] = s * c.w;
+        },
+        [&](int c, int k, Piece<3>& p) {
+          p.load(Cm + (size_t)k * d + c);
+#pragma unroll
+          for (int j = 0; j < 8; j++) p.v[j] += Cm[(size_t)(c + j) * d + k];
+        });
+  blk.finish();
+  T* Ob = dX + b * ax.sb + h * ax.sh + (int64_t)i0 * ax.sl;
   bool bad = false;
-#pragma unroll
-  for (int i = 0; i < 4; i++) {
-    const int r = ty + 16 * i;
-    if (i0 + r >= L) continue;
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-      const int c = c0 + tx + 16 * j;
-      if (c < d) {
-        const float v = qk_scale * fmaf(rs[r], quad[i][j], acc[i][j]);
-        if (!isfinite(v)) bad = true;
-        fs_store(Ob + (int64_t)(i0 + r) * ax.sl + c, v);
-      }
+  blk.rows([&](int r, int c, float4 v) {
+    if (i0 + r >= L) return;
+    if (cscalar) {
+      const float s = 2.f * gamma * rs_s[r];
+      const float4 x = load4(Xb + (int64_t)r * ax.sl + c);
+      v.x = fmaf(s, x.x, v.x); v.y = fmaf(s, x.y, v.y); v.z = fmaf(s, x.z, v.z); v.w = fmaf(s, x.w, v.w);
     }
-  }
+    v.x *= qk_scale; v.y *= qk_scale; v.z *= qk_scale; v.w *= qk_scale;
+    if (!isfinite(v.x) || !isfinite(v.y) || !isfinite(v.z) || !isfinite(v.w)) bad = true;
+    store4(Ob + (int64_t)r * ax.sl + c, v);
+  });
   if (bad) atomicExch(status, FSHARP_E_NONFINITE);
+  blk.end();
 }
 
-int slices_for(const fsharp_ctx* ctx, int BH, int L, int* slice_len) {
-  int nsl = (4 * ctx->sm_count + BH - 1) / BH;
-  const int maxsl = (L + 255) / 256;
-  if (nsl > maxsl) nsl = maxsl;
-  if (nsl > 65535 / BH) nsl = 65535 / BH;
-  if (nsl < 1) nsl = 1;
-  const int slen = (L + nsl - 1) / nsl;
-  *slice_len = slen;
-  return (L + slen - 1) / slen;
-}
+struct Yes { static constexpr bool value = true; };
+struct No { static constexpr bool value = false; };
 
 template <typename T>
 int backward_t(fsharp_ctx* ctx, const void* Qv, const void* Kv, const void* Vv, const void* dYv, const fsharp_dims* dm,
@@ -357,97 +335,85 @@ int backward_t(fsharp_ctx* ctx, const void* Qv, const void* Kv, const void* Vv, 
                WsAlloc* ws) {
   const T* Q = (const T*)Qv; const T* K = (const T*)Kv; const T* V = (const T*)Vv; const T* dY = (const T*)dYv;
   const int B = dm->B, H = dm->H, BH = B * H, Lq = dm->Lq, Lk = dm->Lk, d = dm->d, dv = dm->dv, M = dm->M;
-  const int N = dv + 1;
-  BwdDims q{H, Lq, Lk, d, dv, M, N, causal ? 1 : 0, causal ? chunk : 0, causal ? Lq / chunk : 1};
-  const int C = q.C, nch = q.nch;
+  const int NP = dv + 16, C = causal ? inner_chunk(chunk) : 0, nch = causal ? (Lq + C - 1) / C : 1;
+  const int mt = (M + ROWS - 1) / ROWS, ctiles = (dv + 63) / 64, qt = (Lq + ROWS - 1) / ROWS, kt = (Lk + ROWS - 1) / ROWS;
+  const BwdDims q{H, Lq, Lk, d, dv, M, NP, causal ? 1 : 0, C, nch};
   TensorAddr aq = fs_addr(dm->q_stride, H, Lq, d), ak = fs_addr(dm->k_stride, H, Lk, d);
   TensorAddr av = fs_addr(dm->v_stride, H, Lk, dv), ay = fs_addr(dm->y_stride, H, Lq, dv);
   float* phiQ = ws->take<float>((size_t)BH * Lq * M);
   float* phiK = ws->take<float>((size_t)BH * Lk * M);
-  float* EQ = ws->take<float>((size_t)BH * Lq * M);
-  float* EK = ws->take<float>((size_t)BH * Lk * M);
-  float* rowc = ws->take<float>((size_t)BH * (Lq > Lk ? Lq : Lk));
+  float* E = ws->take<float>((size_t)BH * (Lq > Lk ? Lq : Lk) * M);      // one side after the other
+  float* rs = ws->take<float>((size_t)mt * BH * (Lq > Lk ? Lq : Lk));
+  float* rowcq = ws->take<float>((size_t)BH * Lq);
+  float* rowck = ws->take<float>((size_t)BH * Lk);
   unsigned* gmax = ws->take<unsigned>((size_t)BH);
   float* lsq = ws->take<float>((size_t)BH * Lq);
   float* lsk = ws->take<float>((size_t)BH);
-  float* ND = ws->take<float>((size_t)BH * Lq * N);
-  float* KV = ws->take<float>((size_t)BH * nch * M * N);
-  float* Rt = ws->take<float>((size_t)BH * nch * M * N);
+  float* G = ws->take<float>((size_t)BH * Lq * NP);
+  float* KV = ws->take<float>((size_t)BH * nch * M * NP);
+  float* Rt = ws->take<float>((size_t)BH * nch * M * NP);
   float* sc = causal ? ws->take<float>((size_t)BH * nch * C * C) : nullptr;
   float* gv = causal ? ws->take<float>((size_t)BH * nch * C * C) : nullptr;
-  cudaStream_t st = ctx->stream;
-
-  FS_TRY(fs_simt_featurize(ctx, K, dtype, ak, B, H, Lk, d, M, dm->pool, prep, 2, qk_scale, FSHARP_STAB_GROUP, rowc,
-                           gmax, phiK, lsk));
-  FS_TRY(fs_simt_featurize(ctx, Q, dtype, aq, B, H, Lq, d, M, dm->pool, prep, 1, qk_scale, FSHARP_STAB_ROW, rowc,
-                           gmax, phiQ, lsq));
-  const dim3 gstate((M + TM - 1) / TM, (N + TN - 1) / TN, 1);
-  const int64_t elems = (int64_t)M * N;
+  uint8_t* img = ws->take<uint8_t>(feat3::image_bytes(fs_groups(dm), d, M, 2));
+  int* status = ctx->d_status;
+  const int64_t elems = (int64_t)M * NP;
   const dim3 gscan((unsigned)((elems + NTH - 1) / NTH), BH);
-  int slen = 0, nsl = 1;
-  // 1. key-side sums: the total (bidirectional) or the sum over earlier chunks (causal)
-  if (!causal) {
-    nsl = slices_for(ctx, BH, Lk, &slen);
-    FS_CUDA_OK(cudaMemsetAsync(KV, 0, (size_t)BH * M * N * sizeof(float), st));
-    bwd_state_kernel<T, false><<<dim3(gstate.x, gstate.y, BH * nsl), NTH, 0, st>>>(phiK, V, av, nullptr, q, Lk, slen, nsl, 0, KV);
-    FS_LAUNCH_CHECK(ctx);
-  } else {
-    bwd_state_kernel<T, false><<<dim3(gstate.x, gstate.y, BH * nch), NTH, 0, st>>>(phiK, V, av, nullptr, q, Lk, C, nch, 1, KV);
-    FS_LAUNCH_CHECK(ctx);
-    bwd_scan_kernel<<<gscan, NTH, 0, st>>>(KV, nch, elems, 0);
-    FS_LAUNCH_CHECK(ctx);
-    bwd_tri_kernel<T, 0><<<dim3(C / TM, C / TN, BH * nch), NTH, 0, st>>>(phiQ, phiK, nullptr, V, av, q, sc);
-    FS_LAUNCH_CHECK(ctx);
-  }
-  // 2. numerators and normalisers, then G in their place
-  bwd_numden_kernel<T><<<dim3((Lq + TM - 1) / TM, (N + TN - 1) / TN, BH), NTH, 0, st>>>(phiQ, KV, sc, V, av, q, ND);
-  FS_LAUNCH_CHECK(ctx);
-  {
+
+  const feat3::Task tasks[2] = {{K, ak, Lk, 2, FSHARP_STAB_GROUP, rowck, gmax, phiK, lsk},
+                                {Q, aq, Lq, 1, FSHARP_STAB_ROW, rowcq, nullptr, phiQ, lsq}};
+  FS_TRY(feat3::run(ctx, tasks, 2, dtype, B, H, d, M, dm->pool, prep, qk_scale, img));
+  // sums over tokens: the total (bidirectional), or one per chunk turned into the sum over earlier / later chunks (causal)
+  auto sums = [&](auto from_g, const float* F, int L, float* out, int reverse) -> int {
+    constexpr bool FG = decltype(from_g)::value;
+    int slen = C, nsl = nch;
+    if (!causal) {
+      nsl = fs_token_slices(ctx, BH * mt * ctiles, BH, L, &slen);
+      FS_CUDA_OK(cudaMemsetAsync(out, 0, (size_t)BH * elems * sizeof(float), ctx->stream));
+    }
+    FS_TRY(mma3::launch(ctx, FS_K_BWD_STATE, state_kernel<T, FG>, dim3(mt, ctiles, BH * nsl), F, V, av, G, H, L, M, dv, slen, nsl,
+                        causal ? 1 : 0, out, status));
+    if (causal) {
+      FS_TIME_BEGIN(ctx, FS_K_PREFIX);
+      prefix_kernel<<<gscan, NTH, 0, ctx->stream>>>(out, nch, elems, reverse, nullptr);
+      FS_TIME_END(ctx);
+      FS_LAUNCH_CHECK(ctx);
+    }
+    return FSHARP_OK;
+  };
+  const dim3 gtri(causal ? C / ROWS : 1, causal ? C / ROWS : 1, BH * nch);
+  FS_TRY(sums(No{}, phiK, Lk, KV, 0));
+  if (causal) FS_TRY(mma3::launch(ctx, FS_K_SCORES, scores_kernel, gtri, phiQ, phiK, Lq, M, C, nch, sc, status));
+  FS_TRY(mma3::launch(ctx, FS_K_BWD_NUMDEN, bwd_numden_kernel<T>, dim3(qt, ctiles, BH), phiQ, KV, sc, V, av, dY, ay, q, G, status));
+  if (ctiles > 1) {
     int gx = (Lq + 7) / 8;
     if (gx > 4 * ctx->sm_count) gx = 4 * ctx->sm_count;
-    bwd_g_kernel<T><<<dim3(gx, BH), NTH, 0, st>>>(ND, dY, ay, q, ctx->d_status);
+    FS_TIME_BEGIN(ctx, FS_K_BWD_NUMDEN);
+    bwd_g_kernel<T><<<dim3(gx, BH), NTH, 0, ctx->stream>>>(G, dY, ay, q, status);
+    FS_TIME_END(ctx);
     FS_LAUNCH_CHECK(ctx);
   }
-  const float* G = ND;
-  // 3. query-side sums R: the total, or the sum over later chunks
-  if (!causal) {
-    nsl = slices_for(ctx, BH, Lq, &slen);
-    FS_CUDA_OK(cudaMemsetAsync(Rt, 0, (size_t)BH * M * N * sizeof(float), st));
-    bwd_state_kernel<T, true><<<dim3(gstate.x, gstate.y, BH * nsl), NTH, 0, st>>>(phiQ, V, av, G, q, Lq, slen, nsl, 0, Rt);
-    FS_LAUNCH_CHECK(ctx);
-  } else {
-    bwd_state_kernel<T, true><<<dim3(gstate.x, gstate.y, BH * nch), NTH, 0, st>>>(phiQ, V, av, G, q, Lq, C, nch, 1, Rt);
-    FS_LAUNCH_CHECK(ctx);
-    bwd_scan_kernel<<<gscan, NTH, 0, st>>>(Rt, nch, elems, 1);
-    FS_LAUNCH_CHECK(ctx);
-    bwd_tri_kernel<T, 1><<<dim3(C / TM, C / TN, BH * nch), NTH, 0, st>>>(phiQ, phiK, G, V, av, q, gv);
-    FS_LAUNCH_CHECK(ctx);
-  }
-  // 4. gradients with respect to the exponents, dV, then dQ and dK
-  bwd_dfeat_kernel<T, 1><<<dim3((Lq + TM - 1) / TM, (M + TN - 1) / TN, BH), NTH, 0, st>>>(phiQ, phiK, G, KV, gv, V, av, q, EQ);
-  FS_LAUNCH_CHECK(ctx);
-  bwd_dfeat_kernel<T, 2><<<dim3((Lk + TM - 1) / TM, (M + TN - 1) / TN, BH), NTH, 0, st>>>(phiQ, phiK, G, Rt, gv, V, av, q, EK);
-  FS_LAUNCH_CHECK(ctx);
-  bwd_dv_kernel<T><<<dim3((Lk + TM - 1) / TM, (dv + TN - 1) / TN, BH), NTH, 0, st>>>(phiK, Rt, sc, G, q, (T*)dVv, av);
-  FS_LAUNCH_CHECK(ctx);
-  bwd_dx_kernel<T><<<dim3((Lq + TM - 1) / TM, (d + TN - 1) / TN, BH), NTH, 0, st>>>(EQ, Q, aq, H, Lq, d, M, dm->pool, 1, prep,
-                                                                                  qk_scale, (T*)dQv, ctx->d_status);
-  FS_LAUNCH_CHECK(ctx);
-  bwd_dx_kernel<T><<<dim3((Lk + TM - 1) / TM, (d + TN - 1) / TN, BH), NTH, 0, st>>>(EK, K, ak, H, Lk, d, M, dm->pool, 2, prep,
-                                                                                  qk_scale, (T*)dKv, ctx->d_status);
-  FS_LAUNCH_CHECK(ctx);
-  return FSHARP_OK;
+  FS_TRY(sums(Yes{}, phiQ, Lq, Rt, 1));
+  if (causal) FS_TRY(mma3::launch(ctx, FS_K_SCORES, bwd_tri_kernel<T>, gtri, G, V, av, q, gv, status));
+  FS_TRY(mma3::launch(ctx, FS_K_BWD_DFEAT, bwd_dfeat_kernel<T, 1>, dim3(mt, qt, BH), phiQ, phiK, G, KV, gv, V, av, q, E, rs, status));
+  FS_TRY(mma3::launch(ctx, FS_K_BWD_DX, bwd_dx_kernel<T>, dim3(qt, 1, BH), E, rs, mt, Q, aq, H, Lq, d, M, dm->pool, 1, prep, qk_scale,
+                      (T*)dQv, status));
+  FS_TRY(mma3::launch(ctx, FS_K_BWD_DFEAT, bwd_dfeat_kernel<T, 2>, dim3(mt, kt, BH), phiQ, phiK, G, Rt, gv, V, av, q, E, rs, status));
+  FS_TRY(mma3::launch(ctx, FS_K_BWD_DX, bwd_dx_kernel<T>, dim3(kt, 1, BH), E, rs, mt, K, ak, H, Lk, d, M, dm->pool, 2, prep, qk_scale,
+                      (T*)dKv, status));
+  return mma3::launch(ctx, FS_K_BWD_DV, bwd_dv_kernel<T>, dim3(kt, 1, BH), phiK, Rt, sc, G, q, (T*)dVv, av, status);
 }
 
 }  // namespace
 
 size_t fs_backward_scratch_bytes(const fsharp_dims* dm, int causal, int chunk) {
-  const size_t BH = (size_t)dm->B * dm->H, N = dm->dv + 1, M = dm->M;
-  const size_t Lq = dm->Lq, Lk = dm->Lk, Lmax = Lq > Lk ? Lq : Lk;
-  const size_t nch = causal && chunk > 0 ? Lq / chunk : 1;
-  size_t b = 2 * ws_round(BH * Lq * M * 4) + 2 * ws_round(BH * Lk * M * 4) + ws_round(BH * Lmax * 4) + ws_round(BH * 4) +
-             ws_round(BH * Lq * 4) + ws_round(BH * 4) + ws_round(BH * Lq * N * 4) + 2 * ws_round(BH * nch * M * N * 4);
-  if (causal) b += 2 * ws_round(BH * nch * (size_t)chunk * chunk * 4);
+  const size_t BH = (size_t)dm->B * dm->H, NP = dm->dv + 16, M = dm->M;
+  const size_t Lq = dm->Lq, Lk = dm->Lk, Lmax = Lq > Lk ? Lq : Lk, C = causal ? inner_chunk(chunk) : 0;
+  const size_t nch = causal ? (Lq + C - 1) / C : 1, mt = (M + ROWS - 1) / ROWS;
+  size_t b = ws_round(BH * Lq * M * 4) + ws_round(BH * Lk * M * 4) + ws_round(BH * Lmax * M * 4) + ws_round(mt * BH * Lmax * 4) +
+             2 * ws_round(BH * Lq * 4) + ws_round(BH * Lk * 4) + 2 * ws_round(BH * 4) + ws_round(BH * Lq * NP * 4) +
+             2 * ws_round(BH * nch * M * NP * 4);
+  b += feat3::image_bytes(fs_groups(dm), dm->d, dm->M, 2);
+  if (causal) b += 2 * ws_round(BH * nch * C * C * 4);
   return b;
 }
 

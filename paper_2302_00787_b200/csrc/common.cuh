@@ -48,12 +48,13 @@ enum { PS_BIAS = 0, PS_CSCALAR = 3, PS_CGAMMA = 4 };
 
 // Kernel ids for the optional per-kernel timing (fsharp_set_timing / fsharp_read_timing).
 enum {
-  FS_K_STATS = 1, FS_K_FIT, FS_K_PREP, FS_K_ROWTERM, FS_K_LOGITS, FS_K_GROUPMAX, FS_K_EXPSHIFT, FS_K_KV,
+  FS_K_STATS = 1, FS_K_FIT, FS_K_PREP, FS_K_ROWTERM, FS_K_FEAT, FS_K_GROUPMAX, FS_K_EXPSHIFT, FS_K_KV,
   FS_K_PREFIX, FS_K_SCORES, FS_K_OUT, FS_K_PAIRS, FS_K_PAIRVAR_PREP, FS_K_PAIRVAR,
   FS_K_TC_KV, FS_K_TC_OUT, FS_K_TC_CAUSAL, FS_K_TC_STATS, FS_K_TC_ROWTERM, FS_K_TC_FEAT, FS_K_TC_LOGITS128, FS_K_TC_SCORES128, FS_K_TC_KV128, FS_K_TC_OUT128,
-  FS_K_PAIR_IMAGES,
+  FS_K_PAIR_IMAGES, FS_K_W3, FS_K_BWD_STATE, FS_K_BWD_NUMDEN, FS_K_BWD_DFEAT, FS_K_BWD_DX, FS_K_BWD_DV,
   FS_K_COUNT
 };
+static_assert(FS_K_COUNT <= 32, "ids are below 32");
 constexpr int FS_TIMING_SLOTS = 4096;
 
 struct fsharp_ctx {
@@ -183,6 +184,21 @@ static inline int fs_groups(const fsharp_dims* dm) {
   return dm->pool == FSHARP_POOL_PER_BH ? dm->B * dm->H : dm->H;
 }
 
+// Slices of a token axis that a sum over tokens is cut into: enough for two waves of two blocks per SM over the `blocks`
+// blocks of one slice, at most 256 tokens (the accumulator's rounding, mma3.cuh, stays that of 16 steps), a multiple of 32,
+// and (unit, slice) has to fit a grid's z coordinate.
+static inline int fs_token_slices(const fsharp_ctx* ctx, int blocks, int BH, int L, int* slice_len) {
+  int nsl = (4 * ctx->sm_count + blocks - 1) / blocks;
+  const int least = (L + 255) / 256, most = (L + 127) / 128;
+  if (nsl < least) nsl = least;
+  if (nsl > most) nsl = most;
+  if (nsl > 65535 / BH) nsl = 65535 / BH;
+  if (nsl < 1) nsl = 1;
+  const int slen = ((L + nsl - 1) / nsl + 31) & ~31;
+  *slice_len = slen;
+  return (L + slen - 1) / slen;
+}
+
 // ---- stage entry points (host side, defined in the .cu files) -------------
 int fs_run_stats(fsharp_ctx* ctx, const void* Q, const void* K, const fsharp_dims* dm, int dtype,
                  float qk_scale, double* stats);
@@ -199,10 +215,10 @@ int fs_run_prep(fsharp_ctx* ctx, const float* Omega, int64_t omega_head_stride, 
 int fs_run_prep_images(fsharp_ctx* ctx, const float* Omega, int64_t omega_head_stride, const double* params,
                        int64_t params_stride, int G, int H, int pool, int d, int M, float* prep, float qk_scale,
                        uint8_t* images, int* flags);
-// rowc: scratch [B*H*L] floats.  gmax: scratch [B*H] words.  phi: [B,H,L,M] floats.
+// rowc: scratch [B*H*L] floats.  gmax: scratch [B*H] words.  phi: [B,H,L,M] floats.  img: scratch (feat3.cuh) or null.
 int fs_simt_featurize(fsharp_ctx* ctx, const void* X, int dtype, TensorAddr ax, int B, int H, int L, int d,
                       int M, int pool, const float* prep, int side, float qk_scale, int stab,
-                      float* rowc, unsigned* gmax, float* phi, float* logscale);
+                      float* rowc, unsigned* gmax, float* phi, float* logscale, uint8_t* img);
 // Exponents of bf16 tokens with d = 128 on the tensor cores (tc_logits128.cu); phi [B*H][L][M] fp32, rowc [B*H][L].
 int fs_tc_logits128_supported(const void* X, int dtype, TensorAddr ax, int L, int d, int M);
 int fs_tc_logits128(fsharp_ctx* ctx, const void* X, TensorAddr ax, int B, int H, int L, int M, int pool, const float* prep,

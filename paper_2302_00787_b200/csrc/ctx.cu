@@ -151,7 +151,7 @@ const char* fsharp_kernel_name(int id) {
     case FS_K_FIT: return "fit_kernel";
     case FS_K_PREP: return "prep_kernel";
     case FS_K_ROWTERM: return "rowterm_kernel";
-    case FS_K_LOGITS: return "logits_kernel";
+    case FS_K_FEAT: return "feat3_kernel";
     case FS_K_GROUPMAX: return "groupmax_kernel";
     case FS_K_EXPSHIFT: return "expshift_kernel";
     case FS_K_KV: return "kv_kernel";
@@ -159,6 +159,12 @@ const char* fsharp_kernel_name(int id) {
     case FS_K_SCORES: return "scores_kernel";
     case FS_K_OUT: return "out_kernel";
     case FS_K_PAIRS: return "tc_pairs_kernel";
+    case FS_K_BWD_STATE: return "state_kernel";
+    case FS_K_BWD_NUMDEN: return "bwd_numden_kernel";
+    case FS_K_BWD_DFEAT: return "bwd_dfeat_kernel";
+    case FS_K_BWD_DX: return "bwd_dx_kernel";
+    case FS_K_BWD_DV: return "bwd_dv_kernel";
+    case FS_K_W3: return "w3_images_kernel";
     case FS_K_PAIR_IMAGES: return "pair_images_kernel";
     case FS_K_PAIRVAR_PREP: return "pairvar_prep_kernel";
     case FS_K_PAIRVAR: return "pairvar_kernel";

@@ -1,0 +1,680 @@
+// Features at fp32 precision (Section 4 definition with Section 2.1's M^-1/2) on the tensor cores, for every shape and both
+// types: phi = exp(e - shift), e_im = bias + a_m + w_m . x_i + c_i, c_i = x_i^T C x_i.
+//
+// The fp32 operands enter the MMAs as three bf16 parts (split3.cuh); bf16 tokens are exact.  The feature matrix is written
+// once: the row shift is found in tensor memory before the exponentials, the group shift by a pass of the same products
+// that writes nothing (the products of a tile cost a quarter of what its 128 x 256 features cost in HBM time).  The kernels
+// they replace (fp32 multiply-adds; exponents written, read for the maximum, read and written again as features) took
+// 441 + 98 + 38 us for 2 x 160 k tokens, d = 64, M = 256, and 360 us for the dense quadratic terms.
+#include "feat3.cuh"
+#include "split3.cuh"
+#include "tc_layout.cuh"
+
+using namespace tc;
+using namespace tcl;
+using feat3::Task;
+
+namespace {
+
+__device__ __forceinline__ int group_of(int bh, int H, int pool) { return pool == FSHARP_POOL_PER_BH ? bh : bh % H; }
+
+// Order-preserving map float -> unsigned, so that atomicMax on words gives the float maximum (0 lies below every float).
+__device__ __forceinline__ unsigned f2ord(float f) {
+  unsigned u = __float_as_uint(f);
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+__device__ __forceinline__ float ord2f(unsigned u) {
+  return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
+}
+
+// Float maximum by integer atomics (start value -inf; bit patterns of non-negative floats ascend, of negative ones descend).
+__device__ __forceinline__ void atomic_max_float(float* p, float v) {
+  v += 0.f;                                        // -0 -> +0
+  if (v >= 0.f) atomicMax(reinterpret_cast<int*>(p), __float_as_int(v));
+  else atomicMin(reinterpret_cast<unsigned*>(p), __float_as_uint(v));
+}
+
+// 32 bytes (eight words) as one store; p is 32-byte aligned
+__device__ __forceinline__ void store32(float* p, const uint32_t* x) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(x[4]),
+               "r"(x[5]), "r"(x[6]), "r"(x[7])
+               : "memory");
+}
+
+struct Args {
+  Task t[2];
+  int first[3];           // running number of work items: task i owns [first[i], first[i + 1])
+  int tiles[2];           // token tiles per (batch, head)
+  int H, M, pool, nmb;
+  const float* prep;
+  const uint8_t* img[2];  // per task: operand images of W (nullptr: blocks build them from prep)
+  float qk_scale;
+  int* status;
+};
+
+// Eight values of a token row as the parts of an MMA operand (16-byte pieces `part` bytes apart).
+__device__ __forceinline__ void put8(uint8_t* dst, uint32_t part, const float* p, bool in) {
+  float v[8] = {};
+  if (in) {
+    const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+  }
+  uint4 h, m, l;
+  split3::split8(v, h, m, l);
+  *reinterpret_cast<uint4*>(dst) = h;
+  *reinterpret_cast<uint4*>(dst + part) = m;
+  *reinterpret_cast<uint4*>(dst + 2 * part) = l;
+}
+
+template <typename T, int D> struct Geo {
+  static constexpr int NKS = (D + 63) / 64;                  // slices of 64 values of K
+  static constexpr int KSTEPS = D < 64 ? D / 16 : 4;         // MMA steps per slice
+  static constexpr int CH = D < 64 ? D / 8 : 8;              // 16-byte pieces of a row and slice
+  static constexpr int AP = sizeof(T) == 2 ? 1 : 3;          // parts of a token
+  static constexpr uint32_t A_BYTES = NKS * AP * TILE_BYTES; // [slice][part][128 rows x 128 bytes]
+};
+
+// Token tile -> operand parts, thread i of N; consecutive lanes take one row's pieces.  The global loads are a step of
+// their own, so that they can be in flight while the buffer is still being read.
+template <typename T, int D, int N> struct Stage {
+  using G = Geo<T, D>;
+  static constexpr int PER_ROW = G::NKS * G::CH, COUNT = TILE * PER_ROW / N;
+  static constexpr int BATCH = COUNT < 8 ? COUNT : 8;           // pieces in flight per thread
+  uint4 r[BATCH][sizeof(T) == 2 ? 1 : 2];
+  __device__ __forceinline__ void load(const T* X, int64_t sl, int rows, int i, int batch) {
+#pragma unroll
+    for (int u = 0; u < BATCH; u++) {
+      const int e = i + (batch * BATCH + u) * N, row = e / PER_ROW, c = e % PER_ROW;
+      const uint4* src = reinterpret_cast<const uint4*>(X + (int64_t)row * sl + 8 * c);
+      const bool in = row < rows;
+      r[u][0] = in ? src[0] : make_uint4(0, 0, 0, 0);
+      if (sizeof(T) == 4) r[u][sizeof(T) == 4 ? 1 : 0] = in ? src[1] : make_uint4(0, 0, 0, 0);
+    }
+  }
+  __device__ __forceinline__ void store(uint8_t* sA, int i, int batch) const {
+#pragma unroll
+    for (int u = 0; u < BATCH; u++) {
+      const int e = i + (batch * BATCH + u) * N, row = e / PER_ROW, c = e % PER_ROW, s = c / 8, cc = c % 8;
+      uint8_t* dst = sA + s * (G::AP * TILE_BYTES) + row * 128 + ((cc ^ (row & 7)) << 4);
+      if (sizeof(T) == 2) {
+        *reinterpret_cast<uint4*>(dst) = r[u][0];
+      } else {
+        const uint4 a = r[u][0], b = r[u][sizeof(T) == 4 ? 1 : 0];
+        const float v[8] = {__uint_as_float(a.x), __uint_as_float(a.y), __uint_as_float(a.z), __uint_as_float(a.w),
+                            __uint_as_float(b.x), __uint_as_float(b.y), __uint_as_float(b.z), __uint_as_float(b.w)};
+        uint4 h, m, l;
+        split3::split8(v, h, m, l);
+        *reinterpret_cast<uint4*>(dst) = h;
+        *reinterpret_cast<uint4*>(dst + TILE_BYTES) = m;
+        *reinterpret_cast<uint4*>(dst + 2 * TILE_BYTES) = l;
+      }
+    }
+  }
+  // all pieces of a tile but those of batch 0, which `load` has fetched ahead
+  __device__ __forceinline__ void finish(uint8_t* sA, const T* X, int64_t sl, int rows, int i) {
+    store(sA, i, 0);
+#pragma unroll
+    for (int b = 1; b < COUNT / BATCH; b++) {
+      load(X, sl, rows, i, b);
+      store(sA, i, b);
+    }
+  }
+};
+
+// Feature blocks of M (all of M when it fits: a row's largest exponent is then known inside the block) and their images:
+// [block][slice][3 parts][rows of 128 bytes, 128-byte swizzle], already scaled by log2e qk_scale.
+template <int D> struct WGeo {
+  static constexpr int NKS = (D + 63) / 64, MB = D == 128 ? 128 : 256;
+};
+template <int D>
+__device__ __forceinline__ void put_w(uint8_t* img, int mb, int f, int c, const float* w, float scale, bool& bad) {
+  float v[8];
+#pragma unroll
+  for (int j = 0; j < 8; j++) {
+    v[j] = scale * w[j];
+    bad |= !isfinite(v[j]);
+  }
+  uint4 h, m, l;
+  split3::split8(v, h, m, l);
+  uint8_t* dst = img + (c / 8) * (3 * mb * 128) + f * 128 + (((c % 8) ^ (f & 7)) << 4);
+  *reinterpret_cast<uint4*>(dst) = h;
+  *reinterpret_cast<uint4*>(dst + mb * 128) = m;
+  *reinterpret_cast<uint4*>(dst + 2 * mb * 128) = l;
+}
+template <int D>
+__global__ void __launch_bounds__(256)
+w3_images_kernel(const float* __restrict__ prep, int side0, int sides, int M, float qk_scale, uint8_t* __restrict__ img,
+                 int* __restrict__ status) {
+  using G = WGeo<D>;
+  const int g = blockIdx.y, k = blockIdx.z;                          // group; which of the `sides` sides
+  const size_t per_group = (size_t)G::NKS * 3 * M * 128;
+  const float* W = prep + ((size_t)g * 2 + (side0 - 1 + k)) * PrepLayout{D, M}.total();
+  uint8_t* out = img + ((size_t)k * gridDim.y + g) * per_group;
+  bool bad = false;
+  for (int e = blockIdx.x * 256 + threadIdx.x; e < M * (D / 8); e += gridDim.x * 256) {
+    const int m = e / (D / 8), c = e % (D / 8), blk = m / G::MB, mb = min(G::MB, M - blk * G::MB);
+    put_w<D>(out + (size_t)blk * G::MB * (G::NKS * 3 * 128), mb, m - blk * G::MB, c, W + (size_t)m * D + 8 * c, FS_LOG2E * qk_scale, bad);
+  }
+  if (bad) atomicExch(status, FSHARP_E_NONFINITE);
+}
+
+// acc[128 x N] = A B^T with A = staged tokens, B = [slice][3 parts][N rows x 128 bytes], by one lane: the products with m or l
+// parts first, h h last (the accumulator is truncated at every step; see tc_pairs.cu).
+// sOne / sRow (may be null): one more step of K = 16 with operands [128 x 16] and [N x 16] in core matrices, for a term per column.
+template <typename T, int D>
+__device__ __forceinline__ void issue_products(uint32_t acc, const uint8_t* sA, const uint8_t* sB, int N, const uint8_t* sOne = nullptr,
+                                               const uint8_t* sRow = nullptr) {
+  using G = Geo<T, D>;
+  const uint32_t idesc = idesc_bf16(128, N, 0, 0);
+  const uint64_t da = smem_desc(smem_u32(sA), 16, 1024, SWZ_128B), db = smem_desc(smem_u32(sB), 16, 1024, SWZ_128B);
+  const uint32_t ah = (uint32_t)(da >> 32), bh = (uint32_t)(db >> 32), P = TILE_BYTES / 16, Q = (uint32_t)N * 8;
+#pragma unroll
+  for (int s = 0; s < G::NKS; s++) {
+    const uint32_t a0 = (uint32_t)da + s * G::AP * P, b0 = (uint32_t)db + s * 3 * Q;
+#pragma unroll
+    for (int k = 0; k < G::KSTEPS; k++) {
+      const uint32_t a = a0 + 2 * k, b = b0 + 2 * k;
+      mma_bf16_lh(acc, a, ah, b + 2 * Q, bh, idesc, (s | k) ? 1u : 0u);
+      if (G::AP == 3) {
+        mma_bf16_lh(acc, a + 2 * P, ah, b, bh, idesc, 1u);
+        mma_bf16_lh(acc, a + P, ah, b + Q, bh, idesc, 1u);
+        mma_bf16_lh(acc, a + P, ah, b, bh, idesc, 1u);
+      }
+      mma_bf16_lh(acc, a, ah, b + Q, bh, idesc, 1u);
+    }
+  }
+  if (sOne != nullptr)
+    mma_bf16(acc, smem_desc(smem_u32(sOne), 128, 256, SWZ_NONE), smem_desc(smem_u32(sRow), 128, 256, SWZ_NONE), idesc, 1u);
+#pragma unroll
+  for (int s = 0; s < G::NKS; s++)
+#pragma unroll
+    for (int k = 0; k < G::KSTEPS; k++)
+      mma_bf16_lh(acc, (uint32_t)da + s * G::AP * P + 2 * k, ah, (uint32_t)db + s * 3 * Q + 2 * k, bh, idesc, 1u);
+}
+
+// ---- c_i = x_i^T C x_i; also clears the maxima that later passes raise ------------------------
+// Block = 128 tokens at a time: T = X C on the tensor cores, c_i = t_i . x_i; C = gamma I needs no product.
+constexpr int RT_THREADS = 256;
+struct RtMisc {
+  uint64_t done;
+  uint32_t tmem_base;
+  int abort_flag;
+  float part[2][TILE];
+};
+template <typename T, int D> constexpr size_t rt_smem() { return 1024 + Geo<T, D>::A_BYTES + Geo<T, D>::NKS * 3 * D * 128 + sizeof(RtMisc); }
+
+template <typename T, int D>
+__global__ void __launch_bounds__(RT_THREADS, D == 128 ? 1 : 3)
+rowterm3_kernel(const __grid_constant__ Args a) {
+  using G = Geo<T, D>;
+  using St = Stage<T, D, RT_THREADS>;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* sA = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint8_t* sC = sA + G::A_BYTES;
+  RtMisc* misc = reinterpret_cast<RtMisc*>(sC + G::NKS * 3 * D * 128);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr uint32_t COLS = D < 32 ? 32 : D;
+  if (tid == 0) {
+    mbar_init(&misc->done, 1);
+    misc->abort_flag = 0;
+    fence_barrier_init();
+  }
+  if (warp == 0) {
+    tmem_alloc(&misc->tmem_base, COLS);
+    tmem_relinquish();
+  }
+  tcgen05_fence_before();
+  __syncthreads();
+  tcgen05_fence_after();
+  const uint32_t tmem = misc->tmem_base;
+  PrepLayout pr{D, a.M};
+  const int total = a.first[2];
+  const int w0 = (int)((int64_t)total * blockIdx.x / gridDim.x), w1 = (int)((int64_t)total * (blockIdx.x + 1) / gridDim.x);
+  int have = -1, phase = 0;                       // (task, group) whose C is staged
+  bool scalar = false, bad = false;
+  float gamma = 0.f;
+  St st;
+  auto tokens = [&](int w, int& rows, int64_t& sl) {
+    const int ti = w >= a.first[1] ? 1 : 0;
+    const Task& t = a.t[ti];
+    const int bh = (w - a.first[ti]) / a.tiles[ti], tile = (w - a.first[ti]) % a.tiles[ti];
+    rows = t.L - tile * TILE;
+    sl = t.ax.sl;
+    return reinterpret_cast<const T*>(t.X) + (bh / a.H) * t.ax.sb + (bh % a.H) * t.ax.sh + (int64_t)tile * TILE * sl;
+  };
+  int rows = 0;
+  int64_t sl = 0;
+  const T* X = nullptr;
+  if (w0 < w1) {
+    X = tokens(w0, rows, sl);
+    st.load(X, sl, rows, tid, 0);
+  }
+  for (int w = w0; w < w1; w++) {
+    const int ti = w >= a.first[1] ? 1 : 0;
+    const Task& t = a.t[ti];
+    const int bh = (w - a.first[ti]) / a.tiles[ti], tile = (w - a.first[ti]) % a.tiles[ti];
+    const int g = group_of(bh, a.H, a.pool), key = ti * 65536 + g;
+    if (key != have) {
+      have = key;
+      const float* pp = a.prep + ((size_t)g * 2 + (t.side - 1)) * pr.total();
+      scalar = pp[pr.scal() + PS_CSCALAR] != 0.f;
+      gamma = pp[pr.scal() + PS_CGAMMA];
+      if (!scalar) {
+        // row j of the operand: column j of C, its index i contiguous (the same matrix in the quadratic form: row j of C)
+        const float* Cm = pp + pr.Cmat();
+        for (int e = tid; e < D * G::NKS * G::CH; e += RT_THREADS) {
+          const int j = e / (G::NKS * G::CH), c = e % (G::NKS * G::CH), s = c / 8, cc = c % 8;
+          put8(sC + s * (3 * D * 128) + j * 128 + ((cc ^ (j & 7)) << 4), D * 128, Cm + j * D + 8 * c, true);
+        }
+      }
+    }
+    const int64_t out0 = (int64_t)bh * t.L + (int64_t)tile * TILE;
+    const int row = tid & 127, half = tid >> 7;
+    const int valid = rows;
+    st.finish(sA, X, sl, rows, tid);
+    if (w + 1 < w1) {                             // the next tile's loads fly under this tile's product
+      X = tokens(w + 1, rows, sl);
+      st.load(X, sl, rows, tid, 0);
+    }
+    if (!scalar) {
+      fence_proxy_async_smem();
+      __syncthreads();
+      if (warp == 0) {
+        tcgen05_fence_after();
+        if (lane == 0) {
+          issue_products<T, D>(tmem, sA, sC, D);
+          mma_commit(&misc->done);
+        }
+        __syncwarp();
+      }
+      mbar_wait(&misc->done, phase & 1, &misc->abort_flag, a.status, false);
+      phase++;
+      __syncwarp();
+      tcgen05_fence_after();
+    } else {
+      __syncthreads();
+    }
+    // x from its parts (the row's pieces are conflict-free to read), half of the columns per warpgroup
+    float sum = 0.f;
+    const uint32_t lanes = tmem + ((uint32_t)(row & ~31) << 16);
+#pragma unroll
+    for (int c = 0; c < D / 16; c++) {
+      const int c8 = half * (D / 16) + c, s = c8 / 8, cc = c8 % 8;            // eight columns
+      const uint8_t* src = sA + s * (G::AP * TILE_BYTES) + row * 128 + ((cc ^ (row & 7)) << 4);
+      float x[8];
+#pragma unroll
+      for (int p = 0; p < G::AP; p++) {
+        const uint4 q = *reinterpret_cast<const uint4*>(src + p * TILE_BYTES);
+        const uint32_t u[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+          const float lo = __uint_as_float(u[j] << 16), hi = __uint_as_float(u[j] & 0xffff0000u);
+          x[2 * j] = p ? x[2 * j] + lo : lo;
+          x[2 * j + 1] = p ? x[2 * j + 1] + hi : hi;
+        }
+      }
+      if (scalar) {
+#pragma unroll
+        for (int j = 0; j < 8; j++) sum = fmaf(x[j], x[j], sum);
+      } else {
+        uint32_t tv[8];
+        tmem_ld8(lanes + c8 * 8, tv);
+        tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 8; j++) sum = fmaf(__uint_as_float(tv[j]), x[j], sum);
+      }
+    }
+    if (!scalar) tcgen05_fence_before();
+    misc->part[half][row] = sum;
+    __syncthreads();
+    if (half == 0 && row < valid) {
+      const float sum2 = misc->part[0][row] + misc->part[1][row];
+      const float c = a.qk_scale * a.qk_scale * (scalar ? gamma * sum2 : sum2);
+      bad |= !isfinite(c);                        // so is x then (or C): one test per token instead of one per exponent
+      t.rowc[out0 + row] = FS_LOG2E * c;
+      if (t.stab == FSHARP_STAB_ROW && a.nmb > 1) t.logscale[out0 + row] = __int_as_float(0xff800000);
+    }
+    if (tile == 0 && tid == 0 && t.gmax) t.gmax[bh] = 0u;
+    // (the next tile's staging overwrites sA: its readers are behind the barrier above)
+  }
+  if (bad) atomicExch(a.status, FSHARP_E_NONFINITE);
+  tcgen05_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tcgen05_fence_after();
+    tmem_dealloc(tmem, COLS);
+  }
+}
+
+// ---- the exponents' maxima (WRITE = false), the features (WRITE = true) -------------------------
+// Persistent blocks, one per SM; a block owns a range of (task, (batch, head), feature block, token tile) and fetches the
+// parts of W = Omega B when the group changes.  Everything is in powers of two (W, a, c and the bias carry log2e), so a
+// feature is one ex2 of one addition: the per-feature term a_m rides on the products as one more K step (its three parts
+// against ones).  Warps 8-11 stage token tiles, warp 12 issues the products, the two warpgroups of warps 0-7 take one
+// accumulator each and work on alternate tiles: thread = token, all columns of a row in one thread, so the row's maximum
+// needs no exchange.  A thread stores its row in whole 32-byte sectors.  Bound of the writing pass: HBM (128 KB per tile of
+// 128 x 256: 5.8 k cycles of this SM's share, against 3.4 k cycles of products).  Tried: a_m from shared memory (a broadcast
+// 16-byte load costs four wavefronts) with a transposing buffer in front of the stores (16 k cycles per tile); TMA store
+// tiles staged in shared memory (11 k; each of them waits for its proxy fence).
+constexpr int FT_STAGE0 = 8, FT_MMA = 12, FT_THREADS = 416;
+struct FtMisc {
+  uint64_t a_full[2], a_free[2], t_full[2], t_free[2], w_full;
+  uint32_t tmem_base;
+  int abort_flag;
+};
+template <typename T, int D> struct FtGeo : Geo<T, D> {
+  static constexpr int MB = WGeo<D>::MB;
+  static constexpr int NBUF = (D == 128 && sizeof(T) == 4) ? 1 : 2;    // token tiles in shared memory
+  static constexpr uint32_t W_BYTES = Geo<T, D>::NKS * 3 * MB * 128;
+  static constexpr uint32_t OFF_A = W_BYTES, OFF_ONE = OFF_A + NBUF * Geo<T, D>::A_BYTES, OFF_ROW = OFF_ONE + TILE * 32, OFF_MISC = OFF_ROW + MB * 32;
+  static constexpr size_t SMEM = 1024 + OFF_MISC + sizeof(FtMisc);
+  static_assert(SMEM <= 232448, "shared memory budget");
+};
+
+template <typename T, int D, bool WRITE>
+__global__ void __launch_bounds__(FT_THREADS, 1)
+feat3_kernel(const __grid_constant__ Args a) {
+  using G = FtGeo<T, D>;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* sW = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint8_t* sA = sW + G::OFF_A;
+  uint8_t* sOne = sW + G::OFF_ONE;
+  uint8_t* sRow = sW + G::OFF_ROW;
+  FtMisc* misc = reinterpret_cast<FtMisc*>(sW + G::OFF_MISC);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) {
+    for (int i = 0; i < 2; i++) {
+      mbar_init(&misc->a_full[i], 4);
+      mbar_init(&misc->a_free[i], 1);
+      mbar_init(&misc->t_full[i], 1);
+      mbar_init(&misc->t_free[i], 4);
+    }
+    mbar_init(&misc->w_full, 1);
+    misc->abort_flag = 0;
+    fence_barrier_init();
+  }
+  if (warp == FT_MMA) {
+    tmem_alloc(&misc->tmem_base, 512);
+    tmem_relinquish();
+  }
+  for (int e = tid; e < (TILE + G::MB) * 8; e += FT_THREADS) reinterpret_cast<uint32_t*>(sOne)[e] = 0u;
+  __syncthreads();
+  if (tid < TILE) {                                                // [1, 1, 1, 0, ...]
+    *reinterpret_cast<uint2*>(sOne + core16_offset(tid, 0)) = make_uint2(0x3f803f80u, 0x00003f80u);
+  }
+  tcgen05_fence_before();
+  __syncthreads();
+  tcgen05_fence_after();
+  const uint32_t tmem = misc->tmem_base;
+  PrepLayout pr{D, a.M};
+  const int total = a.first[2];
+  const int w1 = (int)((int64_t)total * (blockIdx.x + 1) / gridDim.x);
+  int w = (int)((int64_t)total * blockIdx.x / gridDim.x);
+  int n = 0, runs = 0;                                             // tiles and runs done by this block (every role counts alike)
+  bool bad = false;
+  while (w < w1) {
+    // a run: consecutive tiles of one (task, (batch, head), feature block)
+    const int ti = w >= a.first[1] ? 1 : 0;
+    const Task& t = a.t[ti];
+    const int u = (w - a.first[ti]) / a.tiles[ti], tile0 = (w - a.first[ti]) % a.tiles[ti];
+    const int bh = u / a.nmb, mblk = u % a.nmb, m0 = mblk * G::MB, mb = min(G::MB, a.M - m0);
+    const int ntiles = min(a.tiles[ti] - tile0, w1 - w);
+    w += ntiles;
+    const int g = group_of(bh, a.H, a.pool);
+    const float* pp = a.prep + ((size_t)g * 2 + (t.side - 1)) * pr.total();
+    const float bias = FS_LOG2E * pp[pr.scal() + PS_BIAS];
+    __syncthreads();                                               // the previous run's products have been read
+    if (a.img[ti] != nullptr) {
+      if (tid == 0) {
+        const uint32_t bytes = (uint32_t)mb * (G::NKS * 3 * 128);
+        mbar_expect_tx(&misc->w_full, bytes);
+        bulk_load(sW, a.img[ti] + ((size_t)g * a.M + m0) * (G::NKS * 3 * 128), bytes, &misc->w_full);
+      }
+    } else {
+      const float* W = pp + pr.W() + (size_t)m0 * D;
+      for (int e = tid; e < mb * (D / 8); e += FT_THREADS)
+        put_w<D>(sW, mb, e / (D / 8), e % (D / 8), W + (size_t)e * 8, FS_LOG2E * a.qk_scale, bad);
+    }
+    for (int e = tid; e < mb; e += FT_THREADS) {
+      const float v = FS_LOG2E * pp[pr.a() + m0 + e];
+      bad |= !isfinite(v);
+      uint32_t h, m, l;
+      split3::split_pair(v, 0.f, h, m, l);
+      *reinterpret_cast<uint2*>(sRow + core16_offset(e, 0)) = make_uint2((h & 0xffffu) | (m << 16), l & 0xffffu);
+    }
+    bad |= !isfinite(bias);
+    fence_proxy_async_smem();
+    __syncthreads();
+    if (warp >= FT_STAGE0 && warp < FT_MMA) {
+      const T* X = reinterpret_cast<const T*>(t.X) + (bh / a.H) * t.ax.sb + (bh % a.H) * t.ax.sh;
+      const int i = tid - FT_STAGE0 * 32;
+      Stage<T, D, 128> st;
+      st.load(X + (int64_t)tile0 * TILE * t.ax.sl, t.ax.sl, t.L - tile0 * TILE, i, 0);
+      for (int it = 0; it < ntiles; it++, n++) {
+        const int b = n % G::NBUF, tok = (tile0 + it) * TILE;
+        mbar_wait(&misc->a_free[b], ((n / G::NBUF) & 1) ^ 1, &misc->abort_flag, a.status);
+        st.finish(sA + b * G::A_BYTES, X + (int64_t)tok * t.ax.sl, t.ax.sl, t.L - tok, i);
+        fence_proxy_async_smem();
+        mbar_arrive_warp(&misc->a_full[b], lane);
+        if (it + 1 < ntiles) st.load(X + (int64_t)(tok + TILE) * t.ax.sl, t.ax.sl, t.L - tok - TILE, i, 0);
+      }
+    } else if (warp == FT_MMA) {
+      if (a.img[ti] != nullptr) mbar_wait(&misc->w_full, runs & 1, &misc->abort_flag, a.status, false);
+      for (int it = 0; it < ntiles; it++, n++) {
+        const int b = n & 1, ab = n % G::NBUF;
+        mbar_wait(&misc->a_full[ab], (n / G::NBUF) & 1, &misc->abort_flag, a.status);
+        mbar_wait(&misc->t_free[b], ((n >> 1) & 1) ^ 1, &misc->abort_flag, a.status);
+        __syncwarp();
+        tcgen05_fence_after();
+        if (elect_one()) {
+          issue_products<T, D>(tmem + b * 256, sA + ab * G::A_BYTES, sW, mb, sOne, sRow);
+          mma_commit(&misc->t_full[b]);
+          mma_commit(&misc->a_free[ab]);
+        }
+        __syncwarp();
+      }
+    } else {
+      const int wg = warp >> 2;
+      float gmx = -3.0e38f;
+      const float gshift = (WRITE && t.stab == FSHARP_STAB_GROUP) ? ord2f(t.gmax[bh]) : 0.f;
+      const bool own = t.stab == FSHARP_STAB_ROW && a.nmb == 1;
+      const bool wide = WRITE && (reinterpret_cast<uintptr_t>(t.phi) & 31) == 0;
+      constexpr float LN2 = 0.693147180559945f;
+      if (WRITE && t.stab == FSHARP_STAB_GROUP && t.logscale && tile0 == 0 && mblk == 0 && tid == 0) t.logscale[bh] = LN2 * gshift;
+      const uint32_t acc = tmem + wg * 256 + ((uint32_t)((warp & 3) * 32) << 16);
+      for (int it = 0; it < ntiles; it++, n++) {
+        if ((n & 1) != wg) continue;
+        const int tok0 = (tile0 + it) * TILE + (warp & 3) * 32, tok = tok0 + lane;
+        const int64_t at = (int64_t)bh * t.L + tok;
+        const bool in = tok < t.L;
+        const float ci = (in ? t.rowc[at] : 0.f) + bias;
+        float shift = gshift;                          // in powers of two, subtracted from acc + ci
+        if (WRITE && t.stab == FSHARP_STAB_ROW && !own) shift = in ? FS_LOG2E * t.logscale[at] : 0.f;
+        float off = ci - shift;
+        mbar_wait(&misc->t_full[wg], (n >> 1) & 1, &misc->abort_flag, a.status);
+        __syncwarp();
+        tcgen05_fence_after();
+        // The next columns' loads from tensor memory are in flight under the current ones' arithmetic: a warpgroup has one
+        // warp per scheduler, so the latencies are its own to hide.  The last piece may reach past mb: columns of the other
+        // accumulator, whose values are not used.
+        uint32_t v[32];
+        auto fetch = [&](int c) {
+          tmem_ld16(acc + c, *reinterpret_cast<uint32_t(*)[16]>(v));
+          tmem_ld16(acc + min(c + 16, 240), *reinterpret_cast<uint32_t(*)[16]>(v + 16));
+        };
+        auto arrived = [&](uint32_t (&x)[32]) {
+          tmem_wait_ld();
+          pin16(v); pin16(v + 16);
+#pragma unroll
+          for (int j = 0; j < 32; j++) x[j] = v[j];
+        };
+        fetch(0);
+        if (!WRITE || own) {
+          float mx = -3.0e38f, my = -3.0e38f;
+          for (int c = 0; c < mb; c += 32) {
+            uint32_t x[32];
+            arrived(x);
+            fetch(c + 32 < mb ? c + 32 : 0);           // (the features start again at column 0)
+#pragma unroll
+            for (int j = 0; j < 16; j += 4) {
+              mx = max3(mx, __uint_as_float(x[j]), __uint_as_float(x[j + 1]));
+              my = max3(my, __uint_as_float(x[j + 2]), __uint_as_float(x[j + 3]));
+            }
+            if (c + 16 < mb) {
+#pragma unroll
+              for (int j = 16; j < 32; j += 4) {
+                mx = max3(mx, __uint_as_float(x[j]), __uint_as_float(x[j + 1]));
+                my = max3(my, __uint_as_float(x[j + 2]), __uint_as_float(x[j + 3]));
+              }
+            }
+          }
+          mx = fmaxf(mx, my);
+          if (WRITE) {
+            off = -mx;
+            if (t.logscale && in) t.logscale[at] = LN2 * (mx + ci);
+          } else if (t.stab == FSHARP_STAB_GROUP) {
+            if (in) gmx = fmaxf(gmx, mx + ci);
+          } else {
+            // (nudged upwards by the rounding of the two conversions, so that no feature exceeds one)
+            const float ls = LN2 * (mx + ci);
+            if (in) atomic_max_float(t.logscale + at, fmaf(fabsf(ls), 2.4e-7f, ls));
+          }
+        }
+        if (WRITE) {
+          float* out = t.phi + at * a.M + m0;
+          for (int c = 0; c < mb; c += 32) {
+            uint32_t x[32];
+            arrived(x);
+            if (c + 32 < mb) fetch(c + 32);
+#pragma unroll
+            for (int j = 0; j < 32; j++) x[j] = __float_as_uint(ex2(__uint_as_float(x[j]) + off));
+            if (in) {
+              float* dst = out + c;
+              if (wide) {
+#pragma unroll
+                for (int j = 0; j < 4; j++)
+                  if (j < 2 || c + 16 < mb) store32(dst + 8 * j, &x[8 * j]);
+              } else {
+#pragma unroll
+                for (int j = 0; j < 32; j++)
+                  if (j < 16 || c + 16 < mb) dst[j] = __uint_as_float(x[j]);
+              }
+            }
+          }
+        } else {
+          tmem_wait_ld();                              // the wrapped-around fetch
+        }
+        tcgen05_fence_before();
+        mbar_arrive_warp(&misc->t_free[wg], lane);
+      }
+      if (!WRITE && t.stab == FSHARP_STAB_GROUP) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) gmx = fmaxf(gmx, __shfl_xor_sync(0xffffffffu, gmx, o));
+        if (lane == 0) atomicMax(t.gmax + bh, f2ord(gmx));
+      }
+    }
+    runs++;
+  }
+  if (bad) atomicExch(a.status, FSHARP_E_NONFINITE);
+  tcgen05_fence_before();
+  __syncthreads();
+  if (warp == FT_MMA) {
+    tcgen05_fence_after();
+    tmem_dealloc(tmem, 512);
+  }
+}
+
+template <typename T, int D>
+int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, int G_groups, uint8_t* img) {
+  using G = FtGeo<T, D>;
+  a.nmb = (a.M + G::MB - 1) / G::MB;
+  const uint8_t* side_img[2] = {nullptr, nullptr};     // by side - 1
+  // (a set with a row shift over several feature blocks has its maxima pass instead: its blocks convert W themselves)
+  if (img != nullptr && !(ntasks == 1 && tasks[0].stab == FSHARP_STAB_ROW && a.nmb > 1)) {
+    const int side0 = ntasks == 2 ? 1 : tasks[0].side;
+    const size_t per_side = (size_t)G_groups * G::NKS * 3 * a.M * 128;
+    for (int k = 0; k < ntasks; k++) side_img[side0 - 1 + k] = img + k * per_side;
+    const dim3 grid((a.M * (D / 8) + 255) / 256, G_groups, ntasks);
+    FS_TIME_BEGIN(ctx, FS_K_W3);
+    w3_images_kernel<D><<<grid, 256, 0, ctx->stream>>>(a.prep, side0, ntasks, a.M, a.qk_scale, img, ctx->d_status);
+    FS_TIME_END(ctx);
+    FS_LAUNCH_CHECK(ctx);
+  }
+  const auto set = [&](int units_per_bh, bool (*take)(const Task&, int)) {
+    int k = 0;
+    a.first[0] = 0;
+    for (int i = 0; i < ntasks; i++) {
+      if (!take(tasks[i], a.nmb)) continue;
+      a.t[k] = tasks[i];
+      a.img[k] = side_img[tasks[i].side - 1];
+      a.tiles[k] = (tasks[i].L + TILE - 1) / TILE;
+      a.first[k + 1] = a.first[k] + BH * units_per_bh * a.tiles[k];
+      k++;
+    }
+    for (; k < 2; k++) a.first[k + 1] = a.first[k];
+    return a.first[2];
+  };
+  {
+    const int total = set(1, [](const Task&, int) { return true; });
+    constexpr size_t smem = rt_smem<T, D>();
+    FS_CUDA_OK(cudaFuncSetAttribute(rowterm3_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int most = (D == 128 ? 1 : 3) * ctx->sm_count;
+    FS_TIME_BEGIN(ctx, FS_K_ROWTERM);
+    rowterm3_kernel<T, D><<<total < most ? total : most, RT_THREADS, smem, ctx->stream>>>(a);
+    FS_TIME_END(ctx);
+    FS_LAUNCH_CHECK(ctx);
+  }
+  const int maxed = set(a.nmb, [](const Task& t, int nmb) { return t.stab == FSHARP_STAB_GROUP || (t.stab == FSHARP_STAB_ROW && nmb > 1); });
+  if (maxed > 0) {
+    FS_CUDA_OK(cudaFuncSetAttribute(feat3_kernel<T, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM));
+    FS_TIME_BEGIN(ctx, FS_K_GROUPMAX);
+    feat3_kernel<T, D, false><<<maxed < ctx->sm_count ? maxed : ctx->sm_count, FT_THREADS, G::SMEM, ctx->stream>>>(a);
+    FS_TIME_END(ctx);
+    FS_LAUNCH_CHECK(ctx);
+  }
+  const int total = set(a.nmb, [](const Task&, int) { return true; });
+  FS_CUDA_OK(cudaFuncSetAttribute(feat3_kernel<T, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM));
+  FS_TIME_BEGIN(ctx, FS_K_FEAT);
+  feat3_kernel<T, D, true><<<total < ctx->sm_count ? total : ctx->sm_count, FT_THREADS, G::SMEM, ctx->stream>>>(a);
+  FS_TIME_END(ctx);
+  FS_LAUNCH_CHECK(ctx);
+  return FSHARP_OK;
+}
+
+// Two token sets share their launches only while both together leave SMs without a tile: beyond that a launch of its own
+// costs a set nothing, and its blocks keep one W each for longer.
+template <typename T, int D>
+int run_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, int groups, uint8_t* img) {
+  int64_t items = 0;
+  for (int i = 0; i < ntasks; i++) items += (int64_t)BH * ((tasks[i].L + TILE - 1) / TILE) * ((a.M + WGeo<D>::MB - 1) / WGeo<D>::MB);
+  if (items > 2147483647LL) return FSHARP_E_SHAPE;     // items are numbered in 32 bits
+  if (ntasks == 1 || items <= ctx->sm_count) return launch_t<T, D>(ctx, a, tasks, ntasks, BH, groups, img);
+  for (int i = 0; i < ntasks; i++) {
+    FS_TRY((launch_t<T, D>(ctx, a, tasks + i, 1, BH, groups, img)));
+  }
+  return FSHARP_OK;
+}
+
+}  // namespace
+
+size_t feat3::image_bytes(int groups, int d, int M, int ntasks) {
+  return ws_round((size_t)ntasks * groups * ((d + 63) / 64) * 3 * M * 128);
+}
+
+int feat3::run(fsharp_ctx* ctx, const Task* tasks, int ntasks, int dtype, int B, int H, int d, int M, int pool, const float* prep,
+               float qk_scale, uint8_t* img) {
+  Args a{};
+  a.H = H; a.M = M; a.pool = pool; a.prep = prep; a.qk_scale = qk_scale; a.status = ctx->d_status;
+  const int groups = pool == FSHARP_POOL_PER_BH ? B * H : H;
+#define FS_FEAT3(DD)                                                                                          \
+  return dtype == FSHARP_F32 ? run_t<float, DD>(ctx, a, tasks, ntasks, B * H, groups, img)                    \
+                             : run_t<__nv_bfloat16, DD>(ctx, a, tasks, ntasks, B * H, groups, img)
+  switch (d) {
+    case 16: FS_FEAT3(16);
+    case 32: FS_FEAT3(32);
+    case 64: FS_FEAT3(64);
+    case 128: FS_FEAT3(128);
+    default: return FSHARP_E_SHAPE;
+  }
+#undef FS_FEAT3
+}

@@ -107,10 +107,9 @@ extern "C" int fsharp_featurize_static(void* stream, const void* X, const float*
   float* prep = ws.take<float>(prep_f);
   float* rowc = ws.take<float>(BH * L);
   unsigned* gmax = ws.take<unsigned>(BH);
-  // everything in the scratch is written before it is read in this call (the maximum words are
-  // cleared by the feature kernels' own memset), so what an earlier call left behind is harmless
+  // everything in the scratch is written before it is read in this call, so what an earlier call left behind is harmless
   FS_TRY(fs_run_prep(&ctx, Omega, dims->omega_head_stride, params, (int64_t)ParamsLayout{d}.total(), G, dims->H,
                      dims->pool, d, M, prep));
   return fs_simt_featurize(&ctx, X, dtype, fs_addr(st, dims->H, L, d), dims->B, dims->H, L, d, M, dims->pool, prep,
-                           side, qk_scale, stab, rowc, gmax, phi, logscale);
+                           side, qk_scale, stab, rowc, gmax, phi, logscale, nullptr);
 }

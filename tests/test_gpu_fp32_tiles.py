@@ -1,0 +1,93 @@
+"""The fp32-precision kernels (features, attention, kernel operator, backward pass) at the edges of their tiles: 128 tokens,
+feature blocks of 256 (d = 128: 128) in the feature kernels and of 128 in the products, 64 value columns, chunks of 128
+tokens whatever the caller's chunk is; against the checker."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import favor_sharp as fs
+from tests.gpu_util import TOL, dev, gpu_fit, host, oracle_unit, rel_err
+from paper_2302_00787_b200 import binding as fb
+from paper_2302_00787_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+# (d, dv, M, Lq, Lk, causal, chunk, dtype)
+CASES = [
+    (16, 16, 16, 1, 300, False, 0, "f32"),          # one query, fewest features
+    (32, 128, 48, 127, 129, False, 0, "f32"),       # two tiles of value columns
+    (64, 32, 272, 129, 257, False, 0, "bf16"),      # a second feature block of 16
+    (64, 64, 1024, 130, 700, False, 0, "f32"),      # most features: row maxima over four blocks
+    (128, 16, 144, 260, 140, False, 0, "f32"),      # d = 128: feature blocks of 128
+    (16, 64, 208, 64, 64, True, 64, "f32"),         # half a tile
+    (32, 32, 128, 192, 192, True, 64, "bf16"),      # the last inner chunk is half full
+    (64, 128, 80, 384, 384, True, 128, "f32"),
+    (128, 64, 384, 512, 512, True, 256, "bf16"),    # two tiles per chunk
+]
+
+
+def inputs(d, dv, M, Lq, Lk, dtype, seed):
+    w = wl.Workload("tiles", 1, 2, Lq, d, dv, M, dtype, "saderf", False, 0, "orthogonal", seed=seed)
+    Q, _, V1 = wl.make_qkv(w)
+    K, _, V = wl.make_qkv(w.scaled(L=Lk, seed=seed + 1))
+    return Q, K, V, V1, wl.make_omega(w)
+
+
+@pytest.mark.parametrize("d,dv,M,Lq,Lk,causal,chunk,dtype", CASES)
+def test_attention_and_gradients_at_tile_edges(d, dv, M, Lq, Lk, causal, chunk, dtype):
+    ctx = fb.Context(0)
+    Q, K, V, dY, Om = inputs(d, dv, M, Lq, Lk, dtype, 77)
+    dQ, dK, dV, ddY, dOm = dev(Q, dtype), dev(K, dtype), dev(V, dtype), dev(dY, dtype), dev(Om)
+    _, pr = gpu_fit(ctx, dQ, dK, d, "saderf")
+    ctx.set_impl(fb.IMPL_SIMT)
+    at = dict(causal=causal, chunk=chunk)
+    Y = host(ctx.fsharp_attend(dQ, dK, dV, dOm, pr, **at))
+    g = [host(t) for t in ctx.fsharp_attend_backward(dQ, dK, dV, ddY, dOm, pr, **at)]
+    assert ctx.status() == 0
+    prh = pr.cpu().numpy()
+    for h in range(2):
+        assert rel_err(Y[0, h], oracle_unit(Q, K, V, Om, prh[h], d, 0, h, causal)) < TOL[dtype]
+        ref = fs.favor_sharp_attention_vjp(Q[0, h], K[0, h], V[0, h], dY[0, h], Om, fb.unpack_params(prh[h], d), causal=causal)
+        for got, r in zip(g, ref):
+            assert rel_err(got[0, h], r) < TOL[dtype]
+
+
+@pytest.mark.parametrize("d,M,L,dtype", [(16, 16, 1, "f32"), (32, 272, 129, "f32"), (64, 1024, 130, "bf16"), (128, 144, 257, "f32"),
+                                         (128, 1024, 128, "bf16")])
+@pytest.mark.parametrize("stab", [fb.STAB_NONE, fb.STAB_ROW, fb.STAB_GROUP])
+def test_features_at_block_edges(d, M, L, dtype, stab):
+    ctx = fb.Context(0)
+    Q, K, _, _, Om = inputs(d, 16, M, L, max(L, 4 * d), dtype, 5)
+    dQ, dK, dOm = dev(Q, dtype), dev(K, dtype), dev(Om)
+    _, pr = gpu_fit(ctx, dQ if L > 1 else dK, dK, d, "saderf")
+    ctx.set_impl(fb.IMPL_SIMT)
+    phi, ls = ctx.fsharp_featurize(dQ, dOm, pr, 1, stab=stab)
+    assert ctx.status() == 0
+    for h in range(2):
+        p = fb.unpack_params(pr[h], d)
+        e = fs.derf_log_features(Q[0, h], Om, p["A"], p["B1"], p["C1"], p["logD"])
+        shift = {fb.STAB_NONE: 0.0, fb.STAB_ROW: lambda: host(ls)[0, h][:, None], fb.STAB_GROUP: lambda: host(ls)[0, h]}[stab]
+        shift = shift() if callable(shift) else shift
+        expect, got = np.exp(e - shift), host(phi)[0, h]
+        big = expect > 1e-30
+        # an exponent is a sum of d products in fp32: 2^-24 of its largest terms times sqrt(d)
+        tol = 2.0 ** -24 * np.abs(e).max() * np.sqrt(d) + 1e-6
+        assert np.max(np.abs(got[big] / expect[big] - 1)) < tol
+        if stab != fb.STAB_NONE:
+            assert got.max() <= 1.0 + 1e-6
+
+
+def test_unaligned_feature_output_of_the_static_entry_point():
+    """phi of fsharp_featurize_static may start on any 4-byte boundary: the result equals the aligned one's."""
+    ctx = fb.Context(0)
+    Q, K, _, _, Om = inputs(32, 16, 80, 150, 150, "f32", 9)
+    dQ, dK, dOm = dev(Q), dev(K), dev(Om)
+    _, pr = gpu_fit(ctx, dQ, dK, 32, "saderf")
+    out = []
+    for off in (0, 1):
+        phi = torch.empty(1 * 2 * 150 * 80 + off, device="cuda")[off:].view(1, 2, 150, 80)
+        ls = torch.empty(1, 2, 150, device="cuda")
+        assert fb.fsharp_featurize_static(dQ, dOm, pr, 1, phi, ls) == 0
+        out.append(phi)
+    torch.cuda.synchronize()
+    assert torch.equal(out[0], out[1])

@@ -5,7 +5,7 @@ import pytest
 import torch
 
 from oracle import favor_sharp as fs
-from gpu_util import dev, host
+from tests.gpu_util import dev, host
 from paper_2302_00787_b200 import binding as fb
 from paper_2302_00787_b200 import workloads as wl
 
