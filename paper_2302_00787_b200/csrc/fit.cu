@@ -4,7 +4,8 @@
 // a cyclic Jacobi solver then confirms convergence (or completes it).  d = 128: the Jacobi solver alone.
 // ADERF factors M1 by Cholesky (M1 = L L^T) and solves ONE eigenproblem, of L^T M2 L (Theorem 4.2's U and Sigma^2
 // for the factor L^T of M1).
-#include "common.cuh"
+#include "fit_common.cuh"
+#include "fit_wide.cuh"
 
 namespace {
 
@@ -26,13 +27,6 @@ __device__ __forceinline__ double block_reduce(double v, double* red, int op /*0
   double r = red[0];
   __syncthreads();
   return r;
-}
-
-// Lemma A.1 in the cancellation-free form that follows from its proof:
-// 1 - 8A = (2 phi + 1 + s)/2 with s = sqrt((2 phi + 1)^2 + 8 phi).
-__device__ __forceinline__ double lemma_a1(double phi) {
-  double s = sqrt((2.0 * phi + 1.0) * (2.0 * phi + 1.0) + 8.0 * phi);
-  return -(2.0 * phi + (12.0 * phi + 4.0 * phi * phi) / (1.0 + s)) / 16.0;
 }
 
 // Two-sided cyclic Jacobi with the round-robin ("tournament") ordering: every round rotates
@@ -399,21 +393,6 @@ __device__ void jacobi_tables(const ushort2* sched, uchar2* pos, uint2* la, ucha
                        (unsigned)px.x | ((unsigned)py.x << 8) | ((unsigned)px.y << 16) | ((unsigned)py.y << 17));
   }
   __syncthreads();
-}
-
-// 1 / sqrt(t) and 1 / t to rounding: the 20-bit hardware estimate and two Newton steps (t normal and positive,
-// resp. non-zero; no special cases).
-__device__ __forceinline__ double rsqrt_fast(double t) {
-  double q;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(q) : "d"(t));
-  q = fma(q * 0.5, fma(-t * q, q, 1.0), q);
-  return fma(q * 0.5, fma(-t * q, q, 1.0), q);
-}
-__device__ __forceinline__ double recip_fast(double t) {
-  double q;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(q) : "d"(t));
-  q = fma(q, fma(-t, q, 1.0), q);
-  return fma(q, fma(-t, q, 1.0), q);
 }
 
 // Row handled by lane group `grp` when `parts` lanes share a row: with eight lanes per row the two rows of a
@@ -911,6 +890,8 @@ struct FitArgs {
   double ridge;
   int v_in_smem;
   int* status;
+  const double* flags;      // not null: only groups whose flag (one per `flag_stride` doubles) is set are fitted
+  size_t flag_stride;
 };
 
 template <bool V_IN_SMEM>
@@ -918,6 +899,7 @@ __global__ void __launch_bounds__(FIT_THREADS) fit_kernel(FitArgs a) {
   fs_grid_dependency_wait();
   extern __shared__ __align__(16) double sm[];
   const int d = a.d, tid = threadIdx.x, g = blockIdx.x;
+  if (a.flags != nullptr && a.flags[(size_t)g * a.flag_stride] == 0.0) return;
   const int lda = d + 1;
   StatsLayout sl{d};
   ParamsLayout pl{d};
@@ -1351,7 +1333,7 @@ size_t fit_smem_bytes(int d, int v_in_smem) {
 
 }  // namespace
 
-size_t fs_fit_scratch_doubles(int G, int d) { return (size_t)G * 5 * d * d; }
+size_t fs_fit_scratch_doubles(int G, int d) { return (size_t)G * (5 * d * d + (d >= 64 ? fitw::Layout{d}.total() : 0)); }
 
 int fs_run_fit(fsharp_ctx* ctx, const double* stats, int G, int d, int variant, double ridge,
                double* params, double* scratch) {
@@ -1360,6 +1342,16 @@ int fs_run_fit(fsharp_ctx* ctx, const double* stats, int G, int d, int variant, 
   a.stats = stats; a.params = params; a.scratch = scratch; a.d = d; a.variant = variant; a.ridge = ridge;
   a.v_in_smem = d <= 64 ? 1 : 0;
   a.status = ctx->d_status;
+  a.flags = nullptr;
+  a.flag_stride = 0;
+  // eigenproblems of d = 64 and 128 go through the chain of fit_wide.cu; this kernel then only takes what that chain gave up
+  // (the smaller ones fit one block's latency better than six launches)
+  if (d >= 64 && (variant == FSHARP_ADERF || variant == FSHARP_SDERF)) {
+    double* wide = scratch + (size_t)G * 5 * d * d;
+    FS_TRY(fitw::run(ctx, stats, G, d, variant, ridge, params, wide));
+    a.flags = wide + fitw::Layout{d}.scal() + fitw::FS_FLAG;
+    a.flag_stride = fitw::Layout{d}.total();
+  }
   size_t smem = fit_smem_bytes(d, a.v_in_smem);
   if (a.v_in_smem) FS_CUDA_OK(cudaFuncSetAttribute(fit_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   else FS_CUDA_OK(cudaFuncSetAttribute(fit_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -1,0 +1,44 @@
+"""The chain of fit kernels for d = 64 and 128 (ADERF, SDERF) where groups of one launch take different ways: ordinary spectra
+through the chain, equal eigenvalues through the Jacobi solver behind it, more groups than SMs."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import favor_sharp as fs
+from paper_2302_00787_b200 import binding as fb
+from tests.test_gpu_parity import assert_fit_close
+
+pytestmark = pytest.mark.gpu
+
+
+def matrices(d, kind, rng):
+    Qm, _ = np.linalg.qr(rng.standard_normal((d, d)))
+    lam = {"plain": rng.uniform(0.1, 0.9, d), "equal": np.full(d, 0.3), "clusters": np.repeat(np.linspace(0.1, 0.5, 8), d // 8),
+           "wide": np.geomspace(1e-2, 1e2, d)}[kind]
+    M1 = (Qm * lam) @ Qm.T
+    return 0.5 * (M1 + M1.T)
+
+
+@pytest.mark.parametrize("variant", ["sderf", "aderf"])
+@pytest.mark.parametrize("d,copies", [(64, 1), (64, 60), (128, 1)])
+def test_mixed_groups(variant, d, copies):
+    rng = np.random.default_rng(d + copies)
+    kinds = ["plain", "equal", "clusters", "wide"]
+    blobs, refs = [], []
+    for kind in kinds:
+        M1 = matrices(d, kind, rng)
+        M2 = 0.5 * M1 + 0.1 * np.eye(d)
+        mu4, mu5 = 0.01 * rng.standard_normal((2, d)) if kind == "plain" else np.zeros((2, d))
+        refs.append(fs.FITS[variant]({"M1": M1, "M2": M2, "mu4": mu4, "mu5": mu5, "mu3": float(mu4 @ mu5) / d, "d": d}))
+        blobs.append(np.concatenate([M1.ravel(), M2.ravel(), mu4, mu5]))
+    ctx = fb.Context(0)
+    pr = ctx.fsharp_fit_params(torch.from_numpy(np.stack(blobs * copies)).cuda(), d, variant)
+    assert ctx.status() == 0
+    # copies of one matrix get the same bits wherever they run
+    first = pr[:len(kinds)]
+    assert torch.equal(pr.view(copies, len(kinds), -1), first.expand(copies, -1, -1))
+    for g, ref in enumerate(refs):
+        # "wide": either side's eigenvalues of Z are exact to 2^-53 |Z| d, that is 2^-53 d cond(Z) of the smallest, which carries
+        # the largest entries of B1^T B1; Z has the eigenvalues lam (lam / 2 + 1/10), cond 5e6
+        assert_fit_close(fb.unpack_params(first[g], d), ref, d, max(1e-8, 2.0 ** -53 * d * 5e6) if kinds[g] == "wide" else 1e-8)
+    assert first[1, 5 * d * d + 3] >= 0 and first[0, 5 * d * d + 3] == 0      # sweeps: none for the ordinary matrix
