@@ -359,8 +359,8 @@ int backward_t(fsharp_ctx* ctx, const void* Qv, const void* Kv, const void* Vv, 
   const int64_t elems = (int64_t)M * NP;
   const dim3 gscan((unsigned)((elems + NTH - 1) / NTH), BH);
 
-  const feat3::Task tasks[2] = {{K, ak, Lk, 2, FSHARP_STAB_GROUP, rowck, gmax, phiK, lsk},
-                                {Q, aq, Lq, 1, FSHARP_STAB_ROW, rowcq, nullptr, phiQ, lsq}};
+  const feat3::Task tasks[2] = {{K, ak, Lk, 2, FSHARP_STAB_GROUP, rowck, gmax, phiK, nullptr, lsk},
+                                {Q, aq, Lq, 1, FSHARP_STAB_ROW, rowcq, nullptr, phiQ, nullptr, lsq}};
   FS_TRY(feat3::run(ctx, tasks, 2, dtype, B, H, d, M, dm->pool, prep, qk_scale, img));
   // sums over tokens: the total (bidirectional), or one per chunk turned into the sum over earlier / later chunks (causal)
   auto sums = [&](auto from_g, const float* F, int L, float* out, int reverse) -> int {

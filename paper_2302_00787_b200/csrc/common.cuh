@@ -48,9 +48,9 @@ enum { PS_BIAS = 0, PS_CSCALAR = 3, PS_CGAMMA = 4 };
 
 // Kernel ids for the optional per-kernel timing (fsharp_set_timing / fsharp_read_timing).
 enum {
-  FS_K_STATS = 1, FS_K_FIT, FS_K_PREP, FS_K_ROWTERM, FS_K_FEAT, FS_K_GROUPMAX, FS_K_EXPSHIFT, FS_K_KV,
+  FS_K_STATS = 1, FS_K_FIT, FS_K_PREP, FS_K_ROWTERM, FS_K_FEAT, FS_K_GROUPMAX, FS_K_KV,
   FS_K_PREFIX, FS_K_SCORES, FS_K_OUT, FS_K_PAIRS, FS_K_PAIRVAR_PREP, FS_K_PAIRVAR,
-  FS_K_TC_KV, FS_K_TC_OUT, FS_K_TC_CAUSAL, FS_K_TC_STATS, FS_K_TC_ROWTERM, FS_K_TC_FEAT, FS_K_TC_LOGITS128, FS_K_TC_SCORES128, FS_K_TC_KV128, FS_K_TC_OUT128,
+  FS_K_TC_KV, FS_K_TC_OUT, FS_K_TC_CAUSAL, FS_K_TC_STATS, FS_K_TC_ROWTERM, FS_K_TC_FEAT, FS_K_TC_SCORES128, FS_K_TC_KV128, FS_K_TC_OUT128,
   FS_K_PAIR_IMAGES, FS_K_W3, FS_K_BWD_STATE, FS_K_BWD_NUMDEN, FS_K_BWD_DFEAT, FS_K_BWD_DX, FS_K_BWD_DV,
   FS_K_COUNT
 };
@@ -219,13 +219,9 @@ int fs_run_prep_images(fsharp_ctx* ctx, const float* Omega, int64_t omega_head_s
 int fs_simt_featurize(fsharp_ctx* ctx, const void* X, int dtype, TensorAddr ax, int B, int H, int L, int d,
                       int M, int pool, const float* prep, int side, float qk_scale, int stab,
                       float* rowc, unsigned* gmax, float* phi, float* logscale, uint8_t* img);
-// Exponents of bf16 tokens with d = 128 on the tensor cores (tc_logits128.cu); phi [B*H][L][M] fp32, rowc [B*H][L].
-int fs_tc_logits128_supported(const void* X, int dtype, TensorAddr ax, int L, int d, int M);
-int fs_tc_logits128(fsharp_ctx* ctx, const void* X, TensorAddr ax, int B, int H, int L, int M, int pool, const float* prep,
-                    int side, float qk_scale, const float* rowc, float* phi);
-// Masked in-chunk scores from bf16 feature matrices [BH][L][M] on the tensor cores (tc_scores128.cu); sc [BH * L / C][C][C] fp32.
+// Masked in-chunk scores from bf16 feature matrices [BH][L][M] on the tensor cores (tc_scores128.cu); sc16 [BH * L / C][C][C] bf16.
 int fs_tc_scores128_supported(int M, int C);
-int fs_tc_scores128(fsharp_ctx* ctx, const void* phiQ16, const void* phiK16, int BH, int L, int M, int C, float* sc, void* sc16);
+int fs_tc_scores128(fsharp_ctx* ctx, const void* phiQ16, const void* phiK16, int BH, int L, int M, int C, void* sc16);
 // Per-chunk key-side sums from the bf16 copy of phi(K) on the tensor cores (tc_kv128.cu); st [BH * L / C][129][M] fp32.
 int fs_tc_kv128_supported(const void* V, TensorAddr av, int dv, int M, int C);
 int fs_tc_kv128(fsharp_ctx* ctx, const void* phiK16, const void* V, TensorAddr av, int B, int H, int L, int M, int C, float* st);

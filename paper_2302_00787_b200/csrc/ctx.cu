@@ -150,11 +150,10 @@ const char* fsharp_kernel_name(int id) {
     case FS_K_STATS: return "stats_kernel";
     case FS_K_FIT: return "fit_kernel";
     case FS_K_PREP: return "prep_kernel";
-    case FS_K_ROWTERM: return "rowterm_kernel";
+    case FS_K_ROWTERM: return "rowterm3_kernel";
     case FS_K_FEAT: return "feat3_kernel";
-    case FS_K_GROUPMAX: return "groupmax_kernel";
-    case FS_K_EXPSHIFT: return "expshift_kernel";
-    case FS_K_KV: return "kv_kernel";
+    case FS_K_GROUPMAX: return "feat3_max_kernel";
+    case FS_K_KV: return "state_kernel";
     case FS_K_PREFIX: return "prefix_kernel";
     case FS_K_SCORES: return "scores_kernel";
     case FS_K_OUT: return "out_kernel";
@@ -174,7 +173,6 @@ const char* fsharp_kernel_name(int id) {
     case FS_K_TC_STATS: return "tc_stats_kernel";
     case FS_K_TC_ROWTERM: return "tc_rowterm_kernel";
     case FS_K_TC_FEAT: return "tc_feat_kernel";
-    case FS_K_TC_LOGITS128: return "tc_logits128_kernel";
     case FS_K_TC_SCORES128: return "tc_scores128_kernel";
     case FS_K_TC_KV128: return "tc_kv128_kernel";
     case FS_K_TC_OUT128: return "tc_out128_kernel";

@@ -11,107 +11,6 @@
 
 namespace {
 
-__device__ __forceinline__ int group_of(int bh, int H, int pool) { return pool == FSHARP_POOL_PER_BH ? bh : bh % H; }
-
-// ---- per-token quadratic term c_i = x_i^T C x_i --------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(NTH)
-rowterm_kernel(const T* __restrict__ X, TensorAddr ax, int H, int L, int d, int M, int pool, int side,
-               const float* __restrict__ prep, float qk_scale, float* __restrict__ rowc) {
-  extern __shared__ float smf[];
-  const int bh = blockIdx.y, b = bh / H, h = bh % H;
-  PrepLayout pr{d, M};
-  const float* pp = prep + ((size_t)group_of(bh, H, pool) * 2 + (side - 1)) * pr.total();
-  const float* scal = pp + pr.scal();
-  const bool cscalar = scal[PS_CSCALAR] != 0.f;
-  const float gamma = scal[PS_CGAMMA];
-  float* Cs = smf;                   // d*d (only when C is dense)
-  float* xs = smf + (cscalar ? 0 : d * d);   // 8 warps * d
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (!cscalar) {
-    const float* Cm = pp + pr.Cmat();
-    for (int e = tid; e < d * d; e += NTH) Cs[e] = Cm[e];
-  }
-  __syncthreads();
-  const T* Xb = X + b * ax.sb + h * ax.sh;
-  float* xw = xs + warp * d;
-  for (int i = blockIdx.x * 8 + warp; i < L; i += gridDim.x * 8) {
-    for (int j = lane; j < d; j += 32) xw[j] = qk_scale * fs_load(Xb + (int64_t)i * ax.sl + j);
-    __syncwarp();
-    float s = 0.f;
-    if (cscalar) {
-      for (int j = lane; j < d; j += 32) s = fmaf(xw[j], xw[j], s);
-      s *= gamma;
-    } else {
-      for (int j = lane; j < d; j += 32) {
-        float t = 0.f;
-        for (int k = 0; k < d; k++) t = fmaf(xw[k], Cs[k * d + j], t);
-        s = fmaf(t, xw[j], s);
-      }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) rowc[(int64_t)bh * L + i] = s;
-    __syncwarp();
-  }
-}
-
-// Order-preserving map float -> unsigned, so that atomicMax on words gives the float maximum.
-__device__ __forceinline__ unsigned f2ord(float f) {
-  unsigned u = __float_as_uint(f);
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-__device__ __forceinline__ float ord2f(unsigned u) {
-  return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
-}
-
-// ---- largest exponent of each (batch, head) --------------------------------------------
-__global__ void __launch_bounds__(NTH)
-groupmax_kernel(const float* __restrict__ phi, int64_t per_bh, unsigned* __restrict__ gmax) {
-  __shared__ float red[NTH / 32];
-  const int bh = blockIdx.y;
-  const float* p = phi + (int64_t)bh * per_bh;
-  float mx = -3.0e38f;
-  for (int64_t e = blockIdx.x * (int64_t)NTH + threadIdx.x; e < per_bh; e += (int64_t)gridDim.x * NTH)
-    mx = fmaxf(mx, p[e]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int i = 1; i < NTH / 32; i++) mx = fmaxf(mx, red[i]);
-    atomicMax(&gmax[bh], f2ord(mx));
-  }
-}
-
-// ---- bf16 features exp(e - shift), one warp per row ------------------------------------------
-// shift: the row's largest exponent (ROW) or the (batch, head)'s (GROUP)
-__global__ void __launch_bounds__(NTH)
-expshift_kernel(const float* __restrict__ logits, int L, int M, int stab, const unsigned* __restrict__ gmax,
-                __nv_bfloat16* __restrict__ phi16, int* __restrict__ status) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int bh = blockIdx.y;
-  const float gshift = stab == FSHARP_STAB_GROUP ? ord2f(gmax[bh]) : 0.f;
-  for (int i = blockIdx.x * 8 + warp; i < L; i += gridDim.x * 8) {
-    const float* row = logits + ((int64_t)bh * L + i) * M;
-    float s = gshift;
-    if (stab == FSHARP_STAB_ROW) {
-      float mx = -3.0e38f;
-      for (int m = lane; m < M; m += 32) mx = fmaxf(mx, row[m]);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      s = mx;
-    }
-    bool bad = false;
-    for (int m = lane; m < M; m += 32) {
-      const float e = row[m];
-      if (!isfinite(e)) bad = true;
-      phi16[((int64_t)bh * L + i) * M + m] = __float2bfloat16_rn(expf(e - s));
-    }
-    if (bad) atomicExch(status, FSHARP_E_NONFINITE);
-  }
-}
-
 // ---- Y = num / den -------------------------------------------------------------------
 // Bidirectional: [num | den] = phiQ (S^T [V | 1]).  Causal: per chunk, phiQ_c times the
 // prefix state plus the masked scores times [V_c | 1].
@@ -178,44 +77,6 @@ out_kernel(const float* __restrict__ phiQ, const float* __restrict__ KV, const f
   blk.end();
 }
 
-// bf16 features of bf16 tokens with d = 128 (the chain of tensor-core kernels): the exponents by tc_logits128, then
-// shift and exponential.
-int featurize128(fsharp_ctx* ctx, const void* X, TensorAddr ax, int B, int H, int L, int M, int pool, const float* prep,
-                 int side, float qk_scale, int stab, float* rowc, unsigned* gmax, float* phi, __nv_bfloat16* phi16) {
-  constexpr int d = 128;
-  const int BH = B * H;
-  {
-    int gx = (L + 7) / 8;
-    if (gx > 4 * ctx->sm_count) gx = 4 * ctx->sm_count;
-    // shared memory: dense C (d*d) + one x per warp; sized for the dense case
-    size_t smem = ((size_t)d * d + 8 * (size_t)d) * sizeof(float);
-    FS_CUDA_OK(cudaFuncSetAttribute(rowterm_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    FS_TIME_BEGIN(ctx, FS_K_ROWTERM);
-    rowterm_kernel<__nv_bfloat16><<<dim3(gx, BH), NTH, smem, ctx->stream>>>((const __nv_bfloat16*)X, ax, H, L, d, M, pool, side, prep,
-                                                                           qk_scale, rowc);
-    FS_TIME_END(ctx);
-    FS_LAUNCH_CHECK(ctx);
-  }
-  FS_TRY(fs_tc_logits128(ctx, X, ax, B, H, L, M, pool, prep, side, qk_scale, rowc, phi));
-  int gx = (L + 7) / 8;
-  if (gx > 4 * ctx->sm_count) gx = 4 * ctx->sm_count;
-  if (stab == FSHARP_STAB_GROUP) {
-    FS_CUDA_OK(cudaMemsetAsync(gmax, 0, (size_t)BH * sizeof(unsigned), ctx->stream));
-    int64_t per_bh = (int64_t)L * M;
-    int gm = (int)((per_bh + 16 * NTH - 1) / (16 * NTH));
-    if (gm > 64) gm = 64;
-    FS_TIME_BEGIN(ctx, FS_K_GROUPMAX);
-    groupmax_kernel<<<dim3(gm, BH), NTH, 0, ctx->stream>>>(phi, per_bh, gmax);
-    FS_TIME_END(ctx);
-    FS_LAUNCH_CHECK(ctx);
-  }
-  FS_TIME_BEGIN(ctx, FS_K_EXPSHIFT);
-  expshift_kernel<<<dim3(gx, BH), NTH, 0, ctx->stream>>>(phi, L, M, stab, gmax, phi16, ctx->d_status);
-  FS_TIME_END(ctx);
-  FS_LAUNCH_CHECK(ctx);
-  return FSHARP_OK;
-}
-
 template <typename T>
 int attend_t(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const fsharp_dims* dm, int causal,
              int chunk, float qk_scale, const float* prep, void* Y, WsAlloc* ws, bool unnormalised) {
@@ -223,27 +84,22 @@ int attend_t(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const
   const int NP = dv + 16, ctiles = (dv + 63) / 64;
   TensorAddr aq = fs_addr(dm->q_stride, H, Lq, d), ak = fs_addr(dm->k_stride, H, Lk, d);
   TensorAddr av = fs_addr(dm->v_stride, H, Lk, dv), ay = fs_addr(dm->y_stride, H, Lq, dv);
-  float* phiQ = ws->take<float>((size_t)BH * Lq * M);
-  float* phiK = ws->take<float>((size_t)BH * Lk * M);
+  // causal, bf16 tensors, d = dv = 128: scores, per-chunk sums and query side from bf16 features
+  const bool tc = causal && !unnormalised && sizeof(T) == 2 && d == 128 && ctx->impl != FSHARP_IMPL_SIMT &&
+                  fs_tc_scores128_supported(M, chunk) && fs_tc_kv128_supported(V, av, dv, M, chunk) && fs_tc_out128_supported(Y, ay);
+  float* phiQ = tc ? nullptr : ws->take<float>((size_t)BH * Lq * M);
+  float* phiK = tc ? nullptr : ws->take<float>((size_t)BH * Lk * M);
+  __nv_bfloat16* phiQ16 = tc ? ws->take<__nv_bfloat16>((size_t)BH * Lq * M) : nullptr;
+  __nv_bfloat16* phiK16 = tc ? ws->take<__nv_bfloat16>((size_t)BH * Lk * M) : nullptr;
   float* rowc = ws->take<float>((size_t)BH * Lk);
   unsigned* gmax = ws->take<unsigned>((size_t)BH);
   float* rowcq = ws->take<float>((size_t)BH * Lq);
   float* lsq = ws->take<float>((size_t)BH * Lq);
   float* lsk = ws->take<float>((size_t)BH);
   uint8_t* img = ws->take<uint8_t>(feat3::image_bytes(fs_groups(dm), d, M, 2));
-  // causal, bf16 tensors, dv = 128: scores, per-chunk sums and query side from bf16 copies of the features
-  const bool tc = causal && !unnormalised && sizeof(T) == 2 && ctx->impl != FSHARP_IMPL_SIMT &&
-                  fs_tc_logits128_supported(Q, FSHARP_BF16, aq, Lq, d, M) && fs_tc_scores128_supported(M, chunk) && fs_tc_kv128_supported(V, av, dv, M, chunk) && fs_tc_out128_supported(Y, ay);
-  __nv_bfloat16* phiQ16 = tc ? ws->take<__nv_bfloat16>((size_t)BH * Lq * M) : nullptr;
-  __nv_bfloat16* phiK16 = tc ? ws->take<__nv_bfloat16>((size_t)BH * Lk * M) : nullptr;
-  if (tc) {
-    FS_TRY(featurize128(ctx, K, ak, B, H, Lk, M, dm->pool, prep, 2, qk_scale, FSHARP_STAB_GROUP, rowc, gmax, phiK, phiK16));
-    FS_TRY(featurize128(ctx, Q, aq, B, H, Lq, M, dm->pool, prep, 1, qk_scale, FSHARP_STAB_ROW, rowcq, gmax, phiQ, phiQ16));
-  } else {
-    const feat3::Task tasks[2] = {{K, ak, Lk, 2, FSHARP_STAB_GROUP, rowc, gmax, phiK, lsk},
-                                  {Q, aq, Lq, 1, FSHARP_STAB_ROW, rowcq, nullptr, phiQ, lsq}};
-    FS_TRY(feat3::run(ctx, tasks, 2, sizeof(T) == 2 ? FSHARP_BF16 : FSHARP_F32, B, H, d, M, dm->pool, prep, qk_scale, img));
-  }
+  const feat3::Task tasks[2] = {{K, ak, Lk, 2, FSHARP_STAB_GROUP, rowc, gmax, phiK, phiK16, lsk},
+                                {Q, aq, Lq, 1, FSHARP_STAB_ROW, rowcq, nullptr, phiQ, phiQ16, lsq}};
+  FS_TRY(feat3::run(ctx, tasks, 2, sizeof(T) == 2 ? FSHARP_BF16 : FSHARP_F32, B, H, d, M, dm->pool, prep, qk_scale, img));
   const dim3 gout((Lq + mma3::ROWS - 1) / mma3::ROWS, ctiles, BH);
   const dim3 gkv((M + mma3::ROWS - 1) / mma3::ROWS, ctiles, 1);
   if (!causal) {
@@ -268,7 +124,7 @@ int attend_t(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const
     prefix_kernel<<<dim3((unsigned)((elems + NTH - 1) / NTH), BH), NTH, 0, ctx->stream>>>(st, nch, elems, 0, st16);
     FS_TIME_END(ctx);
     FS_LAUNCH_CHECK(ctx);
-    FS_TRY(fs_tc_scores128(ctx, phiQ16, phiK16, BH, Lq, M, C, nullptr, sc16));
+    FS_TRY(fs_tc_scores128(ctx, phiQ16, phiK16, BH, Lq, M, C, sc16));
     return fs_tc_out128(ctx, phiQ16, st16, sc16, V, av, Y, ay, B, H, Lq, M, C);
   }
   const int C = inner_chunk(chunk), nch = (Lq + C - 1) / C;
@@ -292,21 +148,25 @@ int attend_t(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const
 int fs_simt_featurize(fsharp_ctx* ctx, const void* X, int dtype, TensorAddr ax, int B, int H, int L, int d,
                       int M, int pool, const float* prep, int side, float qk_scale, int stab,
                       float* rowc, unsigned* gmax, float* phi, float* logscale, uint8_t* img) {
-  const feat3::Task task{X, ax, L, side, stab, rowc, gmax, phi, logscale};
+  const feat3::Task task{X, ax, L, side, stab, rowc, gmax, phi, nullptr, logscale};
   return feat3::run(ctx, &task, 1, dtype, B, H, d, M, pool, prep, qk_scale, img);
 }
 
 size_t fs_simt_attend_scratch_bytes(const fsharp_dims* dm, int causal, int chunk) {
   const size_t BH = (size_t)dm->B * dm->H, NP = dm->dv + 16;
-  size_t b = ws_round(BH * dm->Lq * dm->M * 4) + ws_round(BH * dm->Lk * dm->M * 4) + ws_round(BH * dm->Lk * 4) +
-             ws_round(BH * 4) + 2 * ws_round(BH * dm->Lq * 4) + ws_round(BH * 4) + feat3::image_bytes(fs_groups(dm), dm->d, dm->M, 2);
+  const size_t shifts = ws_round(BH * dm->Lk * 4) + 2 * ws_round(BH * 4) + 2 * ws_round(BH * dm->Lq * 4) +
+                        feat3::image_bytes(fs_groups(dm), dm->d, dm->M, 2);
+  size_t b = ws_round(BH * dm->Lq * dm->M * 4) + ws_round(BH * dm->Lk * dm->M * 4) + shifts;
   if (!causal) {
     b += ws_round(BH * dm->M * NP * 4);
   } else {
     const size_t C = inner_chunk(chunk), nch = (dm->Lq + C - 1) / C;
     b += ws_round(BH * nch * dm->M * NP * 4) + ws_round(BH * nch * C * C * 4);
-    b += ws_round(BH * dm->Lq * dm->M * 2) + ws_round(BH * dm->Lk * dm->M * 2);      // bf16 copies of the features
-    b += ws_round(BH * nch * dm->M * NP * 2) + ws_round(BH * nch * C * C * 2);       // ... of the running sums and the scores
+    // the chain on bf16 features: half the bytes for the features, sums in fp32 and bf16, scores in bf16
+    const size_t N = dm->dv + 1;
+    const size_t t = ws_round(BH * dm->Lq * dm->M * 2) + ws_round(BH * dm->Lk * dm->M * 2) + shifts +
+                     ws_round(BH * nch * dm->M * N * 4) + ws_round(BH * nch * dm->M * N * 2) + ws_round(BH * nch * C * C * 2);
+    if (t > b) b = t;
   }
   return b;
 }

@@ -79,8 +79,8 @@ prefix_kernel(float* __restrict__ st, int nchunks, int64_t elems, int reverse, _
       for (int u = 0; u < 8; u++) {
         const int c = reverse ? nchunks - 1 - (c0 + u) : c0 + u;
         if (c0 + u < nchunks) {
-          base[c * elems + e] = run;
-          if (st16) st16[((int64_t)bh * nchunks + c) * elems + e] = __float2bfloat16_rn(run);   // (for the tensor-core query side)
+          if (!st16) base[c * elems + e] = run;
+          else st16[((int64_t)bh * nchunks + c) * elems + e] = __float2bfloat16_rn(run);   // (what the tensor-core query side reads)
         }
         run += v[u];
       }

@@ -122,11 +122,12 @@ template <typename T, int D, int N> struct Stage {
 };
 
 // Feature blocks of M (all of M when it fits: a row's largest exponent is then known inside the block) and their images:
-// [block][slice][3 parts][rows of 128 bytes, 128-byte swizzle], already scaled by log2e qk_scale.
-template <int D> struct WGeo {
-  static constexpr int NKS = (D + 63) / 64, MB = D == 128 ? 128 : 256;
+// [block][slice][BP parts][rows of 128 bytes, 128-byte swizzle], already scaled by log2e qk_scale.
+// BP = 2 (16 significant bits of W) goes with features that are rounded to bf16.
+template <int D, int BP> struct WGeo {
+  static constexpr int NKS = (D + 63) / 64, MB = D == 128 && BP == 3 ? 128 : 256;
 };
-template <int D>
+template <int D, int BP>
 __device__ __forceinline__ void put_w(uint8_t* img, int mb, int f, int c, const float* w, float scale, bool& bad) {
   float v[8];
 #pragma unroll
@@ -136,32 +137,32 @@ __device__ __forceinline__ void put_w(uint8_t* img, int mb, int f, int c, const 
   }
   uint4 h, m, l;
   split3::split8(v, h, m, l);
-  uint8_t* dst = img + (c / 8) * (3 * mb * 128) + f * 128 + (((c % 8) ^ (f & 7)) << 4);
+  uint8_t* dst = img + (c / 8) * (BP * mb * 128) + f * 128 + (((c % 8) ^ (f & 7)) << 4);
   *reinterpret_cast<uint4*>(dst) = h;
   *reinterpret_cast<uint4*>(dst + mb * 128) = m;
-  *reinterpret_cast<uint4*>(dst + 2 * mb * 128) = l;
+  if (BP == 3) *reinterpret_cast<uint4*>(dst + 2 * mb * 128) = l;
 }
-template <int D>
+template <int D, int BP>
 __global__ void __launch_bounds__(256)
 w3_images_kernel(const float* __restrict__ prep, int side0, int sides, int M, float qk_scale, uint8_t* __restrict__ img,
                  int* __restrict__ status) {
-  using G = WGeo<D>;
+  using G = WGeo<D, BP>;
   const int g = blockIdx.y, k = blockIdx.z;                          // group; which of the `sides` sides
-  const size_t per_group = (size_t)G::NKS * 3 * M * 128;
+  const size_t per_group = (size_t)G::NKS * BP * M * 128;
   const float* W = prep + ((size_t)g * 2 + (side0 - 1 + k)) * PrepLayout{D, M}.total();
   uint8_t* out = img + ((size_t)k * gridDim.y + g) * per_group;
   bool bad = false;
   for (int e = blockIdx.x * 256 + threadIdx.x; e < M * (D / 8); e += gridDim.x * 256) {
     const int m = e / (D / 8), c = e % (D / 8), blk = m / G::MB, mb = min(G::MB, M - blk * G::MB);
-    put_w<D>(out + (size_t)blk * G::MB * (G::NKS * 3 * 128), mb, m - blk * G::MB, c, W + (size_t)m * D + 8 * c, FS_LOG2E * qk_scale, bad);
+    put_w<D, BP>(out + (size_t)blk * G::MB * (G::NKS * BP * 128), mb, m - blk * G::MB, c, W + (size_t)m * D + 8 * c, FS_LOG2E * qk_scale, bad);
   }
   if (bad) atomicExch(status, FSHARP_E_NONFINITE);
 }
 
-// acc[128 x N] = A B^T with A = staged tokens, B = [slice][3 parts][N rows x 128 bytes], by one lane: the products with m or l
-// parts first, h h last (the accumulator is truncated at every step; see tc_pairs.cu).
+// acc[128 x N] = A B^T with A = staged tokens, B = [slice][BP parts][N rows x 128 bytes], by one lane: the products with m or l
+// parts (those of the first USE parts of B) first, h h last (the accumulator is truncated at every step; see tc_pairs.cu).
 // sOne / sRow (may be null): one more step of K = 16 with operands [128 x 16] and [N x 16] in core matrices, for a term per column.
-template <typename T, int D>
+template <typename T, int D, int BP = 3, int USE = BP>
 __device__ __forceinline__ void issue_products(uint32_t acc, const uint8_t* sA, const uint8_t* sB, int N, const uint8_t* sOne = nullptr,
                                                const uint8_t* sRow = nullptr) {
   using G = Geo<T, D>;
@@ -169,27 +170,27 @@ __device__ __forceinline__ void issue_products(uint32_t acc, const uint8_t* sA, 
   const uint64_t da = smem_desc(smem_u32(sA), 16, 1024, SWZ_128B), db = smem_desc(smem_u32(sB), 16, 1024, SWZ_128B);
   const uint32_t ah = (uint32_t)(da >> 32), bh = (uint32_t)(db >> 32), P = TILE_BYTES / 16, Q = (uint32_t)N * 8;
 #pragma unroll
-  for (int s = 0; s < G::NKS; s++) {
-    const uint32_t a0 = (uint32_t)da + s * G::AP * P, b0 = (uint32_t)db + s * 3 * Q;
+  for (int s = 0; s < (USE > 1 ? G::NKS : 0); s++) {
+    const uint32_t a0 = (uint32_t)da + s * G::AP * P, b0 = (uint32_t)db + s * BP * Q;
 #pragma unroll
     for (int k = 0; k < G::KSTEPS; k++) {
       const uint32_t a = a0 + 2 * k, b = b0 + 2 * k;
-      mma_bf16_lh(acc, a, ah, b + 2 * Q, bh, idesc, (s | k) ? 1u : 0u);
+      if (USE == 3) mma_bf16_lh(acc, a, ah, b + 2 * Q, bh, idesc, (s | k) ? 1u : 0u);
       if (G::AP == 3) {
         mma_bf16_lh(acc, a + 2 * P, ah, b, bh, idesc, 1u);
         mma_bf16_lh(acc, a + P, ah, b + Q, bh, idesc, 1u);
         mma_bf16_lh(acc, a + P, ah, b, bh, idesc, 1u);
       }
-      mma_bf16_lh(acc, a, ah, b + Q, bh, idesc, 1u);
+      mma_bf16_lh(acc, a, ah, b + Q, bh, idesc, USE == 3 || (s | k) ? 1u : 0u);
     }
   }
   if (sOne != nullptr)
-    mma_bf16(acc, smem_desc(smem_u32(sOne), 128, 256, SWZ_NONE), smem_desc(smem_u32(sRow), 128, 256, SWZ_NONE), idesc, 1u);
+    mma_bf16(acc, smem_desc(smem_u32(sOne), 128, 256, SWZ_NONE), smem_desc(smem_u32(sRow), 128, 256, SWZ_NONE), idesc, USE > 1 ? 1u : 0u);
 #pragma unroll
   for (int s = 0; s < G::NKS; s++)
 #pragma unroll
     for (int k = 0; k < G::KSTEPS; k++)
-      mma_bf16_lh(acc, (uint32_t)da + s * G::AP * P + 2 * k, ah, (uint32_t)db + s * 3 * Q + 2 * k, bh, idesc, 1u);
+      mma_bf16_lh(acc, (uint32_t)da + s * G::AP * P + 2 * k, ah, (uint32_t)db + s * BP * Q + 2 * k, bh, idesc, 1u);
 }
 
 // ---- c_i = x_i^T C x_i; also clears the maxima that later passes raise ------------------------
@@ -362,19 +363,23 @@ struct FtMisc {
   uint32_t tmem_base;
   int abort_flag;
 };
-template <typename T, int D> struct FtGeo : Geo<T, D> {
-  static constexpr int MB = WGeo<D>::MB;
+template <typename T, int D, int BP> struct FtGeo : Geo<T, D> {
+  static_assert(BP == 3 || Geo<T, D>::AP == 1, "two parts of W: bf16 tokens");
+  static constexpr int MB = WGeo<D, BP>::MB;
   static constexpr int NBUF = (D == 128 && sizeof(T) == 4) ? 1 : 2;    // token tiles in shared memory
-  static constexpr uint32_t W_BYTES = Geo<T, D>::NKS * 3 * MB * 128;
+  static constexpr uint32_t W_BYTES = Geo<T, D>::NKS * BP * MB * 128;
   static constexpr uint32_t OFF_A = W_BYTES, OFF_ONE = OFF_A + NBUF * Geo<T, D>::A_BYTES, OFF_ROW = OFF_ONE + TILE * 32, OFF_MISC = OFF_ROW + MB * 32;
   static constexpr size_t SMEM = 1024 + OFF_MISC + sizeof(FtMisc);
   static_assert(SMEM <= 232448, "shared memory budget");
 };
 
-template <typename T, int D, bool WRITE>
+// BP = 2: bf16 features of the chain of d = 128 kernels, whose shifts may be any value near the maximum (they cancel in the
+// normalisation, and bf16 has the range of fp32): the maxima pass then takes the leading part of W alone.
+template <typename T, int D, bool WRITE, int BP>
 __global__ void __launch_bounds__(FT_THREADS, 1)
 feat3_kernel(const __grid_constant__ Args a) {
-  using G = FtGeo<T, D>;
+  using G = FtGeo<T, D, BP>;
+  constexpr bool OUT16 = BP == 2;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sW = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* sA = sW + G::OFF_A;
@@ -426,14 +431,14 @@ feat3_kernel(const __grid_constant__ Args a) {
     __syncthreads();                                               // the previous run's products have been read
     if (a.img[ti] != nullptr) {
       if (tid == 0) {
-        const uint32_t bytes = (uint32_t)mb * (G::NKS * 3 * 128);
+        const uint32_t bytes = (uint32_t)mb * (G::NKS * BP * 128);
         mbar_expect_tx(&misc->w_full, bytes);
-        bulk_load(sW, a.img[ti] + ((size_t)g * a.M + m0) * (G::NKS * 3 * 128), bytes, &misc->w_full);
+        bulk_load(sW, a.img[ti] + ((size_t)g * a.M + m0) * (G::NKS * BP * 128), bytes, &misc->w_full);
       }
     } else {
       const float* W = pp + pr.W() + (size_t)m0 * D;
       for (int e = tid; e < mb * (D / 8); e += FT_THREADS)
-        put_w<D>(sW, mb, e / (D / 8), e % (D / 8), W + (size_t)e * 8, FS_LOG2E * a.qk_scale, bad);
+        put_w<D, BP>(sW, mb, e / (D / 8), e % (D / 8), W + (size_t)e * 8, FS_LOG2E * a.qk_scale, bad);
     }
     for (int e = tid; e < mb; e += FT_THREADS) {
       const float v = FS_LOG2E * pp[pr.a() + m0 + e];
@@ -467,7 +472,7 @@ feat3_kernel(const __grid_constant__ Args a) {
         __syncwarp();
         tcgen05_fence_after();
         if (elect_one()) {
-          issue_products<T, D>(tmem + b * 256, sA + ab * G::A_BYTES, sW, mb, sOne, sRow);
+          issue_products<T, D, BP, OUT16 && !WRITE ? 1 : BP>(tmem + b * 256, sA + ab * G::A_BYTES, sW, mb, sOne, sRow);
           mma_commit(&misc->t_full[b]);
           mma_commit(&misc->a_free[ab]);
         }
@@ -478,7 +483,7 @@ feat3_kernel(const __grid_constant__ Args a) {
       float gmx = -3.0e38f;
       const float gshift = (WRITE && t.stab == FSHARP_STAB_GROUP) ? ord2f(t.gmax[bh]) : 0.f;
       const bool own = t.stab == FSHARP_STAB_ROW && a.nmb == 1;
-      const bool wide = WRITE && (reinterpret_cast<uintptr_t>(t.phi) & 31) == 0;
+      const bool wide = WRITE && !OUT16 && (reinterpret_cast<uintptr_t>(t.phi) & 31) == 0;
       constexpr float LN2 = 0.693147180559945f;
       if (WRITE && t.stab == FSHARP_STAB_GROUP && t.logscale && tile0 == 0 && mblk == 0 && tid == 0) t.logscale[bh] = LN2 * gshift;
       const uint32_t acc = tmem + wg * 256 + ((uint32_t)((warp & 3) * 32) << 16);
@@ -541,7 +546,8 @@ feat3_kernel(const __grid_constant__ Args a) {
           }
         }
         if (WRITE) {
-          float* out = t.phi + at * a.M + m0;
+          float* out = OUT16 ? nullptr : t.phi + at * a.M + m0;
+          __nv_bfloat16* out16 = OUT16 ? t.phi16 + at * a.M + m0 : nullptr;
           for (int c = 0; c < mb; c += 32) {
             uint32_t x[32];
             arrived(x);
@@ -550,7 +556,13 @@ feat3_kernel(const __grid_constant__ Args a) {
             for (int j = 0; j < 32; j++) x[j] = __float_as_uint(ex2(__uint_as_float(x[j]) + off));
             if (in) {
               float* dst = out + c;
-              if (wide) {
+              if (OUT16) {                               // (M is a multiple of 128 and the scratch aligned)
+                uint32_t h[16];
+#pragma unroll
+                for (int j = 0; j < 16; j++) h[j] = pack_bf16(__uint_as_float(x[2 * j]), __uint_as_float(x[2 * j + 1]));
+                store32(reinterpret_cast<float*>(out16 + c), h);
+                store32(reinterpret_cast<float*>(out16 + c + 16), h + 8);
+              } else if (wide) {
 #pragma unroll
                 for (int j = 0; j < 4; j++)
                   if (j < 2 || c + 16 < mb) store32(dst + 8 * j, &x[8 * j]);
@@ -584,19 +596,19 @@ feat3_kernel(const __grid_constant__ Args a) {
   }
 }
 
-template <typename T, int D>
+template <typename T, int D, int BP>
 int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, int G_groups, uint8_t* img) {
-  using G = FtGeo<T, D>;
+  using G = FtGeo<T, D, BP>;
   a.nmb = (a.M + G::MB - 1) / G::MB;
   const uint8_t* side_img[2] = {nullptr, nullptr};     // by side - 1
   // (a set with a row shift over several feature blocks has its maxima pass instead: its blocks convert W themselves)
   if (img != nullptr && !(ntasks == 1 && tasks[0].stab == FSHARP_STAB_ROW && a.nmb > 1)) {
     const int side0 = ntasks == 2 ? 1 : tasks[0].side;
-    const size_t per_side = (size_t)G_groups * G::NKS * 3 * a.M * 128;
+    const size_t per_side = (size_t)G_groups * G::NKS * BP * a.M * 128;
     for (int k = 0; k < ntasks; k++) side_img[side0 - 1 + k] = img + k * per_side;
     const dim3 grid((a.M * (D / 8) + 255) / 256, G_groups, ntasks);
     FS_TIME_BEGIN(ctx, FS_K_W3);
-    w3_images_kernel<D><<<grid, 256, 0, ctx->stream>>>(a.prep, side0, ntasks, a.M, a.qk_scale, img, ctx->d_status);
+    w3_images_kernel<D, BP><<<grid, 256, 0, ctx->stream>>>(a.prep, side0, ntasks, a.M, a.qk_scale, img, ctx->d_status);
     FS_TIME_END(ctx);
     FS_LAUNCH_CHECK(ctx);
   }
@@ -626,16 +638,16 @@ int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, in
   }
   const int maxed = set(a.nmb, [](const Task& t, int nmb) { return t.stab == FSHARP_STAB_GROUP || (t.stab == FSHARP_STAB_ROW && nmb > 1); });
   if (maxed > 0) {
-    FS_CUDA_OK(cudaFuncSetAttribute(feat3_kernel<T, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM));
+    FS_CUDA_OK(cudaFuncSetAttribute(feat3_kernel<T, D, false, BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM));
     FS_TIME_BEGIN(ctx, FS_K_GROUPMAX);
-    feat3_kernel<T, D, false><<<maxed < ctx->sm_count ? maxed : ctx->sm_count, FT_THREADS, G::SMEM, ctx->stream>>>(a);
+    feat3_kernel<T, D, false, BP><<<maxed < ctx->sm_count ? maxed : ctx->sm_count, FT_THREADS, G::SMEM, ctx->stream>>>(a);
     FS_TIME_END(ctx);
     FS_LAUNCH_CHECK(ctx);
   }
   const int total = set(a.nmb, [](const Task&, int) { return true; });
-  FS_CUDA_OK(cudaFuncSetAttribute(feat3_kernel<T, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM));
+  FS_CUDA_OK(cudaFuncSetAttribute(feat3_kernel<T, D, true, BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM));
   FS_TIME_BEGIN(ctx, FS_K_FEAT);
-  feat3_kernel<T, D, true><<<total < ctx->sm_count ? total : ctx->sm_count, FT_THREADS, G::SMEM, ctx->stream>>>(a);
+  feat3_kernel<T, D, true, BP><<<total < ctx->sm_count ? total : ctx->sm_count, FT_THREADS, G::SMEM, ctx->stream>>>(a);
   FS_TIME_END(ctx);
   FS_LAUNCH_CHECK(ctx);
   return FSHARP_OK;
@@ -643,14 +655,17 @@ int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, in
 
 // Two token sets share their launches only while both together leave SMs without a tile: beyond that a launch of its own
 // costs a set nothing, and its blocks keep one W each for longer.
-template <typename T, int D>
+template <typename T, int D, int BP>
 int run_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, int groups, uint8_t* img) {
+  if constexpr (BP == 3 && D == 128 && sizeof(T) == 2) {
+    if (tasks[0].phi16 != nullptr) return run_t<T, D, 2>(ctx, a, tasks, ntasks, BH, groups, img);
+  }
   int64_t items = 0;
-  for (int i = 0; i < ntasks; i++) items += (int64_t)BH * ((tasks[i].L + TILE - 1) / TILE) * ((a.M + WGeo<D>::MB - 1) / WGeo<D>::MB);
+  for (int i = 0; i < ntasks; i++) items += (int64_t)BH * ((tasks[i].L + TILE - 1) / TILE) * ((a.M + WGeo<D, BP>::MB - 1) / WGeo<D, BP>::MB);
   if (items > 2147483647LL) return FSHARP_E_SHAPE;     // items are numbered in 32 bits
-  if (ntasks == 1 || items <= ctx->sm_count) return launch_t<T, D>(ctx, a, tasks, ntasks, BH, groups, img);
+  if (ntasks == 1 || (items <= ctx->sm_count && BP == 3)) return launch_t<T, D, BP>(ctx, a, tasks, ntasks, BH, groups, img);
   for (int i = 0; i < ntasks; i++) {
-    FS_TRY((launch_t<T, D>(ctx, a, tasks + i, 1, BH, groups, img)));
+    FS_TRY((launch_t<T, D, BP>(ctx, a, tasks + i, 1, BH, groups, img)));
   }
   return FSHARP_OK;
 }
@@ -667,8 +682,8 @@ int feat3::run(fsharp_ctx* ctx, const Task* tasks, int ntasks, int dtype, int B,
   a.H = H; a.M = M; a.pool = pool; a.prep = prep; a.qk_scale = qk_scale; a.status = ctx->d_status;
   const int groups = pool == FSHARP_POOL_PER_BH ? B * H : H;
 #define FS_FEAT3(DD)                                                                                          \
-  return dtype == FSHARP_F32 ? run_t<float, DD>(ctx, a, tasks, ntasks, B * H, groups, img)                    \
-                             : run_t<__nv_bfloat16, DD>(ctx, a, tasks, ntasks, B * H, groups, img)
+  return dtype == FSHARP_F32 ? run_t<float, DD, 3>(ctx, a, tasks, ntasks, B * H, groups, img)                    \
+                             : run_t<__nv_bfloat16, DD, 3>(ctx, a, tasks, ntasks, B * H, groups, img)
   switch (d) {
     case 16: FS_FEAT3(16);
     case 32: FS_FEAT3(32);
