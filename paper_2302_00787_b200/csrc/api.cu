@@ -15,8 +15,9 @@ int fs_tc_key_state_splits(const fsharp_ctx* ctx, const fsharp_dims* dm, int* ti
 size_t fs_tc_key_state_scratch_bytes(const fsharp_ctx* ctx, const fsharp_dims* dm);
 int fs_tc_key_state(fsharp_ctx* ctx, const void* K, const void* V, const fsharp_dims* dm, const uint8_t* images,
                     const int* flags, float* state, float* shifts, WsAlloc* ws);
+size_t fs_tc_query_side_scratch_bytes(const fsharp_dims* dm);
 int fs_tc_query_side(fsharp_ctx* ctx, const void* Q, const fsharp_dims* dm, const uint8_t* images, const float* partial,
-                     const float* shifts, int nsplit, void* Y);
+                     const float* shifts, int nsplit, void* Y, WsAlloc* ws);
 size_t fs_tc_causal_prefix_scratch_bytes(const fsharp_ctx* ctx, const fsharp_dims* dm, int nprefix);
 int fs_tc_causal_prefix(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const fsharp_dims* dm, const uint8_t* images,
                         const int* flags, const float* pre_state, const float* pre_shifts, int nprefix, void* Y, WsAlloc* ws);
@@ -269,7 +270,7 @@ int fsharp_attend_with_state(fsharp_ctx* ctx, const void* Q, const void* K, cons
   const int G = fs_groups(dims);
   const size_t prep_f = (size_t)G * 2 * PrepLayout{dims->d, dims->M}.total();
   const size_t img_bytes = ws_round((size_t)G * 2 * tcl::IMG_BYTES) + ws_round((size_t)G * 2 * tcl::FLAG_WORDS * 4 + 64);
-  FS_TRY(fs_ws_reserve(ctx, ws_round(prep_f * 4) + img_bytes + (causal ? fs_tc_causal_prefix_scratch_bytes(ctx, &qd, n_states) : 0)));
+  FS_TRY(fs_ws_reserve(ctx, ws_round(prep_f * 4) + img_bytes + (causal ? fs_tc_causal_prefix_scratch_bytes(ctx, &qd, n_states) : fs_tc_query_side_scratch_bytes(&qd))));
   WsAlloc ws{ctx->ws, 0};
   float* prep = ws.take<float>(prep_f);
   uint8_t* images = ws.take<uint8_t>((size_t)G * 2 * tcl::IMG_BYTES);
@@ -277,7 +278,7 @@ int fsharp_attend_with_state(fsharp_ctx* ctx, const void* Q, const void* K, cons
   FS_TRY(fs_run_prep_images(ctx, Omega, dims->omega_head_stride, params, (int64_t)ParamsLayout{dims->d}.total(), G,
                             dims->H, dims->pool, dims->d, dims->M, prep, qk_scale, images, flags));
   if (causal) return fs_tc_causal_prefix(ctx, Q, K, V, &qd, images, flags, states, shifts, n_states, Y, &ws);
-  return fs_tc_query_side(ctx, Q, &qd, images, states, shifts, n_states, Y);
+  return fs_tc_query_side(ctx, Q, &qd, images, states, shifts, n_states, Y, &ws);
 }
 
 int fsharp_kernel_apply(fsharp_ctx* ctx, const void* X, const void* Y, const void* Cmat, const float* Omega,
@@ -334,7 +335,14 @@ int fsharp_forward_host(fsharp_ctx* ctx, const void* Q, const void* K, const voi
   size_t inner = ws_round((size_t)G2 * 2 * PrepLayout{dd.d, dd.M}.total() * 4);
   {
     size_t a = fs_simt_attend_scratch_bytes(&dd, causal, chunk);
-    size_t b = fs_tc_supported(&dd, dtype, causal, chunk, qk_scale) ? fs_tc_attend_scratch_bytes(ctx, &dd, causal, chunk) : 0;
+    size_t b = 0;
+    if (fs_tc_supported(&dd, dtype, causal, chunk, qk_scale)) {
+      // (the nested calls see one batch element at a time, whose pieces may be cut finer)
+      fsharp_dims one = dd;
+      if (dd.pool == FSHARP_POOL_PER_BH) one.B = 1;
+      const size_t whole = fs_tc_attend_scratch_bytes(ctx, &dd, causal, chunk), part = fs_tc_attend_scratch_bytes(ctx, &one, causal, chunk);
+      b = whole > part ? whole : part;
+    }
     size_t c = ws_round(fs_fit_scratch_doubles(G, dd.d) * 8);
     size_t use = ctx->impl == FSHARP_IMPL_SIMT ? a : (b ? b : a);
     inner += use > c ? use : c;

@@ -51,7 +51,7 @@ enum {
   FS_K_STATS = 1, FS_K_FIT, FS_K_PREP, FS_K_ROWTERM, FS_K_FEAT, FS_K_GROUPMAX, FS_K_KV,
   FS_K_PREFIX, FS_K_SCORES, FS_K_OUT, FS_K_PAIRS, FS_K_PAIRVAR_PREP, FS_K_PAIRVAR,
   FS_K_TC_KV, FS_K_TC_OUT, FS_K_TC_CAUSAL, FS_K_TC_STATS, FS_K_TC_ROWTERM, FS_K_TC_FEAT, FS_K_TC_SCORES128, FS_K_TC_KV128, FS_K_TC_OUT128,
-  FS_K_PAIR_IMAGES, FS_K_W3, FS_K_BWD_STATE, FS_K_BWD_NUMDEN, FS_K_BWD_DFEAT, FS_K_BWD_DX, FS_K_BWD_DV,
+  FS_K_PAIR_IMAGES, FS_K_W3, FS_K_BWD_STATE, FS_K_BWD_NUMDEN, FS_K_BWD_DFEAT, FS_K_BWD_DX, FS_K_BWD_DV, FS_K_TC_MERGE,
   FS_K_COUNT
 };
 static_assert(FS_K_COUNT <= 32, "ids are below 32");

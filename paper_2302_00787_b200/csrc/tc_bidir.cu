@@ -20,13 +20,15 @@
 #include "common.cuh"
 #include "tc_common.cuh"
 #include "tc_layout.cuh"
+#include "tc_work.cuh"
 
 using namespace tc;
 using namespace tcl;
 
 namespace {
 
-constexpr int MAX_KEY_SPLIT = 64;    // splits of the key range of one (batch, head)
+constexpr int MAX_KEY_SPLIT = 64;    // key states of one (batch, head) that a caller may hand in
+constexpr int MAX_PIECES = 160;      // pieces of the key range of one (batch, head) that are merged
 constexpr int PREFETCH_TILES = 4;   // tiles pulled into L2 ahead of the shared-memory ring
 
 // ------------------------------------------------------------------------------------------
@@ -39,8 +41,19 @@ constexpr int PREFETCH_TILES = 4;   // tiles pulled into L2 ahead of the shared-
 // The accumulator of half h is acc_h = phi_h^T [V | 1] (128 feature lanes x 80 columns: the phi half
 // tile is the M-side operand, [V | 1] the N = 80 side), so a contraction step costs 80 columns of the
 // tensor pipe instead of 128, and every epilogue thread (= one feature) takes part when the state leaves.
+
+// What the query side reads of one (batch, head) (see merge_kernel): the state [4 feature blocks][80 rows x 64 features] fp16,
+// 128-byte swizzle, then g.
+constexpr uint32_t MRG_GOP = KVT_BYTES, GOP_BYTES = TC_M * 32, MRG_BYTES = KVT_BYTES + GOP_BYTES;
+// g_m as an fp16 value and its fp16 remainder: K elements 0 and 1 of row m of the operand
+__device__ __forceinline__ void write_g(uint8_t* gop, int m, float gm) {
+  const __half hi = __float2half_rn(gm), lo = __float2half_rn(gm - __half2float(hi));
+  uint8_t* rowp = gop + (m >> 3) * 256 + (m & 7) * 16;
+  *reinterpret_cast<uint4*>(rowp) = make_uint4((uint32_t)__half_as_ushort(hi) | ((uint32_t)__half_as_ushort(lo) << 16), 0, 0, 0);
+  *reinterpret_cast<uint4*>(rowp + 128) = make_uint4(0, 0, 0, 0);
+}
+
 constexpr int KV_KSTAGES = 3;       // key tiles in flight (TMA, conversion to fp16, logits MMA)
-constexpr bool KV_TURNS = false;    // the two feature halves take turns at the exponentials
 constexpr int KV_POLY_PAIRS = 2;    // of every four pairs of exponentials, this many run on the multiply-add pipe (measured: 1 and 3 are slower)
 struct KvSmem {
   static constexpr uint32_t X0 = 0, V0 = KV_KSTAGES * TILE_BYTES, ONES = V0 + 2 * TILE_BYTES, W = ONES + TILE_BYTES,
@@ -52,15 +65,14 @@ static_assert(KvSmem::PHI % 1024 == 0 && KvSmem::W % 1024 == 0 && KvSmem::ONES %
 struct KvMisc {
   // key and value tiles have barriers of their own: a key tile is free again once the logits MMA that read it
   // has completed, long before the contraction that reads the value tile of the same stage
+  // acc_free[h]: the state of half h has been read, the next piece's contraction may overwrite it
   uint64_t fullK[KV_KSTAGES], convK[KV_KSTAGES], emptyK[KV_KSTAGES], fullV[2], emptyV[2], logits_full, logits_free, phi_full[2],
-      phi_free[2], const_bar;
-  // turn[h]: half h may run its exponentials.  The halves take turns (each arrives on the other's barrier when its
-  // exponentials are done), so one half has the exponential unit to itself while the other half's contraction
-  // runs on the tensor cores and its warps load and scan the next tile's logits.
-  uint64_t turn[2];
+      phi_free[2], acc_free[2], const_bar;
   uint32_t tmem_base;
   int abort_flag;
   int tile_max[2][4];     // per half: [0..2] rotating slots of the per-tile maximum
+  float ref[2];           // half 0's shift at the first tile of the current piece (slot: piece & 1)
+  int cursor[EPI_THREADS / 32];   // where an epilogue warp's iterator stands
 };
 static_assert(sizeof(KvMisc) <= 256, "misc block");
 
@@ -70,20 +82,22 @@ constexpr int HALF_THREADS = EPI_THREADS / 2;
 __global__ void __launch_bounds__(TC_THREADS, 1)
 tc_kv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
              const uint8_t* __restrict__ images, const float* __restrict__ crow, int H, int pool, int L, int Lpad,
-             int tiles_per_split, int nsplit, float* __restrict__ partial, float* __restrict__ shifts,
+             const TileWork work, float* __restrict__ partial, float* __restrict__ shifts, uint8_t* __restrict__ merged,
              int* __restrict__ status) {
   fs_grid_dependency_wait();
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  // (declared with its alignment, so that every address below is a constant: rounded up at run time the base lives in
+  // registers, and next to the 128 logits of a thread it was spilled and reloaded at every barrier)
+  extern __shared__ __align__(1024) uint8_t sm[];
+  if (smem_u32(sm) & 1023u) {                  // uniform over the block, before anything is allocated
+    if (threadIdx.x == 0) atomicExch(status, FSHARP_E_INTERNAL);
+    return;
+  }
   KvMisc* misc = reinterpret_cast<KvMisc*>(sm + KvSmem::MISC);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int split = blockIdx.x, bh = blockIdx.y, b = bh / H, h = bh % H;
-  const int g = pool == FSHARP_POOL_PER_BH ? bh : h;
-  const int total_tiles = (L + TILE - 1) / TILE;
-  const int tile0 = split * tiles_per_split;
-  const int ntiles = min(tiles_per_split, total_tiles - tile0);
-  const uint8_t* img = images + ((size_t)g * 2 + 1) * IMG_BYTES;        // side 2 (keys)
+  auto group = [&](int bh) { return pool == FSHARP_POOL_PER_BH ? bh : bh % H; };
   volatile int* abortp = &misc->abort_flag;
+  TileIter ti;                                 // every warp walks the same tiles; n counts them
+  ti.begin(work, blockIdx.x, gridDim.x);
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < KV_KSTAGES; i++) {
@@ -96,7 +110,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       mbar_init(&misc->emptyV[i], 2);
       mbar_init(&misc->phi_full[i], HALF_THREADS / 32);
       mbar_init(&misc->phi_free[i], 1);
-      mbar_init(&misc->turn[i], HALF_THREADS / 32);
+      mbar_init(&misc->acc_free[i], HALF_THREADS / 32);
       for (int j = 0; j < 4; j++) misc->tile_max[i][j] = f2ord(-INFINITY);
     }
     mbar_init(&misc->logits_full, 1);
@@ -148,60 +162,51 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     if (lane == 0) {
       prefetch_tmap(&tmK);
       prefetch_tmap(&tmV);
-      mbar_expect_tx(&misc->const_bar, IMG_W_BYTES);
-      bulk_load(sm + KvSmem::W, img + IMG_WH, IMG_W_BYTES, &misc->const_bar);
-      // tiles ahead of the shared-memory ring are pulled into L2
-      for (int it = 0; it < min(ntiles, PREFETCH_TILES); it++) {
-        tma_prefetch_4d(&tmK, 0, (tile0 + it) * TILE, h, b);
-        tma_prefetch_4d(&tmV, 0, (tile0 + it) * TILE, h, b);
-      }
     }
-    // Key tile `it` is loaded as soon as the logits MMA of tile it - 3 has completed; the warp then converts its half
-    // of key tile it - 1, which has landed meanwhile; the value tile follows one iteration behind (its stage is held
-    // until the contraction of tile it - 2 has completed).  So the next tile's logits never wait for a value tile.
-    int issuedK = 0, issuedV = 0;
+    // Key tile n is loaded as soon as the logits MMA of tile n - 3 has completed; the warp then converts its half
+    // of key tile n - 1, which has landed meanwhile; the value tile follows one iteration behind (its stage is held
+    // until the contraction of tile n - 2 has completed).  So the next tile's logits never wait for a value tile.
+    int issuedK = 0, issuedV = 0, b = 0, h = 0, vtok = 0, vb = 0, vh = 0;
     auto load_v = [&](int j) {
       const int sj = j & 1;
       if (!__all_sync(0xffffffffu, mbar_wait(&misc->emptyV[sj], ((j >> 1) & 1) ^ 1, abortp, status))) return false;
       if (lane == 0) {
         mbar_expect_tx(&misc->fullV[sj], TILE_BYTES);
-        tma_load_4d(sm + KvSmem::V0 + sj * TILE_BYTES, &tmV, &misc->fullV[sj], 0, (tile0 + j) * TILE, h, b);
+        tma_load_4d(sm + KvSmem::V0 + sj * TILE_BYTES, &tmV, &misc->fullV[sj], 0, vtok, vh, vb);
       }
       issuedV = j + 1;
       return true;
     };
     bool okp = true;
-    for (int it = 0; it < ntiles && okp; it++) {
-      const int st = it % KV_KSTAGES;
-      if (!__all_sync(0xffffffffu, mbar_wait(&misc->emptyK[st], ((it / KV_KSTAGES) & 1) ^ 1, abortp, status))) { okp = false; break; }
+    for (; okp && ti.next(work); issuedK++) {
+      const int n = issuedK, st = n % KV_KSTAGES;
+      if (ti.first()) { b = ti.bh / H; h = ti.bh - b * H; }       // (divisions for every tile cost this warp 10 % of a tile)
+      if (!__all_sync(0xffffffffu, mbar_wait(&misc->emptyK[st], ((n / KV_KSTAGES) & 1) ^ 1, abortp, status))) { okp = false; break; }
       if (lane == 0) {
-        if (it + PREFETCH_TILES < ntiles) {
-          tma_prefetch_4d(&tmK, 0, (tile0 + it + PREFETCH_TILES) * TILE, h, b);
-          tma_prefetch_4d(&tmV, 0, (tile0 + it + PREFETCH_TILES) * TILE, h, b);
-        }
         mbar_expect_tx(&misc->fullK[st], TILE_BYTES);
-        tma_load_4d(sm + KvSmem::X0 + st * TILE_BYTES, &tmK, &misc->fullK[st], 0, (tile0 + it) * TILE, h, b);
+        tma_load_4d(sm + KvSmem::X0 + st * TILE_BYTES, &tmK, &misc->fullK[st], 0, ti.tile() * TILE, h, b);
       }
-      issuedK = it + 1;
-      if (it >= 1) {
-        okp = convert_half(it - 1, 1);
-        if (okp) okp = load_v(it - 1);
+      // tiles ahead of the ring are pulled into L2 (of this piece: a second iterator's registers would spill, and the spill's
+      // way to L2 is what a tile of this warp's schedule costs)
+      if (lane == 0 && ti.idx + PREFETCH_TILES < ti.ntiles) {
+        tma_prefetch_4d(&tmK, 0, (ti.tile() + PREFETCH_TILES) * TILE, h, b);
+        tma_prefetch_4d(&tmV, 0, (ti.tile() + PREFETCH_TILES) * TILE, h, b);
       }
+      if (n >= 1) okp = convert_half(n - 1, 1) && load_v(n - 1);
+      vtok = ti.tile() * TILE;
+      vb = b;
+      vh = h;
     }
-    if (okp && ntiles > 0) {
-      okp = convert_half(ntiles - 1, 1);
-      if (okp) load_v(ntiles - 1);
-    }
+    if (okp && issuedK > 0 && convert_half(issuedK - 1, 1)) load_v(issuedK - 1);
     // no copy of this block may still be in flight when it exits
     if (lane == 0) {
-      mbar_wait(&misc->const_bar, 0, abortp, status, false);
-      for (int it = max(0, issuedK - KV_KSTAGES); it < issuedK; it++)
-        mbar_wait(&misc->fullK[it % KV_KSTAGES], (it / KV_KSTAGES) & 1, abortp, status, false);
-      for (int it = max(0, issuedV - 2); it < issuedV; it++) mbar_wait(&misc->fullV[it & 1], (it >> 1) & 1, abortp, status, false);
+      for (int n = max(0, issuedK - KV_KSTAGES); n < issuedK; n++)
+        mbar_wait(&misc->fullK[n % KV_KSTAGES], (n / KV_KSTAGES) & 1, abortp, status, false);
+      for (int n = max(0, issuedV - 2); n < issuedV; n++) mbar_wait(&misc->fullV[n & 1], (n >> 1) & 1, abortp, status, false);
     }
   } else if (warp == WARP_MMA + 2) {
-    for (int it = 0; it < ntiles; it++)
-      if (!convert_half(it, 0)) break;
+    for (int n = 0; ti.next(work); n++)
+      if (!convert_half(n, 0)) break;
   } else if (warp == WARP_MMA) {
     // ---------------- logits MMAs: the whole warp walks the schedule (descriptor arithmetic and waits stay
     // warp-uniform), one elected lane issues
@@ -210,12 +215,24 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     const uint64_t dW = smem_desc(smem_u32(sm + KvSmem::W), 16, 1024, SWZ_128B);
     uint32_t xl = (uint32_t)dX0, wl = (uint32_t)dW;
     const uint32_t xh = (uint32_t)(dX0 >> 32), wh = (uint32_t)(dW >> 32);
-    for (int it = 0; it < ntiles; it++) {
-      const int st = it % KV_KSTAGES;
+    // W of another group is fetched here as well, when the last logits with the old one have completed (the epilogue is busy
+    // with that tile's exponentials meanwhile)
+    int have = -1, loads = 0;
+    for (int n = 0; ti.next(work); n++) {
+      const int st = n % KV_KSTAGES;
       opaque(xl); opaque(wl);
-      if (it == 0 && !__all_sync(0xffffffffu, mbar_wait(&misc->const_bar, 0, abortp, status))) break;
-      if (!__all_sync(0xffffffffu, mbar_wait(&misc->convK[st], (it / KV_KSTAGES) & 1, abortp, status))) break;
-      if (it > 0 && !__all_sync(0xffffffffu, mbar_wait(&misc->logits_free, (it - 1) & 1, abortp, status))) break;
+      if (const int g = ti.first() ? group(ti.bh) : have; g != have) {
+        have = g;
+        if (n > 0 && !__all_sync(0xffffffffu, mbar_wait(&misc->logits_full, (n - 1) & 1, abortp, status))) break;
+        if (lane == 0) {
+          mbar_expect_tx(&misc->const_bar, IMG_W_BYTES);
+          bulk_load(sm + KvSmem::W, images + ((size_t)g * 2 + 1) * IMG_BYTES + IMG_WH, IMG_W_BYTES, &misc->const_bar);   // side 2 (keys)
+        }
+        __syncwarp();
+        if (!__all_sync(0xffffffffu, mbar_wait(&misc->const_bar, loads++ & 1, abortp, status, false))) break;
+      }
+      if (!__all_sync(0xffffffffu, mbar_wait(&misc->convK[st], (n / KV_KSTAGES) & 1, abortp, status))) break;
+      if (n > 0 && !__all_sync(0xffffffffu, mbar_wait(&misc->logits_free, (n - 1) & 1, abortp, status))) break;
       tcgen05_fence_after();
       if (elect_one()) {
 #pragma unroll
@@ -240,15 +257,17 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     uint32_t pl = (uint32_t)dPhi, v0l = (uint32_t)dVst0, v1l = (uint32_t)dVst1;
     const uint32_t ph = (uint32_t)(dPhi >> 32), v0h = (uint32_t)(dVst0 >> 32), v1h = (uint32_t)(dVst1 >> 32);
     bool ok = true;
-    for (int it = 0; ok && it < ntiles; it++) {
-      const int st = it & 1;
+    for (int n = 0, pieces = 0; ok && ti.next(work); n++) {
+      const int st = n & 1;
       opaque(pl); opaque(v0l); opaque(v1l);
-      if (!__all_sync(0xffffffffu, mbar_wait(&misc->fullV[st], (it >> 1) & 1, abortp, status))) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(&misc->fullV[st], (n >> 1) & 1, abortp, status))) break;
       const uint32_t vl = st ? v1l : v0l, vh = st ? v1h : v0h;
-      const uint32_t acc0 = it > 0 ? 1u : 0u;
+      const uint32_t acc0 = ti.first() ? 0u : 1u;
+      if (ti.first()) pieces++;
 #pragma unroll
       for (int hh = 0; hh < 2; hh++) {
-        if (!__all_sync(0xffffffffu, mbar_wait(&misc->phi_full[hh], it & 1, abortp, status))) { ok = false; break; }
+        if (ti.first() && !__all_sync(0xffffffffu, mbar_wait(&misc->acc_free[hh], pieces & 1, abortp, status))) { ok = false; break; }
+        if (!__all_sync(0xffffffffu, mbar_wait(&misc->phi_full[hh], n & 1, abortp, status))) { ok = false; break; }
         tcgen05_fence_after();
         if (elect_one()) {
 #pragma unroll
@@ -273,11 +292,8 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
     const uint32_t acc_addr = lane_addr + KV_COL_ACC + hf * TC_NV;      // this thread's lane: feature hf * 128 + row
     int* tmax = misc->tile_max[hf];
-    const float* cptr = crow + (size_t)bh * Lpad + (size_t)tile0 * TILE + row;
     float s = 0.f;
-    float cj = ntiles > 0 ? cptr[0] : 0.f;
     bool alive = true;
-    if (KV_TURNS && hf == 1) mbar_arrive_warp(&misc->turn[0], lane);     // half 0 goes first
     // accumulator of this half -> partial `slot` (the contraction that feeds it has completed)
     auto write_partial = [&](size_t slot) {
       __syncwarp();
@@ -298,12 +314,61 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       if (q == 0 && lane == 0) shifts[slot * 2 + hf] = s;
       tcgen05_fence_before();
     };
-    for (int it = 0; it < ntiles && alive; it++) {
-      FS_DBG(tile0 + it < total_tiles && (size_t)tile0 * TILE + (size_t)(it + 1) * TILE <= (size_t)Lpad, status);
+    // A unit that this block has all of needs no merging: its operands (see merge_kernel) are written from here.  The
+    // scales' exponents are relative to the first tile's shift of half 0, which half 0 has set before its share of that
+    // tile's contraction, and so before the contraction that half 1 has waited for.
+    auto write_merged = [&](int bh, int g, float ref) {
+      __syncwarp();
+      tcgen05_fence_after();
+      const int m = hf * 128 + row;
+      const float* a2 = reinterpret_cast<const float*>(images + (size_t)g * 2 * IMG_BYTES + IMG_A2);
+      const float rel = a2[m] - a2[0];             // (on its way during the pass over the accumulator)
+      float am = 0.f;
+#pragma unroll
+      for (int c = 0; c < 5; c++) {
+        uint32_t a[16];
+        tmem_ld16(acc_addr + c * 16, a);
+        tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 16; j++) am = fmaxf(am, fabsf(__uint_as_float(a[j])));
+      }
+      int ex = 0;
+      if (am > 0.f && isfinite(am)) frexpf(am, &ex);
+      const float sc = exp2f((float)-ex);
+      uint8_t* out = merged + (size_t)bh * MRG_BYTES;
+      uint8_t* kcol = out + (m >> 6) * KVT_BLOCK_BYTES;
+#pragma unroll
+      for (int c = 0; c < 5; c++) {
+        uint32_t a[16];
+        tmem_ld16(acc_addr + c * 16, a);
+        tmem_wait_ld();
+        // (rows 65..79 are products with the zero columns of the ones tile)
+#pragma unroll
+        for (int j = 0; j < 16; j++)
+          *reinterpret_cast<__half*>(kcol + sw128_offset(c * 16 + j, m & 63)) = __float2half_rn(__uint_as_float(a[j]) * sc);
+      }
+      write_g(out + MRG_GOP, m, (float)ex + (s - ref) + rel);
+      tcgen05_fence_before();
+    };
+    // Piece by piece, tile by tile.  Next to the 128 logits of a tile there is no register for the iterator in the inner loop
+    // (two spilled words, reloaded all over the unrolled code, make a tile half as long again), so its position waits in
+    // shared memory.  n: tiles of this block so far.
+    int n = 0, pieces = 0;
+    if (lane == 0) misc->cursor[warp] = ti.c;
+    __syncwarp();
+    while (alive) {
+    ti.begin(work, blockIdx.x, gridDim.x);
+    ti.c = *(volatile int*)&misc->cursor[warp];
+    if (!ti.next_piece(work)) break;
+    const float* cptr = crow + (size_t)ti.bh * Lpad + (size_t)ti.tile0 * TILE + row;
+    const int ntiles = ti.ntiles;
+    int left = L - ti.tile0 * TILE - row;        // keys from this thread's row on
+    float cj = cptr[0];
+    for (int it = 0; it < ntiles; it++, n++, left -= TILE) {
       FS_DBG(KV_COL_ACC + hf * TC_NV + TC_NV <= TMEM_COLS && row < TILE, status);
       FS_DBG(KvSmem::PHI + hf * 2 * TILE_BYTES + TILE_BYTES + row * 128 + 128 <= KvSmem::MISC, status);
       const float cnext = it + 1 < ntiles ? cptr[(size_t)(it + 1) * TILE] : 0.f;     // in flight during this tile
-      if (!mbar_wait(&misc->logits_full, it & 1, abortp, status, false)) { alive = false; break; }
+      if (!mbar_wait(&misc->logits_full, n & 1, abortp, status, false)) { alive = false; break; }
       __syncwarp();
       tcgen05_fence_after();
       uint32_t v[128];
@@ -317,7 +382,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       tmem_wait_ld();
       tcgen05_fence_before();
       mbar_arrive_warp(&misc->logits_free, lane);
-      const bool valid = (tile0 + it) * TILE + row < L;
+      const bool valid = left > 0;
       // Exact maximum of this half of the tile, taken BEFORE the exponentials:
       // it overlaps the contraction of the previous tile, and nothing stands between the last exponential and
       // the arrival that starts this tile's contraction.
@@ -334,14 +399,16 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
         const float hm = fmaxf(fmaxf(mxp[0], mxp[1]), fmaxf(mxp[2], mxp[3]));
         float mx = valid ? hm + cj : -INFINITY;
         const int wm = __reduce_max_sync(0xffffffffu, f2ord(mx));       // one instruction for the warp's maximum
-        if (lane == 0) atomicMax(&tmax[it % 3], wm);
-        if (q == 0 && lane == 0) tmax[(it + 1) % 3] = f2ord(-INFINITY);           // next tile's slot; idle since tile it-2
+        if (lane == 0) atomicMax(&tmax[n % 3], wm);
+        if (q == 0 && lane == 0) tmax[(n + 1) % 3] = f2ord(-INFINITY);           // next tile's slot; idle since tile n - 2
         named_bar_sync(1 + hf, HALF_THREADS);
-        tm = ord2f(tmax[it % 3]);
+        tm = ord2f(tmax[n % 3]);
       }
-      // the previous tile's contraction has read the phi half tile and updated the accumulator
-      if (it > 0 && !mbar_wait(&misc->phi_free[hf], (it - 1) & 1, abortp, status, false)) { alive = false; break; }
+      // the previous tile's contraction has read the phi half tile and updated the accumulator (that of a piece's last tile
+      // has been waited for already)
+      if (it > 0 && !mbar_wait(&misc->phi_free[hf], (n - 1) & 1, abortp, status, false)) { alive = false; break; }
       if (it == 0) {
+        if (hf == 0 && row == 0) misc->ref[pieces & 1] = tm;
         s = tm;                      // first tile: the shift is the exact maximum
       } else if (tm - s > SHIFT_HEADROOM_LOG2) {
         // rare (the running maximum grows a handful of times per sequence): the shift moves up to this tile's
@@ -363,7 +430,6 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       }
       uint8_t* prow = sm + KvSmem::PHI + hf * 2 * TILE_BYTES + row * 128;
       const float rc = cj - s;
-      if (KV_TURNS && !mbar_wait(&misc->turn[hf], it & 1, abortp, status, false)) { alive = false; break; }
 #pragma unroll
       for (int c = 0; c < 16; c++) {
         uint32_t p[4];
@@ -385,12 +451,21 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       fence_proxy_async_smem();
       tcgen05_fence_before();
       mbar_arrive_warp(&misc->phi_full[hf], lane);
-      if (KV_TURNS) mbar_arrive_warp(&misc->turn[hf ^ 1], lane);
       cj = cnext;
     }
-    // write this split's partial phi_h^T [V | 1] (rows 0..64 of the state) and its shift
-    if (alive && ntiles > 0 && mbar_wait(&misc->phi_free[hf], (ntiles - 1) & 1, abortp, status, false))
-      write_partial((size_t)bh * nsplit + split);
+    if (!alive) break;
+    // write this piece's partial phi_h^T [V | 1] (rows 0..64 of the state) and its shift
+    if (!mbar_wait(&misc->phi_free[hf], (n - 1) & 1, abortp, status, false)) break;
+    ti.begin(work, blockIdx.x, gridDim.x);
+    ti.c = *(volatile int*)&misc->cursor[warp];
+    ti.next_piece(work);
+    __syncwarp();
+    if (lane == 0) misc->cursor[warp] = ti.c;
+    if (merged != nullptr && ti.ntiles == work.tiles) write_merged(ti.bh, group(ti.bh), *(volatile float*)&misc->ref[pieces & 1]);
+    else write_partial((size_t)ti.slot(work));
+    mbar_arrive_warp(&misc->acc_free[hf], lane);
+    pieces++;
+    }
   }
   tcgen05_fence_before();
   __syncthreads();
@@ -403,8 +478,8 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
 // ------------------------------------------------------------------------------------------
 // query side
 // ------------------------------------------------------------------------------------------
-// Every block first merges the key-side partials of its (batch, head) into shared memory: common
-// shift, sum over the splits, and a scale of its own for every feature.  The query side contracts
+// merge_kernel turns the key-side partials of every (batch, head) into two operands: common shift, sum over the pieces, and a
+// scale of its own for every feature.  The query side contracts
 // phi(Q) with this state in fp16, whose exponent range is narrow, and what a feature contributes to
 // an output is phi(Q)_m times the size of column m of the state.  So every column m is brought to
 // order one by a power of two 2^-e_m, and g_m = e_m + a2_m - max a2 (the per-feature term w^T A w
@@ -414,27 +489,112 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
 // [1, 1, 0, ...] in every row (tensor memory) and whose B operand holds g as an fp16 value and its
 // fp16 remainder.  The query tile is converted from bf16 to fp16 in shared memory (exact for |x| in
 // [2^-14, 65504]), so the logits need one fp16 image of W instead of a bf16 value and its remainder.
+//
+// (Every block of tc_out_kernel used to do this for itself, ten microseconds of loads before its first tile: 768 sequences of
+// 512 tokens, 100 us for the query side; 16 sequences with 32 handed-on states, 85 us.)
+
+constexpr int MERGE_FEATURES = 32, MERGE_ROWS = 9;     // features per block; rows per warp (65 rows over 8 warps)
+
+// grid (TC_M / 32, units; cuts: one per end of a block's range of the stream, since a unit that one block has all of is written
+// by the key side: 768 units of 4 tiles, 6144 blocks 20 us, 1176 blocks 11 us), 512 threads: lane = feature, warp w of either half = rows w, w + 8, ...; the halves take the pieces in
+// turn, three of them (27 loads a thread) in flight: a sum over 40 pieces is bound by the latency of its loads (16 units of 37
+// handed-on states: 26 us with one half and two pieces in flight, 11 us now).
+__global__ void __launch_bounds__(512)
+merge_kernel(const float* __restrict__ partial, const float* __restrict__ shifts, const uint8_t* __restrict__ images, const TileWork work,
+             int blocks, int cuts, int H, int pool, uint8_t* __restrict__ merged) {
+  fs_grid_dependency_wait();
+  __shared__ float fac[MAX_PIECES], red[2][16], amax_s[8][MERGE_FEATURES], other[8][MERGE_ROWS][MERGE_FEATURES];
+  const int tid = threadIdx.x, lane = tid & 31, half = tid >> 8, warp = tid >> 5 & 7;
+  const int bh = cuts ? cut_unit(work, blockIdx.y, blocks) : blockIdx.y;
+  if (bh < 0) return;
+  const int m = blockIdx.x * MERGE_FEATURES + lane, hh = m >> 7;
+  const int g = pool == FSHARP_POOL_PER_BH ? bh : bh % H, n = work_pieces(work, bh, blocks);
+  const size_t slot0 = (size_t)bh * work.slots;
+  const float* a2 = reinterpret_cast<const float*>(images + (size_t)g * 2 * IMG_BYTES + IMG_A2);
+  const float* base = partial + slot0 * TC_NV * TC_M + m;
+  // the first piece's rows are on their way while the shifts are compared
+  float val[MERGE_ROWS];
+#pragma unroll
+  for (int i = 0; i < MERGE_ROWS; i++)
+    val[i] = half < n && warp + 8 * i <= TC_DV ? base[(size_t)(half * TC_NV + warp + 8 * i) * TC_M] : 0.f;
+  float amx = a2[tid & 255], smx = -INFINITY;
+  for (int p = tid; p < 2 * n; p += 512) smx = fmaxf(smx, shifts[slot0 * 2 + p]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    amx = fmaxf(amx, __shfl_xor_sync(0xffffffffu, amx, o));
+    smx = fmaxf(smx, __shfl_xor_sync(0xffffffffu, smx, o));
+  }
+  if (lane == 0) { red[0][tid >> 5] = amx; red[1][tid >> 5] = smx; }
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 16; w++) { amx = fmaxf(amx, red[0][w]); smx = fmaxf(smx, red[1][w]); }
+  if (tid < n) fac[tid] = exp2f(shifts[(slot0 + tid) * 2 + hh] - smx);       // (all features of a block are in one half)
+  __syncthreads();
+  const float f0 = half < n ? fac[half] : 0.f;
+#pragma unroll
+  for (int i = 0; i < MERGE_ROWS; i++) val[i] *= f0;
+#pragma unroll 3
+  for (int p = half + 2; p < n; p += 2) {
+    const float f = fac[p];
+    const float* bp = base + (size_t)p * TC_NV * TC_M;
+#pragma unroll
+    for (int i = 0; i < MERGE_ROWS; i++)
+      if (warp + 8 * i <= TC_DV) val[i] = fmaf(bp[(warp + 8 * i) * TC_M], f, val[i]);
+  }
+  if (half == 1) {
+#pragma unroll
+    for (int i = 0; i < MERGE_ROWS; i++) other[warp][i][lane] = val[i];
+  }
+  __syncthreads();
+  float am = 0.f;
+  if (half == 0) {
+#pragma unroll
+    for (int i = 0; i < MERGE_ROWS; i++) {
+      val[i] += other[warp][i][lane];
+      am = fmaxf(am, fabsf(val[i]));
+    }
+    amax_s[warp][lane] = am;
+  }
+  __syncthreads();
+  if (half == 1) return;
+#pragma unroll
+  for (int w = 0; w < 8; w++) am = fmaxf(am, amax_s[w][lane]);
+  int ex = 0;
+  if (am > 0.f && isfinite(am)) frexpf(am, &ex);                // am = f 2^ex, f in [1/2, 1)
+  const float sc = exp2f((float)-ex);
+  uint8_t* out = merged + (size_t)bh * MRG_BYTES;
+  uint8_t* kcol = out + (m >> 6) * KVT_BLOCK_BYTES;
+#pragma unroll
+  for (int i = 0; i < TC_NV / 8; i++) {
+    const int r = warp + 8 * i;
+    *reinterpret_cast<__half*>(kcol + sw128_offset(r, m & 63)) = __float2half_rn(r <= TC_DV ? val[i < MERGE_ROWS ? i : 0] * sc : 0.f);
+  }
+  if (warp == 0) {
+    write_g(out + MRG_GOP, m, (float)ex + a2[m] - amx);
+  }
+}
+
 constexpr int OUT_STAGES = 3;
 constexpr int WARP_OUT_MMA2 = WARP_MMA + 1, WARP_OUT_CVT = WARP_MMA + 2;
 // Of every four pairs of exponentials, this many run on the multiply-add pipe (exp2_poly2).
 constexpr int OUT_POLY_PAIRS = 1;
 struct OutSmem {
-  // PHI also serves the merge (shifts and their factors) and, 2 KB per epilogue warp inside the rows that warp
-  // itself writes next, the output rows on their way out
+  // PHI also serves, 2 KB per epilogue warp inside the rows that warp itself writes next, the output rows on their way out
   static constexpr uint32_t X0 = 0, WH = OUT_STAGES * TILE_BYTES, PHI = WH + IMG_W_BYTES, KVT = PHI + 4 * TILE_BYTES,
                             ROWMAX = KVT + KVT_BYTES,
                             // g as an MMA operand: [256 features x 16] fp16, no swizzle (the two 16-byte K pieces of a
                             // row 128 bytes apart, 8-row groups 256 bytes apart)
-                            GOP = ROWMAX + 2 * 2 * TILE * 4, GOP_BYTES = TC_M * 32, MISC = GOP + GOP_BYTES, TOTAL = MISC + 256;
+                            GOP = ROWMAX + 2 * 2 * TILE * 4, MISC = GOP + GOP_BYTES, TOTAL = MISC + 256;
 };
 static_assert(OutSmem::PHI % 1024 == 0 && OutSmem::KVT % 1024 == 0 && OutSmem::WH % 1024 == 0, "alignment");
 static_assert(OutSmem::TOTAL + 1024 <= 232448, "shared memory budget");
 
 struct OutMisc {
   // full: the tile has landed; conv: it has been converted to fp16; phi_full[f]: the 64-feature block f of the phi
-  // tile is written (the four warps of its half arrive); g_ready: the merge has written its operands
+  // tile is written (the four warps of its half arrive); one_ready: the A operand of the g step is written;
+  // const_bar: W and g have landed; kvt_bar: the state has
   uint64_t full[OUT_STAGES], conv[OUT_STAGES], empty[OUT_STAGES], logits_full, logits_free, phi_full[TC_M / 64], phi_free, const_bar,
-      g_ready;
+      kvt_bar, one_ready;
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -443,23 +603,22 @@ static_assert(sizeof(OutMisc) <= 256, "misc block");
 constexpr uint32_t OUT_COL_LOGITS = 0, OUT_COL_OUT = 256, OUT_COL_ONE = 496;
 
 __global__ void __launch_bounds__(TC_THREADS, 1)
-tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const uint8_t* __restrict__ images,
-              const float* __restrict__ partial, const float* __restrict__ shifts, int nsplit, int H, int pool, int L,
-              int tiles_per_split,
-              __nv_bfloat16* __restrict__ Y, TensorAddr ay, int* __restrict__ status) {
+tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const uint8_t* __restrict__ images, const uint8_t* __restrict__ merged,
+              int H, int pool, int L, const TileWork work, __nv_bfloat16* __restrict__ Y, TensorAddr ay, int* __restrict__ status) {
   fs_grid_dependency_wait();
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  // (declared with its alignment, so that every address below is a constant: rounded up at run time the base lives in
+  // registers, and next to the 128 logits of a thread it was spilled and reloaded at every barrier)
+  extern __shared__ __align__(1024) uint8_t sm[];
+  if (smem_u32(sm) & 1023u) {                  // uniform over the block, before anything is allocated
+    if (threadIdx.x == 0) atomicExch(status, FSHARP_E_INTERNAL);
+    return;
+  }
   OutMisc* misc = reinterpret_cast<OutMisc*>(sm + OutSmem::MISC);
   float* rowmax = reinterpret_cast<float*>(sm + OutSmem::ROWMAX);   // [tile % 2][half][row]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int split = blockIdx.x, bh = blockIdx.y, b = bh / H, h = bh % H;
-  const int g = pool == FSHARP_POOL_PER_BH ? bh : h;
-  const int total_tiles = (L + TILE - 1) / TILE;
-  const int tile0 = split * tiles_per_split;
-  const int ntiles = min(tiles_per_split, total_tiles - tile0);
-  const uint8_t* img = images + ((size_t)g * 2 + 0) * IMG_BYTES;        // side 1 (queries)
   volatile int* abortp = &misc->abort_flag;
+  TileIter ti;                                 // every warp walks the same tiles; n counts them
+  ti.begin(work, blockIdx.x, gridDim.x);
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < OUT_STAGES; i++) { mbar_init(&misc->full[i], 1); mbar_init(&misc->conv[i], 2); mbar_init(&misc->empty[i], 1); }
@@ -468,7 +627,8 @@ tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const uint8_t* __restrict
     for (int i = 0; i < TC_M / 64; i++) mbar_init(&misc->phi_full[i], EPI_THREADS / 64);
     mbar_init(&misc->phi_free, 1);
     mbar_init(&misc->const_bar, 1);
-    mbar_init(&misc->g_ready, EPI_THREADS / 32);
+    mbar_init(&misc->kvt_bar, 1);
+    mbar_init(&misc->one_ready, EPI_THREADS / 64);
     misc->abort_flag = 0;
     fence_barrier_init();
   }
@@ -503,37 +663,32 @@ tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const uint8_t* __restrict
     return true;
   };
   if (warp == WARP_TMA) {
-    // The whole warp walks the schedule; lane 0 issues the copies.  After the copy of tile it has been issued the
-    // warp converts its half of tile it - 1, which has landed meanwhile.
-    if (lane == 0) {
-      prefetch_tmap(&tmQ);
-      mbar_expect_tx(&misc->const_bar, IMG_W_BYTES);
-      bulk_load(sm + OutSmem::WH, img + IMG_WH, IMG_W_BYTES, &misc->const_bar);
-      for (int it = 0; it < min(ntiles, PREFETCH_TILES); it++) tma_prefetch_4d(&tmQ, 0, (tile0 + it) * TILE, h, b);
-    }
-    int issued = 0;
+    // The whole warp walks the schedule; lane 0 issues the copies.  After the copy of tile n has been issued the
+    // warp converts its half of tile n - 1, which has landed meanwhile.
+    if (lane == 0) prefetch_tmap(&tmQ);
+    int issued = 0, b = 0, h = 0;
     bool okp = true;
-    for (int it = 0; it < ntiles; it++) {
-      const int st = it % OUT_STAGES;
-      if (!__all_sync(0xffffffffu, mbar_wait(&misc->empty[st], ((it / OUT_STAGES) & 1) ^ 1, abortp, status))) { okp = false; break; }
+    for (; okp && ti.next(work); issued++) {
+      const int n = issued, st = n % OUT_STAGES;
+      if (ti.first()) { b = ti.bh / H; h = ti.bh - b * H; }
+      if (!__all_sync(0xffffffffu, mbar_wait(&misc->empty[st], ((n / OUT_STAGES) & 1) ^ 1, abortp, status))) { okp = false; break; }
       if (lane == 0) {
-        if (it + PREFETCH_TILES < ntiles) tma_prefetch_4d(&tmQ, 0, (tile0 + it + PREFETCH_TILES) * TILE, h, b);
         mbar_expect_tx(&misc->full[st], TILE_BYTES);
-        tma_load_4d(sm + OutSmem::X0 + st * TILE_BYTES, &tmQ, &misc->full[st], 0, (tile0 + it) * TILE, h, b);
+        tma_load_4d(sm + OutSmem::X0 + st * TILE_BYTES, &tmQ, &misc->full[st], 0, ti.tile() * TILE, h, b);
       }
-      issued = it + 1;
-      if (it > 0 && !convert_half(it - 1, 1)) { okp = false; break; }
+      if (lane == 0 && ti.idx + PREFETCH_TILES < ti.ntiles)
+        tma_prefetch_4d(&tmQ, 0, (ti.tile() + PREFETCH_TILES) * TILE, h, b);
+      if (n > 0) okp = convert_half(n - 1, 1);
     }
-    if (okp && ntiles > 0) convert_half(ntiles - 1, 1);
+    if (okp && issued > 0) convert_half(issued - 1, 1);
     // no copy of this block may still be in flight when it exits
     if (lane == 0) {
-      mbar_wait(&misc->const_bar, 0, abortp, status, false);
-      for (int it = max(0, issued - OUT_STAGES); it < issued; it++)
-        mbar_wait(&misc->full[it % OUT_STAGES], (it / OUT_STAGES) & 1, abortp, status, false);
+      for (int n = max(0, issued - OUT_STAGES); n < issued; n++)
+        mbar_wait(&misc->full[n % OUT_STAGES], (n / OUT_STAGES) & 1, abortp, status, false);
     }
   } else if (warp == WARP_OUT_CVT) {
-    for (int it = 0; it < ntiles; it++)
-      if (!convert_half(it, 0)) break;
+    for (int n = 0; ti.next(work); n++)
+      if (!convert_half(n, 0)) break;
   } else if (warp == WARP_MMA) {
     // ---------------- logits MMAs: the whole warp walks the schedule, one elected lane issues
     constexpr uint32_t ID_LOGITS = idesc_f16(128, TC_M, 0, 0);
@@ -554,15 +709,28 @@ tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const uint8_t* __restrict
       __syncwarp();
     };
 #define OUT_WAIT(bar, par) if (!__all_sync(0xffffffffu, mbar_wait((bar), (par), abortp, status))) break
-    for (int it = 0; it < ntiles; it++) {
-      const int st = it % OUT_STAGES;
+    bool ready = __all_sync(0xffffffffu, mbar_wait(&misc->one_ready, 0, abortp, status));
+    int unit = -1, have = -1, loads = 0;
+    for (int n = 0; ready && ti.next(work); n++) {
+      const int st = n % OUT_STAGES;
       opaque(xl); opaque(wl); opaque(gl);
-      if (it == 0) {
-        OUT_WAIT(&misc->const_bar, 0);
-        OUT_WAIT(&misc->g_ready, 0);
+      if (ti.bh != unit) {
+        // another (batch, head): its g, and its W if the group changes, once the last logits with the old ones have completed
+        // (the epilogue is busy with that tile's exponentials meanwhile)
+        unit = ti.bh;
+        const int g = pool == FSHARP_POOL_PER_BH ? unit : unit % H;
+        if (n > 0) OUT_WAIT(&misc->logits_full, (n - 1) & 1);
+        if (lane == 0) {
+          mbar_expect_tx(&misc->const_bar, GOP_BYTES + (g != have ? IMG_W_BYTES : 0));
+          bulk_load(sm + OutSmem::GOP, merged + (size_t)unit * MRG_BYTES + MRG_GOP, GOP_BYTES, &misc->const_bar);
+          if (g != have) bulk_load(sm + OutSmem::WH, images + (size_t)g * 2 * IMG_BYTES + IMG_WH, IMG_W_BYTES, &misc->const_bar);   // side 1 (queries)
+        }
+        __syncwarp();
+        have = g;
+        if (!__all_sync(0xffffffffu, mbar_wait(&misc->const_bar, loads++ & 1, abortp, status, false))) break;
       }
-      OUT_WAIT(&misc->conv[st], (it / OUT_STAGES) & 1);
-      if (it > 0) OUT_WAIT(&misc->logits_free, (it - 1) & 1);
+      OUT_WAIT(&misc->conv[st], (n / OUT_STAGES) & 1);
+      if (n > 0) OUT_WAIT(&misc->logits_free, (n - 1) & 1);
       // (Every barrier this warp waits on is one whose next phase cannot complete before this warp has moved on: a
       // wait by parity on a barrier that may run two phases ahead of its waiter would never end.  phi_free is such
       // a barrier for this warp, so the logits are not ordered behind the contraction of an earlier tile.)
@@ -580,16 +748,29 @@ tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const uint8_t* __restrict
     uint32_t pl = (uint32_t)dPhi, kl = (uint32_t)dKvt;
     const uint32_t ph = (uint32_t)(dPhi >> 32), kh = (uint32_t)(dKvt >> 32);
     bool ok = true;
-    for (int it = 0; ok && it < ntiles; it++) {
+    int unit = -1, loads = 0;
+    for (int n = 0; ok && ti.next(work); n++) {
       opaque(pl); opaque(kl);
+      if (ti.bh != unit) {
+        // another state, once the last contraction with the old one has completed (phi_free is committed by this warp: it
+        // cannot run ahead); it lands under the first tile's exponentials
+        unit = ti.bh;
+        if (n > 0 && !__all_sync(0xffffffffu, mbar_wait(&misc->phi_free, (n - 1) & 1, abortp, status))) break;
+        if (lane == 0) {
+          mbar_expect_tx(&misc->kvt_bar, KVT_BYTES);
+          bulk_load(sm + OutSmem::KVT, merged + (size_t)unit * MRG_BYTES, KVT_BYTES, &misc->kvt_bar);
+        }
+        __syncwarp();
+        if (!__all_sync(0xffffffffu, mbar_wait(&misc->kvt_bar, loads++ & 1, abortp, status, false))) break;
+      }
       // An epilogue thread arrives on its half's first block only after it has read the previous tile's output
       // row, so the accumulator may be overwritten once the first blocks of BOTH halves are in.
-      if (!__all_sync(0xffffffffu, mbar_wait(&misc->phi_full[0], it & 1, abortp, status))) break;
-      if (!__all_sync(0xffffffffu, mbar_wait(&misc->phi_full[2], it & 1, abortp, status))) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(&misc->phi_full[0], n & 1, abortp, status))) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(&misc->phi_full[2], n & 1, abortp, status))) break;
 #pragma unroll
       for (int o = 0; o < TC_M / 64; o++) {
         const int fb = ((o & 1) << 1) | (o >> 1);      // 0, 2, 1, 3
-        if (o >= 2 && !__all_sync(0xffffffffu, mbar_wait(&misc->phi_full[fb], it & 1, abortp, status))) { ok = false; break; }
+        if (o >= 2 && !__all_sync(0xffffffffu, mbar_wait(&misc->phi_full[fb], n & 1, abortp, status))) { ok = false; break; }
         tcgen05_fence_after();
         if (elect_one()) {
 #pragma unroll
@@ -611,69 +792,18 @@ tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const uint8_t* __restrict
     const int q = warp & 3, hf = warp >> 2;
     const int row = q * 32 + lane;
     const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
-    __nv_bfloat16* Yb = Y + b * ay.sb + h * ay.sh;
     bool alive = true;
-    {
-      // merge (see above); thread = feature m, whose half (m / 128) is also the thread's half below, so the
-      // arrivals that release a 64-feature block to the MMA warp cover the writers of that block of the state
-      const int m = threadIdx.x, hh = m >> 7;
-      float* sft = reinterpret_cast<float*>(sm + OutSmem::PHI);          // shifts, then their factors (the phi tile is idle)
-      float* red = sft + 2 * MAX_KEY_SPLIT;
-      const float a2m = reinterpret_cast<const float*>(img + IMG_A2)[m];
-      float wmx = a2m;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) wmx = fmaxf(wmx, __shfl_xor_sync(0xffffffffu, wmx, o));
-      if (lane == 0) red[warp] = wmx;
-      if (m < 2 * nsplit) sft[m] = shifts[(size_t)bh * nsplit * 2 + m];
-      named_bar_sync(1, EPI_THREADS);
-      float a2max = red[0], smax = -INFINITY;
-#pragma unroll
-      for (int i = 1; i < EPI_THREADS / 32; i++) a2max = fmaxf(a2max, red[i]);
-      for (int p = 0; p < 2 * nsplit; p++) smax = fmaxf(smax, sft[p]);
-      named_bar_sync(1, EPI_THREADS);
-      if (m < 2 * nsplit) sft[m] = exp2f(sft[m] - smax);
-      named_bar_sync(1, EPI_THREADS);
-      const float* base = partial + (size_t)bh * nsplit * TC_NV * TC_M + m;
-      float val[TC_DV + 1];
-#pragma unroll
-      for (int n = 0; n <= TC_DV; n++) val[n] = 0.f;
-      for (int p = 0; p < nsplit; p++) {        // 65 independent loads in flight per split
-        const float f = sft[2 * p + hh];
-        const float* bp = base + (size_t)p * TC_NV * TC_M;
-#pragma unroll
-        for (int n = 0; n <= TC_DV; n++) val[n] = fmaf(bp[n * TC_M], f, val[n]);
-      }
-      float amax = 0.f;
-#pragma unroll
-      for (int n = 0; n <= TC_DV; n++) amax = fmaxf(amax, fabsf(val[n]));
-      int ex = 0;
-      if (amax > 0.f && isfinite(amax)) frexpf(amax, &ex);          // amax = f 2^ex, f in [1/2, 1)
-      const float sc = exp2f((float)-ex);
-      uint8_t* kcol = sm + OutSmem::KVT + (m >> 6) * KVT_BLOCK_BYTES;
-#pragma unroll
-      for (int n = 0; n < TC_NV; n++)
-        *reinterpret_cast<__half*>(kcol + sw128_offset(n, m & 63)) = __float2half_rn(n <= TC_DV ? val[n <= TC_DV ? n : 0] * sc : 0.f);
-      // g_m as an fp16 value and its fp16 remainder: K elements 0 and 1 of row m of the operand
-      {
-        const float gm = (float)ex + a2m - a2max;
-        const __half hi = __float2half_rn(gm), lo = __float2half_rn(gm - __half2float(hi));
-        uint8_t* rowp = sm + OutSmem::GOP + (m >> 3) * 256 + (m & 7) * 16;
-        *reinterpret_cast<uint4*>(rowp) = make_uint4((uint32_t)__half_as_ushort(hi) | ((uint32_t)__half_as_ushort(lo) << 16), 0, 0, 0);
-        *reinterpret_cast<uint4*>(rowp + 128) = make_uint4(0, 0, 0, 0);
-      }
-      // the A operand of that step: 1, 1, 0, ... (fp16) in every row
-      if (hf == 0) {
-        asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %2, %2, %2, %2, %2, %2};" ::"r"(lane_addr + OUT_COL_ONE),
-                     "r"(0x3C003C00u), "r"(0u) : "memory");
-        tmem_wait_st();
-      }
-      named_bar_sync(1, EPI_THREADS);          // the shifts' factors have been read: the phi tile may be written
-      fence_proxy_async_smem();
+    // the A operand of the g step: 1, 1, 0, ... (fp16) in every row
+    if (hf == 0) {
+      asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %2, %2, %2, %2, %2, %2};" ::"r"(lane_addr + OUT_COL_ONE),
+                   "r"(0x3C003C00u), "r"(0u) : "memory");
+      tmem_wait_st();
       tcgen05_fence_before();
-      mbar_arrive_warp(&misc->g_ready, lane);
+      mbar_arrive_warp(&misc->one_ready, lane);
     }
-    // Y rows of tile j (its contraction has completed): 32 of the 64 columns per thread
-    auto write_out = [&](int j) {
+    // Y rows of a tile (its contraction has completed): 32 of the 64 columns per thread
+    auto write_out = [&](int bh, int tile) {
+      __nv_bfloat16* Yb = Y + (bh / H) * ay.sb + (bh % H) * ay.sh;
       __syncwarp();
       tcgen05_fence_after();
       uint32_t n0[32], d0[16];
@@ -682,7 +812,7 @@ tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const uint8_t* __restrict
       tmem_ld16(base + hf * 32 + 16, reinterpret_cast<uint32_t(&)[16]>(n0[16]));
       tmem_ld16(base + TC_DV, d0);
       tmem_wait_ld();
-      const int64_t r0 = (int64_t)(tile0 + j) * TILE + q * 32;       // first row of this warp
+      const int64_t r0 = (int64_t)tile * TILE + q * 32;       // first row of this warp
       const float den = __uint_as_float(d0[0]);
       if (r0 + lane < L && (!(den > 0.f) || !isfinite(den))) atomicExch(status, FSHARP_E_NONFINITE);
       float inv;                       // outputs are rounded to bf16: the approximate reciprocal (1 ulp) is exact enough
@@ -707,10 +837,11 @@ tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const uint8_t* __restrict
       }
       __syncwarp();
     };
-    for (int it = 0; it < ntiles && alive; it++) {
-      FS_DBG(tile0 + it < total_tiles && OUT_COL_OUT + TC_NV <= OUT_COL_ONE && OUT_COL_ONE + 8 <= TMEM_COLS, status);
+    int n = 0, last_bh = 0, last_tile = 0;
+    for (; alive && ti.next(work); n++) {
+      FS_DBG(ti.tile() * TILE < L && OUT_COL_OUT + TC_NV <= OUT_COL_ONE && OUT_COL_ONE + 8 <= TMEM_COLS, status);
       FS_DBG(OutSmem::PHI + hf * 2 * TILE_BYTES + TILE_BYTES + row * 128 + 128 <= OutSmem::KVT && row < TILE, status);
-      if (!mbar_wait(&misc->logits_full, it & 1, abortp, status, false)) { alive = false; break; }
+      if (!mbar_wait(&misc->logits_full, n & 1, abortp, status, false)) { alive = false; break; }
       __syncwarp();
       tcgen05_fence_after();
       uint32_t v[128];
@@ -731,14 +862,16 @@ tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const uint8_t* __restrict
       float mx = fmaxf(fmaxf(mxp[0], mxp[1]), fmaxf(mxp[2], mxp[3]));
       // the other half of the row: its thread sits in warp q of the other warpgroup (slots rotate over two tiles:
       // a slot is rewritten only after both warps have passed the next tile's barrier)
-      rowmax[(it & 1) * 2 * TILE + hf * TILE + row] = mx;
+      rowmax[(n & 1) * 2 * TILE + hf * TILE + row] = mx;
       named_bar_sync(2 + q, 64);
-      mx = fmaxf(mx, rowmax[(it & 1) * 2 * TILE + (hf ^ 1) * TILE + row]);
-      if (it > 0) {
+      mx = fmaxf(mx, rowmax[(n & 1) * 2 * TILE + (hf ^ 1) * TILE + row]);
+      if (n > 0) {
         // contraction of the previous tile done: its phi tile and its outputs are ours again
-        if (!mbar_wait(&misc->phi_free, (it - 1) & 1, abortp, status, false)) { alive = false; break; }
-        write_out(it - 1);
+        if (!mbar_wait(&misc->phi_free, (n - 1) & 1, abortp, status, false)) { alive = false; break; }
+        write_out(last_bh, last_tile);
       }
+      last_bh = ti.bh;
+      last_tile = ti.tile();
       uint8_t* prow = sm + OutSmem::PHI + hf * 2 * TILE_BYTES + row * 128;
 #pragma unroll
       for (int c = 0; c < 16; c++) {
@@ -766,7 +899,7 @@ tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const uint8_t* __restrict
         }
       }
     }
-    if (alive && ntiles > 0 && mbar_wait(&misc->phi_free, (ntiles - 1) & 1, abortp, status, false)) write_out(ntiles - 1);
+    if (alive && n > 0 && mbar_wait(&misc->phi_free, (n - 1) & 1, abortp, status, false)) write_out(last_bh, last_tile);
   }
   tcgen05_fence_before();
   __syncthreads();
@@ -793,6 +926,20 @@ int pick_split(int units, int tiles, int sms, int max_split, int* tiles_per_spli
   return best;
 }
 
+// One block per SM (or per tile), every block the same number of tiles.  A piece costs a block about as much as a tile, so
+// cutting a unit once more than equal ranges need never pays; more than MAX_PIECES pieces of a unit are not merged.
+TileWork stream_work(const fsharp_ctx* ctx, int units, int tiles, int* blocks) {
+  const int64_t total = (int64_t)units * tiles;
+  int64_t n = total < ctx->sm_count ? total : ctx->sm_count;
+  const int64_t most = (int64_t)units * (MAX_PIECES - 2);              // (a unit's pieces: its share of the blocks and one)
+  if (n > most) n = most;
+  const int least = (int)(total / n);
+  TileWork w{units, tiles, tiles, 1, 1, (tiles + least - 1) / least + 1};
+  if (w.slots > tiles) w.slots = tiles;
+  if (blocks) *blocks = (int)n;
+  return w;
+}
+
 }  // namespace
 
 // ------------------------------------------------------------------------------------------
@@ -801,15 +948,15 @@ int pick_split(int units, int tiles, int sms, int max_split, int* tiles_per_spli
 namespace tchost {
 int make_map_tokens(CUtensorMap* map, const void* base, TensorAddr a, int B, int H, int L, int inner);
 }  // namespace tchost
-int fs_tc_rowterm(fsharp_ctx* ctx, const void* K, const fsharp_dims* dm, const uint8_t* images, const int* flags, int Lpad,
-                  int tiles_per_split, int nsplit, float* crow);
+int fs_tc_rowterm(fsharp_ctx* ctx, const void* K, const fsharp_dims* dm, const uint8_t* images, const int* flags, int Lpad, float* crow);
 size_t fs_tc_bidir_scratch_bytes(const fsharp_ctx* ctx, const fsharp_dims* dm);
 int fs_tc_bidir(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const fsharp_dims* dm, const uint8_t* images,
                 const int* flags, void* Y, WsAlloc* ws);
 int fs_tc_key_side(fsharp_ctx* ctx, const void* K, const void* V, const fsharp_dims* dm, const uint8_t* images,
                    const int* flags, int tiles_per_split, int nsplit, float* crow, float* partial, float* shifts);
+size_t fs_tc_query_side_scratch_bytes(const fsharp_dims* dm);
 int fs_tc_query_side(fsharp_ctx* ctx, const void* Q, const fsharp_dims* dm, const uint8_t* images, const float* partial,
-                     const float* shifts, int nsplit, void* Y);
+                     const float* shifts, int nsplit, void* Y, WsAlloc* ws);
 int fs_tc_key_state_splits(const fsharp_ctx* ctx, const fsharp_dims* dm, int* tiles_per_split);
 size_t fs_tc_key_state_scratch_bytes(const fsharp_ctx* ctx, const fsharp_dims* dm);
 int fs_tc_key_state(fsharp_ctx* ctx, const void* K, const void* V, const fsharp_dims* dm, const uint8_t* images,
@@ -846,10 +993,53 @@ size_t fs_tc_bidir_scratch_bytes(const fsharp_ctx* ctx, const fsharp_dims* dm) {
   const size_t BH = (size_t)dm->B * dm->H;
   const size_t G = fs_groups(dm);
   return ws_round(G * 2 * IMG_BYTES) + ws_round(G * 2 * FLAG_WORDS * 4 + 64) +
-         ws_round(BH * MAX_KEY_SPLIT * TC_M * TC_NV * 4) + 2 * ws_round(BH * MAX_KEY_SPLIT * 2 * 4) +
-         ws_round(BH * (size_t)((dm->Lk + TILE - 1) / TILE) * TILE * 4) +
-         ws_round(BH * TC_NV * TC_M * 2) + ws_round(BH * TC_M * 4);
+         ws_round(BH * (size_t)stream_work(ctx, (int)BH, (dm->Lk + TILE - 1) / TILE, nullptr).slots * (TC_M * TC_NV * 4)) +
+         ws_round(BH * (size_t)((dm->Lk + TILE - 1) / TILE + 1) * 2 * 4) + ws_round(BH * (size_t)((dm->Lk + TILE - 1) / TILE) * TILE * 4) + ws_round(BH * MRG_BYTES);
 }
+
+namespace {
+int key_side(fsharp_ctx* ctx, const void* K, const void* V, const fsharp_dims* dm, const uint8_t* images, const int* flags,
+             const TileWork& work, int blocks, float* crow, float* partial, float* shifts, uint8_t* merged) {
+  FS_RANGE("key side");
+  const int B = dm->B, H = dm->H, Lk = dm->Lk;
+  const int Lpad = (Lk + TILE - 1) / TILE * TILE;
+  FS_TRY(fs_tc_rowterm(ctx, K, dm, images, flags, Lpad, crow));
+  CUtensorMap tmK, tmV;
+  FS_TRY(tchost::make_map_tokens(&tmK, K, fs_addr(dm->k_stride, H, Lk, dm->d), B, H, Lk, dm->d));
+  FS_TRY(tchost::make_map_tokens(&tmV, V, fs_addr(dm->v_stride, H, Lk, dm->dv), B, H, Lk, dm->dv));
+  FS_CUDA_OK(cudaFuncSetAttribute(tc_kv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KvSmem::TOTAL + 1024));
+  FS_TIME_BEGIN(ctx, FS_K_TC_KV);
+  (void)fs_launch_chained(tc_kv_kernel, dim3(blocks), dim3(TC_THREADS), KvSmem::TOTAL + 1024, ctx->stream,
+      tmK, tmV, images, crow, H, dm->pool, Lk, Lpad, work, partial, shifts, merged, ctx->d_status);
+  FS_TIME_END(ctx);
+  FS_LAUNCH_CHECK(ctx);
+  return FSHARP_OK;
+}
+
+int query_side(fsharp_ctx* ctx, const void* Q, const fsharp_dims* dm, const uint8_t* images, const float* partial, const float* shifts,
+               const TileWork& keys, int key_blocks, int cuts, uint8_t* merged, void* Y) {
+  FS_RANGE("query side");
+  const int B = dm->B, H = dm->H, BH = B * H, Lq = dm->Lq;
+  if (const int n = cuts ? key_blocks - 1 : BH; n > 0) {
+    FS_TIME_BEGIN(ctx, FS_K_TC_MERGE);
+    (void)fs_launch_chained(merge_kernel, dim3(TC_M / MERGE_FEATURES, n), dim3(512), 0, ctx->stream, partial, shifts, images, keys,
+                            key_blocks, cuts, H, dm->pool, merged);
+    FS_TIME_END(ctx);
+    FS_LAUNCH_CHECK(ctx);
+  }
+  CUtensorMap tmQ;
+  FS_TRY(tchost::make_map_tokens(&tmQ, Q, fs_addr(dm->q_stride, H, Lq, dm->d), B, H, Lq, dm->d));
+  FS_CUDA_OK(cudaFuncSetAttribute(tc_out_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OutSmem::TOTAL + 1024));
+  int blocks = 0;
+  const TileWork work = stream_work(ctx, BH, (Lq + TILE - 1) / TILE, &blocks);
+  FS_TIME_BEGIN(ctx, FS_K_TC_OUT);
+  (void)fs_launch_chained(tc_out_kernel, dim3(blocks), dim3(TC_THREADS), OutSmem::TOTAL + 1024, ctx->stream,
+      tmQ, images, merged, H, dm->pool, Lq, work, (__nv_bfloat16*)Y, fs_addr(dm->y_stride, H, Lq, dm->dv), ctx->d_status);
+  FS_TIME_END(ctx);
+  FS_LAUNCH_CHECK(ctx);
+  return FSHARP_OK;
+}
+}  // namespace
 
 // Key side: the per-key quadratic term, then the feature / contraction kernel.  crow: [B*H][Lpad] floats,
 // Lpad = ceil(Lk / 128) * 128; partial: [B*H][nsplit][80][256] floats; shifts: [B*H][nsplit][2].
@@ -857,56 +1047,31 @@ size_t fs_tc_bidir_scratch_bytes(const fsharp_ctx* ctx, const fsharp_dims* dm) {
 // first nsplit * tiles_per_split tiles (the causal path asks for the segments that have a successor only).
 int fs_tc_key_side(fsharp_ctx* ctx, const void* K, const void* V, const fsharp_dims* dm, const uint8_t* images,
                    const int* flags, int tiles_per_split, int nsplit, float* crow, float* partial, float* shifts) {
-  FS_RANGE("key side");
-  const int B = dm->B, H = dm->H, Lk = dm->Lk;
-  const int Lpad = (Lk + TILE - 1) / TILE * TILE;
-  FS_TRY(fs_tc_rowterm(ctx, K, dm, images, flags, Lpad, tiles_per_split, nsplit, crow));
-  CUtensorMap tmK, tmV;
-  FS_TRY(tchost::make_map_tokens(&tmK, K, fs_addr(dm->k_stride, H, Lk, dm->d), B, H, Lk, dm->d));
-  FS_TRY(tchost::make_map_tokens(&tmV, V, fs_addr(dm->v_stride, H, Lk, dm->dv), B, H, Lk, dm->dv));
-  FS_CUDA_OK(cudaFuncSetAttribute(tc_kv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KvSmem::TOTAL + 1024));
-  FS_TIME_BEGIN(ctx, FS_K_TC_KV);
-  (void)fs_launch_chained(tc_kv_kernel, dim3(nsplit, B * H), dim3(TC_THREADS), KvSmem::TOTAL + 1024, ctx->stream,
-      tmK, tmV, images, crow, H, dm->pool, Lk, Lpad, tiles_per_split, nsplit, partial, shifts, ctx->d_status);
-  FS_TIME_END(ctx);
-  FS_LAUNCH_CHECK(ctx);
-  return FSHARP_OK;
+  const int BH = dm->B * dm->H;
+  const TileWork work{BH, (dm->Lk + TILE - 1) / TILE, tiles_per_split, nsplit, 0, nsplit};
+  const int blocks = BH * nsplit < ctx->sm_count ? BH * nsplit : ctx->sm_count;
+  return key_side(ctx, K, V, dm, images, flags, work, blocks, crow, partial, shifts, nullptr);
 }
 
 int fs_tc_bidir(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const fsharp_dims* dm, const uint8_t* images,
                 const int* flags, void* Y, WsAlloc* ws) {
-  const int B = dm->B, H = dm->H, BH = B * H, Lq = dm->Lq, Lk = dm->Lk;
-
-  // key side: the split of the key range that minimises (waves of blocks) x (tiles per block)
-  const int ktiles = (Lk + TILE - 1) / TILE;
-  int tps = 0;
-  int nsplit = pick_split(BH, ktiles, ctx->sm_count, MAX_KEY_SPLIT, &tps);
-  float* partial = ws->take<float>((size_t)BH * MAX_KEY_SPLIT * TC_M * TC_NV);
-  float* shifts = ws->take<float>((size_t)BH * MAX_KEY_SPLIT * 2);
-  const int Lpad = ktiles * TILE;
-  float* crow = ws->take<float>((size_t)BH * Lpad);
-  FS_TRY(fs_tc_key_side(ctx, K, V, dm, images, flags, tps, nsplit, crow, partial, shifts));
-
-  return fs_tc_query_side(ctx, Q, dm, images, partial, shifts, nsplit, Y);
+  const int BH = dm->B * dm->H, Lk = dm->Lk;
+  int blocks = 0;
+  const TileWork work = stream_work(ctx, BH, (Lk + TILE - 1) / TILE, &blocks);
+  float* partial = ws->take<float>((size_t)BH * work.slots * TC_M * TC_NV);
+  float* shifts = ws->take<float>((size_t)BH * work.slots * 2);
+  float* crow = ws->take<float>((size_t)BH * work.tiles * TILE);
+  uint8_t* merged = ws->take<uint8_t>((size_t)BH * MRG_BYTES);
+  FS_TRY(key_side(ctx, K, V, dm, images, flags, work, blocks, crow, partial, shifts, merged));
+  return query_side(ctx, Q, dm, images, partial, shifts, work, blocks, 1, merged, Y);
 }
 
 // Query side alone: partial [B*H][nsplit][80][256], shifts [B*H][nsplit][2] are key-side sums of disjoint key ranges
-// (of this call's key side, or handed in by the caller).
+// handed in by the caller.
+size_t fs_tc_query_side_scratch_bytes(const fsharp_dims* dm) { return ws_round((size_t)dm->B * dm->H * MRG_BYTES); }
 int fs_tc_query_side(fsharp_ctx* ctx, const void* Q, const fsharp_dims* dm, const uint8_t* images, const float* partial,
-                     const float* shifts, int nsplit, void* Y) {
-  FS_RANGE("query side");
-  const int B = dm->B, H = dm->H, BH = B * H, Lq = dm->Lq;
+                     const float* shifts, int nsplit, void* Y, WsAlloc* ws) {
   if (nsplit < 1 || nsplit > MAX_KEY_SPLIT) return FSHARP_E_LIMIT;
-  CUtensorMap tmQ;
-  FS_TRY(tchost::make_map_tokens(&tmQ, Q, fs_addr(dm->q_stride, H, Lq, dm->d), B, H, Lq, dm->d));
-  FS_CUDA_OK(cudaFuncSetAttribute(tc_out_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OutSmem::TOTAL + 1024));
-  const int qtiles = (Lq + TILE - 1) / TILE;
-  int qtps = 0;
-  int qsplit = pick_split(BH, qtiles, ctx->sm_count, 1 << 20, &qtps);
-  FS_TIME_BEGIN(ctx, FS_K_TC_OUT);
-  (void)fs_launch_chained(tc_out_kernel, dim3(qsplit, BH), dim3(TC_THREADS), OutSmem::TOTAL + 1024, ctx->stream,
-      tmQ, images, partial, shifts, nsplit, H, dm->pool, Lq, qtps, (__nv_bfloat16*)Y, fs_addr(dm->y_stride, H, Lq, dm->dv), ctx->d_status);
-  FS_TIME_END(ctx);
-  FS_LAUNCH_CHECK(ctx);
-  return FSHARP_OK;
+  const TileWork states{dm->B * dm->H, nsplit, 1, nsplit, 0, nsplit};
+  return query_side(ctx, Q, dm, images, partial, shifts, states, 1, 0, ws->take<uint8_t>((size_t)dm->B * dm->H * MRG_BYTES), Y);
 }

@@ -736,8 +736,7 @@ namespace tchost {
 int make_map_tokens(CUtensorMap* map, const void* base, TensorAddr a, int B, int H, int L, int inner);
 int make_map_out(CUtensorMap* map, void* base, TensorAddr a, int B, int H, int L, int inner);
 }  // namespace tchost
-int fs_tc_rowterm(fsharp_ctx* ctx, const void* K, const fsharp_dims* dm, const uint8_t* images, const int* flags, int Lpad,
-                  int tiles_per_split, int nsplit, float* crow);
+int fs_tc_rowterm(fsharp_ctx* ctx, const void* K, const fsharp_dims* dm, const uint8_t* images, const int* flags, int Lpad, float* crow);
 int fs_tc_key_side(fsharp_ctx* ctx, const void* K, const void* V, const fsharp_dims* dm, const uint8_t* images,
                    const int* flags, int tiles_per_split, int nsplit, float* crow, float* partial, float* shifts);
 int fs_tc_causal_supported(const fsharp_dims* dm, int chunk);
@@ -810,7 +809,7 @@ int fs_tc_causal_prefix(fsharp_ctx* ctx, const void* Q, const void* K, const voi
   if (nseg > 1) {
     FS_TRY(fs_tc_key_side(ctx, K, V, dm, images, flags, per, nseg - 1, crow, partial, shifts));
   } else {
-    FS_TRY(fs_tc_rowterm(ctx, K, dm, images, flags, Lpad, per, 1, crow));
+    FS_TRY(fs_tc_rowterm(ctx, K, dm, images, flags, Lpad, crow));
   }
   int ntot = nseg - 1;
   if (nprefix > 0) {

@@ -184,9 +184,6 @@ int fs_tc_rowterm_side(fsharp_ctx* ctx, const void* X, const fsharp_dims* dm, in
   return FSHARP_OK;
 }
 
-int fs_tc_rowterm(fsharp_ctx* ctx, const void* K, const fsharp_dims* dm, const uint8_t* images, const int* flags, int Lpad,
-                  int tiles_per_split, int nsplit, float* crow) {
-  (void)tiles_per_split;
-  (void)nsplit;
+int fs_tc_rowterm(fsharp_ctx* ctx, const void* K, const fsharp_dims* dm, const uint8_t* images, const int* flags, int Lpad, float* crow) {
   return fs_tc_rowterm_side(ctx, K, dm, 2, images, flags, Lpad, crow);
 }

@@ -1,0 +1,74 @@
+"""The bidirectional tensor-core kernels walk one list of 128-token tiles over all (batch, head) units: a unit may lie within
+one block, be cut by the end of a block's range, or be spread over every block.  Against the checker at the units where the
+ranges end."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import favor_sharp as fs
+from tests.gpu_util import TOL, dev, gpu_fit, host, rel_err
+from paper_2302_00787_b200 import binding as fb
+from paper_2302_00787_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+D, M = 64, 256
+
+# (B, H, Lq, Lk, pool)
+CASES = [
+    (1, 1, 1, 1, fb.POOL_PER_BH),                # one tile, one block
+    (1, 1, 100, 20000, fb.POOL_PER_BH),          # one unit over 148 blocks and more tiles than blocks
+    (1, 1, 20000, 100, fb.POOL_PER_BH),          # ... on the query side; a unit that nothing cuts
+    (1, 3, 300, 6400, fb.POOL_PER_HEAD),         # 150 tiles: blocks of one and two, cut within and at the ends of units
+    (50, 6, 128, 128, fb.POOL_PER_HEAD),         # units of one tile, several per block: nothing is cut
+    (20, 15, 129, 385, fb.POOL_PER_BH),          # units of two (queries) and four tiles (keys), the last one of one token
+    (33, 9, 257, 130, fb.POOL_PER_HEAD),         # W changes within a block, head by head
+]
+
+
+def tensors(B, H, Lq, Lk, spread):
+    w = wl.Workload("stream", B, H, Lq, D, D, M, "bf16", "saderf", False, 0, "orthogonal", seed=5)
+    Q, _, _ = wl.make_qkv(w)
+    K, _, V = wl.make_qkv(w.scaled(L=Lk, seed=6))
+    # the size of the keys differs from tile to tile: running maxima that rise within a piece, pieces with unlike shifts
+    K = K * (1.0 + spread * np.sin(np.arange(Lk) // 128 * 1.7))[None, None, :, None]
+    tq = [dev(x, "bf16") for x in (Q, K, V)]
+    Om = wl.make_omega(w)
+    return [host(x) for x in tq] + [Om], tq + [dev(Om)]
+
+
+def checked_units(U, tiles):
+    """The first and the last unit, and the units around the ends of some blocks' ranges."""
+    n = min(U * tiles, 148)
+    ends = [U * tiles * i // n // tiles for i in (1, n // 3, n // 2, n - 1)]
+    return sorted({0, U - 1} | {min(max(u, 0), U - 1) for e in ends for u in (e - 1, e)})
+
+
+@pytest.mark.parametrize("B,H,Lq,Lk,pool", CASES)
+def test_units_across_blocks(B, H, Lq, Lk, pool):
+    ctx = fb.Context(0)
+    (Q, K, V, Om), (dQ, dK, dV, dOm) = tensors(B, H, Lq, Lk, 0.5)
+    _, pr = gpu_fit(ctx, dQ, dK, D, "saderf", pool)
+    Y = host(ctx.fsharp_attend(dQ, dK, dV, dOm, pr, pool=pool))
+    assert ctx.status() == 0
+    prh = pr.cpu().numpy()
+    for u in sorted(set(checked_units(B * H, -(-Lk // 128))) | set(checked_units(B * H, -(-Lq // 128)))):
+        b, h = divmod(u, H)
+        ref = fs.favor_sharp_attention(Q[b, h], K[b, h], V[b, h], Om, fb.unpack_params(prh[u if pool == fb.POOL_PER_BH else h], D))
+        assert rel_err(Y[b, h], ref) < TOL["bf16"], (b, h)
+
+
+@pytest.mark.parametrize("copies", [1, 2, 3, 7])
+def test_number_of_handed_on_states(copies):
+    """Key states of one range of keys, given `copies` times over (1 .. many pieces per merged unit): every feature sum and
+    every denominator is multiplied by the same number, so the outputs are those of the range alone."""
+    ctx = fb.Context(0)
+    (Q, K, V, Om), (dQ, dK, dV, dOm) = tensors(1, 2, 200, 300, 0.5)
+    _, pr = gpu_fit(ctx, dQ, dK, D, "saderf")
+    st, sh = ctx.fsharp_attend_key_state(dK, dV, dOm, pr)
+    Y = host(ctx.fsharp_attend_with_state(dQ, None, None, dOm, pr, torch.cat([st] * copies, 1), torch.cat([sh] * copies, 1)))
+    assert ctx.status() == 0
+    prh = pr.cpu().numpy()
+    for h in range(2):
+        ref = fs.favor_sharp_attention(Q[0, h], K[0, h], V[0, h], Om, fb.unpack_params(prh[h], D))
+        assert rel_err(Y[0, h], ref) < TOL["bf16"]
