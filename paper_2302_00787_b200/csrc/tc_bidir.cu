@@ -579,14 +579,14 @@ constexpr int WARP_OUT_MMA2 = WARP_MMA + 1, WARP_OUT_CVT = WARP_MMA + 2;
 // Of every four pairs of exponentials, this many run on the multiply-add pipe (exp2_poly2).
 constexpr int OUT_POLY_PAIRS = 1;
 struct OutSmem {
-  // PHI also serves, 2 KB per epilogue warp inside the rows that warp itself writes next, the output rows on their way out
-  static constexpr uint32_t X0 = 0, WH = OUT_STAGES * TILE_BYTES, PHI = WH + IMG_W_BYTES, KVT = PHI + 4 * TILE_BYTES,
-                            ROWMAX = KVT + KVT_BYTES,
+  // STG: 2 KB per epilogue warp, the output rows on their way out
+  static constexpr uint32_t X0 = 0, WH = OUT_STAGES * TILE_BYTES, KVT = WH + IMG_W_BYTES, STG = KVT + KVT_BYTES,
+                            ROWMAX = STG + (EPI_THREADS / 32) * 2048,
                             // g as an MMA operand: [256 features x 16] fp16, no swizzle (the two 16-byte K pieces of a
                             // row 128 bytes apart, 8-row groups 256 bytes apart)
                             GOP = ROWMAX + 2 * 2 * TILE * 4, MISC = GOP + GOP_BYTES, TOTAL = MISC + 256;
 };
-static_assert(OutSmem::PHI % 1024 == 0 && OutSmem::KVT % 1024 == 0 && OutSmem::WH % 1024 == 0, "alignment");
+static_assert(OutSmem::KVT % 1024 == 0 && OutSmem::WH % 1024 == 0, "alignment");
 static_assert(OutSmem::TOTAL + 1024 <= 232448, "shared memory budget");
 
 struct OutMisc {
@@ -599,12 +599,14 @@ struct OutMisc {
   int abort_flag;
 };
 static_assert(sizeof(OutMisc) <= 256, "misc block");
-// TMEM columns: logits, then [num | den], then the A operand of the g step
-constexpr uint32_t OUT_COL_LOGITS = 0, OUT_COL_OUT = 256, OUT_COL_ONE = 496;
+// TMEM columns: logits, then [num | den], the A operand of the g step, phi (fp16, two features per column: the A operand of the
+// contraction).  Phi through shared memory (written by the epilogue, read by the MMA) was 128 of the 300 KB that the pipe, 128
+// bytes per cycle, moved for a tile, and slowed the exponentials beside it: 8 x 8 x 4096 queries __OUT__.
+constexpr uint32_t OUT_COL_LOGITS = 0, OUT_COL_OUT = 256, OUT_COL_ONE = 336, OUT_COL_PHI = 384;
 
 __global__ void __launch_bounds__(TC_THREADS, 1)
-tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const uint8_t* __restrict__ images, const uint8_t* __restrict__ merged,
-              int H, int pool, int L, const TileWork work, __nv_bfloat16* __restrict__ Y, TensorAddr ay, int* __restrict__ status) {
+tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmY, const uint8_t* __restrict__ images, const uint8_t* __restrict__ merged,
+              int H, int pool, int L, const TileWork work, int* __restrict__ status) {
   fs_grid_dependency_wait();
   // (declared with its alignment, so that every address below is a constant: rounded up at run time the base lives in
   // registers, and next to the 128 logits of a thread it was spilled and reloaded at every barrier)
@@ -743,14 +745,13 @@ tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const uint8_t* __restrict
     // blocks of both halves first, so only the last block's MMAs are left when the exponentials end.  One
     // accumulator [num | den] for all 256 features (the two threads of a row agree on the row's shift).
     constexpr uint32_t ID_OUT = idesc_f16(128, TC_NV, 0, 0);      // fp16: phi(Q) <= 1 and a state of order one per feature
-    const uint64_t dPhi = smem_desc(smem_u32(sm + OutSmem::PHI), 16, 1024, SWZ_128B);
     const uint64_t dKvt = smem_desc(smem_u32(sm + OutSmem::KVT), 16, 1024, SWZ_128B);
-    uint32_t pl = (uint32_t)dPhi, kl = (uint32_t)dKvt;
-    const uint32_t ph = (uint32_t)(dPhi >> 32), kh = (uint32_t)(dKvt >> 32);
+    uint32_t kl = (uint32_t)dKvt;
+    const uint32_t kh = (uint32_t)(dKvt >> 32);
     bool ok = true;
     int unit = -1, loads = 0;
     for (int n = 0; ok && ti.next(work); n++) {
-      opaque(pl); opaque(kl);
+      opaque(kl);
       if (ti.bh != unit) {
         // another state, once the last contraction with the old one has completed (phi_free is committed by this warp: it
         // cannot run ahead); it lands under the first tile's exponentials
@@ -775,8 +776,8 @@ tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const uint8_t* __restrict
         if (elect_one()) {
 #pragma unroll
           for (int k = 0; k < 4; k++)
-            mma_bf16_lh(tmem + OUT_COL_OUT, pl + fb * (TILE_BYTES / 16) + 2 * k, ph, kl + fb * (KVT_BLOCK_BYTES / 16) + 2 * k, kh, ID_OUT,
-                        (o > 0 || k > 0) ? 1u : 0u);
+            mma_bf16_ta_lh(tmem + OUT_COL_OUT, tmem + OUT_COL_PHI + fb * 32 + k * 8, kl + fb * (KVT_BLOCK_BYTES / 16) + 2 * k, kh, ID_OUT,
+                           (o > 0 || k > 0) ? 1u : 0u);
           if (o == TC_M / 64 - 1) mma_commit(&misc->phi_free);
         }
         __syncwarp();
@@ -803,23 +804,23 @@ tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const uint8_t* __restrict
     }
     // Y rows of a tile (its contraction has completed): 32 of the 64 columns per thread
     auto write_out = [&](int bh, int tile) {
-      __nv_bfloat16* Yb = Y + (bh / H) * ay.sb + (bh % H) * ay.sh;
       __syncwarp();
       tcgen05_fence_after();
-      uint32_t n0[32], d0[16];
+      uint32_t n0[32], d0;
       const uint32_t base = lane_addr + OUT_COL_OUT;
+      tmem_ld1(base + TC_DV, d0);
       tmem_ld16(base + hf * 32, reinterpret_cast<uint32_t(&)[16]>(n0[0]));
       tmem_ld16(base + hf * 32 + 16, reinterpret_cast<uint32_t(&)[16]>(n0[16]));
-      tmem_ld16(base + TC_DV, d0);
+      if (lane == 0) bulk_wait_read0();                       // the previous tile's rows have left the staging area
       tmem_wait_ld();
-      const int64_t r0 = (int64_t)tile * TILE + q * 32;       // first row of this warp
-      const float den = __uint_as_float(d0[0]);
+      __syncwarp();
+      const int r0 = tile * TILE + q * 32;                    // first row of this warp
+      const float den = __uint_as_float(d0);
       if (r0 + lane < L && (!(den > 0.f) || !isfinite(den))) atomicExch(status, FSHARP_E_NONFINITE);
       float inv;                       // outputs are rounded to bf16: the approximate reciprocal (1 ulp) is exact enough
       asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(den));
-      // The thread's 64 bytes go through shared memory so that a store instruction of the warp covers 8 rows x 64
-      // contiguous bytes.  The staging area lies inside the rows of the phi tile that this warp itself writes next.
-      uint8_t* stg = sm + OutSmem::PHI + hf * 2 * TILE_BYTES + q * 4096;
+      // 32 rows x 64 bytes through shared memory (64-byte swizzle) and one store, which also drops the rows past the end
+      uint8_t* stg = sm + OutSmem::STG + warp * 2048;
 #pragma unroll
       for (int i = 0; i < 4; i++) {
         uint32_t o[4];
@@ -828,19 +829,16 @@ tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const uint8_t* __restrict
           o[e] = pack_bf16(inv * __uint_as_float(n0[8 * i + 2 * e]), inv * __uint_as_float(n0[8 * i + 2 * e + 1]));
         *reinterpret_cast<uint4*>(stg + lane * 64 + ((i ^ ((lane >> 1) & 3)) << 4)) = make_uint4(o[0], o[1], o[2], o[3]);
       }
+      fence_proxy_async_smem();
       __syncwarp();
-#pragma unroll
-      for (int i = 0; i < 4; i++) {
-        const int rr = (lane >> 2) + 8 * i, c = lane & 3;
-        const uint4 val = *reinterpret_cast<const uint4*>(stg + rr * 64 + ((c ^ ((rr >> 1) & 3)) << 4));
-        if (r0 + rr < L) *reinterpret_cast<uint4*>(Yb + (r0 + rr) * ay.sl + hf * 32 + c * 8) = val;
+      if (lane == 0) {
+        if (r0 < L) tma_store_4d(&tmY, stg, hf * 32, r0, bh % H, bh / H);
+        bulk_commit();
       }
-      __syncwarp();
     };
     int n = 0, last_bh = 0, last_tile = 0;
     for (; alive && ti.next(work); n++) {
-      FS_DBG(ti.tile() * TILE < L && OUT_COL_OUT + TC_NV <= OUT_COL_ONE && OUT_COL_ONE + 8 <= TMEM_COLS, status);
-      FS_DBG(OutSmem::PHI + hf * 2 * TILE_BYTES + TILE_BYTES + row * 128 + 128 <= OutSmem::KVT && row < TILE, status);
+      FS_DBG(ti.tile() * TILE < L && OUT_COL_OUT + TC_NV <= OUT_COL_ONE && OUT_COL_ONE + 8 <= OUT_COL_PHI && OUT_COL_PHI + TC_M / 2 <= TMEM_COLS, status);
       if (!mbar_wait(&misc->logits_full, n & 1, abortp, status, false)) { alive = false; break; }
       __syncwarp();
       tcgen05_fence_after();
@@ -872,27 +870,27 @@ tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const uint8_t* __restrict
       }
       last_bh = ti.bh;
       last_tile = ti.tile();
-      uint8_t* prow = sm + OutSmem::PHI + hf * 2 * TILE_BYTES + row * 128;
 #pragma unroll
-      for (int c = 0; c < 16; c++) {
-        uint32_t p[4];
+      for (int c = 0; c < 4; c++) {               // 32 features
+        uint32_t p[16];
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-          uint32_t& e0 = v[c * 8 + 2 * j];
-          uint32_t& e1 = v[c * 8 + 2 * j + 1];
+        for (int j = 0; j < 16; j++) {
+          uint32_t& e0 = v[c * 32 + 2 * j];
+          uint32_t& e1 = v[c * 32 + 2 * j + 1];
           add2(e0, e1, -mx, -mx);
-          if (j < OUT_POLY_PAIRS) {
+          if ((j & 3) < OUT_POLY_PAIRS) {
             exp2_poly2(e0, e1);
             p[j] = pack_f16(__uint_as_float(e0), __uint_as_float(e1));
           } else {
             p[j] = pack_f16(ex2(__uint_as_float(e0)), ex2(__uint_as_float(e1)));
           }
         }
-        *reinterpret_cast<uint4*>(prow + (c >> 3) * TILE_BYTES + (((c & 7) ^ (row & 7)) << 4)) = make_uint4(p[0], p[1], p[2], p[3]);
-        if ((c & 7) == 7) {                     // a 64-feature block of this half is complete
-          fence_proxy_async_smem();
+        __syncwarp();
+        tmem_st16(lane_addr + OUT_COL_PHI + hf * 64 + c * 16, p);
+        if (c & 1) {                              // a 64-feature block of this half is complete
+          tmem_wait_st();
           tcgen05_fence_before();
-          mbar_arrive_warp(&misc->phi_full[hf * 2 + (c >> 3)], lane);
+          mbar_arrive_warp(&misc->phi_full[hf * 2 + (c >> 1)], lane);
           // a real branch after the hand-over: the instruction scheduler would otherwise move the (side-effect-free)
           // exponentials of the second block ahead of it
           if (*abortp) { alive = false; break; }
@@ -900,6 +898,7 @@ tc_out_kernel(const __grid_constant__ CUtensorMap tmQ, const uint8_t* __restrict
       }
     }
     if (alive && n > 0 && mbar_wait(&misc->phi_free, (n - 1) & 1, abortp, status, false)) write_out(last_bh, last_tile);
+    if (lane == 0) bulk_wait0();                 // the block's shared memory outlives its stores
   }
   tcgen05_fence_before();
   __syncthreads();
@@ -947,6 +946,7 @@ TileWork stream_work(const fsharp_ctx* ctx, int units, int tiles, int* blocks) {
 // ------------------------------------------------------------------------------------------
 namespace tchost {
 int make_map_tokens(CUtensorMap* map, const void* base, TensorAddr a, int B, int H, int L, int inner);
+int make_map_out(CUtensorMap* map, void* base, TensorAddr a, int B, int H, int L, int inner);
 }  // namespace tchost
 int fs_tc_rowterm(fsharp_ctx* ctx, const void* K, const fsharp_dims* dm, const uint8_t* images, const int* flags, int Lpad, float* crow);
 size_t fs_tc_bidir_scratch_bytes(const fsharp_ctx* ctx, const fsharp_dims* dm);
@@ -1027,14 +1027,15 @@ int query_side(fsharp_ctx* ctx, const void* Q, const fsharp_dims* dm, const uint
     FS_TIME_END(ctx);
     FS_LAUNCH_CHECK(ctx);
   }
-  CUtensorMap tmQ;
+  CUtensorMap tmQ, tmY;
   FS_TRY(tchost::make_map_tokens(&tmQ, Q, fs_addr(dm->q_stride, H, Lq, dm->d), B, H, Lq, dm->d));
+  FS_TRY(tchost::make_map_out(&tmY, Y, fs_addr(dm->y_stride, H, Lq, dm->dv), B, H, Lq, dm->dv));
   FS_CUDA_OK(cudaFuncSetAttribute(tc_out_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OutSmem::TOTAL + 1024));
   int blocks = 0;
   const TileWork work = stream_work(ctx, BH, (Lq + TILE - 1) / TILE, &blocks);
   FS_TIME_BEGIN(ctx, FS_K_TC_OUT);
   (void)fs_launch_chained(tc_out_kernel, dim3(blocks), dim3(TC_THREADS), OutSmem::TOTAL + 1024, ctx->stream,
-      tmQ, images, merged, H, dm->pool, Lq, work, (__nv_bfloat16*)Y, fs_addr(dm->y_stride, H, Lq, dm->dv), ctx->d_status);
+      tmQ, tmY, images, merged, H, dm->pool, Lq, work, ctx->d_status);
   FS_TIME_END(ctx);
   FS_LAUNCH_CHECK(ctx);
   return FSHARP_OK;
