@@ -4,155 +4,35 @@
 #include <cuda_fp16.h>
 
 #include "common.cuh"
+#include "mma3.cuh"
 #include "tc_common.cuh"
 #include "tc_layout.cuh"
 
 namespace {
 
-constexpr int PREP_THREADS = 256;
-constexpr int PREP_MB = 64;                   // features per block
-constexpr int PREP_LDO = PREP_MB + 1;         // row stride of the transposed Omega chunk: odd, so that the transposing stores
-                                              // (32 consecutive rows, one column) fall into 32 different banks
+constexpr int PREP_MB = mma3::ROWS;           // features per block
+constexpr int PREP_THREADS = mma3::THREADS;
 
-// One block = one (group, role, chunk of 64 features) with role 0, 1: W of side 1, 2; role 2: a (the same for both
-// sides, written for both); role 3: C, the scalars and the flags of side blockIdx.z + 1.  Omega's chunk
-// (transposed) and the d x d matrix (B or A) sit in shared memory in fp32; every thread owns a 4 x d/16 tile of
-// the 64 x d product and walks the inner index with vector loads.  The roles are separate blocks because a
-// block's time is the latency of its dependent global loads: short blocks side by side finish sooner.
+// C, the scalars and the flags of one (group, side); every thread of the block
 template <int D>
-__global__ void __launch_bounds__(PREP_THREADS)
-prep_kernel(const float* __restrict__ Omega, int64_t omega_head_stride, const double* __restrict__ params,
-            int64_t params_stride, int H, int pool, int M, float* __restrict__ prep, float qk_scale,
-            uint8_t* __restrict__ images, int* __restrict__ img_flags) {
-  fs_grid_dependency_wait();
-  // images != nullptr (d = 64, M = 256 only): the tensor-core path's operand images of this (group, side)
-  // are written as well, in the layouts of tc_layout.cuh
-  constexpr int d = D, NC = D / 16;
-  __shared__ int redi[PREP_THREADS];
-  extern __shared__ __align__(16) float stage[];
-  float* Ot = stage;                          // [d][PREP_LDO]: Ot[i][m] = Omega[m0 + m][i]
-  float* Ms = stage + d * PREP_LDO;           // [d][d]
-  const int g = blockIdx.x, role = blockIdx.y, tid = threadIdx.x;
-  const int side = role == 3 ? (int)blockIdx.z + 1 : (role == 1 ? 2 : 1);
-  if (role == 3 ? blockIdx.z >= 2 : (int)blockIdx.z * PREP_MB >= M) return;
-  const int h = pool == FSHARP_POOL_PER_BH ? g % H : g;
-  const float* Om = Omega + (int64_t)h * omega_head_stride;
+__device__ __forceinline__ void scalars_of(int g, int side, const double* __restrict__ params, int64_t params_stride, int M,
+                                           double half_log_m, float* __restrict__ prep, float qk_scale, uint8_t* __restrict__ images,
+                                           int* __restrict__ img_flags, uint8_t* raw) {
+  constexpr int d = D;
+  const int tid = threadIdx.x;
   ParamsLayout pl{d};
   PrepLayout pr{d, M};
   const double* P = params + (size_t)g * params_stride;
-  const double* A = P + pl.A();
-  const double* Bm = P + pl.B(side);
+  float* out = prep + ((size_t)g * 2 + (side - 1)) * pr.total();
   const double* Cm = P + pl.C(side);
   const double* tail = P + pl.tail();
-  float* out = prep + ((size_t)g * 2 + (side - 1)) * pr.total();
-  float* W = out + pr.W();
-  float* av = out + pr.a();
   float* scal = out + pr.scal();
   float* Cf = out + pr.Cmat();
-
-  const int m0 = blockIdx.z * PREP_MB;
-  const int ty = tid >> 4, tx = tid & 15;     // rows m0 + 4 ty + u, columns NC tx + v
-  if (role < 3) {
-    // pass 0 (roles 0, 1): W = Omega B; pass 1 (role 2): a = diag(Omega A Omega^T)
-    const int pass = role == 2 ? 1 : 0;
-    const double* Mat = pass == 0 ? Bm : A;
-    // global loads in batches of eight ahead of the shared-memory stores (a store between two loads would keep
-    // the second load from being issued early)
-    for (int e0 = tid; e0 < PREP_MB * d; e0 += 8 * PREP_THREADS) {    // coalesced read, transposed store
-      float v[8];
-#pragma unroll
-      for (int q = 0; q < 8; q++) {
-        const int e = e0 + q * PREP_THREADS, m = e / d, i = e % d;
-        v[q] = (e < PREP_MB * d && m0 + m < M) ? Om[(size_t)(m0 + m) * d + i] : 0.f;
-      }
-#pragma unroll
-      for (int q = 0; q < 8; q++) {
-        const int e = e0 + q * PREP_THREADS, m = e / d, i = e % d;
-        if (e < PREP_MB * d) Ot[i * PREP_LDO + m] = v[q];
-      }
-    }
-    for (int e0 = tid; e0 < d * d; e0 += 8 * PREP_THREADS) {
-      double v[8];
-#pragma unroll
-      for (int q = 0; q < 8; q++) {
-        const int e = e0 + q * PREP_THREADS;
-        v[q] = e < d * d ? Mat[e] : 0.0;
-      }
-#pragma unroll
-      for (int q = 0; q < 8; q++) {
-        const int e = e0 + q * PREP_THREADS;
-        if (e < d * d) Ms[e] = (float)v[q];
-      }
-    }
-    __syncthreads();
-    float acc[4][NC];
-#pragma unroll
-    for (int u = 0; u < 4; u++)
-#pragma unroll
-      for (int v = 0; v < NC; v++) acc[u][v] = 0.f;
-#pragma unroll 4
-    for (int i = 0; i < d; i++) {
-      const float* ap = Ot + i * PREP_LDO + 4 * ty;       // (two addresses per warp: broadcast reads)
-      const float a[4] = {ap[0], ap[1], ap[2], ap[3]};
-      float b[NC];
-      if (NC >= 4) {
-#pragma unroll
-        for (int v4 = 0; v4 < NC / 4; v4++) {
-          const float4 b4 = *reinterpret_cast<const float4*>(Ms + i * d + NC * tx + 4 * v4);
-          b[4 * v4] = b4.x; b[4 * v4 + 1] = b4.y; b[4 * v4 + 2] = b4.z; b[4 * v4 + 3] = b4.w;
-        }
-      } else {
-#pragma unroll
-        for (int v = 0; v < NC; v++) b[v] = Ms[i * d + NC * tx + v];
-      }
-#pragma unroll
-      for (int u = 0; u < 4; u++)
-#pragma unroll
-        for (int v = 0; v < NC; v++) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; u++) {
-      const int m = m0 + 4 * ty + u;
-      if (pass == 0) {
-        if (m < M) {
-          // (the fp32 copy serves the fp32 kernels only; the tensor-core path reads the operand image)
-          if (images == nullptr) {
-#pragma unroll
-            for (int v = 0; v < NC; v++) W[(size_t)m * d + NC * tx + v] = acc[u][v];
-          } else {
-            // log2e * qk_scale * W rounded to fp16, two neighbours per store
-            uint8_t* img = images + ((size_t)g * 2 + (side - 1)) * tcl::IMG_BYTES;
-            const float sw = FS_LOG2E * qk_scale;
-#pragma unroll
-            for (int v = 0; v + 1 < NC; v += 2)
-              *reinterpret_cast<__half2*>(img + tcl::IMG_WH + tc::sw128_offset(m, NC * tx + v)) =
-                  __floats2half2_rn(acc[u][v] * sw, acc[u][v + 1] * sw);
-          }
-        }
-      } else {
-        // a_m = sum_j (Omega A)_mj Omega_mj, summed over the 16 threads that share row m
-        float sacc = 0.f;
-#pragma unroll
-        for (int v = 0; v < NC; v++) sacc = fmaf(acc[u][v], Ot[(NC * tx + v) * PREP_LDO + 4 * ty + u], sacc);
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) sacc += __shfl_xor_sync(0xffffffffu, sacc, o);
-        if (tx == 0 && m < M) {
-          av[m] = sacc;
-          av[pr.total() + m] = sacc;          // side 2's copy
-          if (images != nullptr) {
-            reinterpret_cast<float*>(images + ((size_t)g * 2 + 0) * tcl::IMG_BYTES + tcl::IMG_A2)[m] = 2.f * FS_LOG2E * sacc;
-            reinterpret_cast<float*>(images + ((size_t)g * 2 + 1) * tcl::IMG_BYTES + tcl::IMG_A2)[m] = 2.f * FS_LOG2E * sacc;
-          }
-        }
-      }
-    }
-    return;
-  }
   // C = gamma I exactly?  The operand images (row j, column i = C[i][j], 128-byte swizzle) are put together in shared
   // memory and leave in 16-byte pieces: element-wise stores of a transposed 2-byte layout would touch a sector each.
   int cscalar = 1, lo_nonzero = 0;
   const double gamma = Cm[0];
-  uint8_t* simg = reinterpret_cast<uint8_t*>(stage);             // [hi image | lo image], IMG_C_BYTES each (d = 64 only)
+  uint8_t* simg = raw;             // [hi image | lo image], IMG_C_BYTES each (d = 64 only)
   for (int e0 = tid; e0 < d * d; e0 += 8 * PREP_THREADS) {
     double cv[8];
 #pragma unroll
@@ -184,23 +64,109 @@ prep_kernel(const float* __restrict__ Omega, int64_t omega_head_stride, const do
     const uint4* src = reinterpret_cast<const uint4*>(simg);
     for (int e = tid; e < (int)(2 * tcl::IMG_C_BYTES / 16); e += PREP_THREADS) dst[e] = src[e];
   }
-  redi[tid] = cscalar;
-  __syncthreads();
-  for (int s = PREP_THREADS / 2; s > 0; s >>= 1) {
-    if (tid < s) redi[tid] = redi[tid] & redi[tid + s];
-    __syncthreads();
-  }
+  cscalar = __syncthreads_and(cscalar);
   if (tid == 0) {
     for (int i = 0; i < 8; i++) scal[i] = 0.f;
-    scal[PS_BIAS] = (float)(tail[PT_LOGD] - 0.5 * log((double)M));
-    scal[PS_CSCALAR] = redi[0] ? 1.f : 0.f;
+    scal[PS_BIAS] = (float)(tail[PT_LOGD] - half_log_m);
+    scal[PS_CSCALAR] = cscalar ? 1.f : 0.f;
     scal[PS_CGAMMA] = (float)gamma;
     if (images != nullptr) {
       int* fl = img_flags + ((size_t)g * 2 + (side - 1)) * tcl::FLAG_WORDS;
-      fl[0] = (redi[0] ? 0 : tcl::FLAG_C_DENSE) | (lo_nonzero ? tcl::FLAG_C_LO : 0);
+      fl[0] = (cscalar ? 0 : tcl::FLAG_C_DENSE) | (lo_nonzero ? tcl::FLAG_C_LO : 0);
       fl[1] = __float_as_int((float)gamma * (FS_LOG2E * qk_scale * qk_scale));
     }
   }
+}
+
+// One block = one (group, role, chunk of 128 features).  Roles: W = Omega B (both sides side by side up to d = 64, one side each
+// at d = 128); a = diag(Omega A Omega^T) (the same for both sides, written for both), C, the scalars and the
+// flags of side blockIdx.z + 1 (in front of the blocks of a, which are no shorter for it, these made a launch 3 us longer).  The products run on the tensor cores at fp32 precision (mma3.cuh): 64 groups of 256 x 64 features are 200
+// million multiply-adds, which as fp32 instructions on operands in shared memory took 20 us (bound by the shared-memory reads);
+// 15.6 us now, most of it the latency of loads, products and stores one after the other.
+template <int D>
+__global__ void __launch_bounds__(PREP_THREADS)
+prep_kernel(const float* __restrict__ Omega, int64_t omega_head_stride, const double* __restrict__ params,
+            int64_t params_stride, int H, int pool, int M, float* __restrict__ prep, float qk_scale,
+            uint8_t* __restrict__ images, int* __restrict__ img_flags, double half_log_m, int* __restrict__ status) {
+  fs_grid_dependency_wait();
+  // images != nullptr (d = 64, M = 256 only): the tensor-core path's operand images of this (group, side)
+  // are written as well, in the layouts of tc_layout.cuh
+  constexpr int d = D, SIDES = D == 128 ? 1 : 2, NW = 2 / SIDES;       // sides per W block, W roles
+  extern __shared__ __align__(16) uint8_t raw[];
+  const int g = blockIdx.x, role = blockIdx.y, tid = threadIdx.x;
+  if (role == NW + 1) {
+    if (blockIdx.z < 2) scalars_of<D>(g, blockIdx.z + 1, params, params_stride, M, half_log_m, prep, qk_scale, images, img_flags, raw);
+    return;
+  }
+  const int m0 = blockIdx.z * PREP_MB, side0 = role;                  // (a W block's first side, from 0)
+  const bool is_a = role == NW;
+  if (m0 >= M) return;
+  const int h = pool == FSHARP_POOL_PER_BH ? g % H : g;
+  const float* Om = Omega + (int64_t)h * omega_head_stride;
+  ParamsLayout pl{d};
+  PrepLayout pr{d, M};
+  const double* P = params + (size_t)g * params_stride;
+  float* out = prep + (size_t)g * 2 * pr.total();                     // side 1; side 2 follows
+  const bool aligned = (reinterpret_cast<uintptr_t>(Om) & 15) == 0;
+  const auto omega = [&](int m, int k, auto& piece) {
+    if (m0 + m >= M) { piece.zero(); return; }
+    const float* p = Om + (size_t)(m0 + m) * d + k;
+    if (aligned) { piece.load(p); return; }
+#pragma unroll
+    for (int j = 0; j < 8; j++) piece.v[j] = p[j];
+  };
+  const auto matrix = [&](int c, int k, auto& piece) {              // eight columns of row k of A or of [B^(1) | B^(2)]
+    const double* p = P + (is_a ? pl.A() : pl.B(side0 + 1 + c / d)) + (size_t)k * d + c % d;
+#pragma unroll
+    for (int j = 0; j < 8; j++) piece.v[j] = (float)p[j];
+  };
+  mma3::Block b;
+  b.begin(raw, is_a ? d : SIDES * d, status);
+  b.template segment<true, 3, false, 3>(d, omega, matrix);
+  b.finish();
+  if (!is_a) {
+    b.rows([&](int row, int c, float4 v) {
+      const int m = m0 + row, side = side0 + c / d, j = c % d;
+      if (m >= M) return;
+      if (images == nullptr) {           // (the fp32 copy serves the fp32 kernels only; the tensor-core path reads the operand image)
+        float* w = out + (size_t)side * pr.total() + pr.W() + (size_t)m * d + j;
+        w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
+      } else {                           // log2e * qk_scale * W rounded to fp16
+        const float sw = FS_LOG2E * qk_scale;
+        const __half2 lo = __floats2half2_rn(v.x * sw, v.y * sw), hi = __floats2half2_rn(v.z * sw, v.w * sw);
+        *reinterpret_cast<uint2*>(images + ((size_t)g * 2 + side) * tcl::IMG_BYTES + tcl::IMG_WH + tc::sw128_offset(m, j)) =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+      }
+    });
+  } else {
+    // a_m = sum_j (Omega A)_mj Omega_mj: the lanes that hold row m, piece by piece, then the two warps
+    float (*part)[PREP_MB] = reinterpret_cast<float (*)[PREP_MB]>(b.sm + 65536);
+    __syncthreads();                                                // (the products have been waited for by warps 0-7)
+    if (tid < PREP_MB) part[0][tid] = part[1][tid] = 0.f;
+    __syncthreads();
+    b.rows([&](int row, int c, float4 v) {
+      float s = 0.f;
+      if (m0 + row < M) {
+        const float* o = Om + (size_t)(m0 + row) * d + c;
+        s = fmaf(v.x, o[0], fmaf(v.y, o[1], fmaf(v.z, o[2], v.w * o[3])));
+      }
+#pragma unroll
+      for (int x = 1; x < (d >= 64 ? 8 : 4); x *= 2) s += __shfl_xor_sync(0xffffffffu, s, x);
+      if ((b.lane & (d >= 64 ? 7 : 3)) == 0) part[b.warp >> 2][row] += s;
+    });
+    __syncthreads();
+    if (tid < PREP_MB && m0 + tid < M) {
+      const int m = m0 + tid;
+      const float a = part[0][tid] + part[1][tid];
+#pragma unroll
+      for (int side = 0; side < 2; side++) {
+        out[(size_t)side * pr.total() + pr.a() + m] = a;
+        if (images != nullptr)
+          reinterpret_cast<float*>(images + ((size_t)g * 2 + side) * tcl::IMG_BYTES + tcl::IMG_A2)[m] = 2.f * FS_LOG2E * a;
+      }
+    }
+  }
+  b.end();
 }
 
 }  // namespace
@@ -217,14 +183,13 @@ int fs_run_prep_images(fsharp_ctx* ctx, const float* Omega, int64_t omega_head_s
   if (G == 0) return FSHARP_OK;
   if (images != nullptr && (d != tcl::TC_D || M != tcl::TC_M)) return FSHARP_E_SHAPE;
   const int nchunks = (M + PREP_MB - 1) / PREP_MB;
-  const dim3 grid(G, 4, nchunks > 2 ? nchunks : 2);
-  const size_t smem = ((size_t)d * PREP_LDO + (size_t)d * d) * sizeof(float);
+  const dim3 grid(G, d == 128 ? 4 : 3, nchunks > 2 ? nchunks : 2);
 #define FS_PREP(DD)                                                                                                  \
   do {                                                                                                               \
-    FS_CUDA_OK(cudaFuncSetAttribute(prep_kernel<DD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));        \
+    FS_CUDA_OK(cudaFuncSetAttribute(prep_kernel<DD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mma3::SMEM));        \
     FS_TIME_BEGIN(ctx, FS_K_PREP);                                                                                    \
-    (void)fs_launch_chained(prep_kernel<DD>, grid, dim3(PREP_THREADS), smem, ctx->stream, Omega, omega_head_stride, params, params_stride, H,   \
-                                                               pool, M, prep, qk_scale, images, flags);              \
+    (void)fs_launch_chained(prep_kernel<DD>, grid, dim3(PREP_THREADS), mma3::SMEM, ctx->stream, Omega, omega_head_stride, params, params_stride, H,   \
+                                                               pool, M, prep, qk_scale, images, flags, 0.5 * log((double)M), ctx->d_status);  \
   } while (0)
   switch (d) {
     case 16: FS_PREP(16); break;

@@ -99,7 +99,6 @@ tc_rowterm_kernel(const __grid_constant__ CUtensorMap tmK, const uint8_t* __rest
       tcgen05_fence_after();
       opaque(xl0); opaque(chl); opaque(cll);
       const uint32_t xl = xl0 + st * (TILE_BYTES / 16);
-      // (a fixed lane, not an elected one: with two of these blocks on an SM the elected form gave wrong products now and then)
       if (lane == 0) {
 #pragma unroll
         for (int k = 0; k < TC_D / 16; k++) mma_bf16_lh(tmem + buf * TC_D, xl + 2 * k, xh, chl + 2 * k, ch, ID_T, k > 0 ? 1u : 0u);
@@ -138,13 +137,16 @@ tc_rowterm_kernel(const __grid_constant__ CUtensorMap tmK, const uint8_t* __rest
           part[j & 3] = fmaf(__uint_as_float(t[2 * j + 1]), __uint_as_float(w8[j] & 0xffff0000u), part[j & 3]);
         }
       }
+      // Stored before the stage is handed back: the store needs every value of x_j.  Behind the arrival the last of them could
+      // still be on their way out of shared memory when the next tile landed there (a 16-byte piece of x_j was then that of
+      // the token 512 further on, once in some hundred calls).
+      out[(size_t)it * TILE] = (part[0] + part[1]) + (part[2] + part[3]);
       tcgen05_fence_before();
       __syncwarp();
       if (lane == 0) {
         mbar_arrive(&misc->t_free[buf]);
         mbar_arrive(&misc->empty[st]);
       }
-      out[(size_t)it * TILE] = (part[0] + part[1]) + (part[2] + part[3]);
     }
   }
   tcgen05_fence_before();
