@@ -408,7 +408,7 @@ constexpr int VC_THREADS = 128, VP = 8;
 template <int D> constexpr size_t vectors_smem() { return ((size_t)(D - 2) * D + 16 * (2 * D + 2)) * sizeof(double); }
 template <int D>
 __global__ void __launch_bounds__(VC_THREADS)
-vectors_kernel(double* __restrict__ scratch, int* __restrict__ status) {
+vectors_kernel(int variant, double* __restrict__ scratch, int* __restrict__ status) {
   fs_grid_dependency_wait();
   constexpr int NU = D / VP;
   extern __shared__ __align__(16) double smv[];
@@ -492,20 +492,28 @@ vectors_kernel(double* __restrict__ scratch, int* __restrict__ status) {
   };
   double sigma;
   {
-    // a grid over the whole interval, one count per thread, then VP points per step inside this group's bracket, to 2^-50
+    // a grid of 512 points over the whole interval: every fourth by one thread each, the three between by this group's lanes;
+    // then VP points per step inside this group's bracket, to 2^-50.  (Where the spectrum is so crowded that the vectors fail the
+    // check below, the precision of sigma decides it, and with it which solver's order of rows a caller gets: the points are
+    // those of the one-block kernel in fit.cu.)
     double a = lo - 0.001 * (hi - lo) - 1e-3, b = hi + 0.001 * (hi - lo) + 1e-3;
-    const double h0 = (b - a) * (1.0 / (VC_THREADS + 1));
-    cnt[tid] = below(fma(h0, (double)(tid + 1), a));
+    constexpr int GRID = 4 * VC_THREADS;
+    const double h0 = (b - a) * (1.0 / (GRID + 1));
+    cnt[tid] = below(fma(h0, (double)(4 * tid + 4), a));
     __syncthreads();
-    int lo_i = 0, hi_i = VC_THREADS;                    // first grid point with more than r eigenvalues below it
+    int lo_i = 0, hi_i = VC_THREADS;                    // first of these points with more than r eigenvalues below it
     while (lo_i < hi_i) {
       const int mid = (lo_i + hi_i) >> 1;
       if (cnt[mid] >= r + 1) hi_i = mid; else lo_i = mid + 1;
     }
-    const double na = lo_i > 0 ? fma(h0, (double)lo_i, a) : a;
-    b = lo_i < VC_THREADS ? fma(h0, (double)(lo_i + 1), a) : b;
+    const int g0 = 4 * lo_i;                            // points g0 .. g0 + 2 of the grid lie below point g0 + 3
+    const bool under = part < 3 && g0 + part < GRID && below(fma(h0, (double)(g0 + part + 1), a)) >= r + 1;
+    const unsigned m3 = (__ballot_sync(0xffffffffu, under) >> (lane & ~(VP - 1))) & 7u;
+    const int gi = lo_i < VC_THREADS ? g0 + (m3 ? __ffs(m3) - 1 : 3) : GRID;        // first point of the grid with more than r below
+    const double na = gi > 0 ? fma(h0, (double)gi, a) : a;
+    b = gi < GRID ? fma(h0, (double)(gi + 1), a) : b;
     a = na;
-    for (int it = 0; it < 14; it++) {
+    for (int it = 0; it < 13; it++) {
       const double h = (b - a) * (1.0 / (VP + 1)), x = fma(h, (double)(part + 1), a);
       const unsigned mask = (__ballot_sync(0xffffffffu, below(x) >= r + 1) >> (lane & ~(VP - 1))) & ((1u << VP) - 1u);
       const int first = mask ? __ffs(mask) - 1 : VP;    // first point with the r-th eigenvalue below it
@@ -522,7 +530,7 @@ vectors_kernel(double* __restrict__ scratch, int* __restrict__ status) {
   // z_{i+1} = -l-_{i+1} z_i with l-_i = e_{i-1} / D-_i.  Two lanes run the two recurrences; the minors are rescaled every
   // eight steps by powers of two, whose exponents the quotients take into account.  A minor that is exactly zero gives a
   // non-finite vector, which the orthogonality check rejects.
-  __shared__ int exps[16][2][D / 8];                    // [q]: exponent taken out before step 8 q + 1
+  __shared__ int exps[16][2][D / 8], cums[16][2][D / 8];      // [q]: exponent taken out before step 8 q + 1; their sums
   if (part < 2) {
     const bool fwd = part == 0;
     double* out = fwd ? Lp : Lm;
@@ -530,7 +538,9 @@ vectors_kernel(double* __restrict__ scratch, int* __restrict__ status) {
     double pm2 = 1.0, pm1 = de[i0].x - sigma;
     out[i0] = pm1;
     int* ex_out = exps[vec][part];
-    ex_out[0] = 0;
+    int* cum_out = cums[vec][part];
+    ex_out[0] = cum_out[0] = 0;
+    int cum = 0;
     for (int s0 = 1; s0 < D; s0 += 8) {                 // eight steps' operands are loaded ahead of the chain
       double dv[8], ev[8], pv[8];
 #pragma unroll
@@ -555,10 +565,38 @@ vectors_kernel(double* __restrict__ scratch, int* __restrict__ status) {
         const double s = __hiloint2double((1023 + sh) << 20, 0);
         pm1 *= s; pm2 *= s;
       }
-      if (s0 + 8 < D) ex_out[(s0 + 8) >> 3] = sh;       // the minors from step s0 + 8 on carry 2^sh against those before
+      cum += sh;
+      if (s0 + 8 < D) {                                 // the minors from step s0 + 8 on carry 2^sh against those before
+        ex_out[(s0 + 8) >> 3] = sh;
+        cum_out[(s0 + 8) >> 3] = cum;
+      }
     }
   }
   __syncwarp();
+  // First steps of the recurrences whose minors, without the rescaling, leave the range of normal numbers.  At d = 64 such a
+  // minor of an ADERF fit counts as zero: many crowded eigenvalues then go to the Jacobi solver, whose order of the rows of B
+  // (Theorem 4.2 leaves it free; here it is that of the eigenvalues) is what callers get for such spectra.  The first of them
+  // still takes part in the choice of the starting index, with the bits it has as a subnormal number.
+  auto subnormal = [](double v, int cum) {
+    const int k = min(max(1074 - cum, -1000), 1000);    // v 2^-cum in units of 2^-1074
+    return rint(v * __hiloint2double((1023 + k) << 20, 0)) * __hiloint2double((1023 - k) << 20, 0);
+  };
+  int deadf = D, deadb = D;
+  if (D == 64 && variant == FSHARP_ADERF) {
+#pragma unroll
+    for (int u = 0; u < NU; u++) {
+      const int i = part + VP * u, sf = i, sb = D - 1 - i;
+      const int ef = ((__double2hiint(Lp[i]) >> 20) & 0x7ff) - cums[vec][0][sf > 0 ? (sf - 1) >> 3 : 0];
+      const int eb = ((__double2hiint(Lm[i]) >> 20) & 0x7ff) - cums[vec][1][sb > 0 ? (sb - 1) >> 3 : 0];
+      if (ef < 1) deadf = min(deadf, sf);
+      if (eb < 1) deadb = min(deadb, sb);
+    }
+#pragma unroll
+    for (int o = VP >> 1; o > 0; o >>= 1) {
+      deadf = min(deadf, __shfl_xor_sync(0xffffffffu, deadf, o));
+      deadb = min(deadb, __shfl_xor_sync(0xffffffffu, deadb, o));
+    }
+  }
   double gbest = 1e300;
   int ibest = 0;
   {
@@ -568,15 +606,19 @@ vectors_kernel(double* __restrict__ scratch, int* __restrict__ status) {
       const int i = part + VP * u;
       // step numbers: forward s = i, backward s = D - 1 - i; a step s = 1 mod 8, s > 1, divides by a minor of the block before
       const int sf = i, sb = D - 1 - i;
-      const double pp = Lp[i], pq = Lm[i];
+      double pp = Lp[i], pq = Lm[i];
       double ppm = i > 0 ? Lp[i - 1] : 1.0, pqp = i < D - 1 ? Lm[i + 1] : 1.0;
       if (sf > 1 && (sf & 7) == 1) ppm *= __hiloint2double((1023 + exps[vec][0][sf >> 3]) << 20, 0);
       if (sb > 1 && (sb & 7) == 1) pqp *= __hiloint2double((1023 + exps[vec][1][sb >> 3]) << 20, 0);
       const double rp = recip_fast(pp), rq = recip_fast(pq);
       lp[u] = ee[i] * ppm * rp;                         // l+_i (unused for i = D - 1: e = 0)
       lm[u] = (i > 0 ? ee[i - 1] : 0.0) * pqp * rq;     // l-_i
+      if (sf == deadf) pp = subnormal(pp, cums[vec][0][sf > 0 ? (sf - 1) >> 3 : 0]);
+      if (sb == deadb) pq = subnormal(pq, cums[vec][1][sb > 0 ? (sb - 1) >> 3 : 0]);
       const double gm = fabs(fma(pp, recip_fast(ppm), fma(pq, recip_fast(pqp), -(dd[i] - sigma))));
-      if (gm < gbest) { gbest = gm; ibest = i; }        // NaN never wins
+      if (sf >= deadf) lp[u] = __longlong_as_double(-1ll);           // NaN: the check below rejects a vector that uses it
+      if (sb >= deadb) lm[u] = __longlong_as_double(-1ll);
+      if (gm < gbest && sf <= deadf && sb <= deadb) { gbest = gm; ibest = i; }        // NaN never wins
     }
     __syncwarp();
 #pragma unroll
@@ -861,7 +903,7 @@ int run_d(fsharp_ctx* ctx, const double* stats, int G, int variant, double ridge
     FITW_LAUNCH(zform_kernel<D>, dim3(G, D / SPLIT<D>), PR_THREADS, 0, stats, ridge, scratch);
   }
   FITW_LAUNCH(tridiag_kernel<D>, dim3(G), Tri<D>::NT, 0, stats, variant, ridge, scratch, ctx->d_status);
-  FITW_LAUNCH(vectors_kernel<D>, dim3(G, D / 16), VC_THREADS, vectors_smem<D>(), scratch, ctx->d_status);
+  FITW_LAUNCH(vectors_kernel<D>, dim3(G, D / 16), VC_THREADS, vectors_smem<D>(), variant, scratch, ctx->d_status);
   FITW_LAUNCH(polish_kernel<D>, dim3(G, D / SPLIT<D>), PR_THREADS, polish_smem<D>(), variant, scratch);
   FITW_LAUNCH(finish_kernel<D>, dim3(G, D / SPLIT<D>), PR_THREADS, 0, variant, scratch, params, ctx->d_status);
 #undef FITW_LAUNCH
