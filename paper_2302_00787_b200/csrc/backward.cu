@@ -36,6 +36,7 @@ template <typename T>
 __global__ void __launch_bounds__(mma3::THREADS, 2)
 bwd_tri_kernel(const float* __restrict__ G, const T* __restrict__ V, TensorAddr av, BwdDims q, float* __restrict__ out,
                int* __restrict__ status) {
+  fs_grid_dependency_wait();
   extern __shared__ uint8_t smem[];
   const int bh = blockIdx.z / q.nch, c = blockIdx.z % q.nch, b = bh / q.H, h = bh % q.H;
   const int i0 = blockIdx.x * ROWS, j0 = blockIdx.y * ROWS, C = q.C, dv = q.dv;
@@ -73,6 +74,7 @@ __global__ void __launch_bounds__(mma3::THREADS, 2)
 bwd_numden_kernel(const float* __restrict__ phiQ, const float* __restrict__ KV, const float* __restrict__ sc,
                   const T* __restrict__ V, TensorAddr av, const T* __restrict__ dY, TensorAddr ay, BwdDims q, float* __restrict__ G,
                   int* __restrict__ status) {
+  fs_grid_dependency_wait();
   extern __shared__ uint8_t smem[];
   __shared__ float inv_s[ROWS], dot_s[ROWS];
   const int bh = blockIdx.z, b = bh / q.H, h = bh % q.H, i0 = blockIdx.x * ROWS;
@@ -142,6 +144,7 @@ bwd_numden_kernel(const float* __restrict__ phiQ, const float* __restrict__ KV, 
 template <typename T>
 __global__ void __launch_bounds__(NTH)
 bwd_g_kernel(float* __restrict__ ND, const T* __restrict__ dY, TensorAddr ay, BwdDims q, int* __restrict__ status) {
+  fs_grid_dependency_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int bh = blockIdx.y, b = bh / q.H, h = bh % q.H, dv = q.dv;
   const T* dYb = dY + b * ay.sb + h * ay.sh;
@@ -171,6 +174,7 @@ __global__ void __launch_bounds__(mma3::THREADS, 2)
 bwd_dfeat_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK, const float* __restrict__ G,
                  const float* __restrict__ St, const float* __restrict__ gv, const T* __restrict__ V, TensorAddr av,
                  BwdDims q, float* __restrict__ E, float* __restrict__ rs, int* __restrict__ status) {
+  fs_grid_dependency_wait();
   extern __shared__ uint8_t smem[];
   __shared__ float rs_s[ROWS];
   const int bh = blockIdx.z, b = bh / q.H, h = bh % q.H;
@@ -240,6 +244,7 @@ template <typename T>
 __global__ void __launch_bounds__(mma3::THREADS, 2)
 bwd_dv_kernel(const float* __restrict__ phiK, const float* __restrict__ Rt, const float* __restrict__ sc,
               const float* __restrict__ G, BwdDims q, T* __restrict__ dV, TensorAddr av, int* __restrict__ status) {
+  fs_grid_dependency_wait();
   extern __shared__ uint8_t smem[];
   const int bh = blockIdx.z, b = bh / q.H, h = bh % q.H, j0 = blockIdx.x * ROWS;
   const int C = q.C, M = q.M, NP = q.NP, dv = q.dv, L = q.Lk;
@@ -270,6 +275,7 @@ __global__ void __launch_bounds__(mma3::THREADS, 2)
 bwd_dx_kernel(const float* __restrict__ E, const float* __restrict__ rs, int mtiles, const T* __restrict__ X, TensorAddr ax, int H, int L,
               int d, int M, int pool, int side, const float* __restrict__ prep, float qk_scale, T* __restrict__ dX,
               int* __restrict__ status) {
+  fs_grid_dependency_wait();
   extern __shared__ uint8_t smem[];
   __shared__ float rs_s[ROWS];
   const int bh = blockIdx.z, b = bh / H, h = bh % H, i0 = blockIdx.x * ROWS;
@@ -374,7 +380,7 @@ int backward_t(fsharp_ctx* ctx, const void* Qv, const void* Kv, const void* Vv, 
                         causal ? 1 : 0, out, status));
     if (causal) {
       FS_TIME_BEGIN(ctx, FS_K_PREFIX);
-      prefix_kernel<<<gscan, NTH, 0, ctx->stream>>>(out, nch, elems, reverse, nullptr);
+      (void)fs_launch_chained(prefix_kernel, gscan, dim3(NTH), 0, ctx->stream, out, nch, elems, reverse, nullptr);
       FS_TIME_END(ctx);
       FS_LAUNCH_CHECK(ctx);
     }
@@ -388,7 +394,7 @@ int backward_t(fsharp_ctx* ctx, const void* Qv, const void* Kv, const void* Vv, 
     int gx = (Lq + 7) / 8;
     if (gx > 4 * ctx->sm_count) gx = 4 * ctx->sm_count;
     FS_TIME_BEGIN(ctx, FS_K_BWD_NUMDEN);
-    bwd_g_kernel<T><<<dim3(gx, BH), NTH, 0, ctx->stream>>>(G, dY, ay, q, status);
+    (void)fs_launch_chained(bwd_g_kernel<T>, dim3(gx, BH), dim3(NTH), 0, ctx->stream, G, dY, ay, q, status);
     FS_TIME_END(ctx);
     FS_LAUNCH_CHECK(ctx);
   }

@@ -20,6 +20,7 @@ out_kernel(const float* __restrict__ phiQ, const float* __restrict__ KV, const f
            const T* __restrict__ V, TensorAddr av, T* __restrict__ Y, TensorAddr ay, int H, int L, int M, int dv,
            int causal, int C, int nchunks, const float* __restrict__ lsq, const float* __restrict__ lsk,
            int* __restrict__ status) {
+  fs_grid_dependency_wait();
   // lsq != nullptr: the unnormalised operator Khat C of Section 2.1 is wanted: row i of the numerator times
   // exp(lsq[i] + lsk[bh]), the shifts that the feature kernels took out of phi(Q) and phi(K)
   extern __shared__ uint8_t smem[];
@@ -121,7 +122,7 @@ int attend_t(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const
     __nv_bfloat16* sc16 = ws->take<__nv_bfloat16>((size_t)BH * nch * C * C);
     FS_TRY(fs_tc_kv128(ctx, phiK16, V, av, B, H, Lk, M, C, st));
     FS_TIME_BEGIN(ctx, FS_K_PREFIX);
-    prefix_kernel<<<dim3((unsigned)((elems + NTH - 1) / NTH), BH), NTH, 0, ctx->stream>>>(st, nch, elems, 0, st16);
+    (void)fs_launch_chained(prefix_kernel, dim3((unsigned)((elems + NTH - 1) / NTH), BH), dim3(NTH), 0, ctx->stream, st, nch, elems, 0, st16);
     FS_TIME_END(ctx);
     FS_LAUNCH_CHECK(ctx);
     FS_TRY(fs_tc_scores128(ctx, phiQ16, phiK16, BH, Lq, M, C, sc16));
@@ -134,7 +135,7 @@ int attend_t(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const
   FS_TRY(mma3::launch(ctx, FS_K_KV, state_kernel<T, false>, dim3(gkv.x, gkv.y, BH * nch), phiK, (const T*)V, av, nullptr, H, Lk, M, dv, C, nch, 1, st,
                       ctx->d_status));
   FS_TIME_BEGIN(ctx, FS_K_PREFIX);
-  prefix_kernel<<<dim3((unsigned)((elems + NTH - 1) / NTH), BH), NTH, 0, ctx->stream>>>(st, nch, elems, 0, nullptr);
+  (void)fs_launch_chained(prefix_kernel, dim3((unsigned)((elems + NTH - 1) / NTH), BH), dim3(NTH), 0, ctx->stream, st, nch, elems, 0, nullptr);
   FS_TIME_END(ctx);
   FS_LAUNCH_CHECK(ctx);
   FS_TRY(mma3::launch(ctx, FS_K_SCORES, scores_kernel, dim3(C / mma3::ROWS, C / mma3::ROWS, BH * nch), phiQ, phiK, Lq, M, C, nch, sc,
@@ -188,6 +189,7 @@ int fs_simt_kernel_apply(fsharp_ctx* ctx, const void* X, const void* Yset, const
 // C + alpha I (Section 2.3's reduction of K^(alpha) to K^(0)).
 namespace {
 __global__ void shift_c_kernel(const double* __restrict__ params, double* __restrict__ out, int d, double alpha, size_t total) {
+  fs_grid_dependency_wait();
   const size_t g = blockIdx.x;
   ParamsLayout pl{d};
   for (size_t e = threadIdx.x; e < total; e += blockDim.x) {
@@ -202,7 +204,7 @@ __global__ void shift_c_kernel(const double* __restrict__ params, double* __rest
 }  // namespace
 int fs_shift_c(fsharp_ctx* ctx, const double* params, double* out, int G, int d, double alpha) {
   if (G == 0) return FSHARP_OK;
-  shift_c_kernel<<<G, 256, 0, ctx->stream>>>(params, out, d, alpha, ParamsLayout{d}.total());
+  (void)fs_launch_chained(shift_c_kernel, dim3(G), dim3(256), 0, ctx->stream, params, out, d, alpha, ParamsLayout{d}.total());
   FS_LAUNCH_CHECK(ctx);
   return FSHARP_OK;
 }

@@ -26,6 +26,7 @@ template <typename T, bool FROM_G>
 __global__ void __launch_bounds__(mma3::THREADS, 2)
 state_kernel(const float* __restrict__ F, const T* __restrict__ V, TensorAddr av, const float* __restrict__ G, int H, int L, int M,
              int dv, int slice_len, int nslices, int per_slice_out, float* __restrict__ out, int* __restrict__ status) {
+  fs_grid_dependency_wait();
   extern __shared__ uint8_t smem[];
   const int bh = blockIdx.z / nslices, sl = blockIdx.z % nslices, b = bh / H, h = bh % H;
   const int m0 = blockIdx.x * mma3::ROWS, NP = dv + 16;
@@ -63,6 +64,7 @@ state_kernel(const float* __restrict__ F, const T* __restrict__ V, TensorAddr av
 // ---- exclusive running sum over the chunks, forwards (earlier chunks) or backwards (later chunks) ------
 __global__ void __launch_bounds__(NTH)
 prefix_kernel(float* __restrict__ st, int nchunks, int64_t elems, int reverse, __nv_bfloat16* __restrict__ st16) {
+  fs_grid_dependency_wait();
   const int bh = blockIdx.y;
   float* base = st + (int64_t)bh * nchunks * elems;
   for (int64_t e = blockIdx.x * (int64_t)NTH + threadIdx.x; e < elems; e += (int64_t)gridDim.x * NTH) {
@@ -92,6 +94,7 @@ prefix_kernel(float* __restrict__ st, int nchunks, int64_t elems, int reverse, _
 __global__ void __launch_bounds__(mma3::THREADS, 2)
 scores_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK, int L, int M, int C, int nchunks,
               float* __restrict__ sc, int* __restrict__ status) {
+  fs_grid_dependency_wait();
   extern __shared__ uint8_t smem[];
   const int bh = blockIdx.z / nchunks, c = blockIdx.z % nchunks;
   const int i0 = blockIdx.x * mma3::ROWS, j0 = blockIdx.y * mma3::ROWS;

@@ -146,6 +146,7 @@ template <int D, int BP>
 __global__ void __launch_bounds__(256)
 w3_images_kernel(const float* __restrict__ prep, int side0, int sides, int M, float qk_scale, uint8_t* __restrict__ img,
                  int* __restrict__ status) {
+  fs_grid_dependency_wait();
   using G = WGeo<D, BP>;
   const int g = blockIdx.y, k = blockIdx.z;                          // group; which of the `sides` sides
   const size_t per_group = (size_t)G::NKS * BP * M * 128;
@@ -207,6 +208,7 @@ template <typename T, int D> constexpr size_t rt_smem() { return 1024 + Geo<T, D
 template <typename T, int D>
 __global__ void __launch_bounds__(RT_THREADS, D == 128 ? 1 : 3)
 rowterm3_kernel(const __grid_constant__ Args a) {
+  fs_grid_dependency_wait();
   using G = Geo<T, D>;
   using St = Stage<T, D, RT_THREADS>;
   extern __shared__ uint8_t smem_raw[];
@@ -378,6 +380,7 @@ template <typename T, int D, int BP> struct FtGeo : Geo<T, D> {
 template <typename T, int D, bool WRITE, int BP>
 __global__ void __launch_bounds__(FT_THREADS, 1)
 feat3_kernel(const __grid_constant__ Args a) {
+  fs_grid_dependency_wait();
   using G = FtGeo<T, D, BP>;
   constexpr bool OUT16 = BP == 2;
   extern __shared__ uint8_t smem_raw[];
@@ -608,7 +611,7 @@ int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, in
     for (int k = 0; k < ntasks; k++) side_img[side0 - 1 + k] = img + k * per_side;
     const dim3 grid((a.M * (D / 8) + 255) / 256, G_groups, ntasks);
     FS_TIME_BEGIN(ctx, FS_K_W3);
-    w3_images_kernel<D, BP><<<grid, 256, 0, ctx->stream>>>(a.prep, side0, ntasks, a.M, a.qk_scale, img, ctx->d_status);
+    (void)fs_launch_chained(w3_images_kernel<D, BP>, grid, dim3(256), 0, ctx->stream, a.prep, side0, ntasks, a.M, a.qk_scale, img, ctx->d_status);
     FS_TIME_END(ctx);
     FS_LAUNCH_CHECK(ctx);
   }
@@ -632,7 +635,7 @@ int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, in
     FS_CUDA_OK(cudaFuncSetAttribute(rowterm3_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int most = (D == 128 ? 1 : 3) * ctx->sm_count;
     FS_TIME_BEGIN(ctx, FS_K_ROWTERM);
-    rowterm3_kernel<T, D><<<total < most ? total : most, RT_THREADS, smem, ctx->stream>>>(a);
+    (void)fs_launch_chained(rowterm3_kernel<T, D>, dim3(total < most ? total : most), dim3(RT_THREADS), smem, ctx->stream, a);
     FS_TIME_END(ctx);
     FS_LAUNCH_CHECK(ctx);
   }
@@ -640,14 +643,14 @@ int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, in
   if (maxed > 0) {
     FS_CUDA_OK(cudaFuncSetAttribute(feat3_kernel<T, D, false, BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM));
     FS_TIME_BEGIN(ctx, FS_K_GROUPMAX);
-    feat3_kernel<T, D, false, BP><<<maxed < ctx->sm_count ? maxed : ctx->sm_count, FT_THREADS, G::SMEM, ctx->stream>>>(a);
+    (void)fs_launch_chained(feat3_kernel<T, D, false, BP>, dim3(maxed < ctx->sm_count ? maxed : ctx->sm_count), dim3(FT_THREADS), G::SMEM, ctx->stream, a);
     FS_TIME_END(ctx);
     FS_LAUNCH_CHECK(ctx);
   }
   const int total = set(a.nmb, [](const Task&, int) { return true; });
   FS_CUDA_OK(cudaFuncSetAttribute(feat3_kernel<T, D, true, BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM));
   FS_TIME_BEGIN(ctx, FS_K_FEAT);
-  feat3_kernel<T, D, true, BP><<<total < ctx->sm_count ? total : ctx->sm_count, FT_THREADS, G::SMEM, ctx->stream>>>(a);
+  (void)fs_launch_chained(feat3_kernel<T, D, true, BP>, dim3(total < ctx->sm_count ? total : ctx->sm_count), dim3(FT_THREADS), G::SMEM, ctx->stream, a);
   FS_TIME_END(ctx);
   FS_LAUNCH_CHECK(ctx);
   return FSHARP_OK;

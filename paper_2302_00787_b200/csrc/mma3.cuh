@@ -273,7 +273,7 @@ template <typename... KArgs, typename... Args>
 inline int launch(fsharp_ctx* ctx, int tag, void (*kernel)(KArgs...), dim3 grid, Args... args) {
   FS_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM));
   FS_TIME_BEGIN(ctx, tag);
-  kernel<<<grid, THREADS, SMEM, ctx->stream>>>(static_cast<KArgs>(args)...);
+  (void)fs_launch_chained(kernel, grid, dim3(THREADS), SMEM, ctx->stream, args...);
   FS_TIME_END(ctx);
   FS_LAUNCH_CHECK(ctx);
   return FSHARP_OK;

@@ -20,6 +20,7 @@ template <typename T, T V> struct integral_constant_t {
 // 172 us at d = 64).
 __global__ void __launch_bounds__(128)
 pairvar_prep_kernel(const double* __restrict__ params, int d, double* __restrict__ ev, int* __restrict__ status) {
+  fs_grid_dependency_wait();
   ParamsLayout pl{d};
   const double* A = params + pl.A();
   const double* B1 = params + pl.B(1);
@@ -71,6 +72,7 @@ template <int D>
 __global__ void __launch_bounds__(NTH)
 pairvar_kernel(const float* __restrict__ X, const float* __restrict__ Y, int64_t np, int M, int R, const double* __restrict__ ev,
                const float* __restrict__ est, double* __restrict__ var, double* __restrict__ pooled) {
+  fs_grid_dependency_wait();
   constexpr int PL = D == 128 ? 2 : 4, P = 32 * PL, NC = D / 8;
   extern __shared__ __align__(16) double smd[];
   double* xs = smd;                       // [D][P]
@@ -220,7 +222,7 @@ int fs_run_pairs(fsharp_ctx* ctx, const float* X, const float* Y, const float* O
   FS_TRY(fs_tc_pairs(ctx, X, Y, npairs, d, M, R, prep, est, ws));
   if (var_cf) {
     FS_TIME_BEGIN(ctx, FS_K_PAIRVAR_PREP);
-    pairvar_prep_kernel<<<d, 128, 0, ctx->stream>>>(params, d, ev, ctx->d_status);
+    (void)fs_launch_chained(pairvar_prep_kernel, dim3(d), dim3(128), 0, ctx->stream, params, d, ev, ctx->d_status);
     FS_TIME_END(ctx);
     FS_LAUNCH_CHECK(ctx);
     if (pooled) FS_CUDA_OK(cudaMemsetAsync(pooled, 0, 2 * sizeof(double), ctx->stream));
@@ -233,7 +235,7 @@ int fs_run_pairs(fsharp_ctx* ctx, const float* X, const float* Y, const float* O
     const int64_t most = (DD < 64 ? 2 : 1) * (int64_t)ctx->sm_count;                                                     \
     if (blocks > most) blocks = most;                                                                                    \
     FS_TIME_BEGIN(ctx, FS_K_PAIRVAR);                                                                                    \
-    pairvar_kernel<DD><<<(unsigned)blocks, NTH, smem, ctx->stream>>>(X, Y, npairs, M, R, ev, est, var_cf, pooled);       \
+    (void)fs_launch_chained(pairvar_kernel<DD>, dim3((unsigned)blocks), dim3(NTH), smem, ctx->stream, X, Y, npairs, M, R, ev, est, var_cf, pooled);       \
     FS_TIME_END(ctx);                                                                                                    \
   } while (0)
     switch (d) {

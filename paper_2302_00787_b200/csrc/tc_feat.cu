@@ -36,6 +36,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 tc_feat_kernel(const __grid_constant__ CUtensorMap tmX, const uint8_t* __restrict__ images, const float* __restrict__ crow,
                const float* __restrict__ prep, int side, int H, int pool, int L, int Lpad, int tiles_per_split, int stab,
                float* __restrict__ phi, float* __restrict__ logscale, int* __restrict__ status) {
+  fs_grid_dependency_wait();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   FtMisc* misc = reinterpret_cast<FtMisc*>(sm + FtSmem::MISC);
@@ -251,7 +252,7 @@ int fs_tc_featurize(fsharp_ctx* ctx, const void* X, const fsharp_dims* dm, int s
   const int tps = (tiles + ns - 1) / ns;
   ns = (tiles + tps - 1) / tps;
   FS_TIME_BEGIN(ctx, FS_K_TC_FEAT);
-  tc_feat_kernel<<<dim3(ns, BH), TC_THREADS, FtSmem::TOTAL + 1024, ctx->stream>>>(
+  (void)fs_launch_chained(tc_feat_kernel, dim3(ns, BH), dim3(TC_THREADS), FtSmem::TOTAL + 1024, ctx->stream, 
       tmX, images, crow, prep, side, H, dm->pool, L, Lpad, tps, stab, phi, logscale, ctx->d_status);
   FS_TIME_END(ctx);
   FS_LAUNCH_CHECK(ctx);

@@ -80,6 +80,7 @@ PairGeom pair_geom(int d, int M, int R) {
 // One thread = 8 values of K of one column of one tile: three parts into the images (rows of 128 bytes, 128-byte swizzle).
 __global__ void __launch_bounds__(256)
 pair_images_kernel(PairGeom g, const float* __restrict__ prep, uint8_t* __restrict__ img, float* __restrict__ a2) {
+  fs_grid_dependency_wait();
   PrepLayout pr{g.d, g.M};
   const int ntiles = g.nqt + g.nunits * g.J;
   const int nmax = g.NT > g.NQ ? g.NT : g.NQ;
@@ -155,6 +156,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1)
 tc_pairs_kernel(PairGeom g, const float* __restrict__ X, const float* __restrict__ Y, int64_t np, const float* __restrict__ prep,
                 const uint8_t* __restrict__ img, const float* __restrict__ a2, int usplit, int units_per_split, int nitems,
                 float* __restrict__ est, int* __restrict__ status) {
+  fs_grid_dependency_wait();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   constexpr int NKS = (2 * D + 63) / 64;
@@ -421,7 +423,7 @@ int fs_tc_pairs(fsharp_ctx* ctx, const float* X, const float* Y, int64_t np, int
   const int nitems = (int)(ptiles * usplit);
   const size_t nthr = (size_t)(g.nqt + g.nunits * g.J) * (g.NT > g.NQ ? g.NT : g.NQ) * g.nks * 8;
   FS_TIME_BEGIN(ctx, FS_K_PAIR_IMAGES);
-  pair_images_kernel<<<(unsigned)((nthr + 255) / 256), 256, 0, ctx->stream>>>(g, prep, img, a2);
+  (void)fs_launch_chained(pair_images_kernel, dim3((unsigned)((nthr + 255) / 256)), dim3(256), 0, ctx->stream, g, prep, img, a2);
   FS_TIME_END(ctx);
   FS_LAUNCH_CHECK(ctx);
   const int grid = nitems < ctx->sm_count ? nitems : ctx->sm_count;
@@ -430,7 +432,7 @@ int fs_tc_pairs(fsharp_ctx* ctx, const float* X, const float* Y, int64_t np, int
   do {                                                                                                                   \
     FS_CUDA_OK(cudaFuncSetAttribute(tc_pairs_kernel<DD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));        \
     FS_TIME_BEGIN(ctx, FS_K_PAIRS);                                                                                       \
-    tc_pairs_kernel<DD><<<grid, PT_THREADS, smem, ctx->stream>>>(g, X, Y, np, prep, img, a2, usplit, ups, nitems, est,    \
+    (void)fs_launch_chained(tc_pairs_kernel<DD>, grid, dim3(PT_THREADS), smem, ctx->stream, g, X, Y, np, prep, img, a2, usplit, ups, nitems, est,    \
                                                                  ctx->d_status);                                         \
     FS_TIME_END(ctx);                                                                                                     \
   } while (0)
