@@ -42,7 +42,7 @@ static_assert(sizeof(StMisc) <= 256, "misc block");
 template <bool WIDE>
 __global__ void __launch_bounds__(ST_THREADS, 2)
 tc_stats_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, int H, int Lq, int Lk,
-                int pool, int Bpool, double qk_scale, int tiles_per_split, double* __restrict__ stats,
+                int Bpool, double qk_scale, int tiles_per_split, double* __restrict__ stats,
                 int* __restrict__ status) {
   using StSmem = StSmemT<WIDE>;
   constexpr int DD = WIDE ? 2 * TC_D : TC_D;          // head dimension
@@ -54,12 +54,15 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // WIDE: blockIdx.z = 4 side + 2 a + b, the column halves of the A and the B operand
   const int side = WIDE ? blockIdx.z >> 2 : blockIdx.z, ha = WIDE ? (blockIdx.z >> 1) & 1 : 0, hb = WIDE ? blockIdx.z & 1 : 0;
-  const int bh = blockIdx.y, b = bh / H, h = bh % H;
+  // One group's tokens are one stream of tiles: the Bpool sequences that the group pools, one after the other.  A block takes a
+  // range of the stream (a block per sequence and range, 64 x 12 sequences of four tiles pooled per head: 1536 blocks, each
+  // adding its 4160 sums into one of 24 matrices, 43 us; 288 blocks of 22 tiles now, 24 us).
+  const int g = blockIdx.y, h = g % H, b0 = g / H;          // (pooled per head: b0 = 0)
   const int L = side ? Lk : Lq;
   const CUtensorMap* tm = side ? &tmK : &tmQ;
-  const int total_tiles = (L + TILE - 1) / TILE;
+  const int seq_tiles = (L + TILE - 1) / TILE;
   const int tile0 = blockIdx.x * tiles_per_split;
-  const int ntiles = min(tiles_per_split, total_tiles - tile0);
+  const int ntiles = min(tiles_per_split, Bpool * seq_tiles - tile0);
   if (ntiles <= 0) return;                    // uniform over the block, before anything is allocated
   volatile int* abortp = &misc->abort_flag;
 
@@ -86,14 +89,15 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   if (warp == ST_WARP_TMA) {
     if (lane == 0) {
       prefetch_tmap(tm);
-      int issued = 0;
+      int issued = 0, b = b0 + tile0 / seq_tiles, t = tile0 % seq_tiles;
       for (int it = 0; it < ntiles; it++) {
         const int st = it % NST;
         if (!mbar_wait(&misc->empty[st], ((it / NST) & 1) ^ 1, abortp, status)) break;
         mbar_expect_tx(&misc->full[st], StSmem::STAGE);
-        tma_load_4d(sm + StSmem::X0 + st * StSmem::STAGE, tm, &misc->full[st], 64 * ha, (tile0 + it) * TILE, h, b);
-        if (WIDE) tma_load_4d(sm + StSmem::X0 + st * StSmem::STAGE + TILE_BYTES, tm, &misc->full[st], 64 * hb, (tile0 + it) * TILE, h, b);
+        tma_load_4d(sm + StSmem::X0 + st * StSmem::STAGE, tm, &misc->full[st], 64 * ha, t * TILE, h, b);
+        if (WIDE) tma_load_4d(sm + StSmem::X0 + st * StSmem::STAGE + TILE_BYTES, tm, &misc->full[st], 64 * hb, t * TILE, h, b);
         issued = it + 1;
+        if (++t == seq_tiles) { t = 0; b++; }
       }
       // no copy of this block may still be in flight when it exits
       for (int it = max(0, issued - NST); it < issued; it++)
@@ -153,7 +157,6 @@ tc_stats_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       mbar_arrive_warp(&misc->acc_free[buf], lane);
     }
     if (alive && row <= TC_D) {
-      const int g = pool == FSHARP_POOL_PER_BH ? bh : h;
       const double inv = 1.0 / ((double)L * (double)Bpool);
       StatsLayout sl{DD};
       double* out = stats + (size_t)g * sl.total();
@@ -207,15 +210,16 @@ int fs_tc_stats_supported(const void* Q, const void* K, const fsharp_dims* dm, i
 int fs_tc_stats(fsharp_ctx* ctx, const void* Q, const void* K, const fsharp_dims* dm, float qk_scale, double* stats) {
   const int B = dm->B, H = dm->H, BH = B * H;
   const int Lmax = dm->Lq > dm->Lk ? dm->Lq : dm->Lk;
-  const int tiles = (Lmax + TILE - 1) / TILE;
+  const int Bpool = dm->pool == FSHARP_POOL_PER_BH ? 1 : B, G = BH / Bpool;
+  const int tiles = Bpool * ((Lmax + TILE - 1) / TILE);                // of one group
   const bool wide = dm->d == 2 * TC_D;
   // two blocks per SM (each block has one MMA-issuing thread, and issuing is what bounds a block): the split of
-  // the token range with the fewest (waves x tiles per block)
+  // a group's tiles with the fewest (waves x tiles per block)
   int best = 1, best_cost = 0x7fffffff, tps = tiles;
-  for (int ns = 1; ns <= tiles; ns++) {
+  for (int ns = 1; ns <= tiles && ns <= 4 * ctx->sm_count; ns++) {
     const int t = (tiles + ns - 1) / ns;
     if ((tiles + t - 1) / t != ns) continue;
-    const long long blocks = (wide ? 8LL : 2LL) * BH * ns;
+    const long long blocks = (wide ? 8LL : 2LL) * G * ns;
     const int waves = (int)((blocks + 2 * ctx->sm_count - 1) / (2 * ctx->sm_count));
     const int cost = waves * (t + 6);        // fill, drain and the final atomics cost about six tiles
     if (cost < best_cost) { best_cost = cost; best = ns; tps = t; }
@@ -223,18 +227,17 @@ int fs_tc_stats(fsharp_ctx* ctx, const void* Q, const void* K, const fsharp_dims
   CUtensorMap tmQ, tmK;
   FS_TRY(tchost::make_map_tokens(&tmQ, Q, fs_addr(dm->q_stride, H, dm->Lq, dm->d), B, H, dm->Lq, dm->d));
   FS_TRY(tchost::make_map_tokens(&tmK, K, fs_addr(dm->k_stride, H, dm->Lk, dm->d), B, H, dm->Lk, dm->d));
-  const int Bpool = dm->pool == FSHARP_POOL_PER_BH ? 1 : B;
   if (wide) {
     FS_CUDA_OK(cudaFuncSetAttribute(tc_stats_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)StSmemT<true>::TOTAL + 1024));
     FS_TIME_BEGIN(ctx, FS_K_TC_STATS);
-    (void)fs_launch_chained(tc_stats_kernel<true>, dim3(best, BH, 8), dim3(ST_THREADS), StSmemT<true>::TOTAL + 1024, ctx->stream,
-        tmQ, tmK, H, dm->Lq, dm->Lk, dm->pool, Bpool, (double)qk_scale, tps, stats, ctx->d_status);
+    (void)fs_launch_chained(tc_stats_kernel<true>, dim3(best, G, 8), dim3(ST_THREADS), StSmemT<true>::TOTAL + 1024, ctx->stream,
+        tmQ, tmK, H, dm->Lq, dm->Lk, Bpool, (double)qk_scale, tps, stats, ctx->d_status);
     FS_TIME_END(ctx);
   } else {
     FS_CUDA_OK(cudaFuncSetAttribute(tc_stats_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)StSmem::TOTAL + 1024));
     FS_TIME_BEGIN(ctx, FS_K_TC_STATS);
-    (void)fs_launch_chained(tc_stats_kernel<false>, dim3(best, BH, 2), dim3(ST_THREADS), StSmem::TOTAL + 1024, ctx->stream,
-        tmQ, tmK, H, dm->Lq, dm->Lk, dm->pool, Bpool, (double)qk_scale, tps, stats, ctx->d_status);
+    (void)fs_launch_chained(tc_stats_kernel<false>, dim3(best, G, 2), dim3(ST_THREADS), StSmem::TOTAL + 1024, ctx->stream,
+        tmQ, tmK, H, dm->Lq, dm->Lk, Bpool, (double)qk_scale, tps, stats, ctx->d_status);
     FS_TIME_END(ctx);
   }
   FS_LAUNCH_CHECK(ctx);

@@ -72,3 +72,33 @@ def test_number_of_handed_on_states(copies):
     for h in range(2):
         ref = fs.favor_sharp_attention(Q[0, h], K[0, h], V[0, h], Om, fb.unpack_params(prh[h], D))
         assert rel_err(Y[0, h], ref) < TOL["bf16"]
+
+
+# (B, H, Lq, Lk, d, pool)
+STATS_CASES = [
+    (1, 1, 1, 1, 64, fb.POOL_PER_HEAD),          # one token
+    (40, 3, 129, 300, 64, fb.POOL_PER_HEAD),     # ranges that begin and end within sequences; a last tile of one token
+    (7, 50, 128, 127, 64, fb.POOL_PER_HEAD),     # one tile per sequence, more groups than ranges
+    (9, 2, 257, 128, 128, fb.POOL_PER_HEAD),     # four blocks of the matrix
+    (2, 2, 20000, 130, 64, fb.POOL_PER_BH),      # sides of unlike length: blocks without a tile
+]
+
+
+@pytest.mark.parametrize("B,H,Lq,Lk,d,pool", STATS_CASES)
+def test_statistics_over_a_stream_of_tiles(B, H, Lq, Lk, d, pool):
+    """Products of bf16 values are exact in fp32; sums of 256 tokens are rounded to fp32 (256 additions: at most 2^-16 of the sum
+    of the magnitudes, here about the diagonal entry), everything after that is fp64."""
+    ctx = fb.Context(0)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    Q, K = (torch.randn(B, H, L, d, generator=gen, device="cuda").add_(0.3).to(torch.bfloat16) for L in (Lq, Lk))
+    st = ctx.fsharp_stats(Q, K, pool=pool).cpu()
+    assert ctx.status() == 0
+    for side, X in enumerate((Q, K)):
+        x = X.double().cpu()
+        x = x.transpose(0, 1).flatten(1, 2) if pool == fb.POOL_PER_HEAD else x.flatten(0, 1)
+        M = x.transpose(1, 2) @ x / x.shape[1]
+        mu = x.mean(1)
+        got = st[:, side * d * d:(side + 1) * d * d].reshape(-1, d, d)
+        gmu = st[:, 2 * d * d + side * d:2 * d * d + (side + 1) * d]
+        assert (got - M).abs().max() <= 2.0 ** -16 * M.abs().max()
+        assert (gmu - mu).abs().max() <= 2.0 ** -16 * x.abs().mean(1).max()
