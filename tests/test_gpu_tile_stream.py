@@ -79,7 +79,8 @@ STATS_CASES = [
     (1, 1, 1, 1, 64, fb.POOL_PER_HEAD),          # one token
     (40, 3, 129, 300, 64, fb.POOL_PER_HEAD),     # ranges that begin and end within sequences; a last tile of one token
     (7, 50, 128, 127, 64, fb.POOL_PER_HEAD),     # one tile per sequence, more groups than ranges
-    (9, 2, 257, 128, 128, fb.POOL_PER_HEAD),     # four blocks of the matrix
+    (9, 2, 257, 128, 128, fb.POOL_PER_HEAD),     # d = 128
+    (1, 1, 3, 40000, 128, fb.POOL_PER_BH),       # one group over all SMs
     (2, 2, 20000, 130, 64, fb.POOL_PER_BH),      # sides of unlike length: blocks without a tile
 ]
 
