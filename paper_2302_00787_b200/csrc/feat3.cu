@@ -14,6 +14,10 @@ using namespace tc;
 using namespace tcl;
 using feat3::Task;
 
+namespace tchost {
+int make_map_tokens(CUtensorMap* map, const void* base, TensorAddr a, int B, int H, int L, int inner);
+}
+
 namespace {
 
 __device__ __forceinline__ int group_of(int bh, int H, int pool) { return pool == FSHARP_POOL_PER_BH ? bh : bh % H; }
@@ -42,6 +46,7 @@ __device__ __forceinline__ void store32(float* p, const uint32_t* x) {
 }
 
 struct Args {
+  CUtensorMap map[2];     // per task: the tokens (BP = 2)
   Task t[2];
   int first[3];           // running number of work items: task i owns [first[i], first[i + 1])
   int tiles[2];           // token tiles per (batch, head)
@@ -359,6 +364,7 @@ rowterm3_kernel(const __grid_constant__ Args a) {
 // 128 x 256: 5.8 k cycles of this SM's share, against 3.4 k cycles of products).  Tried: a_m from shared memory (a broadcast
 // 16-byte load costs four wavefronts) with a transposing buffer in front of the stores (16 k cycles per tile); TMA store
 // tiles staged in shared memory (11 k; each of them waits for its proxy fence).
+constexpr int FT_AHEAD = 4;                                        // tiles pulled into L2 ahead of the two buffers (BP = 2)
 constexpr int FT_STAGE0 = 8, FT_MMA = 12, FT_THREADS = 416;
 struct FtMisc {
   uint64_t a_full[2], a_free[2], t_full[2], t_free[2], w_full;
@@ -392,7 +398,7 @@ feat3_kernel(const __grid_constant__ Args a) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     for (int i = 0; i < 2; i++) {
-      mbar_init(&misc->a_full[i], 4);
+      mbar_init(&misc->a_full[i], OUT16 ? 1 : 4);
       mbar_init(&misc->a_free[i], 1);
       mbar_init(&misc->t_full[i], 1);
       mbar_init(&misc->t_free[i], 4);
@@ -453,7 +459,26 @@ feat3_kernel(const __grid_constant__ Args a) {
     bad |= !isfinite(bias);
     fence_proxy_async_smem();
     __syncthreads();
-    if (warp >= FT_STAGE0 && warp < FT_MMA) {
+    if (OUT16 && warp >= FT_STAGE0 && warp < FT_MMA) {
+      // the tokens are operands as they are: one lane has them copied, panel by panel.  (Through registers, half of a tile's
+      // loads ahead, a tile of the maxima pass took 3.3 k cycles for 1.2 k of products.)
+      if (warp == FT_STAGE0 && lane == 0) {
+        const int b4 = bh / a.H, h4 = bh - b4 * a.H;
+        for (int it = 0; it < ntiles; it++) {
+          const int k = n + it, b = k % G::NBUF, tok = (tile0 + it) * TILE;
+          mbar_wait(&misc->a_free[b], ((k / G::NBUF) & 1) ^ 1, &misc->abort_flag, a.status);
+          mbar_expect_tx(&misc->a_full[b], G::A_BYTES);
+#pragma unroll
+          for (int s = 0; s < G::NKS; s++) tma_load_4d(sA + b * G::A_BYTES + s * TILE_BYTES, &a.map[ti], &misc->a_full[b], 64 * s, tok, h4, b4);
+          if (it + FT_AHEAD < ntiles) {
+#pragma unroll
+            for (int s = 0; s < G::NKS; s++) tma_prefetch_4d(&a.map[ti], 64 * s, tok + FT_AHEAD * TILE, h4, b4);
+          }
+        }
+      }
+      __syncwarp();
+      n += ntiles;
+    } else if (warp >= FT_STAGE0 && warp < FT_MMA) {
       const T* X = reinterpret_cast<const T*>(t.X) + (bh / a.H) * t.ax.sb + (bh % a.H) * t.ax.sh;
       const int i = tid - FT_STAGE0 * 32;
       Stage<T, D, 128> st;
@@ -591,6 +616,10 @@ feat3_kernel(const __grid_constant__ Args a) {
     runs++;
   }
   if (bad) atomicExch(a.status, FSHARP_E_NONFINITE);
+  // no copy of this block may still be in flight when it exits
+  if (OUT16 && warp == FT_STAGE0 && lane == 0)
+    for (int k = max(0, n - G::NBUF); k < n; k++)
+      mbar_wait(&misc->a_full[k % G::NBUF], (k / G::NBUF) & 1, &misc->abort_flag, a.status, false);
   tcgen05_fence_before();
   __syncthreads();
   if (warp == FT_MMA) {
@@ -603,6 +632,9 @@ template <typename T, int D, int BP>
 int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, int G_groups, uint8_t* img) {
   using G = FtGeo<T, D, BP>;
   a.nmb = (a.M + G::MB - 1) / G::MB;
+  CUtensorMap maps[2] = {};
+  if (BP == 2)
+    for (int i = 0; i < ntasks; i++) FS_TRY(tchost::make_map_tokens(&maps[i], tasks[i].X, tasks[i].ax, BH / a.H, a.H, tasks[i].L, D));
   const uint8_t* side_img[2] = {nullptr, nullptr};     // by side - 1
   // (a set with a row shift over several feature blocks has its maxima pass instead: its blocks convert W themselves)
   if (img != nullptr && !(ntasks == 1 && tasks[0].stab == FSHARP_STAB_ROW && a.nmb > 1)) {
@@ -621,6 +653,7 @@ int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, in
     for (int i = 0; i < ntasks; i++) {
       if (!take(tasks[i], a.nmb)) continue;
       a.t[k] = tasks[i];
+      a.map[k] = maps[i];
       a.img[k] = side_img[tasks[i].side - 1];
       a.tiles[k] = (tasks[i].L + TILE - 1) / TILE;
       a.first[k + 1] = a.first[k] + BH * units_per_bh * a.tiles[k];
