@@ -257,12 +257,12 @@ def backward_flops(w):
     return float(per * w.B * w.H)
 
 
-def backward_leg(runners, sm_count, sm_mhz):
-    """fsharp_attend_backward on the bench workloads: CUDA-event time of the call (its kernels run on the fp32 cores),
-    against the fp32 multiply-add peak: SMs x 128 lanes x 2 flops x the SM clock seen under load."""
+def backward_leg(runners):
+    """fsharp_attend_backward on the bench workloads: CUDA-event time of the call, against the rate of its
+    products: three-part fp32 operands on the tensor cores, six bf16 products each."""
     import torch
     res = {}
-    peak = sm_count * 128 * 2 * sm_mhz * 1e6 / 1e12
+    peak = measured_peaks()["bf16_tflops"] / 6
     for r in runners:
         w = r.w
         dQ, dK, dV = r.sets[0]
@@ -283,7 +283,7 @@ def backward_leg(runners, sm_count, sm_mhz):
         ms = e0.elapsed_time(e1) / n
         fl = backward_flops(w)
         res[w.name] = {"ms": ms, "tokens_per_s": w.B * w.L / (ms * 1e-3), "gflop": fl / 1e9,
-                       "roofline": {"bound": "alu", "achieved": fl / (ms * 1e-3) / 1e12, "peak": peak, "unit": "TFLOP/s",
+                       "roofline": {"bound": "tensor", "achieved": fl / (ms * 1e-3) / 1e12, "peak": peak, "unit": "TFLOP/s",
                                     "frac": fl / (ms * 1e-3) / 1e12 / peak},
                        "finite": bool(all(torch.isfinite(t.float()).all().item() for t in grads))}
         del grads, dY
@@ -629,8 +629,7 @@ def main():
                       "note": "one launch fits the groups of all workloads of the step (one block per group); every "
                               "workload's ms_per_step_alone includes a fit launch of its own"}
     if args.backward and world == 1:
-        clk = out["clocks"].get("sm_mhz") or out["clocks"].get("sm_max_mhz") or 1965
-        out["backward"] = backward_leg(runners, torch.cuda.get_device_properties(dev).multi_processor_count, float(clk))
+        out["backward"] = backward_leg(runners)
     if e2e is not None:
         e2e_ms, n_e2e, h2d, d2h = e2e
         out["e2e"] = {"value": tokens_per_step * n_e2e / (e2e_ms * 1e-3), "unit": UNIT, "h2d_bytes_per_step": h2d,
