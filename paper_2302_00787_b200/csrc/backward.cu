@@ -85,6 +85,7 @@ bwd_numden_kernel(const float* __restrict__ phiQ, const float* __restrict__ KV, 
   const int chunk = q.causal ? i0 / C : 0;
   const float* PQ = phiQ + ((int64_t)bh * L + i0) * M;
   const float* S = KV + ((int64_t)bh * q.nch + chunk) * M * NP;
+  mma3::prefetch_rows(PQ, 4LL * M, min(ROWS, L - i0), 4LL * M);
   blk.template segment<true, 3, false, 3>(
       M, [&](int r, int k, Piece<3>& p) { if (i0 + r < L) p.load(PQ + (int64_t)r * M + k); else p.zero(); },
       [&](int c, int k, Piece<3>& p) { p.load(S + (int64_t)k * NP + ct.at(dv, c)); });
@@ -119,19 +120,22 @@ bwd_numden_kernel(const float* __restrict__ phiQ, const float* __restrict__ KV, 
   }
   __syncthreads();
   const T* dYb = dY + b * ay.sb + h * ay.sh + (int64_t)i0 * ay.sl;
-  blk.rows([&](int r, int c, float4 v) {
-    float s = 0.f;
-    if (i0 + r < L && c < dv) {
-      const float inv = inv_s[r];
-      const float4 y = load4(dYb + (int64_t)r * ay.sl + c);
-      s = fmaf(y.x, v.x * inv, fmaf(y.y, v.y * inv, fmaf(y.z, v.z * inv, y.w * (v.w * inv))));
-      *reinterpret_cast<float4*>(Gb + (int64_t)r * NP + c) = make_float4(y.x * inv, y.y * inv, y.z * inv, y.w * inv);
-    }
-    // the lanes of a row are neighbours: eight of them (32 columns at a time) or four
-    s += __shfl_xor_sync(0xffffffffu, s, 1);
-    s += __shfl_xor_sync(0xffffffffu, s, 2);
-    if ((threadIdx.x & 3) == 0) atomicAdd(&dot_s[r], s);
-  });
+  float sum[8] = {};
+  blk.rows([&](int r, int c) { return i0 + r < L && c < dv ? load4(dYb + (int64_t)r * ay.sl + c) : make_float4(0.f, 0.f, 0.f, 0.f); },
+           [&](int r, int c, float4 v, float4 y, int i) {
+             float s = 0.f;
+             if (i0 + r < L && c < dv) {
+               const float inv = inv_s[r];
+               s = fmaf(y.x, v.x * inv, fmaf(y.y, v.y * inv, fmaf(y.z, v.z * inv, y.w * (v.w * inv))));
+               *reinterpret_cast<float4*>(Gb + (int64_t)r * NP + c) = make_float4(y.x * inv, y.y * inv, y.z * inv, y.w * inv);
+             }
+             if (i >= 0) { sum[i < 0 ? 0 : i] += s; return; }
+             // (four neighbouring lanes hold the row's last 16 columns)
+             s += __shfl_xor_sync(0xffffffffu, s, 1);
+             s += __shfl_xor_sync(0xffffffffu, s, 2);
+             if ((threadIdx.x & 3) == 0) atomicAdd(&dot_s[r], s);
+           });
+  blk.add_row_sums(sum, dot_s);
   __syncthreads();
   for (int e = threadIdx.x; e < ROWS * 4; e += mma3::THREADS) {
     const int r = e >> 2, part = e & 3;
@@ -169,6 +173,8 @@ bwd_g_kernel(float* __restrict__ ND, const T* __restrict__ dY, TensorAddr ay, Bw
 // ---- E = dphi * phi (the gradient with respect to the exponents), and its row sums per feature tile ----------------
 // SIDE 1: dphiQ_c = G_c KV_c^T + tril(G_c [V_c | 1]^T) phiK_c;   SIDE 2: dphiK_c = [V_c | 1] R_c^T + tril(...)^T phiQ_c
 // rs [feature tile][BH][L]
+// (2 x 12 x 4096 tokens, M = 256, causal: 183 us with a load of phi, a product and a shared-memory atomic per piece of the
+// epilogue, one after the other; 160 us with the loads of eight pieces issued together and the row sums kept in registers)
 template <typename T, int SIDE>
 __global__ void __launch_bounds__(mma3::THREADS, 2)
 bwd_dfeat_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK, const float* __restrict__ G,
@@ -185,6 +191,12 @@ bwd_dfeat_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK,
   blk.begin(smem, min(ROWS, M - m0), status);
   const float* S = St + ((int64_t)bh * q.nch + chunk) * M * NP + (int64_t)m0 * NP;
   const float* GV = q.causal ? gv + ((int64_t)bh * q.nch + chunk) * C * C : nullptr;
+  const int64_t width = 4LL * min(ROWS, M - m0);
+  if (q.causal) {
+    const float* other = (SIDE == 1 ? phiK : phiQ) + ((int64_t)bh * L + (int64_t)chunk * C + (SIDE == 1 ? 0 : ic)) * M + m0;
+    mma3::prefetch_rows(other, 4LL * M, SIDE == 1 ? min(ic + ROWS, L - chunk * C) : min(C, L - chunk * C) - ic, width);
+  }
+  mma3::prefetch_rows((SIDE == 1 ? phiQ : phiK) + ((int64_t)bh * L + i0) * M + m0, 4LL * M, min(ROWS, L - i0), width);
   if (SIDE == 1) {
     const float* Gb = G + ((int64_t)bh * L + i0) * NP;
     blk.template segment<true, 3, true, 3>(
@@ -221,18 +233,22 @@ bwd_dfeat_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK,
   __syncthreads();
   const int64_t base = ((int64_t)bh * L + i0) * M + m0;
   const float* Ph = (SIDE == 1 ? phiQ : phiK) + base;
-  blk.rows([&](int r, int c, float4 v) {
-    float s = 0.f;
-    if (i0 + r < L) {
-      const float4 f = *reinterpret_cast<const float4*>(Ph + (int64_t)r * M + c);
-      v.x *= f.x; v.y *= f.y; v.z *= f.z; v.w *= f.w;
-      *reinterpret_cast<float4*>(E + base + (int64_t)r * M + c) = v;
-      s = (v.x + v.y) + (v.z + v.w);
-    }
-    s += __shfl_xor_sync(0xffffffffu, s, 1);
-    s += __shfl_xor_sync(0xffffffffu, s, 2);
-    if ((threadIdx.x & 3) == 0) atomicAdd(&rs_s[r], s);
-  });
+  float sum[8] = {};
+  blk.rows([&](int r, int c) { return i0 + r < L ? *reinterpret_cast<const float4*>(Ph + (int64_t)r * M + c) : make_float4(0.f, 0.f, 0.f, 0.f); },
+           [&](int r, int c, float4 v, float4 f, int i) {
+             v.x *= f.x; v.y *= f.y; v.z *= f.z; v.w *= f.w;
+             float s = 0.f;
+             if (i0 + r < L) {
+               *reinterpret_cast<float4*>(E + base + (int64_t)r * M + c) = v;
+               s = (v.x + v.y) + (v.z + v.w);
+             }
+             if (i >= 0) { sum[i < 0 ? 0 : i] += s; return; }
+             // (four neighbouring lanes hold the row's last 16 columns)
+             s += __shfl_xor_sync(0xffffffffu, s, 1);
+             s += __shfl_xor_sync(0xffffffffu, s, 2);
+             if ((threadIdx.x & 3) == 0) atomicAdd(&rs_s[r], s);
+           });
+  blk.add_row_sums(sum, rs_s);
   __syncthreads();
   if (threadIdx.x < ROWS && i0 + (int)threadIdx.x < L)
     rs[((int64_t)blockIdx.x * gridDim.z + bh) * L + i0 + threadIdx.x] = rs_s[threadIdx.x];
@@ -253,6 +269,7 @@ bwd_dv_kernel(const float* __restrict__ phiK, const float* __restrict__ Rt, cons
   blk.begin(smem, dv, status);
   const float* PK = phiK + ((int64_t)bh * L + j0) * M;
   const float* R = Rt + ((int64_t)bh * q.nch + chunk) * M * NP;
+  mma3::prefetch_rows(PK, 4LL * M, min(ROWS, L - j0), 4LL * M);
   blk.template segment<true, 3, false, 3>(
       M, [&](int r, int k, Piece<3>& p) { if (j0 + r < L) p.load(PK + (int64_t)r * M + k); else p.zero(); },
       [&](int c, int k, Piece<3>& p) { p.load(R + (int64_t)k * NP + c); });
@@ -295,6 +312,7 @@ bwd_dx_kernel(const float* __restrict__ E, const float* __restrict__ rs, int mti
   }
   __syncthreads();
   const float* Eb = E + ((int64_t)bh * L + i0) * M;
+  mma3::prefetch_rows(Eb, 4LL * M, min(ROWS, L - i0), 4LL * M);
   const T* Xb = X + b * ax.sb + h * ax.sh + (int64_t)i0 * ax.sl;
   blk.template segment<true, 3, false, 3>(
       M, [&](int r, int k, Piece<3>& p) { if (i0 + r < L) p.load(Eb + (int64_t)r * M + k); else p.zero(); },

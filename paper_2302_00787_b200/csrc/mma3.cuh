@@ -68,6 +68,16 @@ template <> struct Piece<1> {
 template <typename T> struct PartsOf { static constexpr int N = 3; };
 template <> struct PartsOf<__nv_bfloat16> { static constexpr int N = 1; };
 
+// rows of `bytes` contiguous bytes, `stride` bytes apart, asked into L2 by the whole block ahead of its slices: a slice takes 128
+// bytes of a row at a time, one slice ahead of its use, which is not enough against the latency of HBM
+__device__ __forceinline__ void prefetch_rows(const void* base, int64_t stride, int rows, int64_t bytes) {
+  const int lines = (int)((bytes + 127) >> 7);
+  for (int e = threadIdx.x; e < rows * lines; e += THREADS) {
+    const int r = e / lines;
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const char*>(base) + r * stride + (int64_t)(e - r * lines) * 128));
+  }
+}
+
 struct Block {
   uint8_t* sm;
   Misc* misc;
@@ -215,6 +225,13 @@ struct Block {
   // per row where 16 columns are left).  Warps 0-7; the stages serve as a transposing buffer, one 4 KB piece per warp.
   template <class F>
   __device__ __forceinline__ void rows(F emit) {
+    rows([](int, int) { return 0; }, [&](int r, int c, float4 v, int, int) { emit(r, c, v); });
+  }
+  // The same with something fetched for every piece: emit(row, column, float4, load(row, column), i).  The loads of eight pieces
+  // are issued together, ahead of what emit does with them.  i: number of the row among the lane's eight (its row is
+  // 32 (warp % 4) + 4 i + lane / 8), or -1 where 16 columns are left.
+  template <class L, class F>
+  __device__ __forceinline__ void rows(L load, F emit) {
     if (warp == 8) return;
     const int half = ((nt >> 1) + 15) & ~15;
     const int c1 = warp < 4 ? half : nt;
@@ -245,16 +262,32 @@ struct Block {
           const int r = i * 4 + (lane >> 3), cc = lane & 7;
           f[i] = *reinterpret_cast<const float4*>(buf + r * 32 + ((cc ^ (r & 7)) << 2));
         }
+        decltype(load(0, 0)) g[8];
 #pragma unroll
-        for (int i = 0; i < 8; i++) emit(row0 + i * 4 + (lane >> 3), c + (lane & 7) * 4, f[i]);
+        for (int i = 0; i < 8; i++) g[i] = load(row0 + i * 4 + (lane >> 3), c + (lane & 7) * 4);
+#pragma unroll
+        for (int i = 0; i < 8; i++) emit(row0 + i * 4 + (lane >> 3), c + (lane & 7) * 4, f[i], g[i], i);
       } else {
 #pragma unroll
         for (int i = 0; i < 4; i++) {
           const int r = i * 8 + (lane >> 2), cc = lane & 3;
-          emit(row0 + r, c + cc * 4, *reinterpret_cast<const float4*>(buf + r * 32 + ((cc ^ (r & 7)) << 2)));
+          emit(row0 + r, c + cc * 4, *reinterpret_cast<const float4*>(buf + r * 32 + ((cc ^ (r & 7)) << 2)),
+               load(row0 + r, c + cc * 4), -1);
         }
       }
       __syncwarp();
+    }
+  }
+
+  // Sums over the columns that the callers of rows() kept per lane (wide pieces): sum[i] is added to out[row] for the lane's rows.
+  __device__ __forceinline__ void add_row_sums(const float (&sum)[8], float* out) const {
+    if (warp == 8) return;
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+      float s = sum[i];
+#pragma unroll
+      for (int o = 1; o < 8; o *= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if ((lane & 7) == 0) atomicAdd(&out[(warp & 3) * 32 + i * 4 + (lane >> 3)], s);
     }
   }
 
