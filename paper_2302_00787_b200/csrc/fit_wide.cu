@@ -346,11 +346,10 @@ tridiag_kernel(const double* __restrict__ stats, int variant, double ridge, doub
     mu[0][tid] = a;
     mu[1][tid] = b;
   }
-#pragma unroll 16
-  for (int e = tid; e < (int)sl.total() / 2; e += NT) {
-    const double2 v = reinterpret_cast<const double2*>(st)[e];
-    if (!isfinite(v.x) || !isfinite(v.y)) bad = 1.0;
-  }
+  // (one double per load: a caller's statistics are aligned to 8 bytes, no more)
+#pragma unroll 32
+  for (int e = tid; e < (int)sl.total(); e += NT)
+    if (!isfinite(st[e])) bad = 1.0;
   t1 = warp_sum(t1); t2 = warp_sum(t2); mm = warp_sum(mm); bad = warp_sum(bad);
   if (lane == 0) { red[0][warp] = t1; red[1][warp] = t2; red[2][warp] = mm; red[3][warp] = bad; }
   __syncthreads();

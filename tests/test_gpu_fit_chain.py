@@ -42,3 +42,18 @@ def test_mixed_groups(variant, d, copies):
         # the largest entries of B1^T B1; Z has the eigenvalues lam (lam / 2 + 1/10), cond 5e6
         assert_fit_close(fb.unpack_params(first[g], d), ref, d, max(1e-8, 2.0 ** -53 * d * 5e6) if kinds[g] == "wide" else 1e-8)
     assert first[1, 5 * d * d + 3] >= 0 and first[0, 5 * d * d + 3] == 0      # sweeps: none for the ordinary matrix
+
+
+@pytest.mark.parametrize("variant", ["sderf", "aderf"])
+@pytest.mark.parametrize("d", [64, 128])
+def test_statistics_on_any_8_byte_boundary(d, variant):
+    """The statistics blob is an array of doubles: one that starts 8 bytes past a 16-byte boundary gives the same bits."""
+    rng = np.random.default_rng(d)
+    M1, M2 = matrices(d, "plain", rng), matrices(d, "plain", rng)
+    blob = torch.from_numpy(np.tile(np.concatenate([M1.ravel(), M2.ravel(), 0.01 * rng.standard_normal(2 * d)]), (3, 1))).cuda()
+    ctx = fb.Context(0)
+    want = ctx.fsharp_fit_params(blob, d, variant)
+    shifted = torch.empty(blob.numel() + 1, dtype=torch.float64, device="cuda")[1:].view_as(blob).copy_(blob)
+    assert shifted.data_ptr() % 16 == 8
+    assert torch.equal(ctx.fsharp_fit_params(shifted, d, variant), want)
+    assert ctx.status() == 0
