@@ -184,7 +184,8 @@ bwd_dfeat_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK,
   extern __shared__ uint8_t smem[];
   __shared__ float rs_s[ROWS];
   const int bh = blockIdx.z, b = bh / q.H, h = bh % q.H;
-  const int m0 = blockIdx.x * ROWS, i0 = blockIdx.y * ROWS;
+  // (token tiles run along x, the only coordinate that takes more than 65535; the feature tiles of one token tile are neighbours)
+  const int mtiles = (q.M + ROWS - 1) / ROWS, mt = blockIdx.x % mtiles, m0 = mt * ROWS, i0 = blockIdx.x / mtiles * ROWS;
   const int C = q.C, M = q.M, NP = q.NP, dv = q.dv, L = SIDE == 1 ? q.Lq : q.Lk;
   const int chunk = q.causal ? i0 / C : 0, ic = q.causal ? i0 - chunk * C : 0;
   mma3::Block blk;
@@ -251,7 +252,7 @@ bwd_dfeat_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK,
   blk.add_row_sums(sum, rs_s);
   __syncthreads();
   if (threadIdx.x < ROWS && i0 + (int)threadIdx.x < L)
-    rs[((int64_t)blockIdx.x * gridDim.z + bh) * L + i0 + threadIdx.x] = rs_s[threadIdx.x];
+    rs[((int64_t)mt * gridDim.z + bh) * L + i0 + threadIdx.x] = rs_s[threadIdx.x];
   blk.end();
 }
 
@@ -418,10 +419,10 @@ int backward_t(fsharp_ctx* ctx, const void* Qv, const void* Kv, const void* Vv, 
   }
   FS_TRY(sums(Yes{}, phiQ, Lq, Rt, 1));
   if (causal) FS_TRY(mma3::launch(ctx, FS_K_SCORES, bwd_tri_kernel<T>, gtri, G, V, av, q, gv, status));
-  FS_TRY(mma3::launch(ctx, FS_K_BWD_DFEAT, bwd_dfeat_kernel<T, 1>, dim3(mt, qt, BH), phiQ, phiK, G, KV, gv, V, av, q, E, rs, status));
+  FS_TRY(mma3::launch(ctx, FS_K_BWD_DFEAT, bwd_dfeat_kernel<T, 1>, dim3(mt * qt, 1, BH), phiQ, phiK, G, KV, gv, V, av, q, E, rs, status));
   FS_TRY(mma3::launch(ctx, FS_K_BWD_DX, bwd_dx_kernel<T>, dim3(qt, 1, BH), E, rs, mt, Q, aq, H, Lq, d, M, dm->pool, 1, prep, qk_scale,
                       (T*)dQv, status));
-  FS_TRY(mma3::launch(ctx, FS_K_BWD_DFEAT, bwd_dfeat_kernel<T, 2>, dim3(mt, kt, BH), phiQ, phiK, G, Rt, gv, V, av, q, E, rs, status));
+  FS_TRY(mma3::launch(ctx, FS_K_BWD_DFEAT, bwd_dfeat_kernel<T, 2>, dim3(mt * kt, 1, BH), phiQ, phiK, G, Rt, gv, V, av, q, E, rs, status));
   FS_TRY(mma3::launch(ctx, FS_K_BWD_DX, bwd_dx_kernel<T>, dim3(kt, 1, BH), E, rs, mt, K, ak, H, Lk, d, M, dm->pool, 2, prep, qk_scale,
                       (T*)dKv, status));
   return mma3::launch(ctx, FS_K_BWD_DV, bwd_dv_kernel<T>, dim3(kt, 1, BH), phiK, Rt, sc, G, q, (T*)dVv, av, status);

@@ -127,3 +127,23 @@ def test_backward_argument_checks(ctx):
         ctx.fsharp_attend_backward(dQ, dK, dV, flat, dOm, pr)                            # misaligned cotangent
     assert e.value.code == -3
     assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("Lq,Lk", [(8388608 + 5, 200), (200, 8388608 + 5)])
+def test_backward_of_more_than_65535_token_tiles(ctx, Lq, Lk):
+    """A cotangent on a few rows (the first, the last, some of either side of tile 65535) leaves the sums over queries short
+    enough for the checker; every other query's gradient is zero."""
+    gen = torch.Generator(device="cuda").manual_seed(12)
+    Q, K, V = (0.5 * torch.randn(1, 1, L, 16, generator=gen, device="cuda") for L in (Lq, Lk, Lk))
+    rows = sorted({0, 1, 65535 * 128 - 1, 65535 * 128, Lq - 1} if Lq > 65535 * 128 else {0, 77, Lq - 1})
+    dY = torch.zeros(1, 1, Lq, 16, device="cuda")
+    dY[0, 0, rows] = torch.randn(len(rows), 16, generator=gen, device="cuda")
+    Om = wl.iid_omega(16, 16, 3)
+    _, pr = gpu_fit(ctx, Q[:, :, :1000], K[:, :, :1000], 16, "saderf")
+    grads = ctx.fsharp_attend_backward(Q, K, V, dY, dev(Om), pr)
+    assert ctx.status() == 0
+    ref = fs.favor_sharp_attention_vjp(host(Q[0, 0, rows]), host(K[0, 0]), host(V[0, 0]), host(dY[0, 0, rows]), Om,
+                                       fb.unpack_params(pr[0], 16))
+    for got, r in zip((grads[0][0, 0, rows], grads[1][0, 0], grads[2][0, 0]), ref):
+        assert rel_err(host(got), r) < TOL["f32"]
+    assert torch.count_nonzero(grads[0][0, 0].any(dim=1)) <= len(rows)
