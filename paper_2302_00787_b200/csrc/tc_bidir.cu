@@ -53,6 +53,17 @@ __device__ __forceinline__ void write_g(uint8_t* gop, int m, float gm) {
   *reinterpret_cast<uint4*>(rowp + 128) = make_uint4(0, 0, 0, 0);
 }
 
+// Exponent e of the scale 2^-e that brings a feature's column of the state, of largest magnitude am, to order one.  Columns below
+// the normal range (a shift that has grown by some 120 powers of two leaves such remnants) keep what is left of them under the
+// scale 2^126; without the bound the scale is infinite.  A column of zeros counts as below every other: with an exponent of order
+// one its query feature could be a row's largest, and push those that matter under the range of fp16.
+__device__ __forceinline__ int column_exponent(float am) {
+  if (!isfinite(am)) return 0;
+  int ex = -126;
+  if (am > 0.f) frexpf(am, &ex);                 // am = f 2^ex, f in [1/2, 1)
+  return max(ex, -126);
+}
+
 constexpr int KV_KSTAGES = 3;       // key tiles in flight (TMA, conversion to fp16, logits MMA)
 constexpr int KV_POLY_PAIRS = 2;    // of every four pairs of exponentials, this many run on the multiply-add pipe (measured: 1 and 3 are slower)
 struct KvSmem {
@@ -332,8 +343,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
 #pragma unroll
         for (int j = 0; j < 16; j++) am = fmaxf(am, fabsf(__uint_as_float(a[j])));
       }
-      int ex = 0;
-      if (am > 0.f && isfinite(am)) frexpf(am, &ex);
+      const int ex = column_exponent(am);
       const float sc = exp2f((float)-ex);
       uint8_t* out = merged + (size_t)bh * MRG_BYTES;
       uint8_t* kcol = out + (m >> 6) * KVT_BLOCK_BYTES;
@@ -559,8 +569,7 @@ merge_kernel(const float* __restrict__ partial, const float* __restrict__ shifts
   if (half == 1) return;
 #pragma unroll
   for (int w = 0; w < 8; w++) am = fmaxf(am, amax_s[w][lane]);
-  int ex = 0;
-  if (am > 0.f && isfinite(am)) frexpf(am, &ex);                // am = f 2^ex, f in [1/2, 1)
+  const int ex = column_exponent(am);
   const float sc = exp2f((float)-ex);
   uint8_t* out = merged + (size_t)bh * MRG_BYTES;
   uint8_t* kcol = out + (m >> 6) * KVT_BLOCK_BYTES;

@@ -74,6 +74,39 @@ def test_number_of_handed_on_states(copies):
         assert rel_err(Y[0, h], ref) < TOL["bf16"]
 
 
+@pytest.mark.parametrize("H", [1, 148])           # a unit cut between two blocks; units that one block has all of
+@pytest.mark.parametrize("case", ["remnant", "zero"])
+def test_feature_whose_column_of_the_state_all_but_vanishes(H, case):
+    """Feature 5 (whose exponentials flush to zero in both kernels) is seen by the first 128 keys only (remnant: 2^-13 of the others there, and every other feature then grows by 83
+    nats = 2^120) or by no key at all in fp32 (zero); queries may prefer it.  What it contributes is nothing either way, and the
+    outputs are those of the other features."""
+    K = np.zeros((1, H, 256, D))
+    K[..., 0] = 8.0
+    K[..., 1] = 83.0
+    if case == "remnant":
+        K[:, :, :128, 0], K[:, :, :128, 1] = 1.0, 0.0
+    rng = np.random.default_rng(4)
+    K[..., 2:] = rng.choice([-0.25, 0.0, 0.25], K[..., 2:].shape)
+    Q = np.zeros((1, H, 100, D))
+    Q[..., 2:] = rng.choice([-0.25, 0.0, 0.25], Q[..., 2:].shape)
+    if case == "zero":
+        Q[:, :, ::2, 0] = -4.0                   # + 56 nats for feature 5
+    V = wl.bf16_round(rng.standard_normal((1, H, 256, D)))
+    Om = np.zeros((M, D), dtype=np.float32)
+    Om[:, 1] = 1.0
+    Om[:, 2:] = rng.choice([-0.5, 0.5], (M, D - 2))
+    Om[5] = 0.0
+    Om[5, :2] = -14.0, 1.0
+    I = np.eye(D)
+    p = {"A": 0 * I, "B1": I, "B2": I, "C1": 0 * I, "C2": 0 * I, "logD": 0.0}
+    ctx = fb.Context(0)
+    pr = dev(np.stack([fb.pack_params(p, D)] * H))
+    Y = host(ctx.fsharp_attend(dev(Q, "bf16"), dev(K, "bf16"), dev(V, "bf16"), dev(Om), pr))
+    assert ctx.status() == 0
+    for h in sorted({0, H // 2, H - 1}):
+        assert rel_err(Y[0, h], fs.favor_sharp_attention(Q[0, h], K[0, h], V[0, h], Om, p)) < TOL["bf16"]
+
+
 # (B, H, Lq, Lk, d, pool)
 STATS_CASES = [
     (1, 1, 1, 1, 64, fb.POOL_PER_HEAD),          # one token
