@@ -6,6 +6,8 @@
 // that writes nothing (the products of a tile cost a quarter of what its 128 x 256 features cost in HBM time).  The kernels
 // they replace (fp32 multiply-adds; exponents written, read for the maximum, read and written again as features) took
 // 441 + 98 + 38 us for 2 x 160 k tokens, d = 64, M = 256, and 360 us for the dense quadratic terms.
+#include <math.h>
+
 #include "feat3.cuh"
 #include "split3.cuh"
 #include "tc_layout.cuh"
@@ -45,6 +47,22 @@ __device__ __forceinline__ void store32(float* p, const uint32_t* x) {
                : "memory");
 }
 
+// A factor as a float and its remainder: fmaf(hi, x, lo * x) is the product with the unrounded factor, rounded once.  (The same
+// factor multiplies every exponent: rounded to fp32 it moves exponents of 60 nats by 2e-6, all of them in one direction.)
+struct Factor {
+  float hi, lo;
+  __host__ __device__ explicit constexpr Factor(double f = 0.0) : hi((float)f), lo((float)(f - (double)(float)f)) {}
+  __device__ __forceinline__ float times(float x) const { return fmaf(hi, x, lo * x); }
+};
+constexpr double LOG2E = 1.4426950408889634074;
+// The accumulator is cut off after every MMA, never rounded up: over the d / 16 steps of the large products a sum that grows
+// from 0 loses on average LOST_W units of 2^-23 of itself, and what it starts with (a_m) LOST_A units.  Measured by regression
+// of the exponents' errors on w . x and a_m: 0.34, 0.37, 0.51, 0.85 units at d = 16, 32, 64, 128 for the sum.  W and a are scaled up
+// by as much, so that the errors centre on zero.
+template <int D> constexpr double LOST_W = (0.17 + 0.085 * (D / 16)) / 8388608.0;
+template <int D> constexpr double LOST_A = 0.17 * (D / 16) / 8388608.0;
+#define FS_TO_LOG2(x) fmaf(1.44269502f, (x), 1.92596299e-8f * (x))      // x log2(e)
+
 struct Args {
   CUtensorMap map[2];     // per task: the tokens (BP = 2)
   Task t[2];
@@ -53,7 +71,9 @@ struct Args {
   int H, M, pool, nmb;
   const float* prep;
   const uint8_t* img[2];  // per task: operand images of W (nullptr: blocks build them from prep)
-  float qk_scale;
+  Factor wscale;          // log2e qk_scale (1 + LOST_W)
+  float pow2;             // power of two next to qk_scale: tokens times this do not overflow when squared
+  double quad;            // log2e (qk_scale / pow2)^2
   int* status;
 };
 
@@ -133,11 +153,11 @@ template <int D, int BP> struct WGeo {
   static constexpr int NKS = (D + 63) / 64, MB = D == 128 && BP == 3 ? 128 : 256;
 };
 template <int D, int BP>
-__device__ __forceinline__ void put_w(uint8_t* img, int mb, int f, int c, const float* w, float scale, bool& bad) {
+__device__ __forceinline__ void put_w(uint8_t* img, int mb, int f, int c, const float* w, Factor scale, bool& bad) {
   float v[8];
 #pragma unroll
   for (int j = 0; j < 8; j++) {
-    v[j] = scale * w[j];
+    v[j] = scale.times(w[j]);
     bad |= !isfinite(v[j]);
   }
   uint4 h, m, l;
@@ -149,7 +169,7 @@ __device__ __forceinline__ void put_w(uint8_t* img, int mb, int f, int c, const 
 }
 template <int D, int BP>
 __global__ void __launch_bounds__(256)
-w3_images_kernel(const float* __restrict__ prep, int side0, int sides, int M, float qk_scale, uint8_t* __restrict__ img,
+w3_images_kernel(const float* __restrict__ prep, int side0, int sides, int M, Factor scale, uint8_t* __restrict__ img,
                  int* __restrict__ status) {
   fs_grid_dependency_wait();
   using G = WGeo<D, BP>;
@@ -160,7 +180,7 @@ w3_images_kernel(const float* __restrict__ prep, int side0, int sides, int M, fl
   bool bad = false;
   for (int e = blockIdx.x * 256 + threadIdx.x; e < M * (D / 8); e += gridDim.x * 256) {
     const int m = e / (D / 8), c = e % (D / 8), blk = m / G::MB, mb = min(G::MB, M - blk * G::MB);
-    put_w<D, BP>(out + (size_t)blk * G::MB * (G::NKS * BP * 128), mb, m - blk * G::MB, c, W + (size_t)m * D + 8 * c, FS_LOG2E * qk_scale, bad);
+    put_w<D, BP>(out + (size_t)blk * G::MB * (G::NKS * BP * 128), mb, m - blk * G::MB, c, W + (size_t)m * D + 8 * c, scale, bad);
   }
   if (bad) atomicExch(status, FSHARP_E_NONFINITE);
 }
@@ -240,7 +260,7 @@ rowterm3_kernel(const __grid_constant__ Args a) {
   const int w0 = (int)((int64_t)total * blockIdx.x / gridDim.x), w1 = (int)((int64_t)total * (blockIdx.x + 1) / gridDim.x);
   int have = -1, phase = 0;                       // (task, group) whose C is staged
   bool scalar = false, bad = false;
-  float gamma = 0.f;
+  Factor quad;
   St st;
   auto tokens = [&](int w, int& rows, int64_t& sl) {
     const int ti = w >= a.first[1] ? 1 : 0;
@@ -266,7 +286,7 @@ rowterm3_kernel(const __grid_constant__ Args a) {
       have = key;
       const float* pp = a.prep + ((size_t)g * 2 + (t.side - 1)) * pr.total();
       scalar = pp[pr.scal() + PS_CSCALAR] != 0.f;
-      gamma = pp[pr.scal() + PS_CGAMMA];
+      quad = Factor(scalar ? a.quad * (double)pp[pr.scal() + PS_CGAMMA] : a.quad);
       if (!scalar) {
         // row j of the operand: column j of C, its index i contiguous (the same matrix in the quadratic form: row j of C)
         const float* Cm = pp + pr.Cmat();
@@ -303,7 +323,7 @@ rowterm3_kernel(const __grid_constant__ Args a) {
       __syncthreads();
     }
     // x from its parts (the row's pieces are conflict-free to read), half of the columns per warpgroup
-    float sum = 0.f;
+    float sum[4] = {};
     const uint32_t lanes = tmem + ((uint32_t)(row & ~31) << 16);
 #pragma unroll
     for (int c = 0; c < D / 16; c++) {
@@ -321,25 +341,26 @@ rowterm3_kernel(const __grid_constant__ Args a) {
           x[2 * j + 1] = p ? x[2 * j + 1] + hi : hi;
         }
       }
+#pragma unroll
+      for (int j = 0; j < 8; j++) x[j] *= a.pow2;
       if (scalar) {
 #pragma unroll
-        for (int j = 0; j < 8; j++) sum = fmaf(x[j], x[j], sum);
+        for (int j = 0; j < 8; j++) sum[j & 3] = fmaf(x[j], x[j], sum[j & 3]);
       } else {
         uint32_t tv[8];
         tmem_ld8(lanes + c8 * 8, tv);
         tmem_wait_ld();
 #pragma unroll
-        for (int j = 0; j < 8; j++) sum = fmaf(__uint_as_float(tv[j]), x[j], sum);
+        for (int j = 0; j < 8; j++) sum[j & 3] = fmaf(a.pow2 * __uint_as_float(tv[j]), x[j], sum[j & 3]);
       }
     }
     if (!scalar) tcgen05_fence_before();
-    misc->part[half][row] = sum;
+    misc->part[half][row] = (sum[0] + sum[1]) + (sum[2] + sum[3]);
     __syncthreads();
     if (half == 0 && row < valid) {
-      const float sum2 = misc->part[0][row] + misc->part[1][row];
-      const float c = a.qk_scale * a.qk_scale * (scalar ? gamma * sum2 : sum2);
+      const float c = quad.times(misc->part[0][row] + misc->part[1][row]);
       bad |= !isfinite(c);                        // so is x then (or C): one test per token instead of one per exponent
-      t.rowc[out0 + row] = FS_LOG2E * c;
+      t.rowc[out0 + row] = c;
       if (t.stab == FSHARP_STAB_ROW && a.nmb > 1) t.logscale[out0 + row] = __int_as_float(0xff800000);
     }
     if (tile == 0 && tid == 0 && t.gmax) t.gmax[bh] = 0u;
@@ -436,7 +457,7 @@ feat3_kernel(const __grid_constant__ Args a) {
     w += ntiles;
     const int g = group_of(bh, a.H, a.pool);
     const float* pp = a.prep + ((size_t)g * 2 + (t.side - 1)) * pr.total();
-    const float bias = FS_LOG2E * pp[pr.scal() + PS_BIAS];
+    const float bias = FS_TO_LOG2(pp[pr.scal() + PS_BIAS]);
     __syncthreads();                                               // the previous run's products have been read
     if (a.img[ti] != nullptr) {
       if (tid == 0) {
@@ -447,10 +468,10 @@ feat3_kernel(const __grid_constant__ Args a) {
     } else {
       const float* W = pp + pr.W() + (size_t)m0 * D;
       for (int e = tid; e < mb * (D / 8); e += FT_THREADS)
-        put_w<D, BP>(sW, mb, e / (D / 8), e % (D / 8), W + (size_t)e * 8, FS_LOG2E * a.qk_scale, bad);
+        put_w<D, BP>(sW, mb, e / (D / 8), e % (D / 8), W + (size_t)e * 8, a.wscale, bad);
     }
     for (int e = tid; e < mb; e += FT_THREADS) {
-      const float v = FS_LOG2E * pp[pr.a() + m0 + e];
+      const float v = Factor(LOG2E * (1.0 + LOST_A<D>)).times(pp[pr.a() + m0 + e]);
       bad |= !isfinite(v);
       uint32_t h, m, l;
       split3::split_pair(v, 0.f, h, m, l);
@@ -512,8 +533,9 @@ feat3_kernel(const __grid_constant__ Args a) {
       const float gshift = (WRITE && t.stab == FSHARP_STAB_GROUP) ? ord2f(t.gmax[bh]) : 0.f;
       const bool own = t.stab == FSHARP_STAB_ROW && a.nmb == 1;
       const bool wide = WRITE && !OUT16 && (reinterpret_cast<uintptr_t>(t.phi) & 31) == 0;
-      constexpr float LN2 = 0.693147180559945f;
-      if (WRITE && t.stab == FSHARP_STAB_GROUP && t.logscale && tile0 == 0 && mblk == 0 && tid == 0) t.logscale[bh] = LN2 * gshift;
+      // x ln 2, x + y being rounded to x: one rounding in all
+      const auto to_nat = [](float x, float y) { return fmaf(0.693147182f, x, fmaf(0.693147182f, y, -1.90465421e-9f * x)); };
+      if (WRITE && t.stab == FSHARP_STAB_GROUP && t.logscale && tile0 == 0 && mblk == 0 && tid == 0) t.logscale[bh] = to_nat(gshift, 0.f);
       const uint32_t acc = tmem + wg * 256 + ((uint32_t)((warp & 3) * 32) << 16);
       for (int it = 0; it < ntiles; it++, n++) {
         if ((n & 1) != wg) continue;
@@ -521,9 +543,11 @@ feat3_kernel(const __grid_constant__ Args a) {
         const int64_t at = (int64_t)bh * t.L + tok;
         const bool in = tok < t.L;
         const float ci = (in ? t.rowc[at] : 0.f) + bias;
-        float shift = gshift;                          // in powers of two, subtracted from acc + ci
-        if (WRITE && t.stab == FSHARP_STAB_ROW && !own) shift = in ? FS_LOG2E * t.logscale[at] : 0.f;
-        float off = ci - shift;
+        // exponent = acc + add, minus `shift` where that does not come from this block's own maximum: in this order the largest
+        // exponent of the group or row, rounded as it was when the maximum was taken, gives 1 and nothing gives more
+        float add = ci, shift = gshift;
+        if (WRITE && t.stab == FSHARP_STAB_ROW && !own) shift = in ? FS_TO_LOG2(t.logscale[at]) : 0.f;
+        const bool shifted = WRITE && !own && t.stab != FSHARP_STAB_NONE;
         mbar_wait(&misc->t_full[wg], (n >> 1) & 1, &misc->abort_flag, a.status);
         __syncwarp();
         tcgen05_fence_after();
@@ -563,13 +587,14 @@ feat3_kernel(const __grid_constant__ Args a) {
           }
           mx = fmaxf(mx, my);
           if (WRITE) {
-            off = -mx;
-            if (t.logscale && in) t.logscale[at] = LN2 * (mx + ci);
+            add = -mx;
+            const float top = mx + ci, big = fabsf(mx) > fabsf(ci) ? mx : ci, small = fabsf(mx) > fabsf(ci) ? ci : mx;
+            if (t.logscale && in) t.logscale[at] = to_nat(top, small - (top - big));
           } else if (t.stab == FSHARP_STAB_GROUP) {
             if (in) gmx = fmaxf(gmx, mx + ci);
           } else {
             // (nudged upwards by the rounding of the two conversions, so that no feature exceeds one)
-            const float ls = LN2 * (mx + ci);
+            const float ls = to_nat(mx + ci, 0.f);
             if (in) atomic_max_float(t.logscale + at, fmaf(fabsf(ls), 2.4e-7f, ls));
           }
         }
@@ -581,7 +606,13 @@ feat3_kernel(const __grid_constant__ Args a) {
             arrived(x);
             if (c + 32 < mb) fetch(c + 32);
 #pragma unroll
-            for (int j = 0; j < 32; j++) x[j] = __float_as_uint(ex2(__uint_as_float(x[j]) + off));
+            for (int j = 0; j < 32; j += 2) add2(x[j], x[j + 1], add, add);
+            if (shifted) {
+#pragma unroll
+              for (int j = 0; j < 32; j += 2) add2(x[j], x[j + 1], -shift, -shift);
+            }
+#pragma unroll
+            for (int j = 0; j < 32; j++) x[j] = __float_as_uint(ex2(__uint_as_float(x[j])));
             if (in) {
               float* dst = out + c;
               if (OUT16) {                               // (M is a multiple of 128 and the scratch aligned)
@@ -629,8 +660,9 @@ feat3_kernel(const __grid_constant__ Args a) {
 }
 
 template <typename T, int D, int BP>
-int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, int G_groups, uint8_t* img) {
+int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, int G_groups, float qk_scale, uint8_t* img) {
   using G = FtGeo<T, D, BP>;
+  a.wscale = Factor(LOG2E * (1.0 + LOST_W<D>) * (double)qk_scale);
   a.nmb = (a.M + G::MB - 1) / G::MB;
   CUtensorMap maps[2] = {};
   if (BP == 2)
@@ -643,7 +675,7 @@ int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, in
     for (int k = 0; k < ntasks; k++) side_img[side0 - 1 + k] = img + k * per_side;
     const dim3 grid((a.M * (D / 8) + 255) / 256, G_groups, ntasks);
     FS_TIME_BEGIN(ctx, FS_K_W3);
-    (void)fs_launch_chained(w3_images_kernel<D, BP>, grid, dim3(256), 0, ctx->stream, a.prep, side0, ntasks, a.M, a.qk_scale, img, ctx->d_status);
+    (void)fs_launch_chained(w3_images_kernel<D, BP>, grid, dim3(256), 0, ctx->stream, a.prep, side0, ntasks, a.M, a.wscale, img, ctx->d_status);
     FS_TIME_END(ctx);
     FS_LAUNCH_CHECK(ctx);
   }
@@ -692,16 +724,16 @@ int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, in
 // Two token sets share their launches only while both together leave SMs without a tile: beyond that a launch of its own
 // costs a set nothing, and its blocks keep one W each for longer.
 template <typename T, int D, int BP>
-int run_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, int groups, uint8_t* img) {
+int run_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, int groups, float qk_scale, uint8_t* img) {
   if constexpr (BP == 3 && D == 128 && sizeof(T) == 2) {
-    if (tasks[0].phi16 != nullptr) return run_t<T, D, 2>(ctx, a, tasks, ntasks, BH, groups, img);
+    if (tasks[0].phi16 != nullptr) return run_t<T, D, 2>(ctx, a, tasks, ntasks, BH, groups, qk_scale, img);
   }
   int64_t items = 0;
   for (int i = 0; i < ntasks; i++) items += (int64_t)BH * ((tasks[i].L + TILE - 1) / TILE) * ((a.M + WGeo<D, BP>::MB - 1) / WGeo<D, BP>::MB);
   if (items > 2147483647LL) return FSHARP_E_SHAPE;     // items are numbered in 32 bits
-  if (ntasks == 1 || (items <= ctx->sm_count && BP == 3)) return launch_t<T, D, BP>(ctx, a, tasks, ntasks, BH, groups, img);
+  if (ntasks == 1 || (items <= ctx->sm_count && BP == 3)) return launch_t<T, D, BP>(ctx, a, tasks, ntasks, BH, groups, qk_scale, img);
   for (int i = 0; i < ntasks; i++) {
-    FS_TRY((launch_t<T, D, BP>(ctx, a, tasks + i, 1, BH, groups, img)));
+    FS_TRY((launch_t<T, D, BP>(ctx, a, tasks + i, 1, BH, groups, qk_scale, img)));
   }
   return FSHARP_OK;
 }
@@ -715,11 +747,15 @@ size_t feat3::image_bytes(int groups, int d, int M, int ntasks) {
 int feat3::run(fsharp_ctx* ctx, const Task* tasks, int ntasks, int dtype, int B, int H, int d, int M, int pool, const float* prep,
                float qk_scale, uint8_t* img) {
   Args a{};
-  a.H = H; a.M = M; a.pool = pool; a.prep = prep; a.qk_scale = qk_scale; a.status = ctx->d_status;
+  a.H = H; a.M = M; a.pool = pool; a.prep = prep; a.status = ctx->d_status;
+  int e = 0;
+  (void)frexp((double)qk_scale, &e);
+  a.pow2 = (float)ldexp(1.0, e < -100 ? -100 : (e > 100 ? 100 : e));
+  a.quad = LOG2E * (double)qk_scale * (double)qk_scale / ((double)a.pow2 * (double)a.pow2);
   const int groups = pool == FSHARP_POOL_PER_BH ? B * H : H;
 #define FS_FEAT3(DD)                                                                                          \
-  return dtype == FSHARP_F32 ? run_t<float, DD, 3>(ctx, a, tasks, ntasks, B * H, groups, img)                    \
-                             : run_t<__nv_bfloat16, DD, 3>(ctx, a, tasks, ntasks, B * H, groups, img)
+  return dtype == FSHARP_F32 ? run_t<float, DD, 3>(ctx, a, tasks, ntasks, B * H, groups, qk_scale, img)                    \
+                             : run_t<__nv_bfloat16, DD, 3>(ctx, a, tasks, ntasks, B * H, groups, qk_scale, img)
   switch (d) {
     case 16: FS_FEAT3(16);
     case 32: FS_FEAT3(32);

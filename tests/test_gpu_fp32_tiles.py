@@ -91,3 +91,44 @@ def test_unaligned_feature_output_of_the_static_entry_point():
         out.append(phi)
     torch.cuda.synchronize()
     assert torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("d,M,dtype", [(16, 64, "f32"), (64, 256, "f32"), (64, 64, "bf16"), (128, 272, "f32"), (128, 128, "bf16")])
+def test_exponents_are_not_biased(d, M, dtype):
+    """PosRF features of tokens of 2 sigma (exponents of some tens): the errors of the exponents, regressed on their two parts
+    w . x and -|x|^2 / 2, follow neither.  A sum rounded to nearest has errors of either sign; one that is always cut off, or a
+    factor log2(e) q^2 that was rounded before it was applied, is off by one unit in the last place or so of the whole: half a unit
+    (2^-24) is the bound.  (4000 M errors of 1e-6 determine the slopes to some 1e-3 units.)"""
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    X = (2.0 * torch.randn(1, 1, 4000, d, generator=gen, device="cuda")).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    qk = float(np.float32(d ** -0.25))
+    Om = dev(wl.orthogonal_omega(M, d, 1))
+    I = np.eye(d)
+    blob = dev(fb.pack_params({"A": 0 * I, "B1": I, "B2": I, "C1": -0.5 * I, "C2": -0.5 * I, "logD": 0.0}, d)[None])
+    ctx = fb.Context(0)
+    ctx.set_impl(fb.IMPL_SIMT)
+    phi, _ = ctx.fsharp_featurize(X, Om, blob, 1, qk_scale=qk, stab=fb.STAB_NONE)
+    assert ctx.status() == 0
+    x = qk * X[0, 0].double()
+    wx, c = x @ Om.double().T, -0.5 * (x * x).sum(1, keepdim=True)
+    e = wx + c - 0.5 * np.log(M)
+    ok = (phi[0, 0] > 1e-30) & (phi[0, 0] < 1e30)
+    parts = torch.stack([wx[ok], c.expand_as(wx)[ok], torch.ones_like(wx[ok])], 1)
+    slope = torch.linalg.lstsq(parts, (phi[0, 0].double().log() - e)[ok][:, None]).solution[:2, 0]
+    assert slope.abs().max() < 2.0 ** -24
+
+
+@pytest.mark.parametrize("d,M,side", [(64, 256, 2), (64, 512, 1), (128, 256, 1), (32, 64, 2)])
+def test_no_feature_exceeds_one(d, M, side):
+    """Shifts that come from a pass of their own (the group's, and the row's when M needs several feature blocks): the largest
+    exponent must not come out above the shift that was taken from it, however far the parts of a sum are from the sum."""
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    X = 2.0 * torch.randn(8, 4, 500, d, generator=gen, device="cuda")
+    qk = d ** -0.25
+    ctx = fb.Context(0)
+    pr = ctx.fsharp_fit_params(ctx.fsharp_stats(X, X, qk_scale=qk), d, "saderf")
+    phi, _ = ctx.fsharp_featurize(X, dev(wl.orthogonal_omega(M, d, 1)), pr, side, qk_scale=qk,
+                                  stab=fb.STAB_GROUP if side == 2 else fb.STAB_ROW)
+    assert ctx.status() == 0
+    top = phi.amax(dim=(2, 3) if side == 2 else 3)
+    assert top.max() <= 1.0 and top.min() > 1.0 - 1e-4
