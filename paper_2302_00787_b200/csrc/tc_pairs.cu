@@ -18,6 +18,11 @@
 // point: the five products with m or l parts (2^-8 of the result and less) are therefore accumulated first and the h h
 // products last, so that only the last 2 d / 16 steps round at the size of the result (mean error of an estimate at
 // d = 64: 5.3e-6 with the products in any order, 0.9e-6 so, 0.8e-6 for the fp32 kernel).
+// What those steps lose on average of a sum is put back as a factor on W and C (lost()): the mean error of the estimates was
+// 0.40, 0.45, 1.25, 1.95 units of 2^-23 of the exponents' products at d = 16, 32, 64, 128 (PosRF, GERF and ADERF; all of one sign).
+// Relative error of the estimates for points of norm 2, without it / with it / fp32 multiply-adds: d = M = 64, ADERF 2.3e-6 /
+// 0.9e-6 / 1.2e-6; d = 128, M = 256, GERF 5.1e-6 / 2.2e-6 / 1.8e-6, SDERF, whose products are nearly all of one sign and lose
+// more, 5.7e-6 / 2.4e-6 / 0.8e-6.  (Two accumulators for the h h products at d = 128: SDERF 2.3e-6, and 13 % longer.)
 // Bound: tensor pipe (d = 64: 48 MMAs of N = 128 per tile, 3.1 k cycles, against 1.5 k issue cycles of exponentials per
 // warpgroup).
 #include "common.cuh"
@@ -77,6 +82,9 @@ PairGeom pair_geom(int d, int M, int R) {
   return g;
 }
 
+// mean loss, relative, of a sum over n steps
+__device__ __forceinline__ float lost(int n) { return (n <= 4 ? 0.4f : n <= 8 ? 1.25f : 1.95f) * 1.1920929e-7f; }
+
 // One thread = 8 values of K of one column of one tile: three parts into the images (rows of 128 bytes, 128-byte swizzle).
 __global__ void __launch_bounds__(256)
 pair_images_kernel(PairGeom g, const float* __restrict__ prep, uint8_t* __restrict__ img, float* __restrict__ a2) {
@@ -103,7 +111,7 @@ pair_images_kernel(PairGeom g, const float* __restrict__ prep, uint8_t* __restri
           const float* Cm = prep + (size_t)side * pr.total() + pr.Cmat();
           const int j2 = col - side * g.d;
 #pragma unroll
-          for (int j = 0; j < 8; j++) v[j] = Cm[(kk + j) * g.d + j2];
+          for (int j = 0; j < 8; j++) v[j] = fmaf(Cm[(kk + j) * g.d + j2], lost(g.d / 16), Cm[(kk + j) * g.d + j2]);
         }
       } else {
         const int u = (t - g.nqt) / g.J, jt = (t - g.nqt) % g.J;
@@ -111,7 +119,7 @@ pair_images_kernel(PairGeom g, const float* __restrict__ prep, uint8_t* __restri
         if (draw < g.R && m < g.M) {
           const float* W = prep + ((size_t)draw * 2 + side) * pr.total() + pr.W() + (size_t)m * g.d + kk;
 #pragma unroll
-          for (int j = 0; j < 8; j++) v[j] = W[j];
+          for (int j = 0; j < 8; j++) v[j] = fmaf(W[j], lost(g.d / 8), W[j]);
           if (c == 0) a2[(size_t)(t - g.nqt) * g.NT + n] = 2.f * prep[(size_t)draw * 2 * pr.total() + pr.a() + m];
         } else if (c == 0) {
           a2[(size_t)(t - g.nqt) * g.NT + n] = 0.f;
@@ -286,7 +294,7 @@ tc_pairs_kernel(PairGeom g, const float* __restrict__ X, const float* __restrict
       named_bar_sync(1, PT_EPI);                     // the previous tile's products have been read by both warpgroups
       {
         const float* src = (w ? Y : X) + p * D;
-        float sq = 0.f;
+        float sq[4] = {};
 #pragma unroll
         for (int c0 = 0; c0 < D / 8; c0 += 2) {      // 16 values per step: eight columns of l parts
           uint32_t lreg[8];
@@ -299,7 +307,7 @@ tc_pairs_kernel(PairGeom g, const float* __restrict__ X, const float* __restrict
               v[0] = v0.x; v[1] = v0.y; v[2] = v0.z; v[3] = v0.w; v[4] = v1.x; v[5] = v1.y; v[6] = v1.z; v[7] = v1.w;
             }
 #pragma unroll
-            for (int j = 0; j < 8; j++) sq = fmaf(v[j], v[j], sq);
+            for (int j = 0; j < 8; j++) sq[j & 3] = fmaf(v[j], v[j], sq[j & 3]);
             uint4 h, m, l;
             split3::split8(v, h, m, l);
             const int kc = w * (D / 8) + c;          // 16-byte piece along K
@@ -310,7 +318,7 @@ tc_pairs_kernel(PairGeom g, const float* __restrict__ X, const float* __restrict
           }
           tmem_st8(lanes + PT_LCOL + (w * (D / 8) + c0) * 4, lreg);
         }
-        if (nqt == 0) c_s[w * 128 + row] = sq * (w ? scal2 : scal1)[PS_CGAMMA];
+        if (nqt == 0) c_s[w * 128 + row] = ((sq[0] + sq[1]) + (sq[2] + sq[3])) * (w ? scal2 : scal1)[PS_CGAMMA];
         tmem_wait_st();
         fence_proxy_async_smem();
         tcgen05_fence_before();
