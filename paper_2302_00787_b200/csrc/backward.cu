@@ -42,7 +42,7 @@ bwd_tri_kernel(const float* __restrict__ G, const T* __restrict__ V, TensorAddr 
   const int i0 = blockIdx.x * ROWS, j0 = blockIdx.y * ROWS, C = q.C, dv = q.dv;
   if (j0 > i0) return;
   mma3::Block blk;
-  blk.begin(smem, ROWS, status);
+  blk.begin(smem, ROWS, q.NP, status);
   const int rows = min(C, q.Lq - c * C);
   const float* Gc = G + ((int64_t)bh * q.Lq + (int64_t)c * C + i0) * q.NP;
   const T* Vc = V + b * av.sb + h * av.sh + ((int64_t)c * C + j0) * av.sl;
@@ -81,7 +81,7 @@ bwd_numden_kernel(const float* __restrict__ phiQ, const float* __restrict__ KV, 
   const int C = q.C, M = q.M, NP = q.NP, dv = q.dv, L = q.Lq;
   const ColTile ct(dv, blockIdx.y);
   mma3::Block blk;
-  blk.begin(smem, ct.nt(), status);
+  blk.begin(smem, ct.nt(), M + (q.causal ? C : 0), status);
   const int chunk = q.causal ? i0 / C : 0;
   const float* PQ = phiQ + ((int64_t)bh * L + i0) * M;
   const float* S = KV + ((int64_t)bh * q.nch + chunk) * M * NP;
@@ -189,7 +189,7 @@ bwd_dfeat_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK,
   const int C = q.C, M = q.M, NP = q.NP, dv = q.dv, L = SIDE == 1 ? q.Lq : q.Lk;
   const int chunk = q.causal ? i0 / C : 0, ic = q.causal ? i0 - chunk * C : 0;
   mma3::Block blk;
-  blk.begin(smem, min(ROWS, M - m0), status);
+  blk.begin(smem, min(ROWS, M - m0), NP + (q.causal ? C : 0), status);
   const float* S = St + ((int64_t)bh * q.nch + chunk) * M * NP + (int64_t)m0 * NP;
   const float* GV = q.causal ? gv + ((int64_t)bh * q.nch + chunk) * C * C : nullptr;
   const int64_t width = 4LL * min(ROWS, M - m0);
@@ -264,26 +264,26 @@ bwd_dv_kernel(const float* __restrict__ phiK, const float* __restrict__ Rt, cons
   fs_grid_dependency_wait();
   extern __shared__ uint8_t smem[];
   const int bh = blockIdx.z, b = bh / q.H, h = bh % q.H, j0 = blockIdx.x * ROWS;
-  const int C = q.C, M = q.M, NP = q.NP, dv = q.dv, L = q.Lk;
+  const int C = q.C, M = q.M, NP = q.NP, L = q.Lk, cols = tile_columns(q.dv, M), c0 = blockIdx.y * cols;
   const int chunk = q.causal ? j0 / C : 0, jc = q.causal ? j0 - chunk * C : 0;
   mma3::Block blk;
-  blk.begin(smem, dv, status);
+  blk.begin(smem, cols, M + (q.causal ? C - jc : 0), status);
   const float* PK = phiK + ((int64_t)bh * L + j0) * M;
   const float* R = Rt + ((int64_t)bh * q.nch + chunk) * M * NP;
   mma3::prefetch_rows(PK, 4LL * M, min(ROWS, L - j0), 4LL * M);
   blk.template segment<true, 3, false, 3>(
       M, [&](int r, int k, Piece<3>& p) { if (j0 + r < L) p.load(PK + (int64_t)r * M + k); else p.zero(); },
-      [&](int c, int k, Piece<3>& p) { p.load(R + (int64_t)k * NP + c); });
+      [&](int c, int k, Piece<3>& p) { p.load(R + (int64_t)k * NP + c0 + c); });
   if (q.causal) {
     const float* SC = sc + ((int64_t)bh * q.nch + chunk) * C * C;
     const float* Gc = G + ((int64_t)bh * L + (int64_t)chunk * C + jc) * NP;
     blk.template segment<false, 3, false, 3>(
         min(C, L - chunk * C) - jc, [&](int r, int k, Piece<3>& p) { p.load(SC + (int64_t)(jc + k) * C + jc + r); },
-        [&](int c, int k, Piece<3>& p) { p.load(Gc + (int64_t)k * NP + c); });
+        [&](int c, int k, Piece<3>& p) { p.load(Gc + (int64_t)k * NP + c0 + c); });
   }
   blk.finish();
   T* Ob = dV + b * av.sb + h * av.sh + (int64_t)j0 * av.sl;
-  blk.rows([&](int r, int c, float4 v) { if (j0 + r < L) store4(Ob + (int64_t)r * av.sl + c, v); });
+  blk.rows([&](int r, int c, float4 v) { if (j0 + r < L) store4(Ob + (int64_t)r * av.sl + c0 + c, v); });
   blk.end();
 }
 
@@ -296,7 +296,7 @@ bwd_dx_kernel(const float* __restrict__ E, const float* __restrict__ rs, int mti
   fs_grid_dependency_wait();
   extern __shared__ uint8_t smem[];
   __shared__ float rs_s[ROWS];
-  const int bh = blockIdx.z, b = bh / H, h = bh % H, i0 = blockIdx.x * ROWS;
+  const int bh = blockIdx.z, b = bh / H, h = bh % H, i0 = blockIdx.x * ROWS, cols = tile_columns(d, M), c0 = blockIdx.y * cols;
   PrepLayout pr{d, M};
   const float* pp = prep + ((size_t)(pool == FSHARP_POOL_PER_BH ? bh : h) * 2 + (side - 1)) * pr.total();
   const float* W = pp + pr.W();
@@ -304,7 +304,7 @@ bwd_dx_kernel(const float* __restrict__ E, const float* __restrict__ rs, int mti
   const bool cscalar = pp[pr.scal() + PS_CSCALAR] != 0.f;
   const float gamma = pp[pr.scal() + PS_CGAMMA];
   mma3::Block blk;
-  blk.begin(smem, d, status);
+  blk.begin(smem, cols, M + d, status);
   if (threadIdx.x < ROWS) {
     float s = 0.f;
     if (i0 + (int)threadIdx.x < L)
@@ -317,7 +317,7 @@ bwd_dx_kernel(const float* __restrict__ E, const float* __restrict__ rs, int mti
   const T* Xb = X + b * ax.sb + h * ax.sh + (int64_t)i0 * ax.sl;
   blk.template segment<true, 3, false, 3>(
       M, [&](int r, int k, Piece<3>& p) { if (i0 + r < L) p.load(Eb + (int64_t)r * M + k); else p.zero(); },
-      [&](int c, int k, Piece<3>& p) { p.load(W + (size_t)k * d + c); });
+      [&](int c, int k, Piece<3>& p) { p.load(W + (size_t)k * d + c0 + c); });
   if (!cscalar)
     blk.template segment<true, 3, false, 3>(
         d,
@@ -329,14 +329,15 @@ bwd_dx_kernel(const float* __restrict__ E, const float* __restrict__ rs, int mti
           p.v[4] = s * c.x; p.v[5] = s * c.y; p.v[6] = s * c.z; p.v[7] = s * c.w;
         },
         [&](int c, int k, Piece<3>& p) {
-          p.load(Cm + (size_t)k * d + c);
+          p.load(Cm + (size_t)k * d + c0 + c);
 #pragma unroll
-          for (int j = 0; j < 8; j++) p.v[j] += Cm[(size_t)(c + j) * d + k];
+          for (int j = 0; j < 8; j++) p.v[j] += Cm[(size_t)(c0 + c + j) * d + k];
         });
   blk.finish();
   T* Ob = dX + b * ax.sb + h * ax.sh + (int64_t)i0 * ax.sl;
   bool bad = false;
-  blk.rows([&](int r, int c, float4 v) {
+  blk.rows([&](int r, int column, float4 v) {
+    const int c = c0 + column;
     if (i0 + r >= L) return;
     if (cscalar) {
       const float s = 2.f * gamma * rs_s[r];
@@ -405,9 +406,10 @@ int backward_t(fsharp_ctx* ctx, const void* Qv, const void* Kv, const void* Vv, 
     }
     return FSHARP_OK;
   };
-  const dim3 gtri(causal ? C / ROWS : 1, causal ? C / ROWS : 1, BH * nch);
+  const dim3 gtri(causal ? C / ROWS : 1, causal ? C / ROWS : 1, BH * nch), gsc(gtri.x, causal ? C / tile_columns(ROWS, M) : 1, BH * nch);
+  const int dtiles = d / tile_columns(d, M);
   FS_TRY(sums(No{}, phiK, Lk, KV, 0));
-  if (causal) FS_TRY(mma3::launch(ctx, FS_K_SCORES, scores_kernel, gtri, phiQ, phiK, Lq, M, C, nch, sc, status));
+  if (causal) FS_TRY(mma3::launch(ctx, FS_K_SCORES, scores_kernel, gsc, phiQ, phiK, Lq, M, C, nch, sc, status));
   FS_TRY(mma3::launch(ctx, FS_K_BWD_NUMDEN, bwd_numden_kernel<T>, dim3(qt, ctiles, BH), phiQ, KV, sc, V, av, dY, ay, q, G, status));
   if (ctiles > 1) {
     int gx = (Lq + 7) / 8;
@@ -420,12 +422,12 @@ int backward_t(fsharp_ctx* ctx, const void* Qv, const void* Kv, const void* Vv, 
   FS_TRY(sums(Yes{}, phiQ, Lq, Rt, 1));
   if (causal) FS_TRY(mma3::launch(ctx, FS_K_SCORES, bwd_tri_kernel<T>, gtri, G, V, av, q, gv, status));
   FS_TRY(mma3::launch(ctx, FS_K_BWD_DFEAT, bwd_dfeat_kernel<T, 1>, dim3(mt * qt, 1, BH), phiQ, phiK, G, KV, gv, V, av, q, E, rs, status));
-  FS_TRY(mma3::launch(ctx, FS_K_BWD_DX, bwd_dx_kernel<T>, dim3(qt, 1, BH), E, rs, mt, Q, aq, H, Lq, d, M, dm->pool, 1, prep, qk_scale,
+  FS_TRY(mma3::launch(ctx, FS_K_BWD_DX, bwd_dx_kernel<T>, dim3(qt, dtiles, BH), E, rs, mt, Q, aq, H, Lq, d, M, dm->pool, 1, prep, qk_scale,
                       (T*)dQv, status));
   FS_TRY(mma3::launch(ctx, FS_K_BWD_DFEAT, bwd_dfeat_kernel<T, 2>, dim3(mt * kt, 1, BH), phiQ, phiK, G, Rt, gv, V, av, q, E, rs, status));
-  FS_TRY(mma3::launch(ctx, FS_K_BWD_DX, bwd_dx_kernel<T>, dim3(kt, 1, BH), E, rs, mt, K, ak, H, Lk, d, M, dm->pool, 2, prep, qk_scale,
+  FS_TRY(mma3::launch(ctx, FS_K_BWD_DX, bwd_dx_kernel<T>, dim3(kt, dtiles, BH), E, rs, mt, K, ak, H, Lk, d, M, dm->pool, 2, prep, qk_scale,
                       (T*)dKv, status));
-  return mma3::launch(ctx, FS_K_BWD_DV, bwd_dv_kernel<T>, dim3(kt, 1, BH), phiK, Rt, sc, G, q, (T*)dVv, av, status);
+  return mma3::launch(ctx, FS_K_BWD_DV, bwd_dv_kernel<T>, dim3(kt, dv / tile_columns(dv, M), BH), phiK, Rt, sc, G, q, (T*)dVv, av, status);
 }
 
 }  // namespace

@@ -29,7 +29,7 @@ out_kernel(const float* __restrict__ phiQ, const float* __restrict__ KV, const f
   const int i0 = blockIdx.x * mma3::ROWS;
   const ColTile ct(dv, blockIdx.y);
   mma3::Block blk;
-  blk.begin(smem, ct.nt(), status);
+  blk.begin(smem, ct.nt(), M + (causal ? C : 0), status);
   const float* PQ = phiQ + ((int64_t)bh * L + i0) * M;
   const int chunk = causal ? i0 / C : 0;
   const float* S = KV + (int64_t)(causal ? bh * nchunks + chunk : bh) * M * NP;
@@ -138,7 +138,7 @@ int attend_t(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const
   (void)fs_launch_chained(prefix_kernel, dim3((unsigned)((elems + NTH - 1) / NTH), BH), dim3(NTH), 0, ctx->stream, st, nch, elems, 0, nullptr);
   FS_TIME_END(ctx);
   FS_LAUNCH_CHECK(ctx);
-  FS_TRY(mma3::launch(ctx, FS_K_SCORES, scores_kernel, dim3(C / mma3::ROWS, C / mma3::ROWS, BH * nch), phiQ, phiK, Lq, M, C, nch, sc,
+  FS_TRY(mma3::launch(ctx, FS_K_SCORES, scores_kernel, dim3(C / mma3::ROWS, C / tile_columns(mma3::ROWS, M), BH * nch), phiQ, phiK, Lq, M, C, nch, sc,
                       ctx->d_status));
   return mma3::launch(ctx, FS_K_OUT, out_kernel<T>, gout, phiQ, st, sc, (const T*)V, av, (T*)Y, ay, H, Lq, M, dv, 1, C, nch, nullptr,
                       nullptr, ctx->d_status);

@@ -34,7 +34,7 @@ state_kernel(const float* __restrict__ F, const T* __restrict__ V, TensorAddr av
   if (j0 >= j1) return;
   const ColTile ct(dv, blockIdx.y);
   mma3::Block blk;
-  blk.begin(smem, ct.nt(), status);
+  blk.begin(smem, ct.nt(), j1 - j0, status);
   const float* P = F + ((int64_t)bh * L + j0) * M + m0;
   const float* Gb = FROM_G ? G + ((int64_t)bh * L + j0) * NP : nullptr;
   const T* Vb = V + b * av.sb + h * av.sh + (int64_t)j0 * av.sl;
@@ -90,6 +90,9 @@ prefix_kernel(float* __restrict__ st, int nchunks, int64_t elems, int reverse, _
   }
 }
 
+// Columns of a tile of a product over M features (mma3.cuh: LONG_K).
+__host__ __device__ inline int tile_columns(int columns, int M) { return M > mma3::LONG_K && columns > 64 ? 64 : columns; }
+
 // ---- masked in-chunk scores: sc[bh, c][i][j] = (j <= i) phiQ_i . phiK_j; tiles above the diagonal are neither written nor read
 __global__ void __launch_bounds__(mma3::THREADS, 2)
 scores_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK, int L, int M, int C, int nchunks,
@@ -97,10 +100,10 @@ scores_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK, in
   fs_grid_dependency_wait();
   extern __shared__ uint8_t smem[];
   const int bh = blockIdx.z / nchunks, c = blockIdx.z % nchunks;
-  const int i0 = blockIdx.x * mma3::ROWS, j0 = blockIdx.y * mma3::ROWS;
-  if (j0 > i0) return;
+  const int cols = tile_columns(mma3::ROWS, M), i0 = blockIdx.x * mma3::ROWS, j0 = blockIdx.y * cols;
+  if (j0 >= i0 + mma3::ROWS) return;
   mma3::Block blk;
-  blk.begin(smem, mma3::ROWS, status);
+  blk.begin(smem, cols, M, status);
   const int rows = min(C, L - c * C);                                  // the last chunk may be short
   const float* PQ = phiQ + ((int64_t)bh * L + (int64_t)c * C) * M;
   const float* PK = phiK + ((int64_t)bh * L + (int64_t)c * C) * M;

@@ -8,7 +8,11 @@
 // conversion and epilogue run under the other's products.  Per slice of 128 x 128: 12 MMAs of 65 cycles (both operands
 // fp32) against about 400 issue cycles of conversion.
 // Two accumulators: h h products in one, everything with an m or l part in the other.  The tensor core truncates the
-// accumulator at every MMA, so the large sum must not take the small products' steps too (tc_pairs.cu has the figures).
+// accumulator at every MMA, so the large sum must not take the small products' steps too (tc_pairs.cu has the figures).  Where
+// K exceeds 128 and the columns leave room (80 of them at most) the h h products take turns in two accumulators, slice by
+// slice, so that each is truncated half as often; callers with K > 256 cut wider products into tiles of 64 columns for it.
+// (Attention outputs, d = 64, L = 2048, relative error at M = 512 and 1024: 2.3e-6 and 4.9e-6 with one, 1.3e-6 and 2.5e-6 with
+// two, 1.5e-6 and 1.6e-6 for fp32 multiply-adds.)
 //
 // Operand slices: contracted index contiguous ("K-major"): rows of 64 bytes, 64-byte swizzle; row / column index
 // contiguous ("MN-major"): panels of 64 x 32, rows of 128 bytes, 128-byte swizzle.  Nothing is transposed on the way.
@@ -21,7 +25,9 @@ namespace mma3 {
 constexpr int THREADS = 288, PRODUCERS = 256, KS = 32, ROWS = 128;
 constexpr uint32_t PART = 8192;                       // 128 x 32 bf16
 constexpr uint32_t STAGE = 6 * PART;                  // A: h, m, l; B: h, m, l
-constexpr uint32_t TMEM = 256, CORR = 128;            // main accumulator at column 0, the small products' at 128
+// main accumulator at column 0, the small products' at 128; or the two main ones at 0 and SECOND, the small products' at CORR2
+constexpr uint32_t TMEM = 256, CORR = 128, SECOND = 80, CORR2 = 160;
+constexpr int LONG_K = 256;                           // from here on two main accumulators are worth narrower tiles
 
 struct Misc {
   uint64_t full[2], empty[2], done;
@@ -82,16 +88,20 @@ struct Block {
   uint8_t* sm;
   Misc* misc;
   int* status;
-  uint32_t tmem;
+  uint32_t tmem, corr;                                // corr: first column of the small products' accumulator
+  bool two;                                           // two main accumulators
   int nt, it;                                         // columns of the product; slices so far
   int warp, lane;
 
-  // every thread of the block; `columns` a multiple of 16, at most 128
-  __device__ __forceinline__ void begin(uint8_t* raw, int columns, int* status_word) {
+  // every thread of the block; `columns` a multiple of 16, at most 128; K: length of all segments together (where it
+  // exceeds 128 there are two slices at least)
+  __device__ __forceinline__ void begin(uint8_t* raw, int columns, int K, int* status_word) {
     sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~(uintptr_t)1023);
     misc = reinterpret_cast<Misc*>(sm + 2 * STAGE);
     status = status_word;
     nt = columns;
+    two = columns <= (int)SECOND && K > 128;
+    corr = two ? CORR2 : CORR;
     it = 0;
     warp = threadIdx.x >> 5;
     lane = threadIdx.x & 31;
@@ -135,17 +145,18 @@ struct Block {
 #pragma unroll
           for (int k = 0; k < 2; k++) {
             if (k < steps) {
-              const uint32_t a = al + k * ka, b = bl + k * kb, more = (it | k) ? 1u : 0u;
+              const uint32_t a = al + k * ka, b = bl + k * kb, more = (it | k) ? 1u : 0u, small = tmem + corr;
               if (AP == 3) {
-                tc::mma_bf16_lh(tmem + CORR, a + 2 * P, ah, b, bh, idesc, more);
-                tc::mma_bf16_lh(tmem + CORR, a + P, ah, b, bh, idesc, 1u);
+                tc::mma_bf16_lh(small, a + 2 * P, ah, b, bh, idesc, more);
+                tc::mma_bf16_lh(small, a + P, ah, b, bh, idesc, 1u);
               }
               if (BP == 3) {
-                tc::mma_bf16_lh(tmem + CORR, a, ah, b + 2 * P, bh, idesc, AP == 3 ? 1u : more);
-                tc::mma_bf16_lh(tmem + CORR, a, ah, b + P, bh, idesc, 1u);
+                tc::mma_bf16_lh(small, a, ah, b + 2 * P, bh, idesc, AP == 3 ? 1u : more);
+                tc::mma_bf16_lh(small, a, ah, b + P, bh, idesc, 1u);
               }
-              if (AP == 3 && BP == 3) tc::mma_bf16_lh(tmem + CORR, a + P, ah, b + P, bh, idesc, 1u);
-              tc::mma_bf16_lh(tmem, a, ah, b, bh, idesc, more);
+              if (AP == 3 && BP == 3) tc::mma_bf16_lh(small, a + P, ah, b + P, bh, idesc, 1u);
+              const bool other = two && (it & 1);
+              tc::mma_bf16_lh(other ? tmem + SECOND : tmem, a, ah, b, bh, idesc, it > (two ? 1 : 0) || k > 0 ? 1u : 0u);
             }
           }
           tc::mma_commit(&misc->empty[st]);
@@ -208,15 +219,16 @@ struct Block {
 
   // One column of the product; thread (warps 0-3) = row.
   __device__ __forceinline__ float column(int c) const {
-    uint32_t a[8], b[8];
+    uint32_t a[8], b[8], d[8];
     const uint32_t at = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(c & ~7);
     tc::tmem_ld8(at, a);
-    tc::tmem_ld8(at + CORR, b);
+    tc::tmem_ld8(at + corr, b);
+    if (two) tc::tmem_ld8(at + SECOND, d);
     tc::tmem_wait_ld();
     float v = 0.f;
 #pragma unroll
     for (int j = 0; j < 8; j++)
-      if (j == (c & 7)) v = __uint_as_float(a[j]) + __uint_as_float(b[j]);
+      if (j == (c & 7)) v = __uint_as_float(a[j]) + (two ? __uint_as_float(b[j]) + __uint_as_float(d[j]) : __uint_as_float(b[j]));
     return v;
   }
 
@@ -245,8 +257,15 @@ struct Block {
         if (q < wide) {
           uint32_t a[16], b[16];
           tc::tmem_ld16(lanes + c + q * 16, a);
-          tc::tmem_ld16(lanes + CORR + c + q * 16, b);
+          tc::tmem_ld16(lanes + corr + c + q * 16, b);
           tc::tmem_wait_ld();
+          if (two) {
+            uint32_t d[16];
+            tc::tmem_ld16(lanes + SECOND + c + q * 16, d);
+            tc::tmem_wait_ld();
+#pragma unroll
+            for (int j = 0; j < 16; j++) b[j] = __float_as_uint(__uint_as_float(b[j]) + __uint_as_float(d[j]));
+          }
 #pragma unroll
           for (int j = 0; j < 4; j++)
             *reinterpret_cast<float4*>(buf + lane * 32 + (((q * 4 + j) ^ (lane & 7)) << 2)) =

@@ -121,7 +121,7 @@ prep_kernel(const float* __restrict__ Omega, int64_t omega_head_stride, const do
     for (int j = 0; j < 8; j++) piece.v[j] = (float)p[j];
   };
   mma3::Block b;
-  b.begin(raw, is_a ? d : SIDES * d, status);
+  b.begin(raw, is_a ? d : SIDES * d, d, status);
   b.template segment<true, 3, false, 3>(d, omega, matrix);
   b.finish();
   if (!is_a) {
