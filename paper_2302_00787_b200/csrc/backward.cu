@@ -12,7 +12,9 @@
 // Causal sequences go chunk by chunk: KV_i = (sum over earlier chunks) + the masked part inside the
 // chunk, R_j = (sum over later chunks) + the masked part, with tril(P_c S_c^T) and tril(G_c [V_c | 1]^T)
 // formed per chunk.  The feature kernels' shifts (per query row, per (batch, head) for the keys)
-// cancel in every product above exactly as they do in Y.
+// cancel in every product above exactly as they do in Y.  Their factor 2^LIFT on either side (feat3.cuh)
+// would leave G with 2^-2 LIFT; it is given half of that back, so that R and G KV^T are what they are without the factor (a
+// query that sees distant keys only has G near the top of the range), and the gradients' last products take off 2^LIFT.
 #include "f32_parts.cuh"
 #include "feat3.cuh"
 
@@ -20,6 +22,8 @@ namespace {
 
 using mma3::Piece;
 using mma3::ROWS;
+
+constexpr float LIFTED = (float)(1 << feat3::LIFT), UNLIFT = 1.f / LIFTED;
 
 struct BwdDims {
   int H, Lq, Lk, d, dv, M, NP, causal, C, nch;      // NP = dv + 16: [V | 1] rows, G rows and sums are padded to it
@@ -127,7 +131,8 @@ bwd_numden_kernel(const float* __restrict__ phiQ, const float* __restrict__ KV, 
              if (i0 + r < L && c < dv) {
                const float inv = inv_s[r];
                s = fmaf(y.x, v.x * inv, fmaf(y.y, v.y * inv, fmaf(y.z, v.z * inv, y.w * (v.w * inv))));
-               *reinterpret_cast<float4*>(Gb + (int64_t)r * NP + c) = make_float4(y.x * inv, y.y * inv, y.z * inv, y.w * inv);
+               const float gi = LIFTED * inv;
+               *reinterpret_cast<float4*>(Gb + (int64_t)r * NP + c) = make_float4(y.x * gi, y.y * gi, y.z * gi, y.w * gi);
              }
              if (i >= 0) { sum[i < 0 ? 0 : i] += s; return; }
              // (four neighbouring lanes hold the row's last 16 columns)
@@ -139,7 +144,7 @@ bwd_numden_kernel(const float* __restrict__ phiQ, const float* __restrict__ KV, 
   __syncthreads();
   for (int e = threadIdx.x; e < ROWS * 4; e += mma3::THREADS) {
     const int r = e >> 2, part = e & 3;
-    if (i0 + r < L) *reinterpret_cast<float4*>(Gb + (int64_t)r * NP + dv + 4 * part) = make_float4(part ? 0.f : -dot_s[r] * inv_s[r], 0.f, 0.f, 0.f);
+    if (i0 + r < L) *reinterpret_cast<float4*>(Gb + (int64_t)r * NP + dv + 4 * part) = make_float4(part ? 0.f : -dot_s[r] * (LIFTED * inv_s[r]), 0.f, 0.f, 0.f);
   }
   blk.end();
 }
@@ -154,17 +159,17 @@ bwd_g_kernel(float* __restrict__ ND, const T* __restrict__ dY, TensorAddr ay, Bw
   const T* dYb = dY + b * ay.sb + h * ay.sh;
   for (int i = blockIdx.x * 8 + warp; i < q.Lq; i += gridDim.x * 8) {
     float* row = ND + ((int64_t)bh * q.Lq + i) * q.NP;
-    const float den = row[dv], inv = 1.f / den;
+    const float den = row[dv], inv = 1.f / den, gi = LIFTED * inv;
     float s = 0.f;
     for (int c = 4 * lane; c < dv; c += 128) {
       const float4 y = load4(dYb + (int64_t)i * ay.sl + c), n = *reinterpret_cast<const float4*>(row + c);
       s = fmaf(y.x, n.x * inv, fmaf(y.y, n.y * inv, fmaf(y.z, n.z * inv, fmaf(y.w, n.w * inv, s))));
-      *reinterpret_cast<float4*>(row + c) = make_float4(y.x * inv, y.y * inv, y.z * inv, y.w * inv);
+      *reinterpret_cast<float4*>(row + c) = make_float4(y.x * gi, y.y * gi, y.z * gi, y.w * gi);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
-      row[dv] = -s * inv;
+      row[dv] = -s * gi;
       if (!(den > 0.f) || !isfinite(den)) atomicExch(status, FSHARP_E_NONFINITE);
     }
   }
@@ -237,7 +242,7 @@ bwd_dfeat_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK,
   float sum[8] = {};
   blk.rows([&](int r, int c) { return i0 + r < L ? *reinterpret_cast<const float4*>(Ph + (int64_t)r * M + c) : make_float4(0.f, 0.f, 0.f, 0.f); },
            [&](int r, int c, float4 v, float4 f, int i) {
-             v.x *= f.x; v.y *= f.y; v.z *= f.z; v.w *= f.w;
+             v.x = UNLIFT * v.x * f.x; v.y = UNLIFT * v.y * f.y; v.z = UNLIFT * v.z * f.z; v.w = UNLIFT * v.w * f.w;
              float s = 0.f;
              if (i0 + r < L) {
                *reinterpret_cast<float4*>(E + base + (int64_t)r * M + c) = v;
@@ -283,7 +288,9 @@ bwd_dv_kernel(const float* __restrict__ phiK, const float* __restrict__ Rt, cons
   }
   blk.finish();
   T* Ob = dV + b * av.sb + h * av.sh + (int64_t)j0 * av.sl;
-  blk.rows([&](int r, int c, float4 v) { if (j0 + r < L) store4(Ob + (int64_t)r * av.sl + c0 + c, v); });
+  blk.rows([&](int r, int c, float4 v) {
+    if (j0 + r < L) store4(Ob + (int64_t)r * av.sl + c0 + c, make_float4(UNLIFT * v.x, UNLIFT * v.y, UNLIFT * v.z, UNLIFT * v.w));
+  });
   blk.end();
 }
 
@@ -385,8 +392,8 @@ int backward_t(fsharp_ctx* ctx, const void* Qv, const void* Kv, const void* Vv, 
   const int64_t elems = (int64_t)M * NP;
   const dim3 gscan((unsigned)((elems + NTH - 1) / NTH), BH);
 
-  const feat3::Task tasks[2] = {{K, ak, Lk, 2, FSHARP_STAB_GROUP, rowck, gmax, phiK, nullptr, lsk},
-                                {Q, aq, Lq, 1, FSHARP_STAB_ROW, rowcq, nullptr, phiQ, nullptr, lsq}};
+  const feat3::Task tasks[2] = {{K, ak, Lk, 2, FSHARP_STAB_GROUP, rowck, gmax, phiK, nullptr, lsk, feat3::LIFT},
+                                {Q, aq, Lq, 1, FSHARP_STAB_ROW, rowcq, nullptr, phiQ, nullptr, lsq, feat3::LIFT}};
   FS_TRY(feat3::run(ctx, tasks, 2, dtype, B, H, d, M, dm->pool, prep, qk_scale, img));
   // sums over tokens: the total (bidirectional), or one per chunk turned into the sum over earlier / later chunks (causal)
   auto sums = [&](auto from_g, const float* F, int L, float* out, int reverse) -> int {

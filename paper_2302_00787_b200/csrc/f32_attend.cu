@@ -98,8 +98,8 @@ int attend_t(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const
   float* lsq = ws->take<float>((size_t)BH * Lq);
   float* lsk = ws->take<float>((size_t)BH);
   uint8_t* img = ws->take<uint8_t>(feat3::image_bytes(fs_groups(dm), d, M, 2));
-  const feat3::Task tasks[2] = {{K, ak, Lk, 2, FSHARP_STAB_GROUP, rowc, gmax, phiK, phiK16, lsk},
-                                {Q, aq, Lq, 1, FSHARP_STAB_ROW, rowcq, nullptr, phiQ, phiQ16, lsq}};
+  const feat3::Task tasks[2] = {{K, ak, Lk, 2, FSHARP_STAB_GROUP, rowc, gmax, phiK, phiK16, lsk, feat3::LIFT},
+                                {Q, aq, Lq, 1, FSHARP_STAB_ROW, rowcq, nullptr, phiQ, phiQ16, lsq, feat3::LIFT}};
   FS_TRY(feat3::run(ctx, tasks, 2, sizeof(T) == 2 ? FSHARP_BF16 : FSHARP_F32, B, H, d, M, dm->pool, prep, qk_scale, img));
   const dim3 gout((Lq + mma3::ROWS - 1) / mma3::ROWS, ctiles, BH);
   const dim3 gkv((M + mma3::ROWS - 1) / mma3::ROWS, ctiles, 1);
@@ -149,7 +149,7 @@ int attend_t(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const
 int fs_simt_featurize(fsharp_ctx* ctx, const void* X, int dtype, TensorAddr ax, int B, int H, int L, int d,
                       int M, int pool, const float* prep, int side, float qk_scale, int stab,
                       float* rowc, unsigned* gmax, float* phi, float* logscale, uint8_t* img) {
-  const feat3::Task task{X, ax, L, side, stab, rowc, gmax, phi, nullptr, logscale};
+  const feat3::Task task{X, ax, L, side, stab, rowc, gmax, phi, nullptr, logscale, 0};
   return feat3::run(ctx, &task, 1, dtype, B, H, d, M, pool, prep, qk_scale, img);
 }
 

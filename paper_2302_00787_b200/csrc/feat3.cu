@@ -40,6 +40,13 @@ __device__ __forceinline__ void atomic_max_float(float* p, float v) {
   else atomicMin(reinterpret_cast<unsigned*>(p), __float_as_uint(v));
 }
 
+// 2^x with subnormal results
+__device__ __forceinline__ float ex2_full(float x) {
+  float y;
+  asm("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 // 32 bytes (eight words) as one store; p is 32-byte aligned
 __device__ __forceinline__ void store32(float* p, const uint32_t* x) {
   asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(x[4]),
@@ -530,7 +537,7 @@ feat3_kernel(const __grid_constant__ Args a) {
     } else {
       const int wg = warp >> 2;
       float gmx = -3.0e38f;
-      const float gshift = (WRITE && t.stab == FSHARP_STAB_GROUP) ? ord2f(t.gmax[bh]) : 0.f;
+      const float gshift = (WRITE && t.stab == FSHARP_STAB_GROUP) ? ord2f(t.gmax[bh]) - t.lift : 0.f;
       const bool own = t.stab == FSHARP_STAB_ROW && a.nmb == 1;
       const bool wide = WRITE && !OUT16 && (reinterpret_cast<uintptr_t>(t.phi) & 31) == 0;
       // x ln 2, x + y being rounded to x: one rounding in all
@@ -587,14 +594,14 @@ feat3_kernel(const __grid_constant__ Args a) {
           }
           mx = fmaxf(mx, my);
           if (WRITE) {
-            add = -mx;
+            add = t.lift - mx;
             const float top = mx + ci, big = fabsf(mx) > fabsf(ci) ? mx : ci, small = fabsf(mx) > fabsf(ci) ? ci : mx;
-            if (t.logscale && in) t.logscale[at] = to_nat(top, small - (top - big));
+            if (t.logscale && in) t.logscale[at] = to_nat(top - t.lift, small - (top - big));
           } else if (t.stab == FSHARP_STAB_GROUP) {
             if (in) gmx = fmaxf(gmx, mx + ci);
           } else {
             // (nudged upwards by the rounding of the two conversions, so that no feature exceeds one)
-            const float ls = to_nat(mx + ci, 0.f);
+            const float ls = to_nat(mx + ci - t.lift, 0.f);
             if (in) atomic_max_float(t.logscale + at, fmaf(fabsf(ls), 2.4e-7f, ls));
           }
         }
@@ -612,7 +619,7 @@ feat3_kernel(const __grid_constant__ Args a) {
               for (int j = 0; j < 32; j += 2) add2(x[j], x[j + 1], -shift, -shift);
             }
 #pragma unroll
-            for (int j = 0; j < 32; j++) x[j] = __float_as_uint(ex2(__uint_as_float(x[j])));
+            for (int j = 0; j < 32; j++) x[j] = __float_as_uint(OUT16 ? ex2(__uint_as_float(x[j])) : ex2_full(__uint_as_float(x[j])));
             if (in) {
               float* dst = out + c;
               if (OUT16) {                               // (M is a multiple of 128 and the scratch aligned)

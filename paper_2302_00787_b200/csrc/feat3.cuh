@@ -4,6 +4,12 @@
 
 namespace feat3 {
 
+// Features that stay inside the library (attention, its gradients, the kernel operator) carry a factor 2^LIFT against shifted ones:
+// three bf16 parts hold all 24 bits of a value only above 2^-109 (split3.cuh), fp32 multiply-adds held them down to 2^-126,
+// and a causal query may see nothing but keys that lie far below the sequence's largest.  It cancels wherever shifts do; what
+// it costs is the top of the range: a product of both sides overflows 2^32 earlier.
+constexpr int LIFT = 16;
+
 struct Task {
   const void* X;          // tokens, strides ax (elements)
   TensorAddr ax;
@@ -13,11 +19,9 @@ struct Task {
   float* phi;             // [B*H][L][M], or
   __nv_bfloat16* phi16;   // the same rounded to bf16 (bf16 tokens with d = 128 only; phi is then not written, and the shifts
                           // are those of a maximum taken from the leading parts of W)
-  float* logscale;        // as fsharp_featurize; may be null (FSHARP_STAB_ROW: only when needs_logscale() says so)
+  float* logscale;        // as fsharp_featurize (of the lifted features); may be null where M fits one block of features
+  int lift;               // 0 or LIFT: features times 2^lift (FSHARP_STAB_ROW and _GROUP)
 };
-
-// Features of a block: all of M when M <= this, so that a row's largest exponent is known inside the block.
-inline bool needs_logscale(int d, int M, int stab) { return stab == FSHARP_STAB_ROW && M > (d == 128 ? 128 : 256); }
 
 // Scratch for the operand images of W.
 size_t image_bytes(int groups, int d, int M, int ntasks);

@@ -151,3 +151,52 @@ def test_sums_over_many_features(d, causal):
         tuple(fs.favor_sharp_attention_vjp(Q[0, 0], K[0, 0], V[0, 0], dY[0, 0], Om, p, causal=causal))
     for g, r in zip(got, ref):
         assert np.linalg.norm(g[0, 0] - r) < 2.0 ** -19 * np.linalg.norm(r)
+
+
+@pytest.mark.parametrize("level", [40.0, 80.0])
+@pytest.mark.parametrize("d,dv", [(32, 16), (16, 128)])
+def test_queries_that_see_only_keys_far_below_the_largest(d, dv, level):
+    """Causal, fp32: the features of the first 100 keys lie `level` nats below those of the later ones (at 80 nats most of
+    what counts lies between 2^-115 and 2^-125, still normal numbers).  What the rows that see nothing else get is as exact as anything, and so are its gradients."""
+    rng = np.random.default_rng(8)
+    L, M = 256, 48
+    Q, K = (0.5 * rng.standard_normal((1, 1, L, d)).astype(np.float32) for _ in range(2))
+    V, dY = (rng.standard_normal((1, 1, L, dv)).astype(np.float32) for _ in range(2))
+    Om = rng.standard_normal((M, d)).astype(np.float32)
+    Q[..., 1], K[..., 1], Om[:, 1] = 0.0, 0.0, 1.0
+    K[0, 0, 100:, 1] = level
+    dY[0, 0, 100:] = 0.0
+    I = np.eye(d)
+    p = {"A": 0 * I, "B1": I, "B2": I, "C1": 0 * I, "C2": 0 * I, "logD": 0.0}
+    ctx = fb.Context(0)
+    t = [dev(x) for x in (Q, K, V, dY)]
+    blob = dev(fb.pack_params(p, d)[None])
+    at = dict(causal=True, chunk=64)
+    Y = host(ctx.fsharp_attend(*t[:3], dev(Om), blob, **at))[0, 0]
+    grads = [host(g)[0, 0] for g in ctx.fsharp_attend_backward(*t, dev(Om), blob, **at)]
+    assert ctx.status() == 0
+    ref = fs.favor_sharp_attention(Q[0, 0], K[0, 0], V[0, 0], Om, p, causal=True)
+    # an exponent of 90 nats is known to two units in its last place, 1.5e-5
+    assert rel_err(Y[:100], ref[:100]) < 3e-5 and rel_err(Y[100:], ref[100:]) < 3e-5
+    for g, r in zip(grads, fs.favor_sharp_attention_vjp(Q[0, 0], K[0, 0], V[0, 0], dY[0, 0], Om, p, causal=True)):
+        assert rel_err(g[:100], r[:100]) < 3e-5
+
+
+@pytest.mark.parametrize("d,M", [(64, 256), (32, 512)])
+def test_subnormal_features(d, M):
+    """Features below 2^-126 of the row's largest are what fp32 has there: off by half of 2^-149, and the exponent's own error."""
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    X = 4.0 * torch.randn(1, 1, 2000, d, generator=gen, device="cuda")
+    qk = float(np.float32(d ** -0.25))
+    Om = dev(wl.orthogonal_omega(M, d, 1))
+    I = np.eye(d)
+    blob = dev(fb.pack_params({"A": 0 * I, "B1": 2 * I, "B2": I, "C1": -0.5 * I, "C2": -0.5 * I, "logD": 0.0}, d)[None])
+    ctx = fb.Context(0)
+    phi, ls = ctx.fsharp_featurize(X, Om, blob, 1, qk_scale=qk, stab=fb.STAB_ROW)
+    assert ctx.status() == 0
+    x = qk * X[0, 0].double()
+    e = 2.0 * (x @ Om.double().T) - 0.5 * (x * x).sum(1, keepdim=True) - 0.5 * np.log(M)
+    want = (e - ls[0, 0].double()[:, None]).exp()
+    tiny = (want < 2.0 ** -126) & (want > 2.0 ** -148)
+    assert tiny.sum() > 100
+    assert ((phi[0, 0].double() - want).abs() <= 2.0 ** -149 + 1e-4 * want)[tiny].all()
