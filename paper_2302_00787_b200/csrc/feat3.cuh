@@ -17,8 +17,8 @@ struct Task {
   float* rowc;            // [B*H][L] scratch: the x^T C x terms
   unsigned* gmax;         // [B*H] scratch, FSHARP_STAB_GROUP
   float* phi;             // [B*H][L][M], or
-  __nv_bfloat16* phi16;   // the same rounded to bf16 (bf16 tokens with d = 128 only; phi is then not written, and the shifts
-                          // are those of a maximum taken from the leading parts of W)
+  __nv_bfloat16* phi16;   // the same rounded to bf16 (bf16 tokens with d = 128 only; phi is then not written, and a group's shift
+                          // is that of a maximum taken from the leading parts of W)
   float* logscale;        // as fsharp_featurize (of the lifted features); may be null where M fits one block of features
   int lift;               // 0 or LIFT: features times 2^lift (FSHARP_STAB_ROW and _GROUP)
 };
