@@ -110,6 +110,14 @@ inline cudaError_t fs_launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 b
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
+// Lets `kernel` be launched with any amount of dynamic shared memory that fits beside its own static_bytes.  The limit belongs to
+// the kernel, not to the launch: a launch that sets it to just what it needs takes it from another thread's, whose launch of the same
+// kernel with more then fails.  So it only ever gets this one value.
+constexpr int FS_SMEM_PER_BLOCK = 232448;
+template <class K>
+inline cudaError_t fs_allow_smem(K kernel, size_t static_bytes = 0) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FS_SMEM_PER_BLOCK - (int)static_bytes);
+}
 #endif
 
 void fs_time_begin(fsharp_ctx* ctx, int tag);

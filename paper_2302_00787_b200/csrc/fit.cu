@@ -1353,8 +1353,7 @@ int fs_run_fit(fsharp_ctx* ctx, const double* stats, int G, int d, int variant, 
     a.flag_stride = fitw::Layout{d}.total();
   }
   size_t smem = fit_smem_bytes(d, a.v_in_smem);
-  if (a.v_in_smem) FS_CUDA_OK(cudaFuncSetAttribute(fit_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  else FS_CUDA_OK(cudaFuncSetAttribute(fit_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  FS_CUDA_OK(a.v_in_smem ? fs_allow_smem(fit_kernel<true>) : fs_allow_smem(fit_kernel<false>));
   FS_TIME_BEGIN(ctx, FS_K_FIT);
   if (a.v_in_smem) (void)fs_launch_chained(fit_kernel<true>, dim3(G), dim3(FIT_THREADS), smem, ctx->stream, a);
   else (void)fs_launch_chained(fit_kernel<false>, dim3(G), dim3(FIT_THREADS), smem, ctx->stream, a);

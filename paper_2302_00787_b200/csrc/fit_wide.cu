@@ -873,13 +873,11 @@ finish_kernel(int variant, const double* __restrict__ scratch, double* __restric
 // Dynamic shared memory that spreads `blocks` blocks evenly over the SMs: a launch that begins while its predecessor drains puts
 // as many blocks as fit on the first SMs that come free, where they share one fp64 pipe and one shared-memory pipe (64
 // tridiagonalisations: 70 us so, 51 us spread).
-template <class K>
-size_t spread(const fsharp_ctx* ctx, K kernel, int blocks, size_t need) {
+size_t spread(const fsharp_ctx* ctx, size_t static_bytes, int blocks, size_t need) {
   const int per_sm = (blocks + ctx->sm_count - 1) / ctx->sm_count;
-  cudaFuncAttributes at;
-  if (per_sm > 4 || cudaFuncGetAttributes(&at, kernel) != cudaSuccess) return need;
+  if (per_sm > 4) return need;
   // more than a (per_sm + 1)-th of the SM's 228 KB (1 KB per block is the system's)
-  const size_t room = (size_t)(228 * 1024) / (per_sm + 1) + 128, fixed = at.sharedSizeBytes + 1024;
+  const size_t room = (size_t)(228 * 1024) / (per_sm + 1) + 128, fixed = static_bytes + 1024;
   const size_t want = room > fixed ? room - fixed : 0;
   return want > need ? want : need;
 }
@@ -890,8 +888,10 @@ int run_d(fsharp_ctx* ctx, const double* stats, int G, int variant, double ridge
 #define FITW_LAUNCH(kernel, grid, threads, smem, ...)                                       \
   do {                                                                                      \
     const dim3 gr = grid;                                                                   \
-    const size_t sm = spread(ctx, kernel, (int)(gr.x * gr.y), smem);                        \
-    FS_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)); \
+    cudaFuncAttributes at;                                                                  \
+    FS_CUDA_OK(cudaFuncGetAttributes(&at, kernel));                                         \
+    FS_CUDA_OK(fs_allow_smem(kernel, at.sharedSizeBytes));                                  \
+    const size_t sm = spread(ctx, at.sharedSizeBytes, (int)(gr.x * gr.y), smem);            \
     FS_TIME_BEGIN(ctx, FS_K_FIT);                                                           \
     (void)fs_launch_chained(kernel, gr, dim3(threads), sm, st, __VA_ARGS__);                \
     FS_TIME_END(ctx);                                                                       \

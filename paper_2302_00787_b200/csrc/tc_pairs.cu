@@ -438,7 +438,7 @@ int fs_tc_pairs(fsharp_ctx* ctx, const float* X, const float* Y, int64_t np, int
   const size_t smem = 1024 + (size_t)g.nks * 2 * TILE_BYTES + (size_t)g.stages * g.stage_bytes() + 1024 + sizeof(PtMisc);
 #define FS_TCP(DD)                                                                                                       \
   do {                                                                                                                   \
-    FS_CUDA_OK(cudaFuncSetAttribute(tc_pairs_kernel<DD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));        \
+    FS_CUDA_OK(fs_allow_smem(tc_pairs_kernel<DD>));                                                                       \
     FS_TIME_BEGIN(ctx, FS_K_PAIRS);                                                                                       \
     (void)fs_launch_chained(tc_pairs_kernel<DD>, grid, dim3(PT_THREADS), smem, ctx->stream, g, X, Y, np, prep, img, a2, usplit, ups, nitems, est,    \
                                                                  ctx->d_status);                                         \
