@@ -244,6 +244,14 @@ def measured_peaks():
     return peaks
 
 
+def fit_report(timing, steps, groups):
+    """The joint fit of a step from the timing (total milliseconds, launches) of its kernels over `steps` steps."""
+    ms, launches = timing if timing else (None, 0)
+    return {"launches_per_step": launches / steps, "groups": groups, "ms": ms / steps if timing else None,
+            "note": "one call fits the groups of all workloads of the step, as a chain of launches (d = 64 and 128) or one; ms is their "
+                    "sum, each bracketed by its own pair of events; every workload's ms_per_step_alone includes a fit of its own"}
+
+
 def backward_flops(w):
     """Multiply-adds x 2 of the backward pass as the kernels issue them (Section 2.2 differentiated; the header of
     csrc/backward.cu lists the products): features of both sides, the two key- / query-side sums, numerators and
@@ -401,7 +409,7 @@ def main():
     ap.add_argument("--backward", action="store_true",
                     help="also time fsharp_attend_backward on the workloads (fp32 kernels; a few GB of scratch)")
     ap.add_argument("--fit-per-workload", action="store_true",
-                    help="one fit launch per workload instead of one launch over the groups of all workloads of a step")
+                    help="one fit per workload instead of one over the groups of all workloads of a step")
     ap.add_argument("--kernel-impl", default="auto", choices=["auto", "simt", "tensor"])
     args = ap.parse_args()
 
@@ -428,9 +436,8 @@ def main():
     # weak scaling: every rank runs the whole workload on a draw of its own; no data-path collective
     runners = [Runner(w, args, dev, local_rank, rank_seed(0, rank)) for w in ws]
     stream = torch.cuda.current_stream(dev)
-    # The closed-form fit runs one block per parameter group and is bound by the latency of its factorisations, not by
-    # the number of groups: the workloads of a step that share (d, variant) are fitted by ONE launch over all their
-    # groups.  Their statistics and parameters then live in one buffer each, of which every workload holds a slice.
+    # The closed-form fit is bound by the latency of its factorisations, not by the number of groups: the workloads of a
+    # step that share (d, variant) are fitted by ONE call over all their groups.  Their statistics and parameters then live in one buffer each, of which every workload holds a slice.
     joint_fit = (not args.fit_per_workload and len(runners) > 1
                  and len({(r.w.d, r.w.variant) for r in runners}) == 1)
     if joint_fit:
@@ -607,7 +614,7 @@ def main():
     cfg.update({"kernel_impl": args.kernel_impl, "steps_in_flight": 1,
                 "l2": f"inputs rotate over {args.buffers} resident sets per workload "
                       f"({args.buffers * algorithmic_work(ws[0])['bytes'] / 1e6:.0f} MB > 126 MB L2)",
-                "step": ("stats per workload, one fit launch over the parameter groups of all workloads, then prep + featurize + "
+                "step": ("stats per workload, one fit over the parameter groups of all workloads, then prep + featurize + "
                          "contraction per workload" if joint_fit else "per workload: stats + fit + prep + featurize + contraction")})
     out = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
@@ -623,11 +630,7 @@ def main():
         "workloads": per_workload,
     }
     if joint_fit:
-        fk = per_kernel[0].get("fit_kernel")
-        out["fit"] = {"launches_per_step": 1, "groups": int(st_all.shape[0]),
-                      "ms": fk[0] / fk[1] if fk else None,
-                      "note": "one launch fits the groups of all workloads of the step (one block per group); every "
-                              "workload's ms_per_step_alone includes a fit launch of its own"}
+        out["fit"] = fit_report(per_kernel[0].get("fit_kernel"), ksteps, int(st_all.shape[0]))
     if args.backward and world == 1:
         out["backward"] = backward_leg(runners)
     if e2e is not None:
