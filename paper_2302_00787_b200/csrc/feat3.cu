@@ -750,8 +750,11 @@ int run_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, int g
 
 }  // namespace
 
+// Images of very many groups (none beyond 1 GB) are not worth their memory: a group's tokens are then few, and every block converts
+// the W of its own.
 size_t feat3::image_bytes(int groups, int d, int M, int ntasks) {
-  return ws_round((size_t)ntasks * groups * ((d + 63) / 64) * 3 * M * 128);
+  const size_t bytes = ws_round((size_t)ntasks * groups * ((d + 63) / 64) * 3 * M * 128);
+  return bytes <= ((size_t)1 << 30) ? bytes : 0;
 }
 
 int feat3::run(fsharp_ctx* ctx, const Task* tasks, int ntasks, int dtype, int B, int H, int d, int M, int pool, const float* prep,
@@ -763,6 +766,7 @@ int feat3::run(fsharp_ctx* ctx, const Task* tasks, int ntasks, int dtype, int B,
   a.pow2 = (float)ldexp(1.0, e < -100 ? -100 : (e > 100 ? 100 : e));
   a.quad = LOG2E * (double)qk_scale * (double)qk_scale / ((double)a.pow2 * (double)a.pow2);
   const int groups = pool == FSHARP_POOL_PER_BH ? B * H : H;
+  if (image_bytes(groups, d, M, ntasks) == 0) img = nullptr;
 #define FS_FEAT3(DD)                                                                                          \
   return dtype == FSHARP_F32 ? run_t<float, DD, 3>(ctx, a, tasks, ntasks, B * H, groups, qk_scale, img)                    \
                              : run_t<__nv_bfloat16, DD, 3>(ctx, a, tasks, ntasks, B * H, groups, qk_scale, img)

@@ -23,7 +23,7 @@ struct Task {
   int lift;               // 0 or LIFT: features times 2^lift (FSHARP_STAB_ROW and _GROUP)
 };
 
-// Scratch for the operand images of W.
+// Scratch for the operand images of W (0: none are kept).
 size_t image_bytes(int groups, int d, int M, int ntasks);
 
 // Images of W (img, 16-byte aligned; nullptr: the blocks convert W themselves), quadratic terms, largest exponents where a

@@ -1333,11 +1333,24 @@ size_t fit_smem_bytes(int d, int v_in_smem) {
 
 }  // namespace
 
-size_t fs_fit_scratch_doubles(int G, int d) { return (size_t)G * (5 * d * d + (d >= 64 ? fitw::Layout{d}.total() : 0)); }
+// From d = 64 on the chain keeps eight more matrices per group than the one-block kernel does: groups go through in batches of
+// this many (fourteen blocks per SM), so that a call with very many of them needs no more memory for it (d = 128: 3.6 GB).
+constexpr int FIT_BATCH = 2048;
 
-int fs_run_fit(fsharp_ctx* ctx, const double* stats, int G, int d, int variant, double ridge,
+static size_t group_doubles(int d) { return 5 * (size_t)d * d + (d >= 64 ? fitw::Layout{d}.total() : 0); }
+size_t fs_fit_scratch_doubles(int G, int d) { return (size_t)(d >= 64 && G > FIT_BATCH ? FIT_BATCH : G) * group_doubles(d); }
+
+static int fit_batch(fsharp_ctx* ctx, const double* stats, int G, int d, int variant, double ridge, double* params, double* scratch);
+int fs_run_fit(fsharp_ctx* ctx, const double* stats, int G, int d, int variant, double ridge, double* params, double* scratch) {
+  const int batch = d >= 64 ? FIT_BATCH : G;
+  for (int g = 0; g < G; g += batch)
+    FS_TRY(fit_batch(ctx, stats + (size_t)g * StatsLayout{d}.total(), G - g < batch ? G - g : batch, d, variant, ridge,
+                     params + (size_t)g * ParamsLayout{d}.total(), scratch));
+  return FSHARP_OK;
+}
+
+static int fit_batch(fsharp_ctx* ctx, const double* stats, int G, int d, int variant, double ridge,
                double* params, double* scratch) {
-  if (G == 0) return FSHARP_OK;
   FitArgs a;
   a.stats = stats; a.params = params; a.scratch = scratch; a.d = d; a.variant = variant; a.ridge = ridge;
   a.v_in_smem = d <= 64 ? 1 : 0;

@@ -207,19 +207,33 @@ pairvar_kernel(const float* __restrict__ X, const float* __restrict__ Y, int64_t
 
 }  // namespace
 
+// Draws that go through together: as many as prepared operands and images of 1 GB hold (a multiple of 128, so that column tiles of
+// several draws are cut as in one go), all of them in any study but one of thousands of draws.
+static int draws_per_batch(int d, int M, int R) {
+  const size_t per = 2 * PrepLayout{d, M}.total() * sizeof(float) + fs_tc_pairs_scratch_bytes(d, M, 128) / 128;
+  const size_t n = ((size_t)1 << 30) / per / 128 * 128;
+  return (size_t)R <= n ? R : (int)n;
+}
+
 size_t fs_pairs_scratch_bytes(int d, int M, int R) {
-  return ws_round((size_t)R * 2 * PrepLayout{d, M}.total() * sizeof(float)) +
-         ws_round((3 * (size_t)d * d + 1) * sizeof(double)) + fs_tc_pairs_scratch_bytes(d, M, R);
+  const int n = draws_per_batch(d, M, R);
+  return ws_round((size_t)n * 2 * PrepLayout{d, M}.total() * sizeof(float)) +
+         ws_round((3 * (size_t)d * d + 1) * sizeof(double)) + fs_tc_pairs_scratch_bytes(d, M, n);
 }
 
 int fs_run_pairs(fsharp_ctx* ctx, const float* X, const float* Y, const float* Omega, const double* params,
                  int64_t npairs, int d, int M, int R, float* est, double* var_cf, double* pooled, WsAlloc* ws) {
-  float* prep = ws->take<float>((size_t)R * 2 * PrepLayout{d, M}.total());
+  const int batch = draws_per_batch(d, M, R);
+  float* prep = ws->take<float>((size_t)batch * 2 * PrepLayout{d, M}.total());
   double* ev = ws->take<double>(3 * (size_t)d * d + 1);
-  // one "group" per draw, all reading the same parameter blob
-  FS_TRY(fs_run_prep(ctx, Omega, (int64_t)M * d, params, 0, R, R, FSHARP_POOL_PER_HEAD, d, M, prep));
+  for (int r = 0; r < R; r += batch) {
+    const int n = R - r < batch ? R - r : batch;
+    // one "group" per draw, all reading the same parameter blob
+    FS_TRY(fs_run_prep(ctx, Omega + (int64_t)r * M * d, (int64_t)M * d, params, 0, n, n, FSHARP_POOL_PER_HEAD, d, M, prep));
+    WsAlloc rest = *ws;
+    if (npairs > 0) FS_TRY(fs_tc_pairs(ctx, X, Y, npairs, d, M, n, prep, est + (int64_t)r * npairs, &rest));
+  }
   if (npairs == 0) return FSHARP_OK;
-  FS_TRY(fs_tc_pairs(ctx, X, Y, npairs, d, M, R, prep, est, ws));
   if (var_cf) {
     FS_TIME_BEGIN(ctx, FS_K_PAIRVAR_PREP);
     (void)fs_launch_chained(pairvar_prep_kernel, dim3(d), dim3(128), 0, ctx->stream, params, d, ev, ctx->d_status);

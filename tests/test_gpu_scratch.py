@@ -1,0 +1,60 @@
+"""Scratch memory of calls with very many groups or draws: what is kept per group beyond the prepared operands is bounded."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2302_00787_b200 import binding as fb
+from paper_2302_00787_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+def identity(d):
+    I = np.eye(d)
+    return torch.from_numpy(fb.pack_params({"A": 0 * I, "B1": I, "B2": I, "C1": -0.5 * I, "C2": -0.5 * I, "logD": 0.0}, d)).cuda()
+
+
+@pytest.mark.parametrize("variant", ["sderf", "gerf"])
+def test_fit_of_many_groups(variant):
+    """More groups than one batch takes, the last batch a short one: equal matrices get equal parameters wherever they are."""
+    d, G = 64, 4500
+    rng = np.random.default_rng(1)
+    X = rng.standard_normal((3, 8 * d, d)) / d ** 0.5
+    blob = torch.from_numpy(np.stack([np.concatenate([(x.T @ x / 8).ravel(), (x.T @ x / 8).ravel(), np.zeros(2 * d)]) for x in X])).cuda()
+    ctx = fb.Context(0)
+    want = ctx.fsharp_fit_params(blob, d, variant)
+    pr = ctx.fsharp_fit_params(blob.repeat(G // 3, 1), d, variant)
+    assert ctx.status() == 0 and torch.equal(pr, want.repeat(G // 3, 1))
+    assert ctx.workspace_bytes() < 1.2e9                  # 2048 groups of 13 matrices, an eighth in reserve: 1.0e9
+
+
+def test_features_of_many_groups():
+    """4096 groups of 1024 features: no operand images of W (1.6 GB a side)."""
+    B, H, L, d, M = 64, 64, 8, 16, 1024
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    Q, K, V = (0.5 * torch.randn(B, H, L, d, generator=gen, device="cuda") for _ in range(3))
+    Om = torch.from_numpy(wl.iid_omega(M, d, 1)).cuda()
+    ctx = fb.Context(0)
+    pr = identity(d).expand(B * H, -1).contiguous()
+    Y = ctx.fsharp_attend(Q, K, V, Om, pr)
+    assert ctx.status() == 0 and ctx.workspace_bytes() < 2.2e9      # operands 0.6e9, features 0.3e9, states 0.5e9, an eighth in reserve
+    small = fb.Context(0)
+    for b in (0, B - 1):
+        # (sums of eight keys in one block: the same order of addition)
+        assert torch.allclose(Y[b], small.fsharp_attend(Q[b:b + 1], K[b:b + 1], V[b:b + 1], Om, pr[:H])[0], rtol=1e-5, atol=1e-6)
+
+
+def test_pairs_of_many_draws():
+    """600 draws of 1024 features at d = 128 are two batches; a draw's estimates do not depend on the batch it is in."""
+    d, M, R = 128, 1024, 600
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    X, Y = (0.1 * torch.randn(70, d, generator=gen, device="cuda") for _ in range(2))
+    Om = torch.randn(R, M, d, generator=gen, device="cuda")
+    ctx = fb.Context(0)
+    est, var, pooled = ctx.fsharp_pair_estimate(X, Y, Om, identity(d), want_pooled=True)
+    assert ctx.status() == 0 and ctx.workspace_bytes() < 1.3e9
+    small = fb.Context(0)
+    for r in (0, 383, 384, 599):
+        assert torch.equal(est[r], small.fsharp_pair_estimate(X, Y, Om[r:r + 1], identity(d), want_variance=False)[0][0])
+    ratio = est.double() / (X.double() * Y.double()).sum(1).exp()
+    assert abs(pooled[0].item() / ratio.var(dim=0).mean().item() - 1) < 1e-6
