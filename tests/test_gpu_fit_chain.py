@@ -1,5 +1,5 @@
 """The chain of fit kernels for d = 64 and 128 (ADERF, SDERF) where groups of one launch take different ways: ordinary spectra
-through the chain, equal eigenvalues through the Jacobi solver behind it, more groups than SMs."""
+through the chain, eigenvalues equal to rounding through the Jacobi solver behind it, more groups than SMs."""
 import numpy as np
 import pytest
 import torch
@@ -41,7 +41,10 @@ def test_mixed_groups(variant, d, copies):
         # "wide": either side's eigenvalues of Z are exact to 2^-53 |Z| d, that is 2^-53 d cond(Z) of the smallest, which carries
         # the largest entries of B1^T B1; Z has the eigenvalues lam (lam / 2 + 1/10), cond 5e6
         assert_fit_close(fb.unpack_params(first[g], d), ref, d, max(1e-8, 2.0 ** -53 * d * 5e6) if kinds[g] == "wide" else 1e-8)
-    assert first[1, 5 * d * d + 3] >= 0 and first[0, 5 * d * d + 3] == 0      # sweeps: none for the ordinary matrix
+    # Jacobi sweeps: none in the chain; vectors of eigenvalues that agree to rounding are not orthonormal there, and the Jacobi solver
+    # takes over.  (A multiple of the identity goes there too and needs no sweep.)
+    sweeps = first[:, 5 * d * d + 3].tolist()
+    assert sweeps[0] == 0 and sweeps[kinds.index("clusters")] > 0
 
 
 @pytest.mark.parametrize("variant", ["sderf", "aderf"])
