@@ -6,8 +6,7 @@ contraction over one batch of synthetic input.  Prints ONE JSON line (rank 0).
 
 The default workload is the pair of L = 8192, d = 64, M = 256 configurations, causal (cfg3) and
 bidirectional (cfg3b): a step is one pass of each, `value` counts the tokens of both.  One step is in
-flight at a time (--streams S > 1 keeps S independent steps in flight and reports that figure under
-"overlapped", never as the headline).
+flight at a time.
 """
 from __future__ import annotations
 

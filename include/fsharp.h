@@ -149,14 +149,15 @@ int fsharp_stats(fsharp_ctx* ctx, const void* Q, const void* K, const fsharp_dim
 /* Closed-form minimisers of the shifted log-variance objective (Section 3.1):
  * PosRF and GERF (Section 2.3 / 3.1), SADERF (Section 4.3), ADERF (Theorem 4.2),
  * SDERF (Theorem 4.3), all through Lemma A.1's scalar map.  The symmetric
- * eigenproblems are solved on the device in fp64, one thread block per group
- * (d <= 64: tridiagonalisation, Sturm multisection and twisted-factorisation vectors,
- * confirmed by a cyclic Jacobi solver; d = 128: the Jacobi solver).  ADERF factors
+ * eigenproblems are solved on the device in fp64 (ADERF and SDERF at d = 64 and
+ * 128 by a chain of kernels, the rest and what that chain gives up by one thread block
+ * per group: tridiagonalisation, Sturm multisection and twisted-factorisation vectors,
+ * confirmed or completed by a cyclic Jacobi solver).  ADERF factors
  * M1 = L L^T (Cholesky) and solves one eigenproblem, of L^T M2 L: its eigenvectors
  * and eigenvalues are U and Sigma^2 of the theorem's SVD for the factor L^T of M1
  * (any factor F with F^T F = M1 gives the same B1, B2).  The literal B is "one of
- * the solutions" of the theorems (eigenvector signs and rotations inside equal
- * eigenvalues are free); there is no second, canonical form of the parameters.
+ * the solutions" of the theorems (eigenvector signs, rotations inside equal
+ * eigenvalues and, for ADERF, the order of the rows are free); there is no second, canonical form of the parameters.
  * ridge >= 0 adds ridge * tr(M)/d * I to M1 and M2 first (0 = the paper's formulas).
  * stats: device, G groups.  params: device, G * fsharp_params_doubles(d). */
 int fsharp_fit_params(fsharp_ctx* ctx, const double* stats, int G, int d, int variant,
@@ -202,7 +203,9 @@ int fsharp_featurize_static(void* stream, const void* X, const float* Omega, con
 /* Y [B,H,Lq,dv] (type `dtype`) of Section 2.2 with Khat = P S^T in place of the
  * exact kernel matrix, evaluated as P (S^T [V | 1]) (Section 2.1's O(L M n) order).
  * causal != 0 restricts key j to j <= i and evaluates chunk by chunk with a running
- * prefix of S^T [V | 1]; chunk is ignored when causal == 0. */
+ * prefix of S^T [V | 1]; chunk is ignored when causal == 0.
+ * The fp32-precision kernels keep features times 2^16 on either side (queries whose keys all lie some 80 nats below the
+ * sequence's largest lose nothing): sums of |V| times features (at most 1) above 2^96 overflow. */
 int fsharp_attend(fsharp_ctx* ctx, const void* Q, const void* K, const void* V,
                   const float* Omega, const double* params, const fsharp_dims* dims,
                   int dtype, int causal, int chunk, float qk_scale, void* Y);
@@ -216,7 +219,9 @@ int fsharp_attend(fsharp_ctx* ctx, const void* Q, const void* K, const void* V,
  * and, the exponent of Section 4's feature being w^T B x + x^T C x + terms without x,
  * dx = dlog (Omega B) + rowsum(dlog) (C + C^T) x, dQ = qk_scale dx (likewise dK).  causal, chunk, qk_scale and the
  * argument checks are those of fsharp_attend; Q, K, V are read again (nothing is kept from the forward call).
- * fp32 kernels for every shape and both dtypes (bf16 tensors are widened on load, gradients rounded on store).
+ * fp32-precision kernels for every shape and both dtypes (bf16 tensors are widened on load, gradients rounded on store).
+ * (The products run on the tensor cores from three-part bf16 operands: tensor entries below 2^-109 in magnitude carry
+ * fewer than 24 bits.)
  * All pointers are device pointers, 16-byte aligned; asynchronous on the context's stream.  A normaliser that is
  * zero or not finite, or a gradient that is not finite, latches FSHARP_E_NONFINITE in the status word. */
 int fsharp_attend_backward(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const void* dY,

@@ -1,6 +1,7 @@
-// fp32 CUDA-core path: features (Section 4 definition with Section 2.1's M^-1/2) and the
-// linear-attention contraction (Sections 2.1 / 2.2), bidirectional and causal-chunked.
-// Used for fp32 inputs, for shapes the tensor-core path does not take, and on request.
+// Attention at fp32 precision: features from feat3.cu, the linear-attention contraction (Sections 2.1 / 2.2), bidirectional and
+// causal-chunked, on the tensor cores with three-part bf16 operands (mma3.cuh); and the chain of bf16 kernels for d = dv = 128.
+// Used for fp32 inputs, for shapes the fused tensor-core kernels do not take, and on request (FSHARP_IMPL_SIMT: the name is older
+// than the kernels).
 //
 // Scratch (from the context workspace): the two feature matrices, the per-token
 // quadratic term, S^T [V | 1] (per (batch, head); per chunk when causal) and, when

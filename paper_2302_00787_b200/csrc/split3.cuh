@@ -1,6 +1,7 @@
 // fp32 operands on the bf16 tensor cores without loss: x = h + m + l with h = bf16(x), m = bf16(x - h),
 // l = bf16(x - h - m).  The two differences are exact in fp32 and the three parts carry 8 significant bits each, so
-// h + m + l holds all 24 bits of x (while the parts stay above the smallest bf16, i.e. for |x| > 2^-109).  A product of
+// h + m + l holds all 24 bits of x (while the parts stay above the smallest bf16, i.e. for |x| > 2^-109; features inside the library
+// are lifted for it, feat3.cuh; infinities give NaN).  A product of
 // two fp32 operands is the sum of the six part products hh + hm + mh + mm + hl + lh; what is left out (ml, lm, ll) is
 // below 2^-24 of |x||y|, the rounding of one fp32 multiply-add.  Where one operand is a bf16 tensor its value is its h
 // part and three products (hh, mh, lh) are exact.  Every part product is exact in the fp32 accumulator's adder tree.

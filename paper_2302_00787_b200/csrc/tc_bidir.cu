@@ -4,11 +4,11 @@
 //                               phi = 2^(logits + c_j - s)  -> bf16 tile in shared memory
 //                               KV^T += [V | 1]^T phi                        (tcgen05, TMEM)
 //                               (c_j, the key's quadratic term, comes from tc_rowterm_kernel)
-//   query side (tc_out_kernel): first the merge of the key-side partials of its (batch, head): common
-//                               shift, sum, every feature's column scaled to order one (fp16), the
-//                               scales' exponents g (with a2) kept for the logits; then per tile
-//                               logits + g, phi = 2^(... - max of the half row) in fp16,
-//                               [num | den] = phi KV per feature half, halves combined, Y = num / den
+//   merge_kernel                the units that lie in several blocks' ranges: common shift, sum of the partials, every
+//                               feature's column scaled to order one (fp16), the scales' exponents g (with a2) kept for
+//                               the query logits (a unit that one block holds leaves the key side in this form)
+//   query side (tc_out_kernel): per 128-query tile  logits + g, phi = 2^(... - row maximum) in fp16 (tensor memory),
+//                               [num | den] = phi KV, Y = num / den
 //
 // The feature tiles never leave the SM.  One block = 8 epilogue warps (exponentials), one
 // TMA producer warp and one MMA issuing warp; all exponents are kept in log2 units

@@ -5,7 +5,7 @@
 // One block = one 128 x 128 tile of a chunk's C x C score block.  Tiles above the diagonal are all zero and are only
 // written.  The feature index is the contraction: 64 features of both token tiles per TMA stage (two panels with the
 // 128-byte swizzle), four MMAs of N = 128 per stage into one accumulator in tensor memory; the epilogue masks the
-// diagonal tile and writes the rows (fp32, bf16, or both).
+// diagonal tile and writes the rows (bf16).
 #include "common.cuh"
 #include "tc_common.cuh"
 #include "tc_layout.cuh"
