@@ -334,12 +334,14 @@ int fsharp_forward_host(fsharp_ctx* ctx, const void* Q, const void* K, const voi
   const int G2 = G;
   size_t inner = ws_round((size_t)G2 * 2 * PrepLayout{dd.d, dd.M}.total() * 4);
   {
-    size_t a = fs_simt_attend_scratch_bytes(&dd, causal, chunk);
+    // (the nested calls see one batch element at a time, whose pieces may be cut finer and whose operand images may be kept where
+    // those of all would be too many)
+    fsharp_dims one = dd;
+    if (dd.pool == FSHARP_POOL_PER_BH) one.B = 1;
+    const size_t a1 = fs_simt_attend_scratch_bytes(&dd, causal, chunk), a2 = fs_simt_attend_scratch_bytes(&one, causal, chunk);
+    const size_t a = a1 > a2 ? a1 : a2;
     size_t b = 0;
     if (fs_tc_supported(&dd, dtype, causal, chunk, qk_scale)) {
-      // (the nested calls see one batch element at a time, whose pieces may be cut finer)
-      fsharp_dims one = dd;
-      if (dd.pool == FSHARP_POOL_PER_BH) one.B = 1;
       const size_t whole = fs_tc_attend_scratch_bytes(ctx, &dd, causal, chunk), part = fs_tc_attend_scratch_bytes(ctx, &one, causal, chunk);
       b = whole > part ? whole : part;
     }

@@ -58,3 +58,21 @@ def test_pairs_of_many_draws():
         assert torch.equal(est[r], small.fsharp_pair_estimate(X, Y, Om[r:r + 1], identity(d), want_variance=False)[0][0])
     ratio = est.double() / (X.double() * Y.double()).sum(1).exp()
     assert abs(pooled[0].item() / ratio.var(dim=0).mean().item() - 1) < 1e-6
+
+
+def test_host_buffers_of_many_groups():
+    """The images of all groups would pass the bound, those of one batch element do not and are kept: the staging buffers behind the
+    scratch stay where they are."""
+    B, H, L, d, M = 2, 700, 16, 16, 1024
+    gen = torch.Generator().manual_seed(1)
+    Q, K, V = (0.5 * torch.randn(B, H, L, d, generator=gen) for _ in range(3))
+    Om = torch.from_numpy(wl.iid_omega(M, d, 1))
+    ctx = fb.Context(0)
+    Y = ctx.fsharp_forward_host(Q, K, V, Om, "gerf")
+    held = ctx.workspace_bytes()
+    assert ctx.status() == 0
+    dQ, dK, dV = (t.cuda() for t in (Q, K, V))
+    other = fb.Context(0)
+    pr = other.fsharp_fit_params(other.fsharp_stats(dQ, dK), d, "gerf")
+    assert torch.allclose(Y, other.fsharp_attend(dQ, dK, dV, Om.cuda(), pr).cpu(), rtol=1e-4, atol=1e-5)
+    assert torch.equal(Y, ctx.fsharp_forward_host(Q, K, V, Om, "gerf")) and ctx.workspace_bytes() == held
