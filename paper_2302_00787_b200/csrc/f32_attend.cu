@@ -23,7 +23,8 @@ out_kernel(const float* __restrict__ phiQ, const float* __restrict__ KV, const f
            int* __restrict__ status) {
   fs_grid_dependency_wait();
   // lsq != nullptr: the unnormalised operator Khat C of Section 2.1 is wanted: row i of the numerator times
-  // exp(lsq[i] + lsk[bh]), the shifts that the feature kernels took out of phi(Q) and phi(K)
+  // exp(lsq[i] + lsk[bh]), the shifts that the feature kernels took out of phi(Q) and phi(K), without their factors 2^LIFT (taken
+  // off the sums, not off exp(), which may be next to the smallest number as it is)
   extern __shared__ uint8_t smem[];
   __shared__ float inv_s[mma3::ROWS];
   const int bh = blockIdx.z, b = bh / H, h = bh % H, NP = dv + 16;
@@ -70,11 +71,12 @@ out_kernel(const float* __restrict__ phiQ, const float* __restrict__ KV, const f
     inv_s[threadIdx.x] = inv;
   }
   __syncthreads();
+  const float unlift = lsq != nullptr ? 1.f / (float)(1ull << 2 * feat3::LIFT) : 1.f;
   T* Yb = Y + b * ay.sb + h * ay.sh + (int64_t)i0 * ay.sl;
   blk.rows([&](int r, int c, float4 v) {
     if (i0 + r >= L || c >= ct.wt) return;
     const float inv = inv_s[r];
-    store4(Yb + (int64_t)r * ay.sl + ct.v0 + c, make_float4(v.x * inv, v.y * inv, v.z * inv, v.w * inv));
+    store4(Yb + (int64_t)r * ay.sl + ct.v0 + c, make_float4(unlift * v.x * inv, unlift * v.y * inv, unlift * v.z * inv, unlift * v.w * inv));
   });
   blk.end();
 }

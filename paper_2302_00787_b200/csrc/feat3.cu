@@ -540,7 +540,7 @@ feat3_kernel(const __grid_constant__ Args a) {
     } else {
       const int wg = warp >> 2;
       float gmx = -3.0e38f;
-      const float gshift = (WRITE && t.stab == FSHARP_STAB_GROUP) ? ord2f(t.gmax[bh]) - t.lift : 0.f;
+      const float gshift = (WRITE && t.stab == FSHARP_STAB_GROUP) ? ord2f(t.gmax[bh]) : 0.f;
       const bool own = t.stab == FSHARP_STAB_ROW && a.nmb == 1;
       const bool wide = WRITE && !OUT16 && (reinterpret_cast<uintptr_t>(t.phi) & 31) == 0;
       // x ln 2, x + y being rounded to x: one rounding in all
@@ -555,8 +555,8 @@ feat3_kernel(const __grid_constant__ Args a) {
         const float ci = (in ? t.rowc[at] : 0.f) + bias;
         // exponent = acc + add, minus `shift` where that does not come from this block's own maximum: in this order the largest
         // exponent of the group or row, rounded as it was when the maximum was taken, gives 1 and nothing gives more
-        float add = ci, shift = gshift;
-        if (WRITE && t.stab == FSHARP_STAB_ROW && !own) shift = in ? FS_TO_LOG2(t.logscale[at]) : 0.f;
+        float add = ci, shift = gshift - t.lift;
+        if (WRITE && t.stab == FSHARP_STAB_ROW && !own) shift = (in ? FS_TO_LOG2(t.logscale[at]) : 0.f) - t.lift;
         const bool shifted = WRITE && !own && t.stab != FSHARP_STAB_NONE;
         mbar_wait(&misc->t_full[wg], (n >> 1) & 1, &misc->abort_flag, a.status);
         __syncwarp();
@@ -599,12 +599,12 @@ feat3_kernel(const __grid_constant__ Args a) {
           if (WRITE) {
             add = t.lift - mx;
             const float top = mx + ci, big = fabsf(mx) > fabsf(ci) ? mx : ci, small = fabsf(mx) > fabsf(ci) ? ci : mx;
-            if (t.logscale && in) t.logscale[at] = to_nat(top - t.lift, small - (top - big));
+            if (t.logscale && in) t.logscale[at] = to_nat(top, small - (top - big));
           } else if (t.stab == FSHARP_STAB_GROUP) {
             if (in) gmx = fmaxf(gmx, mx + ci);
           } else {
             // (nudged upwards by the rounding of the two conversions, so that no feature exceeds one)
-            const float ls = to_nat(mx + ci - t.lift, 0.f);
+            const float ls = to_nat(mx + ci, 0.f);
             if (in) atomic_max_float(t.logscale + at, fmaf(fabsf(ls), 2.4e-7f, ls));
           }
         }

@@ -19,7 +19,7 @@ struct Task {
   float* phi;             // [B*H][L][M], or
   __nv_bfloat16* phi16;   // the same rounded to bf16 (bf16 tokens with d = 128 only; phi is then not written, and a group's shift
                           // is that of a maximum taken from the leading parts of W)
-  float* logscale;        // as fsharp_featurize (of the lifted features); may be null where M fits one block of features
+  float* logscale;        // as fsharp_featurize (the shift alone, whatever the lift); may be null where M fits one block of features
   int lift;               // 0 or LIFT: features times 2^lift (FSHARP_STAB_ROW and _GROUP)
 };
 

@@ -200,3 +200,22 @@ def test_subnormal_features(d, M):
     tiny = (want < 2.0 ** -126) & (want > 2.0 ** -148)
     assert tiny.sum() > 100
     assert ((phi[0, 0].double() - want).abs() <= 2.0 ** -149 + 1e-4 * want)[tiny].all()
+
+
+def test_kernel_operator_near_the_smallest_numbers():
+    """Shifts of both sides that together are 85 nats below zero (exp: 1e-37) times sums of some thousands: the outputs are normal
+    numbers, and the largest of them come out like any other."""
+    rng = np.random.default_rng(8)
+    d, M = 32, 64
+    X, Y = (0.5 * rng.standard_normal((1, 1, L, d)).astype(np.float32) for L in (100, 300))
+    Om = rng.standard_normal((M, d)).astype(np.float32)
+    I = np.eye(d)
+    p = {"A": 0 * I, "B1": I, "B2": I, "C1": -0.5 * I, "C2": -0.5 * I, "logD": 0.0}
+    logs = [fs.derf_log_features(x[0, 0], Om, p["A"], I, p["C1"], 0.0) for x in (X, Y)]
+    top = logs[0].max() + logs[1].max()
+    p["logD"] = 0.5 * (-85.0 - top)
+    ctx = fb.Context(0)
+    C = np.ones((1, 1, 300, 16), dtype=np.float32)
+    out = host(ctx.fsharp_kernel_apply(dev(X), dev(Y), dev(C), dev(Om), dev(fb.pack_params(p, d)[None])))
+    assert ctx.status() == 0
+    assert rel_err(out[0, 0], fs.kernel_apply(X[0, 0], Y[0, 0], C[0, 0], Om, p, 0.0)) < TOL["f32"]
