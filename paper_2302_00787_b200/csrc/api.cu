@@ -158,7 +158,7 @@ int fsharp_attend(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, 
   // the fp32 path indexes (batch, head, chunk) through a grid z coordinate: refuse before anything is launched
   if (!use_tc && causal && (int64_t)dims->B * dims->H * (dims->Lq / chunk) > 65535) return FSHARP_E_SHAPE;
   const size_t need = ws_round(prep_f * 4) + (use_tc ? fs_tc_attend_scratch_bytes(ctx, dims, causal, chunk)
-                                                     : fs_simt_attend_scratch_bytes(dims, causal, chunk));
+                                                     : fs_simt_attend_scratch_bytes(ctx, dims, causal, chunk));
   FS_TRY(fs_ws_reserve(ctx, need));
   WsAlloc ws{ctx->ws, 0};
   float* prep = ws.take<float>(prep_f);
@@ -298,7 +298,7 @@ int fsharp_kernel_apply(fsharp_ctx* ctx, const void* X, const void* Y, const voi
   const int G = fs_groups(dims);
   const size_t prep_f = (size_t)G * 2 * PrepLayout{dims->d, dims->M}.total();
   const size_t np = (size_t)G * ParamsLayout{dims->d}.total();
-  FS_TRY(fs_ws_reserve(ctx, ws_round(prep_f * 4) + ws_round(np * 8) + fs_simt_attend_scratch_bytes(dims, 0, 0)));
+  FS_TRY(fs_ws_reserve(ctx, ws_round(prep_f * 4) + ws_round(np * 8) + fs_simt_attend_scratch_bytes(ctx, dims, 0, 0)));
   WsAlloc ws{ctx->ws, 0};
   float* prep = ws.take<float>(prep_f);
   double* shifted = ws.take<double>(np);
@@ -338,7 +338,7 @@ int fsharp_forward_host(fsharp_ctx* ctx, const void* Q, const void* K, const voi
     // those of all would be too many)
     fsharp_dims one = dd;
     if (dd.pool == FSHARP_POOL_PER_BH) one.B = 1;
-    const size_t a1 = fs_simt_attend_scratch_bytes(&dd, causal, chunk), a2 = fs_simt_attend_scratch_bytes(&one, causal, chunk);
+    const size_t a1 = fs_simt_attend_scratch_bytes(ctx, &dd, causal, chunk), a2 = fs_simt_attend_scratch_bytes(ctx, &one, causal, chunk);
     const size_t a = a1 > a2 ? a1 : a2;
     size_t b = 0;
     if (fs_tc_supported(&dd, dtype, causal, chunk, qk_scale)) {

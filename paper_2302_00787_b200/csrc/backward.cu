@@ -407,7 +407,7 @@ int backward_t(fsharp_ctx* ctx, const void* Qv, const void* Kv, const void* Vv, 
                         causal ? 1 : 0, out, status));
     if (causal) {
       FS_TIME_BEGIN(ctx, FS_K_PREFIX);
-      (void)fs_launch_chained(prefix_kernel, gscan, dim3(NTH), 0, ctx->stream, out, nch, elems, reverse, nullptr);
+      (void)fs_launch_chained(prefix_kernel, gscan, dim3(NTH), 0, ctx->stream, out, nch, elems, reverse);
       FS_TIME_END(ctx);
       FS_LAUNCH_CHECK(ctx);
     }

@@ -174,7 +174,6 @@ const char* fsharp_kernel_name(int id) {
     case FS_K_TC_STATS: return "tc_stats_kernel";
     case FS_K_TC_ROWTERM: return "tc_rowterm_kernel";
     case FS_K_TC_FEAT: return "tc_feat_kernel";
-    case FS_K_TC_SCORES128: return "tc_scores128_kernel";
     case FS_K_TC_KV128: return "tc_kv128_kernel";
     case FS_K_TC_OUT128: return "tc_out128_kernel";
     default: return "";

@@ -90,7 +90,7 @@ int attend_t(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const
   TensorAddr av = fs_addr(dm->v_stride, H, Lk, dv), ay = fs_addr(dm->y_stride, H, Lq, dv);
   // causal, bf16 tensors, d = dv = 128: scores, per-chunk sums and query side from bf16 features
   const bool tc = causal && !unnormalised && sizeof(T) == 2 && d == 128 && ctx->impl != FSHARP_IMPL_SIMT &&
-                  fs_tc_scores128_supported(M, chunk) && fs_tc_kv128_supported(V, av, dv, M, chunk) && fs_tc_out128_supported(Y, ay);
+                  fs_tc_kv128_supported(V, av, dv, M, chunk) && fs_tc_out128_supported(Y, ay);
   float* phiQ = tc ? nullptr : ws->take<float>((size_t)BH * Lq * M);
   float* phiK = tc ? nullptr : ws->take<float>((size_t)BH * Lk * M);
   __nv_bfloat16* phiQ16 = tc ? ws->take<__nv_bfloat16>((size_t)BH * Lq * M) : nullptr;
@@ -118,18 +118,21 @@ int attend_t(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const
     return FSHARP_OK;
   }
   if (tc) {
-    const int C = chunk, nch = Lq / C, N = dv + 1;
-    const int64_t elems = (int64_t)M * N;
-    float* st = ws->take<float>((size_t)BH * nch * elems);
-    __nv_bfloat16* st16 = ws->take<__nv_bfloat16>((size_t)BH * nch * elems);
-    __nv_bfloat16* sc16 = ws->take<__nv_bfloat16>((size_t)BH * nch * C * C);
-    FS_TRY(fs_tc_kv128(ctx, phiK16, V, av, B, H, Lk, M, C, st));
-    FS_TIME_BEGIN(ctx, FS_K_PREFIX);
-    (void)fs_launch_chained(prefix_kernel, dim3((unsigned)((elems + NTH - 1) / NTH), BH), dim3(NTH), 0, ctx->stream, st, nch, elems, 0, st16);
-    FS_TIME_END(ctx);
-    FS_LAUNCH_CHECK(ctx);
-    FS_TRY(fs_tc_scores128(ctx, phiQ16, phiK16, BH, Lq, M, C, sc16));
-    return fs_tc_out128(ctx, phiQ16, st16, sc16, V, av, Y, ay, B, H, Lq, M, C);
+    const int C = chunk, nch = Lq / C;
+    const int slots = fs_tc_kv128_slots(ctx, BH, M, nch);
+    const int64_t elems = (int64_t)M * (dv + 1);
+    float* tot = ws->take<float>((size_t)BH * slots * elems);
+    __nv_bfloat16* st16 = ws->take<__nv_bfloat16>((size_t)BH * nch * M * dv);
+    __nv_bfloat16* z16 = ws->take<__nv_bfloat16>((size_t)BH * nch * M);
+    if (slots > 1) {
+      FS_TRY(fs_tc_kv128(ctx, phiK16, V, av, B, H, Lk, M, C, tot, nullptr, nullptr));
+      FS_TIME_BEGIN(ctx, FS_K_PREFIX);
+      (void)fs_launch_chained(prefix_kernel, dim3((unsigned)((elems + NTH - 1) / NTH), BH), dim3(NTH), 0, ctx->stream, tot, slots, elems, 0);
+      FS_TIME_END(ctx);
+      FS_LAUNCH_CHECK(ctx);
+    }
+    FS_TRY(fs_tc_kv128(ctx, phiK16, V, av, B, H, Lk, M, C, tot, st16, z16));
+    return fs_tc_out128(ctx, phiQ16, phiK16, st16, z16, V, av, Y, ay, B, H, Lq, M, C);
   }
   const int C = inner_chunk(chunk), nch = (Lq + C - 1) / C;
   const int64_t elems = (int64_t)M * NP;
@@ -138,7 +141,7 @@ int attend_t(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const
   FS_TRY(mma3::launch(ctx, FS_K_KV, state_kernel<T, false>, dim3(gkv.x, gkv.y, BH * nch), phiK, (const T*)V, av, nullptr, H, Lk, M, dv, C, nch, 1, st,
                       ctx->d_status));
   FS_TIME_BEGIN(ctx, FS_K_PREFIX);
-  (void)fs_launch_chained(prefix_kernel, dim3((unsigned)((elems + NTH - 1) / NTH), BH), dim3(NTH), 0, ctx->stream, st, nch, elems, 0, nullptr);
+  (void)fs_launch_chained(prefix_kernel, dim3((unsigned)((elems + NTH - 1) / NTH), BH), dim3(NTH), 0, ctx->stream, st, nch, elems, 0);
   FS_TIME_END(ctx);
   FS_LAUNCH_CHECK(ctx);
   FS_TRY(mma3::launch(ctx, FS_K_SCORES, scores_kernel, dim3(C / mma3::ROWS, C / tile_columns(mma3::ROWS, M), BH * nch), phiQ, phiK, Lq, M, C, nch, sc,
@@ -156,7 +159,7 @@ int fs_simt_featurize(fsharp_ctx* ctx, const void* X, int dtype, TensorAddr ax, 
   return feat3::run(ctx, &task, 1, dtype, B, H, d, M, pool, prep, qk_scale, img);
 }
 
-size_t fs_simt_attend_scratch_bytes(const fsharp_dims* dm, int causal, int chunk) {
+size_t fs_simt_attend_scratch_bytes(const fsharp_ctx* ctx, const fsharp_dims* dm, int causal, int chunk) {
   const size_t BH = (size_t)dm->B * dm->H, NP = dm->dv + 16;
   const size_t shifts = ws_round(BH * dm->Lk * 4) + 2 * ws_round(BH * 4) + 2 * ws_round(BH * dm->Lq * 4) +
                         feat3::image_bytes(fs_groups(dm), dm->d, dm->M, 2);
@@ -166,11 +169,13 @@ size_t fs_simt_attend_scratch_bytes(const fsharp_dims* dm, int causal, int chunk
   } else {
     const size_t C = inner_chunk(chunk), nch = (dm->Lq + C - 1) / C;
     b += ws_round(BH * nch * dm->M * NP * 4) + ws_round(BH * nch * C * C * 4);
-    // the chain on bf16 features: half the bytes for the features, sums in fp32 and bf16, scores in bf16
-    const size_t N = dm->dv + 1;
-    const size_t t = ws_round(BH * dm->Lq * dm->M * 2) + ws_round(BH * dm->Lk * dm->M * 2) + shifts +
-                     ws_round(BH * nch * dm->M * N * 4) + ws_round(BH * nch * dm->M * N * 2) + ws_round(BH * nch * C * C * 2);
-    if (t > b) b = t;
+    // the chain on bf16 features: half the bytes for the features, running sums in bf16, no scores
+    if (dm->d == 128 && dm->dv == 128 && dm->M % 128 == 0 && (chunk == 128 || chunk == 256)) {
+      const size_t t = ws_round(BH * dm->Lq * dm->M * 2) + ws_round(BH * dm->Lk * dm->M * 2) + shifts +
+                       ws_round(BH * fs_tc_kv128_slots(ctx, (int)BH, dm->M, (int)nch) * dm->M * 129 * 4) + ws_round(BH * nch * dm->M * 128 * 2) +
+                       ws_round(BH * nch * dm->M * 2);
+      if (t > b) b = t;
+    }
   }
   return b;
 }

@@ -63,7 +63,7 @@ state_kernel(const float* __restrict__ F, const T* __restrict__ V, TensorAddr av
 
 // ---- exclusive running sum over the chunks, forwards (earlier chunks) or backwards (later chunks) ------
 __global__ void __launch_bounds__(NTH)
-prefix_kernel(float* __restrict__ st, int nchunks, int64_t elems, int reverse, __nv_bfloat16* __restrict__ st16) {
+prefix_kernel(float* __restrict__ st, int nchunks, int64_t elems, int reverse) {
   fs_grid_dependency_wait();
   const int bh = blockIdx.y;
   float* base = st + (int64_t)bh * nchunks * elems;
@@ -80,10 +80,7 @@ prefix_kernel(float* __restrict__ st, int nchunks, int64_t elems, int reverse, _
 #pragma unroll
       for (int u = 0; u < 8; u++) {
         const int c = reverse ? nchunks - 1 - (c0 + u) : c0 + u;
-        if (c0 + u < nchunks) {
-          if (!st16) base[c * elems + e] = run;
-          else st16[((int64_t)bh * nchunks + c) * elems + e] = __float2bfloat16_rn(run);   // (what the tensor-core query side reads)
-        }
+        if (c0 + u < nchunks) base[c * elems + e] = run;
         run += v[u];
       }
     }

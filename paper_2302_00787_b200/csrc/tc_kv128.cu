@@ -1,13 +1,18 @@
-// Per-chunk key-side sums of the causal form, S_c^T [V_c | 1] (Section 2.1's O(L M n) order, chunk by chunk), on the
-// tensor cores for the shapes that have no fused kernel: bf16 copy of phi(K) [B*H][L][M], V [B,H,L,128] bf16.
-// Output st [B*H * L/C][129][M] fp32, column index first (feature index contiguous), so that a warp's stores coalesce
-// and the query-side product finds the feature index contiguous.
+// Key side of the causal chunked form, the running sums KV_c = sum over the chunks before c of S^T [V | 1] (Section 2.1's
+// O(L M n) order), on the tensor cores for the shapes that have no fused kernel: bf16 copy of phi(K) [B*H][L][M], V [B,H,L,128]
+// bf16.  Output, both bf16: st16 [B*H * L/C][M][128] and the normaliser's column z16 [B*H * L/C][M].
 //
-// One block = (range of chunks, block of 128 features, (batch, head)).  Tokens are the contraction: a stage holds
+// One block = (segment of consecutive chunks, block of 128 features, (batch, head)).  Tokens are the contraction: a stage holds
 // 128 tokens of the feature block (two 64-feature panels) and of V (two 64-column panels), all "MN-major" operands
 // (the contracted index is the row of the tile).  Per 16 tokens: D[:, 0..127] += phi^T V (N = 128) and
 // D[:, 128..143] += phi^T E with E the constant tile whose first column is 1 (N = 16).  Two accumulators in tensor
-// memory: the epilogue writes chunk c while chunk c + 1 is multiplied.
+// memory: the epilogue takes chunk c while chunk c + 1 is multiplied.  A chunk's sum is added in fp32 to the running one, which
+// the epilogue warps keep in registers and write, rounded to bf16, in front of every chunk: nothing else leaves the block.  (Sums
+// of single chunks written in fp32, 505 us for 1 x 16 x 65536 tokens, M = 512, chunks of 256, and scanned by a kernel of its own,
+// 265 us, moved 2.2 GB that never had to.)
+// Segments: as many as there are SMs for all (segment, block, (batch, head)); where there is more than one, a first launch
+// (EMIT = false) adds up the earlier ones, cut finer so that it fills the chip too, and the scan kernel turns the pieces' sums into
+// what precedes every piece.
 #include "common.cuh"
 #include "tc_common.cuh"
 #include "tc_layout.cuh"
@@ -17,8 +22,8 @@ using namespace tcl;
 
 namespace {
 
-constexpr int KV_ST = 2;
-constexpr int KVE_THREADS = 128, KVW_TMA = 4, KVW_MMA = 5, KVT = 192;
+constexpr int KV_ST = 3;
+constexpr int KVE_WARPS = 8, KVW_TMA = 8, KVW_MMA = 9, KVT = 320;
 constexpr uint32_t KV_ACC_COLS = 160;                  // 128 + 16, kept apart by a multiple of 32
 constexpr uint32_t KV_TMEM_COLS = 512;                 // two accumulators (power of two)
 constexpr uint32_t KV_STAGE = 4 * TILE_BYTES;          // feature panels 0, 1, then V panels 0, 1
@@ -34,26 +39,37 @@ struct KvMs {
 static_assert(sizeof(KvMs) <= 256, "misc block");
 static_assert(KvSm::TOTAL + 1024 <= 232448, "shared memory budget");
 
+// cps: chunks per segment; sub: pieces that the launch of the totals cuts a segment into, cpp chunks each (none is empty).
+struct KvCut {
+  int nch, cps, sub, cpp;
+  __host__ __device__ int segments() const { return (nch + cps - 1) / cps; }
+  __host__ __device__ int slots() const { return (segments() - 1) * sub + 1; }       // pieces, and one for what precedes the last segment
+};
+
+template <bool EMIT>
 __global__ void __launch_bounds__(KVT, 1)
-tc_kv128_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CUtensorMap tmV, float* __restrict__ st,
-                int H, int M, int C, int nch, int chunks_per_split, int* __restrict__ status) {
+tc_kv128_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CUtensorMap tmV, float* __restrict__ tot,
+                __nv_bfloat16* __restrict__ st16, __nv_bfloat16* __restrict__ z16, int H, int M, int C, KvCut cut,
+                int* __restrict__ status) {
   fs_grid_dependency_wait();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   KvMs* misc = reinterpret_cast<KvMs*>(sm + KvSm::MISC);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int fblk = blockIdx.y, bh = blockIdx.z, b = bh / H, h = bh % H;
-  const int c0 = blockIdx.x * chunks_per_split;
-  const int ncs = min(chunks_per_split, nch - c0);
+  const int seg = EMIT ? (int)blockIdx.x : (int)blockIdx.x / cut.sub, piece = EMIT ? 0 : (int)blockIdx.x % cut.sub;
+  const int c0 = seg * cut.cps + piece * cut.cpp;
+  const int ncs = min(EMIT ? cut.cps : min(cut.cpp, cut.cps - piece * cut.cpp), cut.nch - c0);
   if (ncs <= 0) return;                        // uniform over the block, before anything is allocated
+  const int sums = EMIT ? ncs - 1 : ncs;       // chunks that are multiplied (nothing follows a segment's last one)
   const int tpc = C / TILE;                    // token tiles per chunk
-  const int ntiles = ncs * tpc;
+  const int ntiles = sums * tpc;
   volatile int* abortp = &misc->abort_flag;
   constexpr int N = 129;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < KV_ST; i++) { mbar_init(&misc->full[i], 1); mbar_init(&misc->empty[i], 1); }
-    for (int i = 0; i < 2; i++) { mbar_init(&misc->acc_full[i], 1); mbar_init(&misc->acc_free[i], KVE_THREADS / 32); }
+    for (int i = 0; i < 2; i++) { mbar_init(&misc->acc_full[i], 1); mbar_init(&misc->acc_free[i], KVE_WARPS); }
     misc->abort_flag = 0;
     fence_barrier_init();
   }
@@ -122,31 +138,61 @@ tc_kv128_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
       __syncwarp();
     }
   } else {
-    // epilogue: thread = feature row of D; columns 0..127 the V part, column 128 the ones column
-    const int row = warp * 32 + lane;
-    const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
-    for (int ch = 0; ch < ncs; ch++) {
+    // epilogue: thread = feature row of D and 64 of its columns; the warps of the first half also take the ones column
+    const int half = warp >> 2, row = (warp & 3) * 32 + lane, f = fblk * 128 + row;
+    const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    float run[64], z = 0.f;
+#pragma unroll
+    for (int j = 0; j < 64; j++) run[j] = 0.f;
+    // totals [(batch, head)][piece][129][M]: the pieces' own sums, or (EMIT) those of the pieces before
+    float* t = tot + (((size_t)bh * cut.slots() + seg * cut.sub + piece) * N + half * 64) * M + f;
+    if (EMIT && seg > 0) {
+#pragma unroll
+      for (int j = 0; j < 64; j++) run[j] = t[(size_t)j * M];
+      if (half == 0) z = t[(size_t)128 * M];
+    }
+    auto emit = [&](int c) {
+      const size_t at = ((size_t)bh * cut.nch + c) * M + f;
+      uint32_t* out = reinterpret_cast<uint32_t*>(st16 + at * 128 + half * 64);
+#pragma unroll
+      for (int q = 0; q < 4; q++) {                    // 32 bytes each
+        uint32_t o[8];
+#pragma unroll
+        for (int j = 0; j < 8; j++) o[j] = pack_bf16(run[q * 16 + 2 * j], run[q * 16 + 2 * j + 1]);
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(out + q * 8), "r"(o[0]), "r"(o[1]), "r"(o[2]),
+                     "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7])
+                     : "memory");
+      }
+      if (half == 0) z16[at] = __float2bfloat16_rn(z);
+    };
+    if (EMIT) emit(c0);
+    for (int ch = 0; ch < sums; ch++) {
       const int buf = ch & 1;
       if (!mbar_wait(&misc->acc_full[buf], (ch >> 1) & 1, abortp, status, false)) break;
       __syncwarp();
       tcgen05_fence_after();
-      float* out = st + ((size_t)bh * nch + c0 + ch) * (size_t)N * M + (size_t)fblk * 128 + row;
 #pragma unroll
-      for (int cc = 0; cc < 8; cc++) {
+      for (int cc = 0; cc < 4; cc++) {
         uint32_t t[16];
-        tmem_ld16(lane_addr + buf * KV_ACC_COLS + cc * 16, t);
+        tmem_ld16(lane_addr + buf * KV_ACC_COLS + half * 64 + cc * 16, t);
         tmem_wait_ld();
 #pragma unroll
-        for (int j = 0; j < 16; j++) out[(size_t)(cc * 16 + j) * M] = __uint_as_float(t[j]);
+        for (int j = 0; j < 16; j++) run[cc * 16 + j] += __uint_as_float(t[j]);
       }
-      {
+      if (half == 0) {
         uint32_t t[8];
         tmem_ld8(lane_addr + buf * KV_ACC_COLS + 128, t);
         tmem_wait_ld();
-        out[(size_t)128 * M] = __uint_as_float(t[0]);
+        z += __uint_as_float(t[0]);
       }
       tcgen05_fence_before();
       mbar_arrive_warp(&misc->acc_free[buf], lane);
+      if (EMIT) emit(c0 + ch + 1);
+    }
+    if (!EMIT) {
+#pragma unroll
+      for (int j = 0; j < 64; j++) t[(size_t)j * M] = run[j];
+      if (half == 0) t[(size_t)128 * M] = z;
     }
   }
   tcgen05_fence_before();
@@ -155,6 +201,21 @@ tc_kv128_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
     tcgen05_fence_after();
     tmem_dealloc(tmem, KV_TMEM_COLS);
   }
+}
+
+KvCut cut_of(const fsharp_ctx* ctx, int BH, int M, int nch) {
+  const int units = BH * (M / 128);
+  int ns = ctx->sm_count / units;
+  ns = ns < 1 ? 1 : (ns > nch ? nch : ns);
+  KvCut cut;
+  cut.nch = nch;
+  cut.cps = (nch + ns - 1) / ns;
+  ns = cut.segments();
+  int k = ns > 1 ? ctx->sm_count / (units * (ns - 1)) : 1;
+  k = k < 1 ? 1 : (k > cut.cps ? cut.cps : k);
+  cut.cpp = (cut.cps + k - 1) / k;
+  cut.sub = (cut.cps + cut.cpp - 1) / cut.cpp;
+  return cut;
 }
 
 }  // namespace
@@ -170,21 +231,25 @@ int fs_tc_kv128_supported(const void* V, TensorAddr av, int dv, int M, int C) {
   return (av.sl * 2) % 16 == 0 && (av.sh * 2) % 16 == 0 && (av.sb * 2) % 16 == 0;
 }
 
-// phiK16 [BH][L][M] bf16, V [B,H,L,128] bf16 (strides av), st [BH * L / C][129][M] fp32 (feature index contiguous)
-int fs_tc_kv128(fsharp_ctx* ctx, const void* phiK16, const void* V, TensorAddr av, int B, int H, int L, int M, int C, float* st) {
-  const int BH = B * H, nch = L / C, nq = M / 128;
+// Totals per (batch, head) of [129][M] fp32; one: there is a single segment and no totals are needed.
+int fs_tc_kv128_slots(const fsharp_ctx* ctx, int BH, int M, int nch) { return cut_of(ctx, BH, M, nch).slots(); }
+
+// phiK16 [BH][L][M] bf16, V [B,H,L,128] bf16 (strides av).  st16 = null: the sums of the pieces of all segments but the last to
+// tot [BH][slots][129][M]; else st16 [BH * L / C][M][128] and z16 [BH * L / C][M], from tot as the exclusive scan over slots.
+int fs_tc_kv128(fsharp_ctx* ctx, const void* phiK16, const void* V, TensorAddr av, int B, int H, int L, int M, int C, float* tot,
+                void* st16, void* z16) {
+  const int BH = B * H, nch = L / C;
+  const KvCut cut = cut_of(ctx, BH, M, nch);
   CUtensorMap tmP, tmV;
   TensorAddr ap{(int64_t)BH * L * M, (int64_t)L * M, (int64_t)M};
   FS_TRY(tchost::make_map_tokens(&tmP, phiK16, ap, 1, BH, L, M));
   FS_TRY(tchost::make_map_tokens(&tmV, V, av, B, H, L, 128));
-  FS_CUDA_OK(cudaFuncSetAttribute(tc_kv128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KvSm::TOTAL + 1024));
-  // about two blocks per SM's worth of work in the grid, each walking a range of chunks
-  int ns = (2 * ctx->sm_count + BH * nq - 1) / (BH * nq);
-  ns = ns < 1 ? 1 : (ns > nch ? nch : ns);
-  const int cps = (nch + ns - 1) / ns;
-  ns = (nch + cps - 1) / cps;
+  const auto kernel = st16 ? tc_kv128_kernel<true> : tc_kv128_kernel<false>;
+  const size_t smem = KvSm::TOTAL + 1024;
+  FS_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   FS_TIME_BEGIN(ctx, FS_K_TC_KV128);
-  tc_kv128_kernel<<<dim3(ns, nq, BH), KVT, KvSm::TOTAL + 1024, ctx->stream>>>(tmP, tmV, st, H, M, C, nch, cps, ctx->d_status);
+  kernel<<<dim3(st16 ? cut.segments() : cut.slots() - 1, M / 128, BH), KVT, smem, ctx->stream>>>(
+      tmP, tmV, tot, (__nv_bfloat16*)st16, (__nv_bfloat16*)z16, H, M, C, cut, ctx->d_status);
   FS_TIME_END(ctx);
   FS_LAUNCH_CHECK(ctx);
   return FSHARP_OK;
