@@ -81,6 +81,8 @@ struct Args {
   Factor wscale;          // log2e qk_scale (1 + LOST_W)
   float pow2;             // power of two next to qk_scale: tokens times this do not overflow when squared
   double quad;            // log2e (qk_scale / pow2)^2
+  bool own_terms;         // the feature kernels compute the quadratic terms of groups with C = gamma I themselves
+  bool row_init;          // a pass raises logscale from -inf
   int* status;
 };
 
@@ -249,6 +251,25 @@ rowterm3_kernel(const __grid_constant__ Args a) {
   RtMisc* misc = reinterpret_cast<RtMisc*>(sC + G::NKS * 3 * D * 128);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr uint32_t COLS = D < 32 ? 32 : D;
+  PrepLayout pr{D, a.M};
+  const int total = a.first[2];
+  const int w0 = (int)((int64_t)total * blockIdx.x / gridDim.x), w1 = (int)((int64_t)total * (blockIdx.x + 1) / gridDim.x);
+  if (a.own_terms) {
+    // nothing but the start values where all groups of this block have C = gamma I
+    bool all = true;
+    for (int w = w0; w < w1;) {
+      const int ti = w >= a.first[1] ? 1 : 0, bh = (w - a.first[ti]) / a.tiles[ti], tile = (w - a.first[ti]) % a.tiles[ti];
+      const Task& t = a.t[ti];
+      all &= a.prep[((size_t)group_of(bh, a.H, a.pool) * 2 + (t.side - 1)) * pr.total() + pr.scal() + PS_CSCALAR] != 0.f;
+      if (tile == 0 && tid == 0 && t.gmax) t.gmax[bh] = 0u;
+      if (t.stab == FSHARP_STAB_ROW && a.row_init) {
+        const int i1 = min(t.L, (tile + min(a.tiles[ti] - tile, w1 - w)) * TILE);
+        for (int i = tile * TILE + tid; i < i1; i += RT_THREADS) t.logscale[(int64_t)bh * t.L + i] = __int_as_float(0xff800000);
+      }
+      w += a.tiles[ti] - tile;
+    }
+    if (all) return;
+  }
   if (tid == 0) {
     mbar_init(&misc->done, 1);
     misc->abort_flag = 0;
@@ -262,9 +283,6 @@ rowterm3_kernel(const __grid_constant__ Args a) {
   __syncthreads();
   tcgen05_fence_after();
   const uint32_t tmem = misc->tmem_base;
-  PrepLayout pr{D, a.M};
-  const int total = a.first[2];
-  const int w0 = (int)((int64_t)total * blockIdx.x / gridDim.x), w1 = (int)((int64_t)total * (blockIdx.x + 1) / gridDim.x);
   int have = -1, phase = 0;                       // (task, group) whose C is staged
   bool scalar = false, bad = false;
   Factor quad;
@@ -368,7 +386,7 @@ rowterm3_kernel(const __grid_constant__ Args a) {
       const float c = quad.times(misc->part[0][row] + misc->part[1][row]);
       bad |= !isfinite(c);                        // so is x then (or C): one test per token instead of one per exponent
       t.rowc[out0 + row] = c;
-      if (t.stab == FSHARP_STAB_ROW && a.nmb > 1) t.logscale[out0 + row] = __int_as_float(0xff800000);
+      if (t.stab == FSHARP_STAB_ROW && a.row_init) t.logscale[out0 + row] = __int_as_float(0xff800000);
     }
     if (tile == 0 && tid == 0 && t.gmax) t.gmax[bh] = 0u;
     // (the next tile's staging overwrites sA: its readers are behind the barrier above)
@@ -395,17 +413,19 @@ rowterm3_kernel(const __grid_constant__ Args a) {
 constexpr int FT_AHEAD = 4;                                        // tiles pulled into L2 ahead of the two buffers (BP = 2)
 constexpr int FT_STAGE0 = 8, FT_MMA = 12, FT_THREADS = 416;
 struct FtMisc {
-  uint64_t a_full[2], a_free[2], t_full[2], t_free[2], w_full;
+  uint64_t a_full[2], a_free[2], t_full[2], t_free[2], max_full[2], w_full;
   uint32_t tmem_base;
   int abort_flag;
 };
+struct FtMax { float row[2][2][TILE]; };       // PAIR: the other block's maxima, two places per warpgroup
 template <typename T, int D, int BP> struct FtGeo : Geo<T, D> {
   static_assert(BP == 3 || Geo<T, D>::AP == 1, "two parts of W: bf16 tokens");
   static constexpr int MB = WGeo<D, BP>::MB;
   static constexpr int NBUF = (D == 128 && sizeof(T) == 4) ? 1 : 2;    // token tiles in shared memory
   static constexpr uint32_t W_BYTES = Geo<T, D>::NKS * BP * MB * 128;
   static constexpr uint32_t OFF_A = W_BYTES, OFF_ONE = OFF_A + NBUF * Geo<T, D>::A_BYTES, OFF_ROW = OFF_ONE + TILE * 32, OFF_MISC = OFF_ROW + MB * 32;
-  static constexpr size_t SMEM = 1024 + OFF_MISC + sizeof(FtMisc);
+  static constexpr uint32_t OFF_MAX = OFF_MISC + sizeof(FtMisc);
+  static constexpr size_t SMEM = 1024 + OFF_MAX + (BP == 2 ? sizeof(FtMax) : 0);
   static_assert(SMEM <= 232448, "shared memory budget");
 };
 
@@ -413,12 +433,18 @@ template <typename T, int D, int BP> struct FtGeo : Geo<T, D> {
 // counts most, is a power of two and loses nothing to bf16 (with a maximum from the leading part of W, half the products, the
 // outputs' error rose from 2.83e-3 to 2.88e-3; 1 x 16 x 65536 tokens, M = 512: the step 3435 us, 3515 us now).  The shift of a group may be any value near
 // its maximum (it cancels in the normalisation, and bf16 has the range of fp32): that pass takes the leading part of W alone.
-template <typename T, int D, bool WRITE, int BP>
+// PAIR: row shifts where M takes two blocks of features: two blocks of a cluster walk the same tiles, one half of the features each, and
+// tell each other their rows' maxima through shared memory.  (A pass of its own for the maxima, 200 us for 1 x 16 x 65536 tokens and
+// M = 512, made all the products of the pass that writes.)
+// BP = 2, C = gamma I: the first pass over the tokens takes x^T C x from the tile in shared memory, in the order of
+// rowterm3_kernel (which read all tokens once more for it: 85 us for the same tokens).
+template <typename T, int D, bool WRITE, int BP, bool PAIR = false>
 __global__ void __launch_bounds__(FT_THREADS, 1)
 feat3_kernel(const __grid_constant__ Args a) {
   fs_grid_dependency_wait();
   using G = FtGeo<T, D, BP>;
   constexpr bool OUT16 = BP == 2;
+  static_assert(!PAIR || (WRITE && OUT16), "pairs write bf16 features");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sW = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* sA = sW + G::OFF_A;
@@ -426,10 +452,14 @@ feat3_kernel(const __grid_constant__ Args a) {
   uint8_t* sRow = sW + G::OFF_ROW;
   FtMisc* misc = reinterpret_cast<FtMisc*>(sW + G::OFF_MISC);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = PAIR ? (int)cluster_rank() : 0;
+  // the first pass over the tokens: its epilogue warps read them too
+  const bool terms = OUT16 && (!WRITE || PAIR || (a.t[0].stab == FSHARP_STAB_ROW && a.nmb == 1));
   if (tid == 0) {
     for (int i = 0; i < 2; i++) {
       mbar_init(&misc->a_full[i], OUT16 ? 1 : 4);
-      mbar_init(&misc->a_free[i], 1);
+      mbar_init(&misc->a_free[i], terms ? 5 : 1);
+      if (PAIR) mbar_init(&misc->max_full[i], 4);
       mbar_init(&misc->t_full[i], 1);
       mbar_init(&misc->t_free[i], 4);
     }
@@ -448,12 +478,14 @@ feat3_kernel(const __grid_constant__ Args a) {
   }
   tcgen05_fence_before();
   __syncthreads();
+  if (PAIR) cluster_sync();                                        // the other block's barriers are initialised
   tcgen05_fence_after();
   const uint32_t tmem = misc->tmem_base;
+  FtMax* maxima = reinterpret_cast<FtMax*>(sW + G::OFF_MAX);
   PrepLayout pr{D, a.M};
-  const int total = a.first[2];
-  const int w1 = (int)((int64_t)total * (blockIdx.x + 1) / gridDim.x);
-  int w = (int)((int64_t)total * blockIdx.x / gridDim.x);
+  const int total = a.first[2], me = PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x, blocks = PAIR ? (int)gridDim.x >> 1 : (int)gridDim.x;
+  const int w1 = (int)((int64_t)total * (me + 1) / blocks);
+  int w = (int)((int64_t)total * me / blocks);
   int n = 0, runs = 0;                                             // tiles and runs done by this block (every role counts alike)
   bool bad = false;
   while (w < w1) {
@@ -461,7 +493,7 @@ feat3_kernel(const __grid_constant__ Args a) {
     const int ti = w >= a.first[1] ? 1 : 0;
     const Task& t = a.t[ti];
     const int u = (w - a.first[ti]) / a.tiles[ti], tile0 = (w - a.first[ti]) % a.tiles[ti];
-    const int bh = u / a.nmb, mblk = u % a.nmb, m0 = mblk * G::MB, mb = min(G::MB, a.M - m0);
+    const int bh = PAIR ? u : u / a.nmb, mblk = PAIR ? rank : u % a.nmb, m0 = mblk * G::MB, mb = min(G::MB, a.M - m0);
     const int ntiles = min(a.tiles[ti] - tile0, w1 - w);
     w += ntiles;
     const int g = group_of(bh, a.H, a.pool);
@@ -541,7 +573,9 @@ feat3_kernel(const __grid_constant__ Args a) {
       const int wg = warp >> 2;
       float gmx = -3.0e38f;
       const float gshift = (WRITE && t.stab == FSHARP_STAB_GROUP) ? ord2f(t.gmax[bh]) : 0.f;
-      const bool own = t.stab == FSHARP_STAB_ROW && a.nmb == 1;
+      const bool own = PAIR || (t.stab == FSHARP_STAB_ROW && a.nmb == 1);
+      const bool scalar = terms && pp[pr.scal() + PS_CSCALAR] != 0.f;
+      const Factor quad(scalar ? a.quad * (double)pp[pr.scal() + PS_CGAMMA] : 0.0);
       const bool wide = WRITE && !OUT16 && (reinterpret_cast<uintptr_t>(t.phi) & 31) == 0;
       // x ln 2, x + y being rounded to x: one rounding in all
       const auto to_nat = [](float x, float y) { return fmaf(0.693147182f, x, fmaf(0.693147182f, y, -1.90465421e-9f * x)); };
@@ -552,7 +586,40 @@ feat3_kernel(const __grid_constant__ Args a) {
         const int tok0 = (tile0 + it) * TILE + (warp & 3) * 32, tok = tok0 + lane;
         const int64_t at = (int64_t)bh * t.L + tok;
         const bool in = tok < t.L;
-        const float ci = (in ? t.rowc[at] : 0.f) + bias;
+        float ci = bias;
+        if (OUT16 && terms) {
+          const int ab = n % G::NBUF, row = (warp & 3) * 32 + lane;
+          if (scalar) {
+            mbar_wait(&misc->a_full[ab], (n / G::NBUF) & 1, &misc->abort_flag, a.status);
+            float half[2] = {};
+#pragma unroll
+            for (int s = 0; s < G::NKS; s++) {
+              float sum[4] = {};
+              const uint8_t* src = sA + ab * G::A_BYTES + s * TILE_BYTES + row * 128;
+#pragma unroll
+              for (int cc = 0; cc < G::CH; cc++) {
+                const uint4 q = *reinterpret_cast<const uint4*>(src + ((cc ^ (row & 7)) << 4));
+                const uint32_t v[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                  const float lo = a.pow2 * __uint_as_float(v[j] << 16), hi = a.pow2 * __uint_as_float(v[j] & 0xffff0000u);
+                  sum[(2 * j) & 3] = fmaf(lo, lo, sum[(2 * j) & 3]);
+                  sum[(2 * j + 1) & 3] = fmaf(hi, hi, sum[(2 * j + 1) & 3]);
+                }
+              }
+              half[s & 1] = (sum[0] + sum[1]) + (sum[2] + sum[3]);
+            }
+            const float c = quad.times(half[0] + half[1]);
+            bad |= in && !isfinite(c);
+            ci += c;
+            if (!WRITE && in && mblk == 0) t.rowc[at] = c;
+          } else {
+            ci += in ? t.rowc[at] : 0.f;
+          }
+          mbar_arrive_warp(&misc->a_free[ab], lane);
+        } else {
+          ci += in ? t.rowc[at] : 0.f;
+        }
         // exponent = acc + add, minus `shift` where that does not come from this block's own maximum: in this order the largest
         // exponent of the group or row, rounded as it was when the maximum was taken, gives 1 and nothing gives more
         float add = ci, shift = gshift - t.lift;
@@ -596,6 +663,17 @@ feat3_kernel(const __grid_constant__ Args a) {
             }
           }
           mx = fmaxf(mx, my);
+          if (PAIR) {
+            // (the other block is at most one of this warpgroup's tiles ahead: its next maxima need this one's)
+            const int k = n >> 1, row = (warp & 3) * 32 + lane;
+            float* place = &maxima->row[wg][k & 1][row];
+            store_cluster(map_cluster(smem_u32(place), rank ^ 1), mx);
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(map_cluster(smem_u32(&misc->max_full[wg]), rank ^ 1));
+            mbar_wait_cluster(&misc->max_full[wg], k & 1, &misc->abort_flag, a.status);
+            __syncwarp();
+            mx = fmaxf(mx, *reinterpret_cast<volatile float*>(place));
+          }
           if (WRITE) {
             add = t.lift - mx;
             const float top = mx + ci, big = fabsf(mx) > fabsf(ci) ? mx : ci, small = fabsf(mx) > fabsf(ci) ? ci : mx;
@@ -663,6 +741,7 @@ feat3_kernel(const __grid_constant__ Args a) {
       mbar_wait(&misc->a_full[k % G::NBUF], (k / G::NBUF) & 1, &misc->abort_flag, a.status, false);
   tcgen05_fence_before();
   __syncthreads();
+  if (PAIR) cluster_sync();                                        // (the other block writes here until its last tile)
   if (warp == FT_MMA) {
     tcgen05_fence_after();
     tmem_dealloc(tmem, 512);
@@ -678,8 +757,11 @@ int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, in
   if (BP == 2)
     for (int i = 0; i < ntasks; i++) FS_TRY(tchost::make_map_tokens(&maps[i], tasks[i].X, tasks[i].ax, BH / a.H, a.H, tasks[i].L, D));
   const uint8_t* side_img[2] = {nullptr, nullptr};     // by side - 1
+  const bool pair = BP == 2 && ntasks == 1 && tasks[0].stab == FSHARP_STAB_ROW && a.nmb == 2;
+  a.own_terms = BP == 2;
+  a.row_init = a.nmb > 1 && !pair;
   // (a set with a row shift over several feature blocks has its maxima pass instead: its blocks convert W themselves)
-  if (img != nullptr && !(ntasks == 1 && tasks[0].stab == FSHARP_STAB_ROW && a.nmb > 1)) {
+  if (img != nullptr && !(ntasks == 1 && tasks[0].stab == FSHARP_STAB_ROW && a.nmb > 1 && !pair)) {
     const int side0 = ntasks == 2 ? 1 : tasks[0].side;
     const size_t per_side = (size_t)G_groups * G::NKS * BP * a.M * 128;
     for (int k = 0; k < ntasks; k++) side_img[side0 - 1 + k] = img + k * per_side;
@@ -713,6 +795,18 @@ int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, in
     (void)fs_launch_chained(rowterm3_kernel<T, D>, dim3(total < most ? total : most), dim3(RT_THREADS), smem, ctx->stream, a);
     FS_TIME_END(ctx);
     FS_LAUNCH_CHECK(ctx);
+  }
+  if constexpr (BP == 2) {
+    if (pair) {
+      const auto kernel = feat3_kernel<T, D, true, BP, true>;
+      const int total = set(1, [](const Task&, int) { return true; }), most = ctx->sm_count / 2;
+      FS_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM));
+      FS_TIME_BEGIN(ctx, FS_K_FEAT);
+      (void)fs_launch_chained_cluster(kernel, dim3(2 * (total < most ? total : most)), dim3(FT_THREADS), 2, G::SMEM, ctx->stream, a);
+      FS_TIME_END(ctx);
+      FS_LAUNCH_CHECK(ctx);
+      return FSHARP_OK;
+    }
   }
   const int maxed = set(a.nmb, [](const Task& t, int nmb) { return t.stab == FSHARP_STAB_GROUP || (t.stab == FSHARP_STAB_ROW && nmb > 1); });
   if (maxed > 0) {

@@ -1,0 +1,40 @@
+"""The chain of kernels for bf16, d = dv = 128, causal (feature maps, running key-side sums, query side) where its work is cut
+differently: one tile, one chunk, one segment for want of SMs, as many segments as chunks, segments whose totals are added up in
+pieces, one, two (whole and half) and three blocks of features; against the fp32-precision kernels."""
+import numpy as np
+import pytest
+import torch
+
+from tests.gpu_util import TOL, dev, gpu_fit, host, rel_err
+from paper_2302_00787_b200 import binding as fb
+from paper_2302_00787_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,H,L,M,chunk,variant", [
+    (1, 1, 128, 128, 128, "sderf"),       # one tile
+    (1, 1, 256, 256, 256, "aderf"),       # one chunk of two tiles: nothing precedes it; a dense C
+    (2, 19, 384, 512, 128, "saderf"),     # 152 (batch, head, feature block)s: one segment each
+    (1, 3, 5120, 128, 256, "sderf"),      # a segment per chunk
+    (1, 16, 1024, 512, 128, "sderf"),     # two segments of four chunks, the first added up in two pieces
+    (1, 5, 2816, 384, 256, "aderf"),      # a last segment of one chunk; the second block of features half full
+    (1, 2, 512, 640, 256, "sderf"),       # three blocks of features: row maxima by a pass of their own
+])
+def test_chain_against_fp32_kernels(B, H, L, M, chunk, variant):
+    ctx = fb.Context(0)
+    w = wl.Workload("chain", B, H, L, 128, 128, M, "bf16", variant, True, chunk, "orthogonal", outlier_frac=0.05, seed=9)
+    Q, K, V = (dev(t, "bf16") for t in wl.make_qkv(w))
+    Om = dev(wl.make_omega(w))
+    _, pr = gpu_fit(ctx, Q, K, 128, "saderf" if L < 512 else variant)
+    at = dict(causal=True, chunk=chunk)
+    Y = host(ctx.fsharp_attend(Q, K, V, Om, pr, **at))
+    assert torch.equal(ctx.fsharp_attend(Q, K, V, Om, pr, **at).float().cpu().double(), torch.from_numpy(Y))
+    ctx.set_impl(fb.IMPL_SIMT)
+    ref = host(ctx.fsharp_attend(Q, K, V, Om, pr, **at))
+    assert ctx.status() == 0
+    for b in range(B):
+        for h in range(H):
+            assert rel_err(Y[b, h], ref[b, h]) < TOL["bf16"]
+    # the first token sees itself alone
+    assert np.abs(Y[:, :, 0] - host(V)[:, :, 0]).max() < 1e-2 * np.abs(host(V)[:, :, 0]).max()
