@@ -8,17 +8,54 @@
 
 namespace {
 
+// A thread has R x R products of one token after the other (rows and columns in pieces of four, one 16-byte load each);
+// the (D / R)^2 threads that cover the matrix form a group, and the groups of a block share out the tokens of a tile.  The next tile's loads
+// are in flight under this one's products.  (A matrix over the whole block at every d, 2 x 2 products at d = 32 for four
+// loads, a tile of 32 tokens at a time and its loads waited for: 24 us for 2 x 32 x 1501 tokens.)
 constexpr int ST_THREADS = 256;
-constexpr int ST_TT = 32;        // tokens per shared-memory tile
-constexpr int ST_FLUSH = 4;      // tiles between fp32 -> fp64 folds
+template <int D> struct StGeo {
+  static constexpr int R = D == 128 ? 8 : 4, TPG = (D / R) * (D / R), NG = ST_THREADS / TPG, TT = 4096 / D;      // tokens per tile
+  static constexpr int FLUSH = 128 / (TT / NG);      // tiles between fp32 -> fp64 folds: 128 tokens of a thread
+  static constexpr int LD = D + 4;
+};
+
+// the tile's values that this thread brings: 16-byte pieces
+template <typename T, int D> struct StTile {
+  static constexpr int E = 16 / sizeof(T), N = 4096 / E / ST_THREADS;
+  uint4 r[N];
+  __device__ __forceinline__ void load(const T* X, int64_t sl, int rows, int tid) {
+#pragma unroll
+    for (int u = 0; u < N; u++) {
+      const int e = (tid + u * ST_THREADS) * E, t = e / D, c = e % D;
+      r[u] = t < rows ? *reinterpret_cast<const uint4*>(X + (int64_t)t * sl + c) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  }
+  __device__ __forceinline__ void store(float* xs, float scale, int tid, bool& bad) const {
+#pragma unroll
+    for (int u = 0; u < N; u++) {
+      const int e = (tid + u * ST_THREADS) * E, t = e / D, c = e % D;
+      const uint32_t w[4] = {r[u].x, r[u].y, r[u].z, r[u].w};
+      float v[E];
+#pragma unroll
+      for (int j = 0; j < E; j++) {
+        v[j] = scale * (sizeof(T) == 4 ? __uint_as_float(w[j]) : __uint_as_float(j & 1 ? w[j / 2] & 0xffff0000u : w[j / 2] << 16));
+        bad |= !isfinite(v[j]);
+      }
+#pragma unroll
+      for (int j = 0; j < E; j += 4) *reinterpret_cast<float4*>(xs + t * StGeo<D>::LD + c + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+    }
+  }
+};
 
 template <typename T, int D>
 __global__ void __launch_bounds__(ST_THREADS)
 stats_kernel(const T* __restrict__ Q, const T* __restrict__ K, TensorAddr aq, TensorAddr ak, int H, int Lq, int Lk,
              int pool, int Bpool, float qk_scale, int tokens_per_split, double* __restrict__ stats,
              int* __restrict__ status) {
-  constexpr int RB = D / 16;
-  __shared__ float xs[ST_TT][D + 1];
+  using G = StGeo<D>;
+  constexpr int R = G::R, NG = G::NG, TT = G::TT, LD = G::LD, SUB = ST_THREADS / D;
+  __shared__ __align__(16) float xs[TT * LD];
+  __shared__ double sums[NG > 1 ? D * D : 1], cols[ST_THREADS];
   const int side = blockIdx.z;           // 0: queries, 1: keys
   const int bh = blockIdx.y;
   const int b = bh / H, h = bh % H;
@@ -29,50 +66,50 @@ stats_kernel(const T* __restrict__ Q, const T* __restrict__ K, TensorAddr aq, Te
   const int t1 = min(L, t0 + tokens_per_split);
   if (t0 >= t1) return;
   const int g = pool == FSHARP_POOL_PER_BH ? bh : h;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int tid = threadIdx.x, grp = tid / G::TPG, tx = tid % G::TPG % (D / R), ty = tid % G::TPG / (D / R);
+  // row / column of the thread's products: pieces of four, D / 2 apart where there are two
+  const auto at = [](int i, int x) { return (i & 3) + 4 * x + (i >> 2) * (D / 2); };
 
-  float acc[RB][RB];
-  double accd[RB][RB];
+  float acc[R][R];
+  double accd[R][R];
 #pragma unroll
-  for (int i = 0; i < RB; i++)
+  for (int i = 0; i < R; i++)
 #pragma unroll
-    for (int j = 0; j < RB; j++) { acc[i][j] = 0.f; accd[i][j] = 0.0; }
-  float colacc = 0.f;
+    for (int j = 0; j < R; j++) { acc[i][j] = 0.f; accd[i][j] = 0.0; }
+  float colacc = 0.f;                    // column tid % D over every SUB-th token
   double colaccd = 0.0;
   bool bad = false;
   int since = 0;
-
-  for (int tb = t0; tb < t1; tb += ST_TT) {
-    for (int e = tid; e < ST_TT * D; e += ST_THREADS) {
-      int t = e / D, c = e % D;
-      float v = 0.f;
-      if (tb + t < t1) v = qk_scale * fs_load(X + (int64_t)(tb + t) * ad.sl + c);
-      if (!isfinite(v)) bad = true;
-      xs[t][c] = v;
-    }
+  StTile<T, D> tile;
+  tile.load(X + (int64_t)t0 * ad.sl, ad.sl, t1 - t0, tid);
+  for (int tb = t0; tb < t1; tb += TT) {
+    tile.store(xs, qk_scale, tid, bad);
     __syncthreads();
+    if (tb + TT < t1) tile.load(X + (int64_t)(tb + TT) * ad.sl, ad.sl, t1 - tb - TT, tid);
+    const int n = min(TT, t1 - tb);      // (rows up to the tile's end are zeros)
 #pragma unroll 4
-    for (int t = 0; t < ST_TT; t++) {
-      float a[RB], bb[RB];
+    for (int t = grp; t < n; t += NG) {
+      float a[R], bb[R];
 #pragma unroll
-      for (int i = 0; i < RB; i++) { a[i] = xs[t][ty + 16 * i]; bb[i] = xs[t][tx + 16 * i]; }
+      for (int i = 0; i < R; i += 4) {
+        const float4 u = *reinterpret_cast<const float4*>(xs + t * LD + at(i, ty)), v = *reinterpret_cast<const float4*>(xs + t * LD + at(i, tx));
+        a[i] = u.x; a[i + 1] = u.y; a[i + 2] = u.z; a[i + 3] = u.w;
+        bb[i] = v.x; bb[i + 1] = v.y; bb[i + 2] = v.z; bb[i + 3] = v.w;
+      }
 #pragma unroll
-      for (int i = 0; i < RB; i++)
+      for (int i = 0; i < R; i++)
 #pragma unroll
-        for (int j = 0; j < RB; j++) acc[i][j] = fmaf(a[i], bb[j], acc[i][j]);
+        for (int j = 0; j < R; j++) acc[i][j] = fmaf(a[i], bb[j], acc[i][j]);
     }
-    if (tid < D) {
-      float s = 0.f;
-      for (int t = 0; t < ST_TT; t++) s += xs[t][tid];
-      colacc += s;
-    }
+#pragma unroll 4
+    for (int t = tid / D; t < n; t += SUB) colacc += xs[t * LD + tid % D];
     __syncthreads();
-    if (++since == ST_FLUSH) {
+    if (++since == G::FLUSH) {
       since = 0;
 #pragma unroll
-      for (int i = 0; i < RB; i++)
+      for (int i = 0; i < R; i++)
 #pragma unroll
-        for (int j = 0; j < RB; j++) { accd[i][j] += (double)acc[i][j]; acc[i][j] = 0.f; }
+        for (int j = 0; j < R; j++) { accd[i][j] += (double)acc[i][j]; acc[i][j] = 0.f; }
       colaccd += (double)colacc;
       colacc = 0.f;
     }
@@ -81,12 +118,33 @@ stats_kernel(const T* __restrict__ Q, const T* __restrict__ K, TensorAddr aq, Te
   StatsLayout sl{D};
   double* out = stats + (size_t)g * sl.total();
   double* Mo = out + sl.M(side + 1);
+  cols[tid] = colaccd + (double)colacc;
+  if (NG > 1) {
+    for (int k = 0; k < NG; k++) {
+      if (grp == k)
 #pragma unroll
-  for (int i = 0; i < RB; i++)
+        for (int i = 0; i < R; i++)
 #pragma unroll
-    for (int j = 0; j < RB; j++)
-      atomicAdd(&Mo[(size_t)(ty + 16 * i) * D + (tx + 16 * j)], (accd[i][j] + (double)acc[i][j]) * inv);
-  if (tid < D) atomicAdd(&out[sl.mu(side + 4) + tid], (colaccd + (double)colacc) * inv);
+          for (int j = 0; j < R; j++) {
+            double* s = &sums[at(i, ty) * D + at(j, tx)];
+            *s = (k ? *s : 0.0) + (accd[i][j] + (double)acc[i][j]);
+          }
+      __syncthreads();
+    }
+    for (int e = tid; e < D * D; e += ST_THREADS) atomicAdd(&Mo[e], sums[e] * inv);
+  } else {
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < R; i++)
+#pragma unroll
+      for (int j = 0; j < R; j++) atomicAdd(&Mo[(size_t)at(i, ty) * D + at(j, tx)], (accd[i][j] + (double)acc[i][j]) * inv);
+  }
+  if (tid < D) {
+    double c = 0.0;
+#pragma unroll
+    for (int k = 0; k < SUB; k++) c += cols[k * D + tid];
+    atomicAdd(&out[sl.mu(side + 4) + tid], c * inv);
+  }
   if (bad) atomicExch(status, FSHARP_E_NONFINITE);
 }
 
@@ -100,7 +158,7 @@ int launch_stats(fsharp_ctx* ctx, const void* Q, const void* K, const fsharp_dim
   if (nsplit > maxsplit) nsplit = maxsplit;
   if (nsplit < 1) nsplit = 1;
   int tps = (Lmax + nsplit - 1) / nsplit;
-  tps = (tps + ST_TT - 1) / ST_TT * ST_TT;
+  tps = (tps + 31) / 32 * 32;
   nsplit = (Lmax + tps - 1) / tps;
   dim3 grid(nsplit, BH, 2);
   TensorAddr aq = fs_addr(dm->q_stride, dm->H, dm->Lq, dm->d);
