@@ -18,6 +18,7 @@ using feat3::Task;
 
 namespace tchost {
 int make_map_tokens(CUtensorMap* map, const void* base, TensorAddr a, int B, int H, int L, int inner);
+int make_map_features(CUtensorMap* map, void* base, int BH, int L, int M, int bf16, int box_bytes);
 }
 
 namespace {
@@ -47,13 +48,6 @@ __device__ __forceinline__ float ex2_full(float x) {
   return y;
 }
 
-// 32 bytes (eight words) as one store; p is 32-byte aligned
-__device__ __forceinline__ void store32(float* p, const uint32_t* x) {
-  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(x[4]),
-               "r"(x[5]), "r"(x[6]), "r"(x[7])
-               : "memory");
-}
-
 // A factor as a float and its remainder: fmaf(hi, x, lo * x) is the product with the unrounded factor, rounded once.  (The same
 // factor multiplies every exponent: rounded to fp32 it moves exponents of 60 nats by 2e-6, all of them in one direction.)
 struct Factor {
@@ -72,6 +66,8 @@ template <int D> constexpr double LOST_A = 0.17 * (D / 16) / 8388608.0;
 
 struct Args {
   CUtensorMap map[2];     // per task: the tokens (BP = 2)
+  CUtensorMap out[2];     // per task: the features, where staged[i]
+  bool staged[2];
   Task t[2];
   int first[3];           // running number of work items: task i owns [first[i], first[i + 1])
   int tiles[2];           // token tiles per (batch, head)
@@ -406,10 +402,12 @@ rowterm3_kernel(const __grid_constant__ Args a) {
 // feature is one ex2 of one addition: the per-feature term a_m rides on the products as one more K step (its three parts
 // against ones).  Warps 8-11 stage token tiles, warp 12 issues the products, the two warpgroups of warps 0-7 take one
 // accumulator each and work on alternate tiles: thread = token, all columns of a row in one thread, so the row's maximum
-// needs no exchange.  A thread stores its row in whole 32-byte sectors.  Bound of the writing pass: HBM (128 KB per tile of
-// 128 x 256: 5.8 k cycles of this SM's share, against 3.4 k cycles of products).  Tried: a_m from shared memory (a broadcast
-// 16-byte load costs four wavefronts) with a transposing buffer in front of the stores (16 k cycles per tile); TMA store
-// tiles staged in shared memory (11 k; each of them waits for its proxy fence).
+// needs no exchange.  A warp's rows go through shared memory and leave as copies of whole lines (32 rows of 128 bytes; 64 where d = 128
+// leaves little room).  Bound of the writing pass: HBM (128 KB per tile of 128 x 256: 6.5 k cycles of this SM's share of the rate of writes)
+// against 3.4 k cycles of products;
+// 2 x 8 x 10007 fp32 tokens, d = 64, M = 256, both sides: 217.6 us with each lane storing its own row in 32-byte pieces (a store instruction
+// then touches 32 lines: 3.5 TB/s at best, whole lines 5.7), 212 us now.  Measured inside: 12 k cycles per tile, the two warpgroups' stores
+// taking turns at some 15 bytes per cycle, and 3.5 k of each 23 k waiting for the next tile's products.
 constexpr int FT_AHEAD = 4;                                        // tiles pulled into L2 ahead of the two buffers (BP = 2)
 constexpr int FT_STAGE0 = 8, FT_MMA = 12, FT_THREADS = 416;
 struct FtMisc {
@@ -418,12 +416,18 @@ struct FtMisc {
   int abort_flag;
 };
 struct FtMax { float row[2][2][TILE]; };       // PAIR: the other block's maxima, two places per warpgroup
-template <typename T, int D, int BP> struct FtGeo : Geo<T, D> {
+template <typename T, int D, int BP, bool WRITE> struct FtGeo : Geo<T, D> {
   static_assert(BP == 3 || Geo<T, D>::AP == 1, "two parts of W: bf16 tokens");
   static constexpr int MB = WGeo<D, BP>::MB;
-  static constexpr int NBUF = (D == 128 && sizeof(T) == 4) ? 1 : 2;    // token tiles in shared memory
+  static constexpr bool SMALL = D == 128;                              // little room beside W and the tokens
+  // token tiles in shared memory (one where fp32 tokens leave room for no second one beside the staged features: their conversion and
+  // the products, 1.5 k + 3.2 k cycles, stay below what the stores of a tile take)
+  static constexpr int NBUF = sizeof(T) == 4 && (D == 128 || WRITE) ? 1 : 2;
+  static constexpr uint32_t STAGE = SMALL ? 2048 : 4096;               // per warp: 32 rows of features, STAGE / 32 bytes each
+  static constexpr int NSTAGE = SMALL ? 1 : 2;
   static constexpr uint32_t W_BYTES = Geo<T, D>::NKS * BP * MB * 128;
-  static constexpr uint32_t OFF_A = W_BYTES, OFF_ONE = OFF_A + NBUF * Geo<T, D>::A_BYTES, OFF_ROW = OFF_ONE + TILE * 32, OFF_MISC = OFF_ROW + MB * 32;
+  static constexpr uint32_t OFF_A = W_BYTES, OFF_OUT = OFF_A + NBUF * Geo<T, D>::A_BYTES, OFF_ONE = OFF_OUT + (WRITE ? 8 * NSTAGE * STAGE : 0),
+                            OFF_ROW = OFF_ONE + TILE * 32, OFF_MISC = OFF_ROW + MB * 32;
   static constexpr uint32_t OFF_MAX = OFF_MISC + sizeof(FtMisc);
   static constexpr size_t SMEM = 1024 + OFF_MAX + (BP == 2 ? sizeof(FtMax) : 0);
   static_assert(SMEM <= 232448, "shared memory budget");
@@ -442,7 +446,7 @@ template <typename T, int D, bool WRITE, int BP, bool PAIR = false>
 __global__ void __launch_bounds__(FT_THREADS, 1)
 feat3_kernel(const __grid_constant__ Args a) {
   fs_grid_dependency_wait();
-  using G = FtGeo<T, D, BP>;
+  using G = FtGeo<T, D, BP, WRITE>;
   constexpr bool OUT16 = BP == 2;
   static_assert(!PAIR || (WRITE && OUT16), "pairs write bf16 features");
   extern __shared__ uint8_t smem_raw[];
@@ -486,6 +490,7 @@ feat3_kernel(const __grid_constant__ Args a) {
   const int total = a.first[2], me = PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x, blocks = PAIR ? (int)gridDim.x >> 1 : (int)gridDim.x;
   const int w1 = (int)((int64_t)total * (me + 1) / blocks);
   int w = (int)((int64_t)total * me / blocks);
+  int copies = 0;
   int n = 0, runs = 0;                                             // tiles and runs done by this block (every role counts alike)
   bool bad = false;
   while (w < w1) {
@@ -576,7 +581,29 @@ feat3_kernel(const __grid_constant__ Args a) {
       const bool own = PAIR || (t.stab == FSHARP_STAB_ROW && a.nmb == 1);
       const bool scalar = terms && pp[pr.scal() + PS_CSCALAR] != 0.f;
       const Factor quad(scalar ? a.quad * (double)pp[pr.scal() + PS_CGAMMA] : 0.0);
-      const bool wide = WRITE && !OUT16 && (reinterpret_cast<uintptr_t>(t.phi) & 31) == 0;
+      // 32 rows of ROW_BYTES of features from the lanes' registers to the warp's place in shared memory, and out by a copy that
+      // drops rows and columns past the end
+      constexpr int ROW_BYTES = G::STAGE / 32;
+      uint8_t* place = sW + G::OFF_OUT + warp * (G::NSTAGE * G::STAGE);
+      const auto put_rows = [&](const uint32_t* x, int column, int row0) {
+        if (lane == 0) {
+          if (G::NSTAGE == 2) bulk_wait_read1(); else bulk_wait_read0();
+        }
+        __syncwarp();
+        uint8_t* dst = place + (G::NSTAGE == 2 ? (copies & 1) * G::STAGE : 0);
+        copies++;
+#pragma unroll
+        for (int j = 0; j < ROW_BYTES / 16; j++) {
+          const int piece = ROW_BYTES == 128 ? j ^ (lane & 7) : j ^ ((lane >> 1) & 3);
+          *reinterpret_cast<uint4*>(dst + lane * ROW_BYTES + piece * 16) = make_uint4(x[4 * j], x[4 * j + 1], x[4 * j + 2], x[4 * j + 3]);
+        }
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+          if (row0 < t.L) tma_store_3d(&a.out[ti], dst, column, row0, bh);
+          bulk_commit();
+        }
+      };
       // x ln 2, x + y being rounded to x: one rounding in all
       const auto to_nat = [](float x, float y) { return fmaf(0.693147182f, x, fmaf(0.693147182f, y, -1.90465421e-9f * x)); };
       if (WRITE && t.stab == FSHARP_STAB_GROUP && t.logscale && tile0 == 0 && mblk == 0 && tid == 0) t.logscale[bh] = to_nat(gshift, 0.f);
@@ -687,8 +714,6 @@ feat3_kernel(const __grid_constant__ Args a) {
           }
         }
         if (WRITE) {
-          float* out = OUT16 ? nullptr : t.phi + at * a.M + m0;
-          __nv_bfloat16* out16 = OUT16 ? t.phi16 + at * a.M + m0 : nullptr;
           for (int c = 0; c < mb; c += 32) {
             uint32_t x[32];
             arrived(x);
@@ -701,23 +726,20 @@ feat3_kernel(const __grid_constant__ Args a) {
             }
 #pragma unroll
             for (int j = 0; j < 32; j++) x[j] = __float_as_uint(OUT16 ? ex2(__uint_as_float(x[j])) : ex2_full(__uint_as_float(x[j])));
-            if (in) {
-              float* dst = out + c;
-              if (OUT16) {                               // (M is a multiple of 128 and the scratch aligned)
-                uint32_t h[16];
+            if (OUT16) {
+              uint32_t h[16];
 #pragma unroll
-                for (int j = 0; j < 16; j++) h[j] = pack_bf16(__uint_as_float(x[2 * j]), __uint_as_float(x[2 * j + 1]));
-                store32(reinterpret_cast<float*>(out16 + c), h);
-                store32(reinterpret_cast<float*>(out16 + c + 16), h + 8);
-              } else if (wide) {
+              for (int j = 0; j < 16; j++) h[j] = pack_bf16(__uint_as_float(x[2 * j]), __uint_as_float(x[2 * j + 1]));
+              put_rows(h, m0 + c, tok0);
+            } else if (a.staged[ti]) {
 #pragma unroll
-                for (int j = 0; j < 4; j++)
-                  if (j < 2 || c + 16 < mb) store32(dst + 8 * j, &x[8 * j]);
-              } else {
+              for (int j = 0; j < 32; j += ROW_BYTES / 4)
+                if (c + j < mb) put_rows(x + j, m0 + c + j, tok0);
+            } else if (in) {
+              float* dst = t.phi + at * a.M + m0 + c;
 #pragma unroll
-                for (int j = 0; j < 32; j++)
-                  if (j < 16 || c + 16 < mb) dst[j] = __uint_as_float(x[j]);
-              }
+              for (int j = 0; j < 32; j++)
+                if (j < 16 || c + 16 < mb) dst[j] = __uint_as_float(x[j]);
             }
           }
         } else {
@@ -736,6 +758,7 @@ feat3_kernel(const __grid_constant__ Args a) {
   }
   if (bad) atomicExch(a.status, FSHARP_E_NONFINITE);
   // no copy of this block may still be in flight when it exits
+  if (WRITE && warp < FT_STAGE0 && lane == 0) bulk_wait0();
   if (OUT16 && warp == FT_STAGE0 && lane == 0)
     for (int k = max(0, n - G::NBUF); k < n; k++)
       mbar_wait(&misc->a_full[k % G::NBUF], (k / G::NBUF) & 1, &misc->abort_flag, a.status, false);
@@ -750,12 +773,20 @@ feat3_kernel(const __grid_constant__ Args a) {
 
 template <typename T, int D, int BP>
 int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, int G_groups, float qk_scale, uint8_t* img) {
-  using G = FtGeo<T, D, BP>;
+  using G = FtGeo<T, D, BP, true>;
+  constexpr size_t max_smem = FtGeo<T, D, BP, false>::SMEM;
   a.wscale = Factor(LOG2E * (1.0 + LOST_W<D>) * (double)qk_scale);
   a.nmb = (a.M + G::MB - 1) / G::MB;
   CUtensorMap maps[2] = {};
   if (BP == 2)
     for (int i = 0; i < ntasks; i++) FS_TRY(tchost::make_map_tokens(&maps[i], tasks[i].X, tasks[i].ax, BH / a.H, a.H, tasks[i].L, D));
+  CUtensorMap outs[2] = {};
+  bool staged[2] = {};
+  for (int i = 0; i < ntasks; i++) {
+    void* phi = BP == 2 ? (void*)tasks[i].phi16 : (void*)tasks[i].phi;
+    staged[i] = reinterpret_cast<uintptr_t>(phi) % 16 == 0;          // (the library's own are)
+    if (staged[i]) FS_TRY(tchost::make_map_features(&outs[i], phi, BH, tasks[i].L, a.M, BP == 2, G::STAGE / 32));
+  }
   const uint8_t* side_img[2] = {nullptr, nullptr};     // by side - 1
   const bool pair = BP == 2 && ntasks == 1 && tasks[0].stab == FSHARP_STAB_ROW && a.nmb == 2;
   a.own_terms = BP == 2;
@@ -778,6 +809,8 @@ int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, in
       if (!take(tasks[i], a.nmb)) continue;
       a.t[k] = tasks[i];
       a.map[k] = maps[i];
+      a.out[k] = outs[i];
+      a.staged[k] = staged[i];
       a.img[k] = side_img[tasks[i].side - 1];
       a.tiles[k] = (tasks[i].L + TILE - 1) / TILE;
       a.first[k + 1] = a.first[k] + BH * units_per_bh * a.tiles[k];
@@ -810,9 +843,9 @@ int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, in
   }
   const int maxed = set(a.nmb, [](const Task& t, int nmb) { return t.stab == FSHARP_STAB_GROUP || (t.stab == FSHARP_STAB_ROW && nmb > 1); });
   if (maxed > 0) {
-    FS_CUDA_OK(cudaFuncSetAttribute(feat3_kernel<T, D, false, BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM));
+    FS_CUDA_OK(cudaFuncSetAttribute(feat3_kernel<T, D, false, BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem));
     FS_TIME_BEGIN(ctx, FS_K_GROUPMAX);
-    (void)fs_launch_chained(feat3_kernel<T, D, false, BP>, dim3(maxed < ctx->sm_count ? maxed : ctx->sm_count), dim3(FT_THREADS), G::SMEM, ctx->stream, a);
+    (void)fs_launch_chained(feat3_kernel<T, D, false, BP>, dim3(maxed < ctx->sm_count ? maxed : ctx->sm_count), dim3(FT_THREADS), max_smem, ctx->stream, a);
     FS_TIME_END(ctx);
     FS_LAUNCH_CHECK(ctx);
   }

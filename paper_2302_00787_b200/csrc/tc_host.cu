@@ -77,6 +77,21 @@ int make_map_out(CUtensorMap* map, void* base, TensorAddr a, int B, int H, int L
   return r == CUDA_SUCCESS ? FSHARP_OK : FSHARP_E_CUDA;
 }
 
+// Features [BH][L][M], fp32 or bf16, as store tiles of 32 rows of box_bytes (64 or 128, staged with the swizzle of that width).
+int make_map_features(CUtensorMap* map, void* base, int BH, int L, int M, int bf16, int box_bytes) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return FSHARP_E_CUDA;
+  const cuuint64_t es = bf16 ? 2 : 4;
+  cuuint64_t dims[3] = {(cuuint64_t)M, (cuuint64_t)L, (cuuint64_t)BH};
+  cuuint64_t strides[2] = {(cuuint64_t)M * es, (cuuint64_t)L * M * es};
+  cuuint32_t box[3] = {(cuuint32_t)(box_bytes / es), 32, 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = fn(map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, box_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                  CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? FSHARP_OK : FSHARP_E_CUDA;
+}
+
 }  // namespace tchost
 
 int fs_tc_supported(const fsharp_dims* dm, int dtype, int causal, int chunk, float qk_scale) {
