@@ -120,6 +120,54 @@ prep_kernel(const float* __restrict__ Omega, int64_t omega_head_stride, const do
 #pragma unroll
     for (int j = 0; j < 8; j++) piece.v[j] = (float)p[j];
   };
+  const auto put_a = [&](int m, float a) {
+#pragma unroll
+    for (int side = 0; side < 2; side++) {
+      out[(size_t)side * pr.total() + pr.a() + m] = a;
+      if (images != nullptr)
+        reinterpret_cast<float*>(images + ((size_t)g * 2 + side) * tcl::IMG_BYTES + tcl::IMG_A2)[m] = 2.f * FS_LOG2E * a;
+    }
+  };
+  if (is_a) {
+    // A is diagonal in all fits: a_m = sum_k A_kk Omega_mk^2, and no product (with one, these blocks and those of W were two
+    // waves of blocks for 64 groups)
+    float* diag = reinterpret_cast<float*>(raw);
+    const double* A = P + pl.A();
+    int off = 0;
+    for (int e0 = tid; e0 < d * d; e0 += 8 * PREP_THREADS) {
+      double v[8];
+#pragma unroll
+      for (int q = 0; q < 8; q++) v[q] = e0 + q * PREP_THREADS < d * d ? A[e0 + q * PREP_THREADS] : 0.0;
+#pragma unroll
+      for (int q = 0; q < 8; q++) {
+        const int e = e0 + q * PREP_THREADS;
+        if (e >= d * d) continue;
+        if (e % (d + 1) == 0) diag[e / (d + 1)] = (float)v[q];
+        else if (v[q] != 0.0) off = 1;
+      }
+    }
+    if (!__syncthreads_or(off)) {
+      const int m = m0 + (tid >> 1), k0 = (tid & 1) * (d / 2);        // two threads per feature
+      if (tid < 2 * PREP_MB) {
+        float s[4] = {};
+        if (m < M) {
+          const float* o = Om + (size_t)m * d + k0;
+#pragma unroll
+          for (int k = 0; k < d / 2; k += 4) {
+            float4 w;
+            if (aligned) w = *reinterpret_cast<const float4*>(o + k);
+            else w = make_float4(o[k], o[k + 1], o[k + 2], o[k + 3]);
+            const float4 a = *reinterpret_cast<const float4*>(diag + k0 + k);
+            s[0] = fmaf(a.x * w.x, w.x, s[0]); s[1] = fmaf(a.y * w.y, w.y, s[1]); s[2] = fmaf(a.z * w.z, w.z, s[2]); s[3] = fmaf(a.w * w.w, w.w, s[3]);
+          }
+        }
+        float a = (s[0] + s[1]) + (s[2] + s[3]);
+        a += __shfl_xor_sync(0xffffffffu, a, 1);
+        if (m < M && (tid & 1) == 0) put_a(m, a);
+      }
+      return;
+    }
+  }
   mma3::Block b;
   b.begin(raw, is_a ? d : SIDES * d, d, status);
   b.template segment<true, 3, false, 3>(d, omega, matrix);
@@ -157,13 +205,7 @@ prep_kernel(const float* __restrict__ Omega, int64_t omega_head_stride, const do
     __syncthreads();
     if (tid < PREP_MB && m0 + tid < M) {
       const int m = m0 + tid;
-      const float a = part[0][tid] + part[1][tid];
-#pragma unroll
-      for (int side = 0; side < 2; side++) {
-        out[(size_t)side * pr.total() + pr.a() + m] = a;
-        if (images != nullptr)
-          reinterpret_cast<float*>(images + ((size_t)g * 2 + side) * tcl::IMG_BYTES + tcl::IMG_A2)[m] = 2.f * FS_LOG2E * a;
-      }
+      put_a(m, part[0][tid] + part[1][tid]);
     }
   }
   b.end();
