@@ -297,14 +297,11 @@ int fsharp_kernel_apply(fsharp_ctx* ctx, const void* X, const void* Y, const voi
   FS_CUDA_OK(cudaSetDevice(ctx->device));
   const int G = fs_groups(dims);
   const size_t prep_f = (size_t)G * 2 * PrepLayout{dims->d, dims->M}.total();
-  const size_t np = (size_t)G * ParamsLayout{dims->d}.total();
-  FS_TRY(fs_ws_reserve(ctx, ws_round(prep_f * 4) + ws_round(np * 8) + fs_simt_attend_scratch_bytes(ctx, dims, 0, 0)));
+  FS_TRY(fs_ws_reserve(ctx, ws_round(prep_f * 4) + fs_simt_attend_scratch_bytes(ctx, dims, 0, 0)));
   WsAlloc ws{ctx->ws, 0};
   float* prep = ws.take<float>(prep_f);
-  double* shifted = ws.take<double>(np);
-  FS_TRY(fs_shift_c(ctx, params, shifted, G, dims->d, alpha));
-  FS_TRY(fs_run_prep(ctx, Omega, dims->omega_head_stride, shifted, (int64_t)ParamsLayout{dims->d}.total(), G, dims->H,
-                     dims->pool, dims->d, dims->M, prep));
+  FS_TRY(fs_run_prep(ctx, Omega, dims->omega_head_stride, params, (int64_t)ParamsLayout{dims->d}.total(), G, dims->H,
+                     dims->pool, dims->d, dims->M, prep, alpha));
   return fs_simt_kernel_apply(ctx, X, Y, Cmat, dims, dtype, qk_scale, prep, out, &ws);
 }
 

@@ -235,13 +235,14 @@ int fs_tc_stats(fsharp_ctx* ctx, const void* Q, const void* K, const fsharp_dims
 int fs_run_fit(fsharp_ctx* ctx, const double* stats, int G, int d, int variant, double ridge,
                double* params, double* scratch);
 size_t fs_fit_scratch_doubles(int G, int d);
-// params_stride: doubles between the blobs of two groups (0 = every group reads the same blob)
+// params_stride: doubles between the blobs of two groups (0 = every group reads the same blob).  alpha: added to the diagonals of C1
+// and C2 (exp(alpha |x|^2) f(w, x) is the DERF with C + alpha I: Section 2.3's reduction of K^(alpha) to K^(0)).
 int fs_run_prep(fsharp_ctx* ctx, const float* Omega, int64_t omega_head_stride, const double* params,
-                int64_t params_stride, int G, int H, int pool, int d, int M, float* prep /* [G][2][PrepLayout] */);
+                int64_t params_stride, int G, int H, int pool, int d, int M, float* prep /* [G][2][PrepLayout] */, double alpha = 0.0);
 // The same, and (images != nullptr; d = 64, M = 256) the tensor-core path's operand images and flag words too.
 int fs_run_prep_images(fsharp_ctx* ctx, const float* Omega, int64_t omega_head_stride, const double* params,
                        int64_t params_stride, int G, int H, int pool, int d, int M, float* prep, float qk_scale,
-                       uint8_t* images, int* flags);
+                       uint8_t* images, int* flags, double alpha = 0.0);
 // rowc: scratch [B*H*L] floats.  gmax: scratch [B*H] words.  phi: [B,H,L,M] floats.  img: scratch (feat3.cuh) or null.
 int fs_simt_featurize(fsharp_ctx* ctx, const void* X, int dtype, TensorAddr ax, int B, int H, int L, int d,
                       int M, int pool, const float* prep, int side, float qk_scale, int stab,
@@ -265,7 +266,6 @@ size_t fs_backward_scratch_bytes(const fsharp_dims* dm, int causal, int chunk);
 int fs_backward(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const void* dY, const fsharp_dims* dm,
                 int dtype, int causal, int chunk, float qk_scale, const float* prep, void* dQ, void* dK, void* dV,
                 WsAlloc* ws);
-int fs_shift_c(fsharp_ctx* ctx, const double* params, double* out, int G, int d, double alpha);
 int fs_run_pairs(fsharp_ctx* ctx, const float* X, const float* Y, const float* Omega, const double* params,
                  int64_t npairs, int d, int M, int R, float* est, double* var_cf, double* pooled, WsAlloc* ws);
 size_t fs_pairs_scratch_bytes(int d, int M, int R);

@@ -192,27 +192,3 @@ int fs_simt_kernel_apply(fsharp_ctx* ctx, const void* X, const void* Yset, const
   if (dtype == FSHARP_F32) return attend_t<float>(ctx, X, Yset, Cmat, dm, 0, 0, qk_scale, prep, out, ws, true);
   return attend_t<__nv_bfloat16>(ctx, X, Yset, Cmat, dm, 0, 0, qk_scale, prep, out, ws, true);
 }
-
-// params_out = params with alpha added to the diagonals of C1 and C2: exp(alpha |x|^2) f(w, x) is the DERF with
-// C + alpha I (Section 2.3's reduction of K^(alpha) to K^(0)).
-namespace {
-__global__ void shift_c_kernel(const double* __restrict__ params, double* __restrict__ out, int d, double alpha, size_t total) {
-  fs_grid_dependency_wait();
-  const size_t g = blockIdx.x;
-  ParamsLayout pl{d};
-  for (size_t e = threadIdx.x; e < total; e += blockDim.x) {
-    double v = params[g * total + e];
-    if (e >= pl.C(1) && e < pl.tail()) {
-      const size_t r = (e - pl.C(1)) % pl.dd();
-      if (r / d == r % d) v += alpha;
-    }
-    out[g * total + e] = v;
-  }
-}
-}  // namespace
-int fs_shift_c(fsharp_ctx* ctx, const double* params, double* out, int G, int d, double alpha) {
-  if (G == 0) return FSHARP_OK;
-  (void)fs_launch_chained(shift_c_kernel, dim3(G), dim3(256), 0, ctx->stream, params, out, d, alpha, ParamsLayout{d}.total());
-  FS_LAUNCH_CHECK(ctx);
-  return FSHARP_OK;
-}

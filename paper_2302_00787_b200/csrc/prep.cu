@@ -17,7 +17,7 @@ constexpr int PREP_THREADS = mma3::THREADS;
 template <int D>
 __device__ __forceinline__ void scalars_of(int g, int side, const double* __restrict__ params, int64_t params_stride, int M,
                                            double half_log_m, float* __restrict__ prep, float qk_scale, uint8_t* __restrict__ images,
-                                           int* __restrict__ img_flags, uint8_t* raw) {
+                                           int* __restrict__ img_flags, double alpha, uint8_t* raw) {
   constexpr int d = D;
   const int tid = threadIdx.x;
   ParamsLayout pl{d};
@@ -31,7 +31,7 @@ __device__ __forceinline__ void scalars_of(int g, int side, const double* __rest
   // C = gamma I exactly?  The operand images (row j, column i = C[i][j], 128-byte swizzle) are put together in shared
   // memory and leave in 16-byte pieces: element-wise stores of a transposed 2-byte layout would touch a sector each.
   int cscalar = 1, lo_nonzero = 0;
-  const double gamma = Cm[0];
+  const double gamma = Cm[0] + alpha;
   uint8_t* simg = raw;             // [hi image | lo image], IMG_C_BYTES each (d = 64 only)
   for (int e0 = tid; e0 < d * d; e0 += 8 * PREP_THREADS) {
     double cv[8];
@@ -39,6 +39,7 @@ __device__ __forceinline__ void scalars_of(int g, int side, const double* __rest
     for (int q = 0; q < 8; q++) {
       const int e = e0 + q * PREP_THREADS;
       cv[q] = e < d * d ? Cm[e] : 0.0;
+      if (e % (d + 1) == 0) cv[q] += alpha;                          // (0, but for the operator with exp(alpha |x|^2))
     }
 #pragma unroll
     for (int q = 0; q < 8; q++) {
@@ -87,7 +88,7 @@ template <int D>
 __global__ void __launch_bounds__(PREP_THREADS)
 prep_kernel(const float* __restrict__ Omega, int64_t omega_head_stride, const double* __restrict__ params,
             int64_t params_stride, int H, int pool, int M, float* __restrict__ prep, float qk_scale,
-            uint8_t* __restrict__ images, int* __restrict__ img_flags, double half_log_m, int* __restrict__ status) {
+            uint8_t* __restrict__ images, int* __restrict__ img_flags, double half_log_m, double alpha, int* __restrict__ status) {
   fs_grid_dependency_wait();
   // images != nullptr (d = 64, M = 256 only): the tensor-core path's operand images of this (group, side)
   // are written as well, in the layouts of tc_layout.cuh
@@ -95,7 +96,7 @@ prep_kernel(const float* __restrict__ Omega, int64_t omega_head_stride, const do
   extern __shared__ __align__(16) uint8_t raw[];
   const int g = blockIdx.x, role = blockIdx.y, tid = threadIdx.x;
   if (role == NW + 1) {
-    if (blockIdx.z < 2) scalars_of<D>(g, blockIdx.z + 1, params, params_stride, M, half_log_m, prep, qk_scale, images, img_flags, raw);
+    if (blockIdx.z < 2) scalars_of<D>(g, blockIdx.z + 1, params, params_stride, M, half_log_m, prep, qk_scale, images, img_flags, alpha, raw);
     return;
   }
   const int m0 = blockIdx.z * PREP_MB, side0 = role;                  // (a W block's first side, from 0)
@@ -214,13 +215,13 @@ prep_kernel(const float* __restrict__ Omega, int64_t omega_head_stride, const do
 }  // namespace
 
 int fs_run_prep(fsharp_ctx* ctx, const float* Omega, int64_t omega_head_stride, const double* params,
-                int64_t params_stride, int G, int H, int pool, int d, int M, float* prep) {
-  return fs_run_prep_images(ctx, Omega, omega_head_stride, params, params_stride, G, H, pool, d, M, prep, 1.f, nullptr, nullptr);
+                int64_t params_stride, int G, int H, int pool, int d, int M, float* prep, double alpha) {
+  return fs_run_prep_images(ctx, Omega, omega_head_stride, params, params_stride, G, H, pool, d, M, prep, 1.f, nullptr, nullptr, alpha);
 }
 
 int fs_run_prep_images(fsharp_ctx* ctx, const float* Omega, int64_t omega_head_stride, const double* params,
                        int64_t params_stride, int G, int H, int pool, int d, int M, float* prep, float qk_scale,
-                       uint8_t* images, int* flags) {
+                       uint8_t* images, int* flags, double alpha) {
   FS_RANGE("operand images");
   if (G == 0) return FSHARP_OK;
   if (images != nullptr && (d != tcl::TC_D || M != tcl::TC_M)) return FSHARP_E_SHAPE;
@@ -231,7 +232,7 @@ int fs_run_prep_images(fsharp_ctx* ctx, const float* Omega, int64_t omega_head_s
     FS_CUDA_OK(cudaFuncSetAttribute(prep_kernel<DD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mma3::SMEM));        \
     FS_TIME_BEGIN(ctx, FS_K_PREP);                                                                                    \
     (void)fs_launch_chained(prep_kernel<DD>, grid, dim3(PREP_THREADS), mma3::SMEM, ctx->stream, Omega, omega_head_stride, params, params_stride, H,   \
-                                                               pool, M, prep, qk_scale, images, flags, 0.5 * log((double)M), ctx->d_status);  \
+                                                               pool, M, prep, qk_scale, images, flags, 0.5 * log((double)M), alpha, ctx->d_status);  \
   } while (0)
   switch (d) {
     case 16: FS_PREP(16); break;
