@@ -39,10 +39,11 @@ __device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
 template <typename T>
 __global__ void __launch_bounds__(mma3::THREADS, 2)
 bwd_tri_kernel(const float* __restrict__ G, const T* __restrict__ V, TensorAddr av, BwdDims q, float* __restrict__ out,
-               int* __restrict__ status) {
+               int flip, int* __restrict__ status) {
   fs_grid_dependency_wait();
+  const int zi = mma3::unit_of(flip);
   extern __shared__ uint8_t smem[];
-  const int bh = blockIdx.z / q.nch, c = blockIdx.z % q.nch, b = bh / q.H, h = bh % q.H;
+  const int bh = zi / q.nch, c = zi % q.nch, b = bh / q.H, h = bh % q.H;
   const int i0 = blockIdx.x * ROWS, j0 = blockIdx.y * ROWS, C = q.C, dv = q.dv;
   if (j0 > i0) return;
   mma3::Block blk;
@@ -59,7 +60,7 @@ bwd_tri_kernel(const float* __restrict__ G, const T* __restrict__ V, TensorAddr 
         else p.unit();
       });
   blk.finish();
-  float* S = out + (int64_t)blockIdx.z * C * C;
+  float* S = out + (int64_t)zi * C * C;
   blk.rows([&](int r, int n, float4 v) {
     const int i = i0 + r, j = j0 + n;
     if (j > i) v.x = 0.f;
@@ -77,11 +78,12 @@ template <typename T>
 __global__ void __launch_bounds__(mma3::THREADS, 2)
 bwd_numden_kernel(const float* __restrict__ phiQ, const float* __restrict__ KV, const float* __restrict__ sc,
                   const T* __restrict__ V, TensorAddr av, const T* __restrict__ dY, TensorAddr ay, BwdDims q, float* __restrict__ G,
-                  int* __restrict__ status) {
+                  int flip, int* __restrict__ status) {
   fs_grid_dependency_wait();
+  const int zi = mma3::unit_of(flip);
   extern __shared__ uint8_t smem[];
   __shared__ float inv_s[ROWS], dot_s[ROWS];
-  const int bh = blockIdx.z, b = bh / q.H, h = bh % q.H, i0 = blockIdx.x * ROWS;
+  const int bh = zi, b = bh / q.H, h = bh % q.H, i0 = blockIdx.x * ROWS;
   const int C = q.C, M = q.M, NP = q.NP, dv = q.dv, L = q.Lq;
   const ColTile ct(dv, blockIdx.y);
   mma3::Block blk;
@@ -89,7 +91,6 @@ bwd_numden_kernel(const float* __restrict__ phiQ, const float* __restrict__ KV, 
   const int chunk = q.causal ? i0 / C : 0;
   const float* PQ = phiQ + ((int64_t)bh * L + i0) * M;
   const float* S = KV + ((int64_t)bh * q.nch + chunk) * M * NP;
-  mma3::prefetch_rows(PQ, 4LL * M, min(ROWS, L - i0), 4LL * M);
   blk.template segment<true, 3, false, 3>(
       M, [&](int r, int k, Piece<3>& p) { if (i0 + r < L) p.load(PQ + (int64_t)r * M + k); else p.zero(); },
       [&](int c, int k, Piece<3>& p) { p.load(S + (int64_t)k * NP + ct.at(dv, c)); });
@@ -184,11 +185,12 @@ template <typename T, int SIDE>
 __global__ void __launch_bounds__(mma3::THREADS, 2)
 bwd_dfeat_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK, const float* __restrict__ G,
                  const float* __restrict__ St, const float* __restrict__ gv, const T* __restrict__ V, TensorAddr av,
-                 BwdDims q, float* __restrict__ E, float* __restrict__ rs, int* __restrict__ status) {
+                 BwdDims q, float* __restrict__ E, float* __restrict__ rs, int flip, int* __restrict__ status) {
   fs_grid_dependency_wait();
+  const int zi = mma3::unit_of(flip);
   extern __shared__ uint8_t smem[];
   __shared__ float rs_s[ROWS];
-  const int bh = blockIdx.z, b = bh / q.H, h = bh % q.H;
+  const int bh = zi, b = bh / q.H, h = bh % q.H;
   // (token tiles run along x, the only coordinate that takes more than 65535; the feature tiles of one token tile are neighbours)
   const int mtiles = (q.M + ROWS - 1) / ROWS, mt = blockIdx.x % mtiles, m0 = mt * ROWS, i0 = blockIdx.x / mtiles * ROWS;
   const int C = q.C, M = q.M, NP = q.NP, dv = q.dv, L = SIDE == 1 ? q.Lq : q.Lk;
@@ -197,12 +199,6 @@ bwd_dfeat_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK,
   blk.begin(smem, min(ROWS, M - m0), NP + (q.causal ? C : 0), status);
   const float* S = St + ((int64_t)bh * q.nch + chunk) * M * NP + (int64_t)m0 * NP;
   const float* GV = q.causal ? gv + ((int64_t)bh * q.nch + chunk) * C * C : nullptr;
-  const int64_t width = 4LL * min(ROWS, M - m0);
-  if (q.causal) {
-    const float* other = (SIDE == 1 ? phiK : phiQ) + ((int64_t)bh * L + (int64_t)chunk * C + (SIDE == 1 ? 0 : ic)) * M + m0;
-    mma3::prefetch_rows(other, 4LL * M, SIDE == 1 ? min(ic + ROWS, L - chunk * C) : min(C, L - chunk * C) - ic, width);
-  }
-  mma3::prefetch_rows((SIDE == 1 ? phiQ : phiK) + ((int64_t)bh * L + i0) * M + m0, 4LL * M, min(ROWS, L - i0), width);
   if (SIDE == 1) {
     const float* Gb = G + ((int64_t)bh * L + i0) * NP;
     blk.template segment<true, 3, true, 3>(
@@ -265,17 +261,17 @@ bwd_dfeat_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK,
 template <typename T>
 __global__ void __launch_bounds__(mma3::THREADS, 2)
 bwd_dv_kernel(const float* __restrict__ phiK, const float* __restrict__ Rt, const float* __restrict__ sc,
-              const float* __restrict__ G, BwdDims q, T* __restrict__ dV, TensorAddr av, int* __restrict__ status) {
+              const float* __restrict__ G, BwdDims q, T* __restrict__ dV, TensorAddr av, int flip, int* __restrict__ status) {
   fs_grid_dependency_wait();
+  const int zi = mma3::unit_of(flip);
   extern __shared__ uint8_t smem[];
-  const int bh = blockIdx.z, b = bh / q.H, h = bh % q.H, j0 = blockIdx.x * ROWS;
+  const int bh = zi, b = bh / q.H, h = bh % q.H, j0 = blockIdx.x * ROWS;
   const int C = q.C, M = q.M, NP = q.NP, L = q.Lk, cols = tile_columns(q.dv, M), c0 = blockIdx.y * cols;
   const int chunk = q.causal ? j0 / C : 0, jc = q.causal ? j0 - chunk * C : 0;
   mma3::Block blk;
   blk.begin(smem, cols, M + (q.causal ? C - jc : 0), status);
   const float* PK = phiK + ((int64_t)bh * L + j0) * M;
   const float* R = Rt + ((int64_t)bh * q.nch + chunk) * M * NP;
-  mma3::prefetch_rows(PK, 4LL * M, min(ROWS, L - j0), 4LL * M);
   blk.template segment<true, 3, false, 3>(
       M, [&](int r, int k, Piece<3>& p) { if (j0 + r < L) p.load(PK + (int64_t)r * M + k); else p.zero(); },
       [&](int c, int k, Piece<3>& p) { p.load(R + (int64_t)k * NP + c0 + c); });
@@ -299,11 +295,12 @@ template <typename T>
 __global__ void __launch_bounds__(mma3::THREADS, 2)
 bwd_dx_kernel(const float* __restrict__ E, const float* __restrict__ rs, int mtiles, const T* __restrict__ X, TensorAddr ax, int H, int L,
               int d, int M, int pool, int side, const float* __restrict__ prep, float qk_scale, T* __restrict__ dX,
-              int* __restrict__ status) {
+              int flip, int* __restrict__ status) {
   fs_grid_dependency_wait();
+  const int zi = mma3::unit_of(flip);
   extern __shared__ uint8_t smem[];
   __shared__ float rs_s[ROWS];
-  const int bh = blockIdx.z, b = bh / H, h = bh % H, i0 = blockIdx.x * ROWS, cols = tile_columns(d, M), c0 = blockIdx.y * cols;
+  const int bh = zi, b = bh / H, h = bh % H, i0 = blockIdx.x * ROWS, cols = tile_columns(d, M), c0 = blockIdx.y * cols;
   PrepLayout pr{d, M};
   const float* pp = prep + ((size_t)(pool == FSHARP_POOL_PER_BH ? bh : h) * 2 + (side - 1)) * pr.total();
   const float* W = pp + pr.W();
@@ -320,7 +317,6 @@ bwd_dx_kernel(const float* __restrict__ E, const float* __restrict__ rs, int mti
   }
   __syncthreads();
   const float* Eb = E + ((int64_t)bh * L + i0) * M;
-  mma3::prefetch_rows(Eb, 4LL * M, min(ROWS, L - i0), 4LL * M);
   const T* Xb = X + b * ax.sb + h * ax.sh + (int64_t)i0 * ax.sl;
   blk.template segment<true, 3, false, 3>(
       M, [&](int r, int k, Piece<3>& p) { if (i0 + r < L) p.load(Eb + (int64_t)r * M + k); else p.zero(); },
@@ -396,7 +392,7 @@ int backward_t(fsharp_ctx* ctx, const void* Qv, const void* Kv, const void* Vv, 
                                 {Q, aq, Lq, 1, FSHARP_STAB_ROW, rowcq, nullptr, phiQ, nullptr, lsq, feat3::LIFT}};
   FS_TRY(feat3::run(ctx, tasks, 2, dtype, B, H, d, M, dm->pool, prep, qk_scale, img));
   // sums over tokens: the total (bidirectional), or one per chunk turned into the sum over earlier / later chunks (causal)
-  auto sums = [&](auto from_g, const float* F, int L, float* out, int reverse) -> int {
+  auto sums = [&](auto from_g, const float* F, int L, float* out, int reverse, int flip) -> int {
     constexpr bool FG = decltype(from_g)::value;
     int slen = C, nsl = nch;
     if (!causal) {
@@ -404,10 +400,10 @@ int backward_t(fsharp_ctx* ctx, const void* Qv, const void* Kv, const void* Vv, 
       FS_CUDA_OK(cudaMemsetAsync(out, 0, (size_t)BH * elems * sizeof(float), ctx->stream));
     }
     FS_TRY(mma3::launch(ctx, FS_K_BWD_STATE, state_kernel<T, FG>, dim3(mt, ctiles, BH * nsl), F, V, av, G, H, L, M, dv, slen, nsl,
-                        causal ? 1 : 0, out, status));
+                        causal ? 1 : 0, out, flip, status));
     if (causal) {
       FS_TIME_BEGIN(ctx, FS_K_PREFIX);
-      (void)fs_launch_chained(prefix_kernel, gscan, dim3(NTH), 0, ctx->stream, out, nch, elems, reverse);
+      (void)fs_launch_chained(prefix_kernel, gscan, dim3(NTH), 0, ctx->stream, out, nch, elems, reverse, 1 - flip);
       FS_TIME_END(ctx);
       FS_LAUNCH_CHECK(ctx);
     }
@@ -415,9 +411,9 @@ int backward_t(fsharp_ctx* ctx, const void* Qv, const void* Kv, const void* Vv, 
   };
   const dim3 gtri(causal ? C / ROWS : 1, causal ? C / ROWS : 1, BH * nch), gsc(gtri.x, causal ? C / tile_columns(ROWS, M) : 1, BH * nch);
   const int dtiles = d / tile_columns(d, M);
-  FS_TRY(sums(No{}, phiK, Lk, KV, 0));
-  if (causal) FS_TRY(mma3::launch(ctx, FS_K_SCORES, scores_kernel, gsc, phiQ, phiK, Lq, M, C, nch, sc, status));
-  FS_TRY(mma3::launch(ctx, FS_K_BWD_NUMDEN, bwd_numden_kernel<T>, dim3(qt, ctiles, BH), phiQ, KV, sc, V, av, dY, ay, q, G, status));
+  FS_TRY(sums(No{}, phiK, Lk, KV, 0, 0));
+  if (causal) FS_TRY(mma3::launch(ctx, FS_K_SCORES, scores_kernel, gsc, phiQ, phiK, Lq, M, C, nch, sc, 1, status));
+  FS_TRY(mma3::launch(ctx, FS_K_BWD_NUMDEN, bwd_numden_kernel<T>, dim3(qt, ctiles, BH), phiQ, KV, sc, V, av, dY, ay, q, G, 0, status));
   if (ctiles > 1) {
     int gx = (Lq + 7) / 8;
     if (gx > 4 * ctx->sm_count) gx = 4 * ctx->sm_count;
@@ -426,15 +422,15 @@ int backward_t(fsharp_ctx* ctx, const void* Qv, const void* Kv, const void* Vv, 
     FS_TIME_END(ctx);
     FS_LAUNCH_CHECK(ctx);
   }
-  FS_TRY(sums(Yes{}, phiQ, Lq, Rt, 1));
-  if (causal) FS_TRY(mma3::launch(ctx, FS_K_SCORES, bwd_tri_kernel<T>, gtri, G, V, av, q, gv, status));
-  FS_TRY(mma3::launch(ctx, FS_K_BWD_DFEAT, bwd_dfeat_kernel<T, 1>, dim3(mt * qt, 1, BH), phiQ, phiK, G, KV, gv, V, av, q, E, rs, status));
+  FS_TRY(sums(Yes{}, phiQ, Lq, Rt, 1, 1));
+  if (causal) FS_TRY(mma3::launch(ctx, FS_K_SCORES, bwd_tri_kernel<T>, gtri, G, V, av, q, gv, 1, status));
+  FS_TRY(mma3::launch(ctx, FS_K_BWD_DFEAT, bwd_dfeat_kernel<T, 1>, dim3(mt * qt, 1, BH), phiQ, phiK, G, KV, gv, V, av, q, E, rs, 0, status));
   FS_TRY(mma3::launch(ctx, FS_K_BWD_DX, bwd_dx_kernel<T>, dim3(qt, dtiles, BH), E, rs, mt, Q, aq, H, Lq, d, M, dm->pool, 1, prep, qk_scale,
-                      (T*)dQv, status));
-  FS_TRY(mma3::launch(ctx, FS_K_BWD_DFEAT, bwd_dfeat_kernel<T, 2>, dim3(mt * kt, 1, BH), phiQ, phiK, G, Rt, gv, V, av, q, E, rs, status));
+                      (T*)dQv, 1, status));
+  FS_TRY(mma3::launch(ctx, FS_K_BWD_DFEAT, bwd_dfeat_kernel<T, 2>, dim3(mt * kt, 1, BH), phiQ, phiK, G, Rt, gv, V, av, q, E, rs, 0, status));
   FS_TRY(mma3::launch(ctx, FS_K_BWD_DX, bwd_dx_kernel<T>, dim3(kt, dtiles, BH), E, rs, mt, K, ak, H, Lk, d, M, dm->pool, 2, prep, qk_scale,
-                      (T*)dKv, status));
-  return mma3::launch(ctx, FS_K_BWD_DV, bwd_dv_kernel<T>, dim3(kt, dv / tile_columns(dv, M), BH), phiK, Rt, sc, G, q, (T*)dVv, av, status);
+                      (T*)dKv, 1, status));
+  return mma3::launch(ctx, FS_K_BWD_DV, bwd_dv_kernel<T>, dim3(kt, dv / tile_columns(dv, M), BH), phiK, Rt, sc, G, q, (T*)dVv, av, 0, status);
 }
 
 }  // namespace

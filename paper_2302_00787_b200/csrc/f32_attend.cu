@@ -19,7 +19,7 @@ template <typename T>
 __global__ void __launch_bounds__(mma3::THREADS, 2)
 out_kernel(const float* __restrict__ phiQ, const float* __restrict__ KV, const float* __restrict__ sc,
            const T* __restrict__ V, TensorAddr av, T* __restrict__ Y, TensorAddr ay, int H, int L, int M, int dv,
-           int causal, int C, int nchunks, const float* __restrict__ lsq, const float* __restrict__ lsk,
+           int causal, int C, int nchunks, const float* __restrict__ lsq, const float* __restrict__ lsk, int flip,
            int* __restrict__ status) {
   fs_grid_dependency_wait();
   // lsq != nullptr: the unnormalised operator Khat C of Section 2.1 is wanted: row i of the numerator times
@@ -27,7 +27,7 @@ out_kernel(const float* __restrict__ phiQ, const float* __restrict__ KV, const f
   // off the sums, not off exp(), which may be next to the smallest number as it is)
   extern __shared__ uint8_t smem[];
   __shared__ float inv_s[mma3::ROWS];
-  const int bh = blockIdx.z, b = bh / H, h = bh % H, NP = dv + 16;
+  const int bh = mma3::unit_of(flip), b = bh / H, h = bh % H, NP = dv + 16;
   const int i0 = blockIdx.x * mma3::ROWS;
   const ColTile ct(dv, blockIdx.y);
   mma3::Block blk;
@@ -112,9 +112,9 @@ int attend_t(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const
     int slen = 0;
     const int nsl = fs_token_slices(ctx, BH * gkv.x * gkv.y, BH, Lk, &slen);
     FS_TRY(mma3::launch(ctx, FS_K_KV, state_kernel<T, false>, dim3(gkv.x, gkv.y, BH * nsl), phiK, (const T*)V, av, nullptr, H, Lk, M, dv, slen, nsl, 0,
-                        KV, ctx->d_status));
+                        KV, 0, ctx->d_status));
     FS_TRY(mma3::launch(ctx, FS_K_OUT, out_kernel<T>, gout, phiQ, KV, nullptr, (const T*)V, av, (T*)Y, ay, H, Lq, M, dv, 0, 0, 1,
-                        unnormalised ? lsq : nullptr, lsk, ctx->d_status));
+                        unnormalised ? lsq : nullptr, lsk, 1, ctx->d_status));
     return FSHARP_OK;
   }
   if (tc) {
@@ -127,7 +127,7 @@ int attend_t(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const
     if (slots > 1) {
       FS_TRY(fs_tc_kv128(ctx, phiK16, V, av, B, H, Lk, M, C, tot, nullptr, nullptr));
       FS_TIME_BEGIN(ctx, FS_K_PREFIX);
-      (void)fs_launch_chained(prefix_kernel, dim3((unsigned)((elems + NTH - 1) / NTH), BH), dim3(NTH), 0, ctx->stream, tot, slots, elems, 0);
+      (void)fs_launch_chained(prefix_kernel, dim3((unsigned)((elems + NTH - 1) / NTH), BH), dim3(NTH), 0, ctx->stream, tot, slots, elems, 0, 0);
       FS_TIME_END(ctx);
       FS_LAUNCH_CHECK(ctx);
     }
@@ -138,16 +138,16 @@ int attend_t(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const
   const int64_t elems = (int64_t)M * NP;
   float* st = ws->take<float>((size_t)BH * nch * elems);
   float* sc = ws->take<float>((size_t)BH * nch * C * C);
-  FS_TRY(mma3::launch(ctx, FS_K_KV, state_kernel<T, false>, dim3(gkv.x, gkv.y, BH * nch), phiK, (const T*)V, av, nullptr, H, Lk, M, dv, C, nch, 1, st,
+  FS_TRY(mma3::launch(ctx, FS_K_KV, state_kernel<T, false>, dim3(gkv.x, gkv.y, BH * nch), phiK, (const T*)V, av, nullptr, H, Lk, M, dv, C, nch, 1, st, 0,
                       ctx->d_status));
   FS_TIME_BEGIN(ctx, FS_K_PREFIX);
-  (void)fs_launch_chained(prefix_kernel, dim3((unsigned)((elems + NTH - 1) / NTH), BH), dim3(NTH), 0, ctx->stream, st, nch, elems, 0);
+  (void)fs_launch_chained(prefix_kernel, dim3((unsigned)((elems + NTH - 1) / NTH), BH), dim3(NTH), 0, ctx->stream, st, nch, elems, 0, 1);
   FS_TIME_END(ctx);
   FS_LAUNCH_CHECK(ctx);
-  FS_TRY(mma3::launch(ctx, FS_K_SCORES, scores_kernel, dim3(C / mma3::ROWS, C / tile_columns(mma3::ROWS, M), BH * nch), phiQ, phiK, Lq, M, C, nch, sc,
+  FS_TRY(mma3::launch(ctx, FS_K_SCORES, scores_kernel, dim3(C / mma3::ROWS, C / tile_columns(mma3::ROWS, M), BH * nch), phiQ, phiK, Lq, M, C, nch, sc, 1,
                       ctx->d_status));
   return mma3::launch(ctx, FS_K_OUT, out_kernel<T>, gout, phiQ, st, sc, (const T*)V, av, (T*)Y, ay, H, Lq, M, dv, 1, C, nch, nullptr,
-                      nullptr, ctx->d_status);
+                      nullptr, 0, ctx->d_status);
 }
 
 }  // namespace

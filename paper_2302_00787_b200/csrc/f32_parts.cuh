@@ -25,10 +25,11 @@ struct ColTile {
 template <typename T, bool FROM_G>
 __global__ void __launch_bounds__(mma3::THREADS, 2)
 state_kernel(const float* __restrict__ F, const T* __restrict__ V, TensorAddr av, const float* __restrict__ G, int H, int L, int M,
-             int dv, int slice_len, int nslices, int per_slice_out, float* __restrict__ out, int* __restrict__ status) {
+             int dv, int slice_len, int nslices, int per_slice_out, float* __restrict__ out, int flip, int* __restrict__ status) {
   fs_grid_dependency_wait();
+  const int zi = mma3::unit_of(flip);
   extern __shared__ uint8_t smem[];
-  const int bh = blockIdx.z / nslices, sl = blockIdx.z % nslices, b = bh / H, h = bh % H;
+  const int bh = zi / nslices, sl = zi % nslices, b = bh / H, h = bh % H;
   const int m0 = blockIdx.x * mma3::ROWS, NP = dv + 16;
   const int j0 = sl * slice_len, j1 = min(L, j0 + slice_len);
   if (j0 >= j1) return;
@@ -51,7 +52,7 @@ state_kernel(const float* __restrict__ F, const T* __restrict__ V, TensorAddr av
         }
       });
   blk.finish();
-  float* O = out + (int64_t)(per_slice_out ? blockIdx.z : bh) * M * NP;
+  float* O = out + (int64_t)(per_slice_out ? zi : bh) * M * NP;
   blk.rows([&](int r, int c, float4 v) {
     if (m0 + r >= M || (c >= ct.wt && blockIdx.y > 0)) return;        // the ones block is written by the first tile
     float4* dst = reinterpret_cast<float4*>(O + (int64_t)(m0 + r) * NP + ct.at(dv, c));
@@ -63,9 +64,9 @@ state_kernel(const float* __restrict__ F, const T* __restrict__ V, TensorAddr av
 
 // ---- exclusive running sum over the chunks, forwards (earlier chunks) or backwards (later chunks) ------
 __global__ void __launch_bounds__(NTH)
-prefix_kernel(float* __restrict__ st, int nchunks, int64_t elems, int reverse) {
+prefix_kernel(float* __restrict__ st, int nchunks, int64_t elems, int reverse, int flip) {
   fs_grid_dependency_wait();
-  const int bh = blockIdx.y;
+  const int bh = flip ? gridDim.y - 1 - blockIdx.y : blockIdx.y;
   float* base = st + (int64_t)bh * nchunks * elems;
   for (int64_t e = blockIdx.x * (int64_t)NTH + threadIdx.x; e < elems; e += (int64_t)gridDim.x * NTH) {
     float run = 0.f;
@@ -93,10 +94,11 @@ __host__ __device__ inline int tile_columns(int columns, int M) { return M > mma
 // ---- masked in-chunk scores: sc[bh, c][i][j] = (j <= i) phiQ_i . phiK_j; tiles above the diagonal are neither written nor read
 __global__ void __launch_bounds__(mma3::THREADS, 2)
 scores_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK, int L, int M, int C, int nchunks,
-              float* __restrict__ sc, int* __restrict__ status) {
+              float* __restrict__ sc, int flip, int* __restrict__ status) {
   fs_grid_dependency_wait();
+  const int zi = mma3::unit_of(flip);
   extern __shared__ uint8_t smem[];
-  const int bh = blockIdx.z / nchunks, c = blockIdx.z % nchunks;
+  const int bh = zi / nchunks, c = zi % nchunks;
   const int cols = tile_columns(mma3::ROWS, M), i0 = blockIdx.x * mma3::ROWS, j0 = blockIdx.y * cols;
   if (j0 >= i0 + mma3::ROWS) return;
   mma3::Block blk;
@@ -108,7 +110,7 @@ scores_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK, in
       M, [&](int r, int k, mma3::Piece<3>& p) { if (i0 + r < rows) p.load(PQ + (int64_t)(i0 + r) * M + k); else p.zero(); },
       [&](int n, int k, mma3::Piece<3>& p) { if (j0 + n < rows) p.load(PK + (int64_t)(j0 + n) * M + k); else p.zero(); });
   blk.finish();
-  float* S = sc + (int64_t)blockIdx.z * C * C;
+  float* S = sc + (int64_t)zi * C * C;
   blk.rows([&](int r, int n, float4 v) {
     const int i = i0 + r, j = j0 + n;
     if (j + 1 > i) v.y = 0.f;

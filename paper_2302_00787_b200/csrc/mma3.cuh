@@ -74,15 +74,10 @@ template <> struct Piece<1> {
 template <typename T> struct PartsOf { static constexpr int N = 3; };
 template <> struct PartsOf<__nv_bfloat16> { static constexpr int N = 1; };
 
-// rows of `bytes` contiguous bytes, `stride` bytes apart, asked into L2 by the whole block ahead of its slices: a slice takes 128
-// bytes of a row at a time, one slice ahead of its use, which is not enough against the latency of HBM
-__device__ __forceinline__ void prefetch_rows(const void* base, int64_t stride, int rows, int64_t bytes) {
-  const int lines = (int)((bytes + 127) >> 7);
-  for (int e = threadIdx.x; e < rows * lines; e += THREADS) {
-    const int r = e / lines;
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const char*>(base) + r * stride + (int64_t)(e - r * lines) * 128));
-  }
-}
+// Which unit (z coordinate) a block takes.  Kernels of a chain walk the units up and down in turn: the matrices that one leaves behind
+// are larger than the L2, and what it touched last is still there for the next one (causal training step of 2 x 12 x 4096 tokens: 1223 -> 1208 us).
+// (A block's rows asked into L2 ahead of its slices: 18 us more, the first slices wait behind all of them.)
+__device__ __forceinline__ int unit_of(int flip) { return flip ? gridDim.z - 1 - blockIdx.z : blockIdx.z; }
 
 struct Block {
   uint8_t* sm;
