@@ -130,9 +130,9 @@ prep_kernel(const float* __restrict__ Omega, int64_t omega_head_stride, const do
     }
   };
   if (is_a) {
-    // A is diagonal in all fits: a_m = sum_k A_kk Omega_mk^2, and no product (with one, these blocks and those of W were two
+    // A is diagonal in all fits: a_m = sum_k A_kk Omega_mk^2, in fp64, and no product (with one, these blocks and those of W were two
     // waves of blocks for 64 groups)
-    float* diag = reinterpret_cast<float*>(raw);
+    double* diag = reinterpret_cast<double*>(raw);
     const double* A = P + pl.A();
     int off = 0;
     for (int e0 = tid; e0 < d * d; e0 += 8 * PREP_THREADS) {
@@ -143,14 +143,14 @@ prep_kernel(const float* __restrict__ Omega, int64_t omega_head_stride, const do
       for (int q = 0; q < 8; q++) {
         const int e = e0 + q * PREP_THREADS;
         if (e >= d * d) continue;
-        if (e % (d + 1) == 0) diag[e / (d + 1)] = (float)v[q];
+        if (e % (d + 1) == 0) diag[e / (d + 1)] = v[q];
         else if (v[q] != 0.0) off = 1;
       }
     }
     if (!__syncthreads_or(off)) {
       const int m = m0 + (tid >> 1), k0 = (tid & 1) * (d / 2);        // two threads per feature
       if (tid < 2 * PREP_MB) {
-        float s[4] = {};
+        double s[4] = {};
         if (m < M) {
           const float* o = Om + (size_t)m * d + k0;
 #pragma unroll
@@ -158,12 +158,14 @@ prep_kernel(const float* __restrict__ Omega, int64_t omega_head_stride, const do
             float4 w;
             if (aligned) w = *reinterpret_cast<const float4*>(o + k);
             else w = make_float4(o[k], o[k + 1], o[k + 2], o[k + 3]);
-            const float4 a = *reinterpret_cast<const float4*>(diag + k0 + k);
-            s[0] = fmaf(a.x * w.x, w.x, s[0]); s[1] = fmaf(a.y * w.y, w.y, s[1]); s[2] = fmaf(a.z * w.z, w.z, s[2]); s[3] = fmaf(a.w * w.w, w.w, s[3]);
+            const float v[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+            for (int j = 0; j < 4; j++) s[j] = fma(diag[k0 + k + j] * v[j], (double)v[j], s[j]);
           }
         }
-        float a = (s[0] + s[1]) + (s[2] + s[3]);
-        a += __shfl_xor_sync(0xffffffffu, a, 1);
+        double sum = (s[0] + s[1]) + (s[2] + s[3]);
+        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+        const float a = (float)sum;
         if (m < M && (tid & 1) == 0) put_a(m, a);
       }
       return;
