@@ -79,12 +79,15 @@ __device__ __forceinline__ void scalars_of(int g, int side, const double* __rest
   }
 }
 
-// One block = one (group, role, chunk of 128 features).  Roles: W = Omega B (both sides side by side up to d = 64, one side each
-// at d = 128); a = diag(Omega A Omega^T) (the same for both sides, written for both), C, the scalars and the
-// flags of side blockIdx.z + 1 (in front of the blocks of a, which are no shorter for it, these made a launch 3 us longer).  The products run on the tensor cores at fp32 precision (mma3.cuh): 64 groups of 256 x 64 features are 200
-// million multiply-adds, which as fp32 instructions on operands in shared memory took 20 us (bound by the shared-memory reads);
-// 15.6 us now, most of it the latency of loads, products and stores one after the other.
-template <int D>
+// One block = one (group, role, chunk of 128 features).  Roles: W = Omega B of SIDES sides; a = diag(Omega A Omega^T), the same for
+// both sides and written for both; C, the scalars and the flags of side blockIdx.z + 1 (in front of the blocks of a, these made a
+// launch 3 us longer, also with the sum for diagonal A).  The products run on the tensor cores at fp32
+// precision (mma3.cuh): 64 groups of 256 x 64 features are 200 million multiply-adds, which as fp32 instructions on operands in shared
+// memory took 20 us (bound by the shared-memory reads).  What is left is the latency of loads, products and stores one after the
+// other, and of a second wave of blocks where there is one.  A W block takes one side while all blocks are resident at once, two on
+// an SM, and both side by side beyond that (with one side each: 16 groups, M = 256, the two calls of the feature case 212 -> 207 us
+// and the slice 130 -> 124.5 us; 64 groups, the bidirectional step 235.5 -> 241.6 us).
+template <int D, int SIDES>
 __global__ void __launch_bounds__(PREP_THREADS)
 prep_kernel(const float* __restrict__ Omega, int64_t omega_head_stride, const double* __restrict__ params,
             int64_t params_stride, int H, int pool, int M, float* __restrict__ prep, float qk_scale,
@@ -92,7 +95,8 @@ prep_kernel(const float* __restrict__ Omega, int64_t omega_head_stride, const do
   fs_grid_dependency_wait();
   // images != nullptr (d = 64, M = 256 only): the tensor-core path's operand images of this (group, side)
   // are written as well, in the layouts of tc_layout.cuh
-  constexpr int d = D, SIDES = D == 128 ? 1 : 2, NW = 2 / SIDES;       // sides per W block, W roles
+  constexpr int d = D, NW = 2 / SIDES;                                 // W roles
+  static_assert(SIDES * D <= 128, "columns of one product");
   extern __shared__ __align__(16) uint8_t raw[];
   const int g = blockIdx.x, role = blockIdx.y, tid = threadIdx.x;
   if (role == NW + 1) {
@@ -228,19 +232,21 @@ int fs_run_prep_images(fsharp_ctx* ctx, const float* Omega, int64_t omega_head_s
   if (G == 0) return FSHARP_OK;
   if (images != nullptr && (d != tcl::TC_D || M != tcl::TC_M)) return FSHARP_E_SHAPE;
   const int nchunks = (M + PREP_MB - 1) / PREP_MB;
-  const dim3 grid(G, d == 128 ? 4 : 3, nchunks > 2 ? nchunks : 2);
-#define FS_PREP(DD)                                                                                                  \
+  const int nz = nchunks > 2 ? nchunks : 2;
+  const bool apart = d == 128 || (int64_t)G * 4 * nz <= 2 * ctx->sm_count;
+  const dim3 grid(G, apart ? 4 : 3, nz);
+#define FS_PREP(DD, SS)                                                                                              \
   do {                                                                                                               \
-    FS_CUDA_OK(cudaFuncSetAttribute(prep_kernel<DD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mma3::SMEM));        \
+    FS_CUDA_OK(cudaFuncSetAttribute(prep_kernel<DD, SS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mma3::SMEM));    \
     FS_TIME_BEGIN(ctx, FS_K_PREP);                                                                                    \
-    (void)fs_launch_chained(prep_kernel<DD>, grid, dim3(PREP_THREADS), mma3::SMEM, ctx->stream, Omega, omega_head_stride, params, params_stride, H,   \
+    (void)fs_launch_chained(prep_kernel<DD, SS>, grid, dim3(PREP_THREADS), mma3::SMEM, ctx->stream, Omega, omega_head_stride, params, params_stride, H,   \
                                                                pool, M, prep, qk_scale, images, flags, 0.5 * log((double)M), alpha, ctx->d_status);  \
   } while (0)
   switch (d) {
-    case 16: FS_PREP(16); break;
-    case 32: FS_PREP(32); break;
-    case 64: FS_PREP(64); break;
-    case 128: FS_PREP(128); break;
+    case 16: if (apart) FS_PREP(16, 1); else FS_PREP(16, 2); break;
+    case 32: if (apart) FS_PREP(32, 1); else FS_PREP(32, 2); break;
+    case 64: if (apart) FS_PREP(64, 1); else FS_PREP(64, 2); break;
+    case 128: FS_PREP(128, 1); break;
     default: return FSHARP_E_SHAPE;
   }
 #undef FS_PREP
