@@ -1,6 +1,6 @@
-// Closed-form parameter fits (Section 3.1, Section 4.3, Theorems 4.2 and 4.3, Lemma A.1), fp64, one thread block
-// per parameter group.  ADERF and SDERF at d = 64 and 128 go through the chain of fit_wide.cu first; here they are fitted for
-// the groups that the chain flags.  Symmetric eigenproblems, d <= 64: Householder tridiagonalisation, Sturm-count multisection,
+// Closed-form parameter fits (Section 3.1, Section 4.3, Theorems 4.2 and 4.3, Lemma A.1), fp64.  PosRF, GERF and SADERF need no
+// eigenproblem (closed_fit_kernel).  ADERF and SDERF: one thread block per parameter group; at d = 64 and 128 they go through the
+// chain of fit_wide.cu first, and here they are fitted for the groups that the chain flags.  Symmetric eigenproblems, d <= 64: Householder tridiagonalisation, Sturm-count multisection,
 // one vector per eigenvalue from the twisted factorisation, reflectors applied back, one symmetric orthogonalisation;
 // a cyclic Jacobi solver then confirms convergence (or completes it).  d = 128: the Jacobi solver alone.
 // ADERF factors M1 by Cholesky (M1 = L L^T) and solves ONE eigenproblem, of L^T M2 L (Theorem 4.2's U and Sigma^2
@@ -13,19 +13,18 @@ namespace {
 constexpr int FIT_THREADS = 512;
 constexpr int JACOBI_MAX_SWEEPS = 40;
 
+// Every thread gets the result; a barrier for the block's shared memory on both sides.
 __device__ __forceinline__ double block_reduce(double v, double* red, int op /*0 sum, 1 max, 2 min*/) {
   const int tid = threadIdx.x;
+  auto both = [op](double a, double b) { return op == 0 ? a + b : (op == 1 ? fmax(a, b) : fmin(a, b)); };
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = both(v, __shfl_xor_sync(0xffffffffu, v, o));
   __syncthreads();
-  red[tid] = v;
+  if ((tid & 31) == 0) red[tid >> 5] = v;
   __syncthreads();
-  for (int s = FIT_THREADS / 2; s > 0; s >>= 1) {
-    if (tid < s) {
-      double a = red[tid], b = red[tid + s];
-      red[tid] = op == 0 ? a + b : (op == 1 ? fmax(a, b) : fmin(a, b));
-    }
-    __syncthreads();
-  }
-  double r = red[0];
+  double r = red[tid & (FIT_THREADS / 32 - 1)];
+#pragma unroll
+  for (int o = FIT_THREADS / 64; o > 0; o >>= 1) r = both(r, __shfl_xor_sync(0xffffffffu, r, o));
   __syncthreads();
   return r;
 }
@@ -1015,41 +1014,7 @@ __global__ void __launch_bounds__(FIT_THREADS) fit_kernel(FitArgs a) {
   bool violated = false;
   int nsweeps = 0;
 
-  if (a.variant == FSHARP_POSRF || a.variant == FSHARP_GERF) {
-    const double S = t1 + t2 + 2.0 * mm;
-    double A = 0.0;
-    if (a.variant == FSHARP_GERF) { phi = S / d; A = lemma_a1(phi); }
-    const double b = sqrt(1.0 - 4.0 * A);
-    for (int e = tid; e < d * d; e += FIT_THREADS) {
-      double dg = (e / d == e % d) ? 1.0 : 0.0;
-      oA[e] = A * dg; oB1[e] = b * dg; oB2[e] = b * dg; oC1[e] = -0.5 * dg; oC2[e] = -0.5 * dg;
-    }
-    logD = 0.25 * d * log(1.0 - 4.0 * A);
-    obj = d * (log(1.0 - 4.0 * A) - 0.5 * log(1.0 - 8.0 * A)) + (2.0 - 8.0 * A) / (1.0 - 8.0 * A) * S - t1 - t2;
-  } else if (a.variant == FSHARP_SADERF) {
-    // Section 4.3: Psi_ll = (M2_ll / M1_ll)^(1/4), then the GERF fit on {Psi x}, {Psi^-1 y}.
-    double sq = 0.0;
-    for (int i = tid; i < d; i += FIT_THREADS) {
-      double m1 = M1[i * d + i] + rg1, m2 = M2[i * d + i] + rg2;
-      if (!(m1 > 0.0) || !(m2 > 0.0)) { violated = true; m1 = fmax(m1, 1e-300); m2 = fmax(m2, 1e-300); }
-      double psi2 = sqrt(m2 / m1);
-      lam[i] = sqrt(psi2);
-      sq += sqrt(m1 * m2);
-    }
-    sq = block_reduce(sq, red, 0);
-    const double S = 2.0 * sq + 2.0 * mm;
-    phi = S / d;
-    const double A = lemma_a1(phi);
-    const double b = sqrt(1.0 - 4.0 * A);
-    for (int e = tid; e < d * d; e += FIT_THREADS) {
-      int i = e / d;
-      double dg = (i == e % d) ? 1.0 : 0.0, psi = lam[i];
-      oA[e] = A * dg; oB1[e] = b * psi * dg; oB2[e] = b / psi * dg;
-      oC1[e] = -0.5 * psi * psi * dg; oC2[e] = -0.5 / (psi * psi) * dg;
-    }
-    logD = 0.25 * d * log(1.0 - 4.0 * A);
-    obj = d * (log(1.0 - 4.0 * A) - 0.5 * log(1.0 - 8.0 * A)) + (2.0 - 8.0 * A) / (1.0 - 8.0 * A) * S - 2.0 * sq;
-  } else if (a.variant == FSHARP_SDERF) {
+  if (a.variant == FSHARP_SDERF) {
     // Theorem 4.3: N = M1 + mu4 mu5^T + mu5 mu4^T + M2, eigenvalues non-ascending.
     for (int e0 = tid; e0 < d * d; e0 += 8 * FIT_THREADS) {          // global loads in batches ahead of the stores
       double m1[8], m2[8];
@@ -1325,6 +1290,93 @@ __global__ void __launch_bounds__(FIT_THREADS) fit_kernel(FitArgs a) {
   if (violated) atomicExch(a.status, FSHARP_E_CONSTRAINT);
 }
 
+// ---- PosRF, GERF, SADERF: closed forms without an eigenproblem -----------------------------------------------------
+// Eight rows of the parameters per block, d / 8 blocks per group: every block works out the scalars from the diagonals and checks its
+// share of the statistics.  (Inside fit_kernel, one block of 512 threads per group and its shared memory, the 64 x 12 x 512 pooled step took 196.6 us, 188.6 now.)
+constexpr int CF_THREADS = 256, CF_ROWS = 8;
+__global__ void __launch_bounds__(CF_THREADS)
+closed_fit_kernel(const double* __restrict__ stats, double* __restrict__ params, int d, int variant, double ridge, int* __restrict__ status) {
+  fs_grid_dependency_wait();
+  __shared__ double red[4][CF_THREADS / 32], psi_s[128];
+  const int g = blockIdx.x, r0 = blockIdx.y * CF_ROWS, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const StatsLayout sl{d};
+  const ParamsLayout pl{d};
+  const double* st = stats + (size_t)g * sl.total();
+  double* out = params + (size_t)g * pl.total();
+  const double *M1 = st + sl.M(1), *M2 = st + sl.M(2);
+  double m1 = 0.0, m2 = 0.0, m45 = 0.0;
+  if (tid < d) {
+    m1 = M1[tid * d + tid];
+    m2 = M2[tid * d + tid];
+    m45 = st[sl.mu(4) + tid] * st[sl.mu(5) + tid];
+  }
+  bool bad = false, violated = false;
+  for (int e = blockIdx.y * CF_THREADS + tid; e < (int)sl.total(); e += gridDim.y * CF_THREADS) bad |= !isfinite(st[e]);
+  auto sum = [&](double v, int slot) {                  // (a slot is used once)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) red[slot][warp] = v;
+    __syncthreads();
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < CF_THREADS / 32; w++) s += red[slot][w];
+    return s;
+  };
+  double t1 = sum(m1, 0), t2 = sum(m2, 1);
+  const double mm = sum(m45, 2);
+  const double rg1 = ridge * t1 / d, rg2 = ridge * t2 / d;
+  t1 += d * rg1;
+  t2 += d * rg2;
+  double S = t1 + t2 + 2.0 * mm, traces = t1 + t2, A = 0.0, phi = 0.0;
+  if (variant == FSHARP_SADERF) {
+    // Section 4.3: Psi_ll = (M2_ll / M1_ll)^(1/4), then the GERF fit on {Psi x}, {Psi^-1 y}.
+    double sq = 0.0;
+    if (tid < d) {
+      m1 += rg1;
+      m2 += rg2;
+      if (!(m1 > 0.0) || !(m2 > 0.0)) { violated = true; m1 = fmax(m1, 1e-300); m2 = fmax(m2, 1e-300); }
+      psi_s[tid] = sqrt(sqrt(m2 / m1));
+      sq = sqrt(m1 * m2);
+    }
+    sq = sum(sq, 3);
+    S = 2.0 * sq + 2.0 * mm;
+    traces = 2.0 * sq;
+  } else if (tid < d) {
+    psi_s[tid] = 1.0;
+  }
+  __syncthreads();
+  if (variant != FSHARP_POSRF) {
+    phi = S / d;
+    A = lemma_a1(phi);
+  }
+  const double b = sqrt(1.0 - 4.0 * A);
+  for (int e = r0 * d + tid; e < (r0 + CF_ROWS) * d; e += CF_THREADS) {
+    const int i = e / d;
+    const double dg = i == e % d ? 1.0 : 0.0, psi = psi_s[i];
+    out[pl.A() + e] = A * dg;
+    out[pl.B(1) + e] = b * psi * dg;
+    out[pl.B(2) + e] = b / psi * dg;
+    out[pl.C(1) + e] = -0.5 * psi * psi * dg;
+    out[pl.C(2) + e] = -0.5 / (psi * psi) * dg;
+  }
+  if (blockIdx.y == 0 && tid < 8) {
+    double v = 0.0;
+    if (tid == PT_LOGD) v = 0.25 * d * log(1.0 - 4.0 * A);
+    if (tid == PT_OBJ) v = d * (log(1.0 - 4.0 * A) - 0.5 * log(1.0 - 8.0 * A)) + (2.0 - 8.0 * A) / (1.0 - 8.0 * A) * S - traces;
+    if (tid == PT_PHI) v = phi;
+    out[pl.tail() + tid] = v;
+  }
+  if (violated) {
+    atomicExch(status, FSHARP_E_CONSTRAINT);            // (stands whatever the other blocks find)
+  } else if (bad) {
+    for (int old = *status; old != FSHARP_E_CONSTRAINT;) {
+      const int seen = atomicCAS(status, old, FSHARP_E_NONFINITE);
+      if (seen == old) break;
+      old = seen;
+    }
+  }
+}
+
 size_t fit_smem_bytes(int d, int v_in_smem) {
   size_t dbl = (size_t)d * (d + 1) * (v_in_smem ? 4 : 1) + 4 * (size_t)d + FIT_THREADS;
   size_t tables = v_in_smem ? ((size_t)(d - 1) * d + (size_t)(d / 2) * (d / 2 + 1) / 2) * sizeof(uchar2) +
@@ -1352,6 +1404,13 @@ int fs_run_fit(fsharp_ctx* ctx, const double* stats, int G, int d, int variant, 
 
 static int fit_batch(fsharp_ctx* ctx, const double* stats, int G, int d, int variant, double ridge,
                double* params, double* scratch) {
+  if (variant != FSHARP_ADERF && variant != FSHARP_SDERF) {
+    FS_TIME_BEGIN(ctx, FS_K_FIT);
+    (void)fs_launch_chained(closed_fit_kernel, dim3(G, d / CF_ROWS), dim3(CF_THREADS), 0, ctx->stream, stats, params, d, variant, ridge, ctx->d_status);
+    FS_TIME_END(ctx);
+    FS_LAUNCH_CHECK(ctx);
+    return FSHARP_OK;
+  }
   FitArgs a;
   a.stats = stats; a.params = params; a.scratch = scratch; a.d = d; a.variant = variant; a.ridge = ridge;
   a.v_in_smem = d <= 64 ? 1 : 0;
@@ -1360,7 +1419,7 @@ static int fit_batch(fsharp_ctx* ctx, const double* stats, int G, int d, int var
   a.flag_stride = 0;
   // eigenproblems of d = 64 and 128 go through the chain of fit_wide.cu; this kernel then only takes what that chain gave up
   // (the smaller ones fit one block's latency better than six launches)
-  if (d >= 64 && (variant == FSHARP_ADERF || variant == FSHARP_SDERF)) {
+  if (d >= 64) {
     double* wide = scratch + (size_t)G * 5 * d * d;
     FS_TRY(fitw::run(ctx, stats, G, d, variant, ridge, params, wide));
     a.flags = wide + fitw::Layout{d}.scal() + fitw::FS_FLAG;
