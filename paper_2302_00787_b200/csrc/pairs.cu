@@ -19,9 +19,10 @@ __host__ __device__ constexpr int pv_blocks(int columns) { return columns * (col
 __device__ __forceinline__ int frag(int k, int j) {
   return ((pv_blocks(j >> 3) + (k >> 3)) * 32 + (j & 7) * 4 + ((k & 7) >> 1)) * 2 + (k & 1);
 }
-// One block per row k, one thread per column: the serial length is that of one inner product (a single block took
-// 172 us at d = 64).
-__global__ void __launch_bounds__(128)
+// One block per row k; 256 / d threads per column share the inner products' terms, whose loads are in flight together.  (One thread
+// per column, four terms at a time: 30 us at d = 64, a third of a call with few pairs; a single block took 172 us.)
+constexpr int PP_THREADS = 256;
+__global__ void __launch_bounds__(PP_THREADS)
 pairvar_prep_kernel(const double* __restrict__ params, int d, double* __restrict__ ev, int* __restrict__ status) {
   fs_grid_dependency_wait();
   ParamsLayout pl{d};
@@ -30,36 +31,50 @@ pairvar_prep_kernel(const double* __restrict__ params, int d, double* __restrict
   const double* B2 = params + pl.B(2);
   const double* C1 = params + pl.C(1);
   const double* C2 = params + pl.C(2);
-  __shared__ double rinv[128], lg[128];
-  const int k = blockIdx.x, j = threadIdx.x;
-  if (j < d) {
+  __shared__ double rinv[128], lg[128], part_s[3][PP_THREADS];
+  const int k = blockIdx.x, tid = threadIdx.x, j = tid % d, parts = PP_THREADS / d, len = d / parts, l0 = tid / d * len;
+  double c1 = 0.0, c2 = 0.0, a = 0.0;
+  if (tid < d) {
     const double v = 1.0 - 8.0 * A[j * d + j];
+    c1 = C1[k * d + j] + C1[j * d + k];
+    c2 = C2[k * d + j] + C2[j * d + k];
+    a = A[k * d + j];
     rinv[j] = 1.0 / v;
     if (k == 0) lg[j] = log(v);
     if (k == 0 && !(v > 0.0)) atomicExch(status, FSHARP_E_CONSTRAINT);
+    if (k != j && a != 0.0) atomicExch(status, FSHARP_E_CONSTRAINT);
   }
   __syncthreads();
-  if (j < d) {
-    if (k != j && A[k * d + j] != 0.0) atomicExch(status, FSHARP_E_CONSTRAINT);
-    double s1 = 0.0, s2 = 0.0, s12 = 0.0;
-#pragma unroll 4
-    for (int l = 0; l < d; l++) {
-      const double r = rinv[l], b1k = B1[l * d + k] * r, b2j = B2[l * d + j];
-      s1 = fma(b1k, B1[l * d + j], s1);
-      s2 = fma(B2[l * d + k] * r, b2j, s2);
-      s12 = fma(b1k, b2j, s12);
+  double s1 = 0.0, s2 = 0.0, s12 = 0.0;
+#pragma unroll 16
+  for (int l = l0; l < l0 + len; l++) {
+    const double r = rinv[l], b1k = B1[l * d + k] * r, b2j = B2[l * d + j];
+    s1 = fma(b1k, B1[l * d + j], s1);
+    s2 = fma(B2[l * d + k] * r, b2j, s2);
+    s12 = fma(b1k, b2j, s12);
+  }
+  part_s[0][tid] = s1;
+  part_s[1][tid] = s2;
+  part_s[2][tid] = s12;
+  __syncthreads();
+  if (tid < d) {
+    for (int p = 1; p < parts; p++) {
+      s1 += part_s[0][p * d + j];
+      s2 += part_s[1][p * d + j];
+      s12 += part_s[2][p * d + j];
     }
-    const double c1 = C1[k * d + j] + C1[j * d + k], c2 = C2[k * d + j] + C2[j * d + k];
     if (k >> 3 <= j >> 3) {
       ev[frag(k, j)] = k < j ? 2.0 * (c1 + 2.0 * s1) : (k == j ? c1 + 2.0 * s1 : 0.0);
       ev[frag(d + k, d + j)] = k < j ? 2.0 * (c2 + 2.0 * s2) : (k == j ? c2 + 2.0 * s2 : 0.0);
     }
     ev[frag(k, d + j)] = 4.0 * s12;
   }
-  if (k == 0 && j == 0) {
+  if (k == 0 && tid < 32) {
     double ld = 0.0;
-    for (int l = 0; l < d; l++) ld += lg[l];
-    ev[64 * pv_blocks(d / 4)] = 4.0 * params[pl.tail() + PT_LOGD] - 0.5 * ld;
+    for (int l = tid; l < d; l += 32) ld += lg[l];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ld += __shfl_xor_sync(0xffffffffu, ld, o);
+    if (tid == 0) ev[64 * pv_blocks(d / 4)] = 4.0 * params[pl.tail() + PT_LOGD] - 0.5 * ld;
   }
 }
 
@@ -244,7 +259,7 @@ int fs_run_pairs(fsharp_ctx* ctx, const float* X, const float* Y, const float* O
   if (npairs == 0) return FSHARP_OK;
   if (var_cf) {
     FS_TIME_BEGIN(ctx, FS_K_PAIRVAR_PREP);
-    (void)fs_launch_chained(pairvar_prep_kernel, dim3(d), dim3(128), 0, ctx->stream, params, d, ev, ctx->d_status);
+    (void)fs_launch_chained(pairvar_prep_kernel, dim3(d), dim3(PP_THREADS), 0, ctx->stream, params, d, ev, ctx->d_status);
     FS_TIME_END(ctx);
     FS_LAUNCH_CHECK(ctx);
     if (pooled) FS_CUDA_OK(cudaMemsetAsync(pooled, 0, 2 * sizeof(double), ctx->stream));
