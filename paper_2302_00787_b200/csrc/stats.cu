@@ -2,7 +2,7 @@
 // mu4 = mean x, mu5 = mean y.
 //
 // One thread block accumulates the Gram matrix of a slice of tokens of one
-// (batch, head, side): products in fp32 over 128 tokens, then folded into fp64
+// (batch, head, side): products in fp32 over 64 tokens, then folded into fp64
 // registers; slices are combined with fp64 atomics.
 #include "common.cuh"
 
@@ -15,7 +15,7 @@ namespace {
 constexpr int ST_THREADS = 256;
 template <int D> struct StGeo {
   static constexpr int R = D == 128 ? 8 : 4, TPG = (D / R) * (D / R), NG = ST_THREADS / TPG, TT = 4096 / D;      // tokens per tile
-  static constexpr int FLUSH = 128 / (TT / NG);      // tiles between fp32 -> fp64 folds: 128 tokens of a thread
+  static constexpr int FLUSH = 64 / (TT / NG);       // tiles between fp32 -> fp64 folds: 64 tokens of a thread
   static constexpr int LD = D + 4;
 };
 
@@ -153,7 +153,8 @@ int launch_stats(fsharp_ctx* ctx, const void* Q, const void* K, const fsharp_dim
                  double* stats) {
   const int BH = dm->B * dm->H;
   const int Lmax = dm->Lq > dm->Lk ? dm->Lq : dm->Lk;
-  int nsplit = (4 * ctx->sm_count + 2 * BH - 1) / (2 * BH);
+  // as many blocks as are resident at once (two on an SM, one at d = 128): every further one is another d^2 fp64 atomics
+  int nsplit = (dm->d == 128 ? 1 : 2) * ctx->sm_count / (2 * BH);
   int maxsplit = (Lmax + 127) / 128;
   if (nsplit > maxsplit) nsplit = maxsplit;
   if (nsplit < 1) nsplit = 1;
