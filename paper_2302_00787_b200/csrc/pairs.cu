@@ -92,7 +92,8 @@ __device__ __forceinline__ void dmma(double (&c)[2], double a, double b) {
 // in which a lane's A values of an 8-block, z[2 t] and z[2 t + 1] (t = lane % 4), belong to the columns of its part of the product,
 // so that z^T (F z) needs no other values of z.  The warps go their own ways (loads of one run under the products of another),
 // the pooling included.  d = 128: half of F fits, so two launches, the first of which leaves its share of the exponent in var.
-// (Scalar multiply-adds, x and y as doubles in shared memory and F through L1, which it did not fit: 1.57 ms for 2^20 pairs, d = 64, R = 32.)
+// (Scalar multiply-adds, x and y as doubles in shared memory and F through L1, which it did not fit: 1.57 ms for 2^20 pairs, d = 64, R = 32; 0.69 ms now, 0.52 at
+// the rate of the fp64 units.  16 warps of eight pairs each instead of eight of sixteen: the same.)
 template <int D> struct PvGeo {
   static constexpr int NB = D / 4, MT = D == 128 ? 1 : 2, P = 64 * MT, SPLIT = D == 128 ? 23 : NB;    // block columns; those of the first launch
   static constexpr int BLOCKS0 = pv_blocks(SPLIT), BLOCKS1 = pv_blocks(NB) - BLOCKS0;

@@ -9,7 +9,7 @@
 // memory: the epilogue takes chunk c while chunk c + 1 is multiplied.  A chunk's sum is added in fp32 to the running one, which
 // the epilogue warps keep in registers and write, rounded to bf16, in front of every chunk: nothing else leaves the block.  (Sums
 // of single chunks written in fp32, 505 us for 1 x 16 x 65536 tokens, M = 512, chunks of 256, and scanned by a kernel of its own,
-// 265 us, moved 2.2 GB that never had to.)
+// 265 us, moved 2.2 GB that never had to; the two launches take 139 and 292 us.)
 // Segments: as many as there are SMs for all (segment, block, (batch, head)); where there is more than one, a first launch
 // (EMIT = false) adds up the earlier ones, cut finer so that it fills the chip too, and the scan kernel turns the pieces' sums into
 // what precedes every piece.
