@@ -390,15 +390,13 @@ int backward_t(fsharp_ctx* ctx, const void* Qv, const void* Kv, const void* Vv, 
 
   const feat3::Task tasks[2] = {{K, ak, Lk, 2, FSHARP_STAB_GROUP, rowck, gmax, phiK, nullptr, lsk, feat3::LIFT},
                                 {Q, aq, Lq, 1, FSHARP_STAB_ROW, rowcq, nullptr, phiQ, nullptr, lsq, feat3::LIFT}};
-  FS_TRY(feat3::run(ctx, tasks, 2, dtype, B, H, d, M, dm->pool, prep, qk_scale, img));
+  // (KV and Rt are neighbours, with less than 256 bytes between them)
+  FS_TRY(feat3::run(ctx, tasks, 2, dtype, B, H, d, M, dm->pool, prep, qk_scale, img, KV, causal ? 0 : (size_t)(Rt - KV) + (size_t)BH * elems));
   // sums over tokens: the total (bidirectional), or one per chunk turned into the sum over earlier / later chunks (causal)
   auto sums = [&](auto from_g, const float* F, int L, float* out, int reverse, int flip) -> int {
     constexpr bool FG = decltype(from_g)::value;
     int slen = C, nsl = nch;
-    if (!causal) {
-      nsl = fs_token_slices(ctx, BH * mt * ctiles, BH, L, &slen);
-      FS_CUDA_OK(cudaMemsetAsync(out, 0, (size_t)BH * elems * sizeof(float), ctx->stream));
-    }
+    if (!causal) nsl = fs_token_slices(ctx, BH * mt * ctiles, BH, L, &slen);
     FS_TRY(mma3::launch(ctx, FS_K_BWD_STATE, state_kernel<T, FG>, dim3(mt, ctiles, BH * nsl), F, V, av, G, H, L, M, dv, slen, nsl,
                         causal ? 1 : 0, out, flip, status));
     if (causal) {

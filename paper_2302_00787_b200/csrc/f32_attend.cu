@@ -103,12 +103,12 @@ int attend_t(fsharp_ctx* ctx, const void* Q, const void* K, const void* V, const
   uint8_t* img = ws->take<uint8_t>(feat3::image_bytes(fs_groups(dm), d, M, 2));
   const feat3::Task tasks[2] = {{K, ak, Lk, 2, FSHARP_STAB_GROUP, rowc, gmax, phiK, phiK16, lsk, feat3::LIFT},
                                 {Q, aq, Lq, 1, FSHARP_STAB_ROW, rowcq, nullptr, phiQ, phiQ16, lsq, feat3::LIFT}};
-  FS_TRY(feat3::run(ctx, tasks, 2, sizeof(T) == 2 ? FSHARP_BF16 : FSHARP_F32, B, H, d, M, dm->pool, prep, qk_scale, img));
+  float* KV = causal ? nullptr : ws->take<float>((size_t)BH * M * NP);
+  FS_TRY(feat3::run(ctx, tasks, 2, sizeof(T) == 2 ? FSHARP_BF16 : FSHARP_F32, B, H, d, M, dm->pool, prep, qk_scale, img, KV,
+                    causal ? 0 : (size_t)BH * M * NP));
   const dim3 gout((Lq + mma3::ROWS - 1) / mma3::ROWS, ctiles, BH);
   const dim3 gkv((M + mma3::ROWS - 1) / mma3::ROWS, ctiles, 1);
   if (!causal) {
-    float* KV = ws->take<float>((size_t)BH * M * NP);
-    FS_CUDA_OK(cudaMemsetAsync(KV, 0, (size_t)BH * M * NP * sizeof(float), ctx->stream));
     int slen = 0;
     const int nsl = fs_token_slices(ctx, BH * gkv.x * gkv.y, BH, Lk, &slen);
     FS_TRY(mma3::launch(ctx, FS_K_KV, state_kernel<T, false>, dim3(gkv.x, gkv.y, BH * nsl), phiK, (const T*)V, av, nullptr, H, Lk, M, dv, slen, nsl, 0,

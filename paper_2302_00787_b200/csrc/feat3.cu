@@ -79,6 +79,8 @@ struct Args {
   double quad;            // log2e (qk_scale / pow2)^2
   bool own_terms;         // the feature kernels compute the quadratic terms of groups with C = gamma I themselves
   bool row_init;          // a pass raises logscale from -inf
+  float4* zero;           // cleared by the kernel of the quadratic terms
+  size_t zero4;
   int* status;
 };
 
@@ -250,6 +252,7 @@ rowterm3_kernel(const __grid_constant__ Args a) {
   PrepLayout pr{D, a.M};
   const int total = a.first[2];
   const int w0 = (int)((int64_t)total * blockIdx.x / gridDim.x), w1 = (int)((int64_t)total * (blockIdx.x + 1) / gridDim.x);
+  for (size_t i = blockIdx.x * (size_t)RT_THREADS + tid; i < a.zero4; i += (size_t)gridDim.x * RT_THREADS) a.zero[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   if (a.own_terms) {
     // nothing but the start values where all groups of this block have C = gamma I
     bool all = true;
@@ -872,6 +875,7 @@ int run_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, int g
   if (ntasks == 1 || (BP == 3 && (D < 128 || items <= ctx->sm_count))) return launch_t<T, D, BP>(ctx, a, tasks, ntasks, BH, groups, qk_scale, img);
   for (int i = 0; i < ntasks; i++) {
     FS_TRY((launch_t<T, D, BP>(ctx, a, tasks + i, 1, BH, groups, qk_scale, img)));
+    a.zero4 = 0;
   }
   return FSHARP_OK;
 }
@@ -886,8 +890,10 @@ size_t feat3::image_bytes(int groups, int d, int M, int ntasks) {
 }
 
 int feat3::run(fsharp_ctx* ctx, const Task* tasks, int ntasks, int dtype, int B, int H, int d, int M, int pool, const float* prep,
-               float qk_scale, uint8_t* img) {
+               float qk_scale, uint8_t* img, float* zero, size_t zero_floats) {
   Args a{};
+  a.zero = reinterpret_cast<float4*>(zero);
+  a.zero4 = zero_floats / 4;
   a.H = H; a.M = M; a.pool = pool; a.prep = prep; a.status = ctx->d_status;
   int e = 0;
   (void)frexp((double)qk_scale, &e);

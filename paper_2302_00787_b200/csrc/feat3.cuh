@@ -27,8 +27,10 @@ struct Task {
 size_t image_bytes(int groups, int d, int M, int ntasks);
 
 // Images of W (img, 16-byte aligned; nullptr: the blocks convert W themselves), quadratic terms, largest exponents where a
-// shift needs them, then the features of all tasks.  Two tasks are of different sides.
+// shift needs them, then the features of all tasks.  Two tasks are of different sides.  zero (16-byte aligned, a multiple of four
+// floats): cleared on the way, for sums that later kernels of the chain add up (a memset between them would end the chain of
+// programmatic dependents).
 int run(fsharp_ctx* ctx, const Task* tasks, int ntasks, int dtype, int B, int H, int d, int M, int pool, const float* prep,
-        float qk_scale, uint8_t* img);
+        float qk_scale, uint8_t* img, float* zero = nullptr, size_t zero_floats = 0);
 
 }  // namespace feat3
