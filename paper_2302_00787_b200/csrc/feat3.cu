@@ -414,11 +414,11 @@ rowterm3_kernel(const __grid_constant__ Args a) {
 constexpr int FT_AHEAD = 4;                                        // tiles pulled into L2 ahead of the two buffers (BP = 2)
 constexpr int FT_STAGE0 = 8, FT_MMA = 12, FT_THREADS = 416;
 struct FtMisc {
-  uint64_t a_full[2], a_free[2], t_full[2], t_free[2], max_full[2], w_full;
+  uint64_t a_full[2], a_free[2], t_full[2], t_free[2], max_full[2][2], w_full;
   uint32_t tmem_base;
   int abort_flag;
 };
-struct FtMax { float row[2][2][TILE]; };       // PAIR: the other block's maxima, two places per warpgroup
+struct FtMax { float row[2][2][TILE]; };       // PAIR: the other block's maxima, two places (and barriers) per warpgroup
 template <typename T, int D, int BP, bool WRITE> struct FtGeo : Geo<T, D> {
   static_assert(BP == 3 || Geo<T, D>::AP == 1, "two parts of W: bf16 tokens");
   static constexpr int MB = WGeo<D, BP>::MB;
@@ -466,7 +466,10 @@ feat3_kernel(const __grid_constant__ Args a) {
     for (int i = 0; i < 2; i++) {
       mbar_init(&misc->a_full[i], OUT16 ? 1 : 4);
       mbar_init(&misc->a_free[i], terms ? 5 : 1);
-      if (PAIR) mbar_init(&misc->max_full[i], 4);
+      if (PAIR) {
+        mbar_init(&misc->max_full[i][0], 4);
+        mbar_init(&misc->max_full[i][1], 4);
+      }
       mbar_init(&misc->t_full[i], 1);
       mbar_init(&misc->t_free[i], 4);
     }
@@ -694,13 +697,16 @@ feat3_kernel(const __grid_constant__ Args a) {
           }
           mx = fmaxf(mx, my);
           if (PAIR) {
-            // (the other block is at most one of this warpgroup's tiles ahead: its next maxima need this one's)
+            // The other block's warps can be one of this warpgroup's tiles ahead, no more: past it they wait for warps here.  So
+            // consecutive tiles have places and barriers of their own (with one barrier, the next tile's four arrivals could
+            // complete a second phase before a slow warp here had seen the first, and its wait for that parity would not end).
             const int k = n >> 1, row = (warp & 3) * 32 + lane;
             float* place = &maxima->row[wg][k & 1][row];
+            uint64_t* bar = &misc->max_full[wg][k & 1];
             store_cluster(map_cluster(smem_u32(place), rank ^ 1), mx);
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(map_cluster(smem_u32(&misc->max_full[wg]), rank ^ 1));
-            mbar_wait_cluster(&misc->max_full[wg], k & 1, &misc->abort_flag, a.status);
+            if (lane == 0) mbar_arrive_cluster(map_cluster(smem_u32(bar), rank ^ 1));
+            mbar_wait_cluster(bar, (k >> 1) & 1, &misc->abort_flag, a.status);
             __syncwarp();
             mx = fmaxf(mx, *reinterpret_cast<volatile float*>(place));
           }

@@ -40,3 +40,28 @@ def test_chain_against_fp32_kernels(B, H, L, M, chunk, variant):
             assert rel_err(Y[b, h], ref[b, h]) < 7 * 2.0 ** -9
     # the first token sees itself alone
     assert np.abs(Y[:, :, 0] - host(V)[:, :, 0]).max() < 1e-2 * np.abs(host(V)[:, :, 0]).max()
+
+
+def row_bound(ctx, Q, K, V, Om, pr, at):
+    """What the chain's roundings may move every output value by, against the fp32 tensors' result.  Numerator and denominator are sums
+    whose terms carry three roundings to bf16 each (phi(Q); phi(K); the score or the running sum), the quotient one more: to first
+    order 7 x 2^-9 of the attention applied to |V|.  Second order and the exponents from two parts of W (16 bits): one more."""
+    return 8 * 2.0 ** -9 * host(ctx.fsharp_attend(Q.float(), K.float(), V.float().abs(), Om, pr, **at))
+
+
+@pytest.mark.parametrize("M,variant", [(512, "sderf"), (384, "aderf")])
+def test_pairs_of_blocks_over_many_tiles(M, variant):
+    """Two blocks of features, 16 (batch, head)s of 40 token tiles: a pair of blocks exchanges its rows' maxima over eight or nine
+    tiles, four or five per warpgroup, so that every place and barrier of the exchange is used again; always the same bits."""
+    ctx = fb.Context(0)
+    w = wl.Workload("chain", 2, 8, 5120, 128, 128, M, "bf16", variant, True, 256, "orthogonal", outlier_frac=0.05, seed=3)
+    Q, K, V = (dev(t, "bf16") for t in wl.make_qkv(w))
+    Om = dev(wl.make_omega(w))
+    _, pr = gpu_fit(ctx, Q, K, 128, variant)
+    at = dict(causal=True, chunk=256)
+    Y = ctx.fsharp_attend(Q, K, V, Om, pr, **at)
+    ref = host(ctx.fsharp_attend(Q.float(), K.float(), V.float(), Om, pr, **at))
+    assert (np.abs(host(Y) - ref) <= row_bound(ctx, Q, K, V, Om, pr, at)).all()
+    for _ in range(100):
+        assert torch.equal(ctx.fsharp_attend(Q, K, V, Om, pr, **at), Y)
+    assert ctx.status() == 0
