@@ -418,7 +418,10 @@ struct FtMisc {
   uint32_t tmem_base;
   int abort_flag;
 };
-struct FtMax { float row[2][2][TILE]; };       // PAIR: the other block's maxima, two places (and barriers) per warpgroup
+struct FtMax {
+  float row[2][2][TILE];      // PAIR: the other block's maxima, two places (and barriers) per warpgroup
+  float term[2][TILE];        // x^T C x of the warpgroups' tiles
+};
 template <typename T, int D, int BP, bool WRITE> struct FtGeo : Geo<T, D> {
   static_assert(BP == 3 || Geo<T, D>::AP == 1, "two parts of W: bf16 tokens");
   static constexpr int MB = WGeo<D, BP>::MB;
@@ -646,6 +649,9 @@ feat3_kernel(const __grid_constant__ Args a) {
             bad |= in && !isfinite(c);
             ci += c;
             if (!WRITE && in && mblk == 0) t.rowc[at] = c;
+            // Stored before the tile is handed back: the store needs every value of the row.  Nothing else uses c on this side of
+            // the arrival, behind which the last loads could still be on their way out of shared memory when the next tile lands.
+            *const_cast<volatile float*>(&maxima->term[wg][row]) = c;
           } else {
             ci += in ? t.rowc[at] : 0.f;
           }

@@ -49,10 +49,11 @@ def row_bound(ctx, Q, K, V, Om, pr, at):
     return 8 * 2.0 ** -9 * host(ctx.fsharp_attend(Q.float(), K.float(), V.float().abs(), Om, pr, **at))
 
 
-@pytest.mark.parametrize("M,variant", [(512, "sderf"), (384, "aderf")])
-def test_pairs_of_blocks_over_many_tiles(M, variant):
-    """Two blocks of features, 16 (batch, head)s of 40 token tiles: a pair of blocks exchanges its rows' maxima over eight or nine
-    tiles, four or five per warpgroup, so that every place and barrier of the exchange is used again; always the same bits."""
+@pytest.mark.parametrize("M,variant", [(512, "sderf"), (384, "aderf"), (256, "sderf")])
+def test_blocks_over_many_tiles(M, variant):
+    """16 (batch, head)s of 40 token tiles.  Two blocks of features: a pair of blocks exchanges its rows' maxima over eight or nine
+    tiles, four or five per warpgroup, so that every place and barrier of the exchange is used again.  C = gamma I: the epilogue's reads
+    of a tile are done before the next one is copied over it.  Always the same bits."""
     ctx = fb.Context(0)
     w = wl.Workload("chain", 2, 8, 5120, 128, 128, M, "bf16", variant, True, 256, "orthogonal", outlier_frac=0.05, seed=3)
     Q, K, V = (dev(t, "bf16") for t in wl.make_qkv(w))
