@@ -1291,14 +1291,15 @@ __global__ void __launch_bounds__(FIT_THREADS) fit_kernel(FitArgs a) {
 }
 
 // ---- PosRF, GERF, SADERF: closed forms without an eigenproblem -----------------------------------------------------
-// Eight rows of the parameters per block, d / 8 blocks per group: every block works out the scalars from the diagonals and checks its
+// A share of the rows of the parameters per block: every block works out the scalars from the diagonals and checks its
 // share of the statistics.  (Inside fit_kernel, one block of 512 threads per group and its shared memory, the 64 x 12 x 512 pooled step took 196.6 us, 188.6 now.)
 constexpr int CF_THREADS = 256, CF_ROWS = 8;
+template <int d>
 __global__ void __launch_bounds__(CF_THREADS)
-closed_fit_kernel(const double* __restrict__ stats, double* __restrict__ params, int d, int variant, double ridge, int* __restrict__ status) {
+closed_fit_kernel(const double* __restrict__ stats, double* __restrict__ params, int variant, double ridge, int* __restrict__ status) {
   fs_grid_dependency_wait();
   __shared__ double red[4][CF_THREADS / 32], psi_s[128];
-  const int g = blockIdx.x, r0 = blockIdx.y * CF_ROWS, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rows = d / gridDim.y, g = blockIdx.x, r0 = blockIdx.y * rows, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const StatsLayout sl{d};
   const ParamsLayout pl{d};
   const double* st = stats + (size_t)g * sl.total();
@@ -1311,6 +1312,7 @@ closed_fit_kernel(const double* __restrict__ stats, double* __restrict__ params,
     m45 = st[sl.mu(4) + tid] * st[sl.mu(5) + tid];
   }
   bool bad = false, violated = false;
+#pragma unroll 8
   for (int e = blockIdx.y * CF_THREADS + tid; e < (int)sl.total(); e += gridDim.y * CF_THREADS) bad |= !isfinite(st[e]);
   auto sum = [&](double v, int slot) {                  // (a slot is used once)
 #pragma unroll
@@ -1350,7 +1352,7 @@ closed_fit_kernel(const double* __restrict__ stats, double* __restrict__ params,
     A = lemma_a1(phi);
   }
   const double b = sqrt(1.0 - 4.0 * A);
-  for (int e = r0 * d + tid; e < (r0 + CF_ROWS) * d; e += CF_THREADS) {
+  for (int e = r0 * d + tid; e < (r0 + rows) * d; e += CF_THREADS) {
     const int i = e / d;
     const double dg = i == e % d ? 1.0 : 0.0, psi = psi_s[i];
     out[pl.A() + e] = A * dg;
@@ -1375,6 +1377,22 @@ closed_fit_kernel(const double* __restrict__ stats, double* __restrict__ params,
       old = seen;
     }
   }
+}
+
+// Blocks per group: eight rows each while all blocks are resident early, two on an SM; beyond that at least 1024 values of each
+// matrix, since every block repeats the scalars' work, and all of a group where that still leaves four blocks per SM.  (SADERF, us, per call.
+// Eight rows at every number of groups, and the statistics scanned one load at a time: d = 64, 2500 groups 303, d = 128, 500 groups 184; one block
+// of fit_kernel per group 204 and 102; now 107 and 86.  100 groups, d = 64: 8.1 with eight rows, 6.6 with sixteen, 7.1 with all.)
+int launch_closed_fit(fsharp_ctx* ctx, const double* stats, int G, int d, int variant, double ridge, double* params) {
+  int per = d / CF_ROWS;
+  const int64_t sm = ctx->sm_count;
+  while (per > 1 && (int64_t)G * per > 2 * sm && (d * d / per < 1024 || (int64_t)G * per >= 8 * sm)) per /= 2;
+  const auto kernel = d == 16 ? closed_fit_kernel<16> : d == 32 ? closed_fit_kernel<32> : d == 64 ? closed_fit_kernel<64> : closed_fit_kernel<128>;
+  FS_TIME_BEGIN(ctx, FS_K_FIT);
+  (void)fs_launch_chained(kernel, dim3(G, per), dim3(CF_THREADS), 0, ctx->stream, stats, params, variant, ridge, ctx->d_status);
+  FS_TIME_END(ctx);
+  FS_LAUNCH_CHECK(ctx);
+  return FSHARP_OK;
 }
 
 size_t fit_smem_bytes(int d, int v_in_smem) {
@@ -1404,13 +1422,7 @@ int fs_run_fit(fsharp_ctx* ctx, const double* stats, int G, int d, int variant, 
 
 static int fit_batch(fsharp_ctx* ctx, const double* stats, int G, int d, int variant, double ridge,
                double* params, double* scratch) {
-  if (variant != FSHARP_ADERF && variant != FSHARP_SDERF) {
-    FS_TIME_BEGIN(ctx, FS_K_FIT);
-    (void)fs_launch_chained(closed_fit_kernel, dim3(G, d / CF_ROWS), dim3(CF_THREADS), 0, ctx->stream, stats, params, d, variant, ridge, ctx->d_status);
-    FS_TIME_END(ctx);
-    FS_LAUNCH_CHECK(ctx);
-    return FSHARP_OK;
-  }
+  if (variant != FSHARP_ADERF && variant != FSHARP_SDERF) return launch_closed_fit(ctx, stats, G, d, variant, ridge, params);
   FitArgs a;
   a.stats = stats; a.params = params; a.scratch = scratch; a.d = d; a.variant = variant; a.ridge = ridge;
   a.v_in_smem = d <= 64 ? 1 : 0;

@@ -60,3 +60,21 @@ def test_statistics_on_any_8_byte_boundary(d, variant):
     assert shifted.data_ptr() % 16 == 8
     assert torch.equal(ctx.fsharp_fit_params(shifted, d, variant), want)
     assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("variant", ["posrf", "gerf", "saderf"])
+@pytest.mark.parametrize("d,G", [(16, 201), (32, 99), (32, 600), (64, 102), (64, 300), (64, 2500), (128, 150), (128, 500), (128, 1200)])
+def test_closed_forms_however_many_groups(d, G, variant):
+    """The closed forms share a group's rows out to fewer blocks the more groups there are: the same bits as group by group; a
+    violated constraint in the last group is reported whichever block finds it."""
+    rng = np.random.default_rng(d)
+    X = rng.standard_normal((3, 4 * d, d)) / d ** 0.5
+    blob = torch.from_numpy(np.stack([np.concatenate([(x.T @ x / 8).ravel(), (x.T @ x / 4).ravel(), 0.1 * x[0], 0.1 * x[1]]) for x in X])).cuda()
+    ctx = fb.Context(0)
+    want = torch.cat([ctx.fsharp_fit_params(blob[g:g + 1], d, variant) for g in range(3)])
+    many = blob.repeat((G + 2) // 3, 1)[:G].contiguous()
+    assert torch.equal(ctx.fsharp_fit_params(many, d, variant), want.repeat((G + 2) // 3, 1)[:G])
+    assert ctx.status() == 0
+    many[G - 1, d * d - 1] = float("nan")                  # (a diagonal entry: SADERF's M1 is no longer positive there)
+    ctx.fsharp_fit_params(many, d, variant)
+    assert ctx.status() == (-6 if variant == "saderf" else -7)
