@@ -78,7 +78,7 @@ int fsharp_fit_params(fsharp_ctx* ctx, const double* stats, int G, int d, int va
   if (!(ridge >= 0.0)) return FSHARP_E_BADARG;
   if (G == 0) return FSHARP_OK;
   FS_CUDA_OK(cudaSetDevice(ctx->device));
-  size_t need = ws_round(fs_fit_scratch_doubles(G, d) * sizeof(double));
+  size_t need = ws_round(fs_fit_scratch_doubles(G, d, variant) * sizeof(double));
   FS_TRY(fs_ws_reserve(ctx, need));
   return fs_run_fit(ctx, stats, G, d, variant, ridge, params, reinterpret_cast<double*>(ctx->ws));
 }
@@ -342,7 +342,7 @@ int fsharp_forward_host(fsharp_ctx* ctx, const void* Q, const void* K, const voi
       const size_t whole = fs_tc_attend_scratch_bytes(ctx, &dd, causal, chunk), part = fs_tc_attend_scratch_bytes(ctx, &one, causal, chunk);
       b = whole > part ? whole : part;
     }
-    size_t c = ws_round(fs_fit_scratch_doubles(G, dd.d) * 8);
+    size_t c = ws_round(fs_fit_scratch_doubles(G, dd.d, variant) * 8);
     size_t use = ctx->impl == FSHARP_IMPL_SIMT ? a : (b ? b : a);
     inner += use > c ? use : c;
   }

@@ -234,7 +234,7 @@ int fs_tc_stats_supported(const void* Q, const void* K, const fsharp_dims* dm, i
 int fs_tc_stats(fsharp_ctx* ctx, const void* Q, const void* K, const fsharp_dims* dm, float qk_scale, double* stats);
 int fs_run_fit(fsharp_ctx* ctx, const double* stats, int G, int d, int variant, double ridge,
                double* params, double* scratch);
-size_t fs_fit_scratch_doubles(int G, int d);
+size_t fs_fit_scratch_doubles(int G, int d, int variant);
 // params_stride: doubles between the blobs of two groups (0 = every group reads the same blob).  alpha: added to the diagonals of C1
 // and C2 (exp(alpha |x|^2) f(w, x) is the DERF with C + alpha I: Section 2.3's reduction of K^(alpha) to K^(0)).
 int fs_run_prep(fsharp_ctx* ctx, const float* Omega, int64_t omega_head_stride, const double* params,

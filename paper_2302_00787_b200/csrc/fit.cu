@@ -1406,13 +1406,18 @@ size_t fit_smem_bytes(int d, int v_in_smem) {
 
 // From d = 64 on the chain keeps eight more matrices per group than the one-block kernel does: groups go through in batches of
 // this many (fourteen blocks per SM), so that a call with very many of them needs no more memory for it (d = 128: 3.6 GB).
+// The closed forms need none, and go through at once.
 constexpr int FIT_BATCH = 2048;
 
+static bool closed_form(int variant) { return variant != FSHARP_ADERF && variant != FSHARP_SDERF; }
 static size_t group_doubles(int d) { return 5 * (size_t)d * d + (d >= 64 ? fitw::Layout{d}.total() : 0); }
-size_t fs_fit_scratch_doubles(int G, int d) { return (size_t)(d >= 64 && G > FIT_BATCH ? FIT_BATCH : G) * group_doubles(d); }
+size_t fs_fit_scratch_doubles(int G, int d, int variant) {
+  return closed_form(variant) ? 0 : (size_t)(d >= 64 && G > FIT_BATCH ? FIT_BATCH : G) * group_doubles(d);
+}
 
 static int fit_batch(fsharp_ctx* ctx, const double* stats, int G, int d, int variant, double ridge, double* params, double* scratch);
 int fs_run_fit(fsharp_ctx* ctx, const double* stats, int G, int d, int variant, double ridge, double* params, double* scratch) {
+  if (closed_form(variant)) return launch_closed_fit(ctx, stats, G, d, variant, ridge, params);
   const int batch = d >= 64 ? FIT_BATCH : G;
   for (int g = 0; g < G; g += batch)
     FS_TRY(fit_batch(ctx, stats + (size_t)g * StatsLayout{d}.total(), G - g < batch ? G - g : batch, d, variant, ridge,
@@ -1422,7 +1427,6 @@ int fs_run_fit(fsharp_ctx* ctx, const double* stats, int G, int d, int variant, 
 
 static int fit_batch(fsharp_ctx* ctx, const double* stats, int G, int d, int variant, double ridge,
                double* params, double* scratch) {
-  if (variant != FSHARP_ADERF && variant != FSHARP_SDERF) return launch_closed_fit(ctx, stats, G, d, variant, ridge, params);
   FitArgs a;
   a.stats = stats; a.params = params; a.scratch = scratch; a.d = d; a.variant = variant; a.ridge = ridge;
   a.v_in_smem = d <= 64 ? 1 : 0;

@@ -25,7 +25,8 @@ def test_fit_of_many_groups(variant):
     want = ctx.fsharp_fit_params(blob, d, variant)
     pr = ctx.fsharp_fit_params(blob.repeat(G // 3, 1), d, variant)
     assert ctx.status() == 0 and torch.equal(pr, want.repeat(G // 3, 1))
-    assert ctx.workspace_bytes() < 1.2e9                  # 2048 groups of 13 matrices, an eighth in reserve: 1.0e9
+    # 2048 groups of 13 matrices, an eighth in reserve: 1.0e9; nothing for a closed form but what a context starts with
+    assert ctx.workspace_bytes() < 1.2e9 if variant in ("aderf", "sderf") else ctx.workspace_bytes() == fb.Context(0).workspace_bytes()
 
 
 def test_features_of_many_groups():
