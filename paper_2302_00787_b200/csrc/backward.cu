@@ -199,6 +199,7 @@ bwd_dfeat_kernel(const float* __restrict__ phiQ, const float* __restrict__ phiK,
   blk.begin(smem, min(ROWS, M - m0), NP + (q.causal ? C : 0), status);
   const float* S = St + ((int64_t)bh * q.nch + chunk) * M * NP + (int64_t)m0 * NP;
   const float* GV = q.causal ? gv + ((int64_t)bh * q.nch + chunk) * C * C : nullptr;
+  mma3::prefetch_rows((SIDE == 1 ? phiQ : phiK) + ((int64_t)bh * L + i0) * M + m0, 4LL * M, min(ROWS, L - i0), 4LL * min(ROWS, M - m0));
   if (SIDE == 1) {
     const float* Gb = G + ((int64_t)bh * L + i0) * NP;
     blk.template segment<true, 3, true, 3>(
@@ -317,6 +318,7 @@ bwd_dx_kernel(const float* __restrict__ E, const float* __restrict__ rs, int mti
   }
   __syncthreads();
   const float* Eb = E + ((int64_t)bh * L + i0) * M;
+  mma3::prefetch_rows(Eb, 4LL * M, min(ROWS, L - i0), 4LL * M);
   const T* Xb = X + b * ax.sb + h * ax.sh + (int64_t)i0 * ax.sl;
   blk.template segment<true, 3, false, 3>(
       M, [&](int r, int k, Piece<3>& p) { if (i0 + r < L) p.load(Eb + (int64_t)r * M + k); else p.zero(); },

@@ -76,8 +76,20 @@ template <> struct PartsOf<__nv_bfloat16> { static constexpr int N = 1; };
 
 // Which unit (z coordinate) a block takes.  Kernels of a chain walk the units up and down in turn: the matrices that one leaves behind
 // are larger than the L2, and what it touched last is still there for the next one (causal training step of 2 x 12 x 4096 tokens: 1223 -> 1208 us).
-// (A block's rows asked into L2 ahead of its slices: 18 us more, the first slices wait behind all of them.)
 __device__ __forceinline__ int unit_of(int flip) { return flip ? gridDim.z - 1 - blockIdx.z : blockIdx.z; }
+
+// rows of `bytes` contiguous bytes, `stride` bytes apart, asked into L2 by the whole block ahead of its slices: a slice takes 128
+// bytes of a row at a time, one slice ahead of its use, which is not enough against the latency of HBM.  For the matrices that a long
+// sequence leaves in HBM: the tokens' own rows of bwd_dfeat and bwd_dx (gradients of 5 x 4 x 16722 bf16 tokens, d = 64, M = 256, 1783 us with none,
+// 1741 with bwd_dfeat's, 1724 with both; of 2 x 12 x 4096, causal, 941 and 937).  The chunk's other rows too: 954, the first slices wait
+// behind all of them; those of bwd_numden and bwd_dv: the same within 1 %.
+__device__ __forceinline__ void prefetch_rows(const void* base, int64_t stride, int rows, int64_t bytes) {
+  const int lines = (int)((bytes + 127) >> 7);
+  for (int e = threadIdx.x; e < rows * lines; e += THREADS) {
+    const int r = e / lines;
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const char*>(base) + r * stride + (int64_t)(e - r * lines) * 128));
+  }
+}
 
 struct Block {
   uint8_t* sm;
