@@ -48,6 +48,13 @@ __device__ __forceinline__ float ex2_full(float x) {
   return y;
 }
 
+// 32 bytes (eight words) as one store; p is 32-byte aligned
+__device__ __forceinline__ void store32(float* p, const uint32_t* x) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(x[4]),
+               "r"(x[5]), "r"(x[6]), "r"(x[7])
+               : "memory");
+}
+
 // A factor as a float and its remainder: fmaf(hi, x, lo * x) is the product with the unrounded factor, rounded once.  (The same
 // factor multiplies every exponent: rounded to fp32 it moves exponents of 60 nats by 2e-6, all of them in one direction.)
 struct Factor {
@@ -588,6 +595,7 @@ feat3_kernel(const __grid_constant__ Args a) {
       float gmx = -3.0e38f;
       const float gshift = (WRITE && t.stab == FSHARP_STAB_GROUP) ? ord2f(t.gmax[bh]) : 0.f;
       const bool own = PAIR || (t.stab == FSHARP_STAB_ROW && a.nmb == 1);
+      const bool wide = WRITE && !OUT16 && (reinterpret_cast<uintptr_t>(t.phi) & 31) == 0;
       const bool scalar = terms && pp[pr.scal() + PS_CSCALAR] != 0.f;
       const Factor quad(scalar ? a.quad * (double)pp[pr.scal() + PS_CGAMMA] : 0.0);
       // 32 rows of ROW_BYTES of features from the lanes' registers to the warp's place in shared memory, and out by a copy that
@@ -752,9 +760,15 @@ feat3_kernel(const __grid_constant__ Args a) {
                 if (c + j < mb) put_rows(x + j, m0 + c + j, tok0);
             } else if (in) {
               float* dst = t.phi + at * a.M + m0 + c;
+              if (wide) {
 #pragma unroll
-              for (int j = 0; j < 32; j++)
-                if (j < 16 || c + 16 < mb) dst[j] = __uint_as_float(x[j]);
+                for (int j = 0; j < 4; j++)
+                  if (j < 2 || c + 16 < mb) store32(dst + 8 * j, &x[8 * j]);
+              } else {
+#pragma unroll
+                for (int j = 0; j < 32; j++)
+                  if (j < 16 || c + 16 < mb) dst[j] = __uint_as_float(x[j]);
+              }
             }
           }
         } else {
@@ -786,6 +800,18 @@ feat3_kernel(const __grid_constant__ Args a) {
   }
 }
 
+// Tiles per block up to which each lane stores its own row: where a block has only a few, nothing runs under the latency of staging and
+// copying, and lines that a row does not fill are written in parts either way.  Staged and direct, us, row shifts, 148 SMs.  d = 64, M = 256,
+// fp32: 24.8 and 24.6 with half a tile per block, 29.2 and 30.7 with one or two, 49.3 and 51.6 with four.  Rows of partial lines, d = 32, M = 208,
+// bf16: 18.0 and 17.4 with one, 40.8 and 39.8 with six, 46.0 and 46.2 with eight; d = 64, M = 48, fp32: 18.2 and 17.8, 33.8 and 33.7, 55.6 and 57.1 with
+// twelve; M = 16, half of a staged tile: 12.7 and 12.3, 35.7 and 33.7 with twenty.  d = 128, in halves of a line: fp32, M = 256, 71.7 and
+// 70.1 with two, 81.6 and 81.6 with three, 91.2 and 92.7 with four; bf16, 96 x 687 tokens, M = 256 (eight tiles per block, in pieces of sequences),
+// 169 and 164, 8 x 9472 87.4 and 89.0; one block of features, M = 64, 32.6 and 32.9 with three.
+int direct_tiles(int bits, int d, int M) {
+  if (d == 128) return bits == 16 && M > 128 ? 8 : 3;
+  return M < 32 ? 1 << 24 : M % 32 ? 6 : 1;
+}
+
 template <typename T, int D, int BP>
 int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, int G_groups, float qk_scale, uint8_t* img) {
   using G = FtGeo<T, D, BP, true>;
@@ -797,9 +823,13 @@ int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, in
     for (int i = 0; i < ntasks; i++) FS_TRY(tchost::make_map_tokens(&maps[i], tasks[i].X, tasks[i].ax, BH / a.H, a.H, tasks[i].L, D));
   CUtensorMap outs[2] = {};
   bool staged[2] = {};
+  int64_t items = 0;
+  for (int i = 0; i < ntasks; i++) items += (int64_t)BH * a.nmb * ((tasks[i].L + TILE - 1) / TILE);
+  const bool few = BP == 3 && items <= (int64_t)direct_tiles(sizeof(T) * 8, D, a.M) * ctx->sm_count;
   for (int i = 0; i < ntasks; i++) {
     void* phi = BP == 2 ? (void*)tasks[i].phi16 : (void*)tasks[i].phi;
-    staged[i] = reinterpret_cast<uintptr_t>(phi) % 16 == 0;          // (the library's own are)
+    const uintptr_t at = reinterpret_cast<uintptr_t>(phi);
+    staged[i] = at % 16 == 0 && !(few && at % 32 == 0);              // (the library's own are on 256-byte boundaries)
     if (staged[i]) FS_TRY(tchost::make_map_features(&outs[i], phi, BH, tasks[i].L, a.M, BP == 2, G::STAGE / 32));
   }
   const uint8_t* side_img[2] = {nullptr, nullptr};     // by side - 1
