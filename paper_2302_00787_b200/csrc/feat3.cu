@@ -260,6 +260,7 @@ rowterm3_kernel(const __grid_constant__ Args a) {
   const int total = a.first[2];
   const int w0 = (int)((int64_t)total * blockIdx.x / gridDim.x), w1 = (int)((int64_t)total * (blockIdx.x + 1) / gridDim.x);
   for (size_t i = blockIdx.x * (size_t)RT_THREADS + tid; i < a.zero4; i += (size_t)gridDim.x * RT_THREADS) a.zero[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (w0 >= w1) return;                           // a block that only clears
   if (a.own_terms) {
     // nothing but the start values where all groups of this block have C = gamma I
     bool all = true;
@@ -869,8 +870,14 @@ int launch_t(fsharp_ctx* ctx, Args& a, const Task* tasks, int ntasks, int BH, in
     constexpr size_t smem = rt_smem<T, D>();
     FS_CUDA_OK(cudaFuncSetAttribute(rowterm3_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int most = (D == 128 ? 1 : 3) * ctx->sm_count;
+    // A block per tile; where tiles are few, enough blocks for what is cleared (four stores per thread), up to one per SM.  (All of it by the
+    // blocks of one or two tiles: the attention of 2 x 64 tokens, d = 128, M = 1024, 84 -> 90 us, 85 so; up to three per SM: 64 x 100 tokens,
+    // d = 64, M = 256, 69.7 -> 71.3.)
+    const size_t clear = (a.zero4 + 4 * RT_THREADS - 1) / (4 * RT_THREADS);
+    int blocks = clear < (size_t)ctx->sm_count ? (int)clear : ctx->sm_count;
+    if (total > blocks) blocks = total < most ? total : most;
     FS_TIME_BEGIN(ctx, FS_K_ROWTERM);
-    (void)fs_launch_chained(rowterm3_kernel<T, D>, dim3(total < most ? total : most), dim3(RT_THREADS), smem, ctx->stream, a);
+    (void)fs_launch_chained(rowterm3_kernel<T, D>, dim3(blocks), dim3(RT_THREADS), smem, ctx->stream, a);
     FS_TIME_END(ctx);
     FS_LAUNCH_CHECK(ctx);
   }

@@ -52,6 +52,30 @@ def test_attention_and_gradients_at_tile_edges(d, dv, M, Lq, Lk, causal, chunk, 
             assert rel_err(got[0, h], r) < TOL[dtype]
 
 
+@pytest.mark.parametrize("d,dv,M,Lq,Lk", [(128, 128, 1024, 3, 5), (16, 16, 16, 1, 1), (32, 128, 1024, 200, 130), (64, 64, 512, 5000, 60)])
+def test_sums_start_from_zero_whatever_the_scratch_held(d, dv, M, Lq, Lk):
+    """The sums over tokens are cleared by the kernel of the quadratic terms, by more blocks than there are tiles where tiles are few."""
+    Q, K, V, dY, Om = inputs(d, dv, M, Lq, Lk, "f32", 5)
+    dQ, dK, dV, ddY, dOm = dev(Q), dev(K), dev(V), dev(dY), dev(Om)
+    ctx, clean = fb.Context(0), fb.Context(0)
+    _, pr = gpu_fit(ctx, dev(inputs(d, dv, M, 600, 600, "f32", 6)[0]), dev(inputs(d, dv, M, 600, 600, "f32", 6)[1]), d, "saderf")
+    big = [dev(t) for t in inputs(d, dv, M, 6000, 6000, "f32", 7)[:4]]
+
+    def calls(c):
+        return (c.fsharp_attend(dQ, dK, dV, dOm, pr), c.fsharp_kernel_apply(dQ, dK, dV, dOm, pr)) + tuple(
+            c.fsharp_attend_backward(dQ, dK, dV, ddY, dOm, pr))
+
+    want = calls(clean)
+    for i in range(5):                                    # the scratch full of another call's features before each
+        ctx.fsharp_attend_backward(*big, dOm, pr)
+        got = calls(ctx)[i]
+        assert torch.allclose(got, want[i], rtol=1e-5, atol=1e-5 * float(want[i].abs().max()))
+    assert ctx.status() == 0 and clean.status() == 0
+    prh = pr.cpu().numpy()
+    for h in range(2):
+        assert rel_err(host(want[0])[0, h], oracle_unit(Q, K, V, Om, prh[h], d, 0, h, False)) < TOL["f32"]
+
+
 @pytest.mark.parametrize("d,M,L,dtype", [(16, 16, 1, "f32"), (32, 272, 129, "f32"), (64, 1024, 130, "bf16"), (128, 144, 257, "f32"),
                                          (128, 1024, 128, "bf16")])
 @pytest.mark.parametrize("stab", [fb.STAB_NONE, fb.STAB_ROW, fb.STAB_GROUP])
