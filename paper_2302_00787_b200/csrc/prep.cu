@@ -39,13 +39,13 @@ __device__ __forceinline__ void scalars_of(int g, int side, const double* __rest
     for (int q = 0; q < 8; q++) {
       const int e = e0 + q * PREP_THREADS;
       cv[q] = e < d * d ? Cm[e] : 0.0;
-      if (e % (d + 1) == 0) cv[q] += alpha;                          // (0, but for the operator with exp(alpha |x|^2))
     }
 #pragma unroll
     for (int q = 0; q < 8; q++) {
       const int e = e0 + q * PREP_THREADS;
       if (e >= d * d) continue;
       const int i = e / d, j = e % d;
+      if (i == j) cv[q] += alpha;                                    // (0, but for the operator with exp(alpha |x|^2))
       if (images == nullptr) Cf[e] = (float)cv[q];
       if (i == j ? (cv[q] != gamma) : (cv[q] != 0.0)) cscalar = 0;
       if (images != nullptr) {
@@ -84,11 +84,12 @@ __device__ __forceinline__ void scalars_of(int g, int side, const double* __rest
 // launch 3 us longer, also with the sum for diagonal A).  The products run on the tensor cores at fp32
 // precision (mma3.cuh): 64 groups of 256 x 64 features are 200 million multiply-adds, which as fp32 instructions on operands in shared
 // memory took 20 us (bound by the shared-memory reads).  What is left is the latency of loads, products and stores one after the
-// other, and of a second wave of blocks where there is one.  A W block takes one side while all blocks are resident at once, two on
-// an SM, and both side by side beyond that (with one side each: 16 groups, M = 256, the two calls of the feature case 212 -> 207 us
-// and the slice 130 -> 124.5 us; 64 groups, the bidirectional step 235.5 -> 241.6 us).
+// other, in as many waves as it takes: two blocks on an SM (96 registers: three warps of each of two blocks' nine share a scheduler.  With more, one
+// block: features of 400 x 128 fp32 tokens, d = 128, M = 512, 744 us, 641 so).  d = 64 and below: a W block takes one side while that
+// makes at most two waves (d = 64) or one, both side by side beyond that (features of 128-token groups, d = 64, M = 256, us, one side and both: 24
+// groups 25.6 and 30.2, 64 36.3 and 40.8, 74 37.4 and 38.1, 200 86.6 and 81.8; d = 32: 37 16.7 and 17.9, 64 18.2 and 18.7, 100 21.6 and 19.8).
 template <int D, int SIDES>
-__global__ void __launch_bounds__(PREP_THREADS)
+__global__ void __launch_bounds__(PREP_THREADS, 2)
 prep_kernel(const float* __restrict__ Omega, int64_t omega_head_stride, const double* __restrict__ params,
             int64_t params_stride, int H, int pool, int M, float* __restrict__ prep, float qk_scale,
             uint8_t* __restrict__ images, int* __restrict__ img_flags, double half_log_m, double alpha, int* __restrict__ status) {
@@ -134,17 +135,18 @@ prep_kernel(const float* __restrict__ Omega, int64_t omega_head_stride, const do
     }
   };
   if (is_a) {
-    // A is diagonal in all fits: a_m = sum_k A_kk Omega_mk^2, in fp64, and no product (with one, these blocks and those of W were two
-    // waves of blocks for 64 groups)
+    // A is diagonal in all fits: a_m = sum_k A_kk Omega_mk^2, in fp64, and no product (which takes the same time, but ends in fp32:
+    // error of the gradients at d = 16 4.3e-7 and 6.4e-7)
     double* diag = reinterpret_cast<double*>(raw);
     const double* A = P + pl.A();
     int off = 0;
-    for (int e0 = tid; e0 < d * d; e0 += 8 * PREP_THREADS) {
-      double v[8];
+    constexpr int BATCH = D == 128 ? 16 : 8;
+    for (int e0 = tid; e0 < d * d; e0 += BATCH * PREP_THREADS) {
+      double v[BATCH];
 #pragma unroll
-      for (int q = 0; q < 8; q++) v[q] = e0 + q * PREP_THREADS < d * d ? A[e0 + q * PREP_THREADS] : 0.0;
+      for (int q = 0; q < BATCH; q++) v[q] = e0 + q * PREP_THREADS < d * d ? A[e0 + q * PREP_THREADS] : 0.0;
 #pragma unroll
-      for (int q = 0; q < 8; q++) {
+      for (int q = 0; q < BATCH; q++) {
         const int e = e0 + q * PREP_THREADS;
         if (e >= d * d) continue;
         if (e % (d + 1) == 0) diag[e / (d + 1)] = v[q];
@@ -233,7 +235,7 @@ int fs_run_prep_images(fsharp_ctx* ctx, const float* Omega, int64_t omega_head_s
   if (images != nullptr && (d != tcl::TC_D || M != tcl::TC_M)) return FSHARP_E_SHAPE;
   const int nchunks = (M + PREP_MB - 1) / PREP_MB;
   const int nz = nchunks > 2 ? nchunks : 2;
-  const bool apart = d == 128 || (int64_t)G * 4 * nz <= 2 * ctx->sm_count;
+  const bool apart = d == 128 || (int64_t)G * 4 * nz <= (d == 64 ? 4 : 2) * ctx->sm_count;
   const dim3 grid(G, apart ? 4 : 3, nz);
 #define FS_PREP(DD, SS)                                                                                              \
   do {                                                                                                               \

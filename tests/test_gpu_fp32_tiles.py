@@ -101,6 +101,22 @@ def test_features_at_block_edges(d, M, L, dtype, stab):
             assert got.max() <= 1.0 + 1e-6
 
 
+@pytest.mark.parametrize("d,M", [(16, 144), (32, 272), (64, 256), (64, 48), (128, 144)])
+def test_operands_of_however_many_groups(d, M):
+    """W is made one side at a time or both side by side, by the number of groups: a group's features have the same bits."""
+    ctx = fb.Context(0)
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    X = torch.randn(1, 3, 70, d, generator=gen, device="cuda") * d ** -0.25
+    Om = dev(wl.orthogonal_omega(M, d, 4))
+    _, pr = gpu_fit(ctx, X, X, d, "saderf")
+    for side in (1, 2):
+        want, _ = ctx.fsharp_featurize(X, Om, pr, side, stab=fb.STAB_ROW)
+        for G in (30, 66, 81, 402):
+            phi, _ = ctx.fsharp_featurize(X.repeat(1, G // 3, 1, 1), Om, pr.repeat(G // 3, 1), side, stab=fb.STAB_ROW)
+            assert torch.equal(phi, want.repeat(1, G // 3, 1, 1))
+    assert ctx.status() == 0
+
+
 def test_unaligned_feature_output_of_the_static_entry_point():
     """phi of fsharp_featurize_static may start on any 4-byte boundary: the result equals the aligned one's."""
     ctx = fb.Context(0)
