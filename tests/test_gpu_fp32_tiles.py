@@ -259,3 +259,24 @@ def test_kernel_operator_near_the_smallest_numbers():
     out = host(ctx.fsharp_kernel_apply(dev(X), dev(Y), dev(C), dev(Om), dev(fb.pack_params(p, d)[None])))
     assert ctx.status() == 0
     assert rel_err(out[0, 0], fs.kernel_apply(X[0, 0], Y[0, 0], C[0, 0], Om, p, 0.0)) < TOL["f32"]
+
+
+@pytest.mark.parametrize("d", [16, 32, 64, 128])
+@pytest.mark.parametrize("B,H,Lq,Lk,pool", [(1, 1, 1, 1, fb.POOL_PER_BH), (1, 3, 33, 5000, fb.POOL_PER_BH), (2, 19, 129, 700, fb.POOL_PER_HEAD),
+                                            (1, 75, 1024, 300, fb.POOL_PER_BH), (1, 2, 9000, 9000, fb.POOL_PER_BH)])
+def test_statistics_however_the_tokens_are_cut(B, H, Lq, Lk, pool, d):
+    """fp32 tensors: slices of both sides' tokens by lengths and numbers of (batch, head)s; against fp64 sums."""
+    ctx = fb.Context(0)
+    gen = torch.Generator(device="cuda").manual_seed(d + Lq)
+    Q, K = (torch.randn(B, H, L, d, generator=gen, device="cuda") + 0.3 for L in (Lq, Lk))
+    st = ctx.fsharp_stats(Q, K, pool=pool)
+    assert ctx.status() == 0
+    for X, at, mu in ((Q, 0, 2 * d * d), (K, d * d, 2 * d * d + d)):
+        x = X.double()
+        x = x.transpose(0, 1).flatten(1, 2) if pool == fb.POOL_PER_HEAD else x.flatten(0, 1)
+        M, m = x.transpose(1, 2) @ x / x.shape[1], x.mean(1)
+        scale = M.diagonal(dim1=1, dim2=2).sqrt()
+        # at most 64 products are added in fp32: 64 roundings of sums that are at most the root of the two diagonals' product
+        tol = 64 * 2.0 ** -24
+        assert ((st[:, at:at + d * d].view(-1, d, d) - M).abs() <= tol * scale[:, :, None] * scale[:, None]).all()
+        assert ((st[:, mu:mu + d] - m).abs() <= tol * scale).all()
