@@ -72,3 +72,27 @@ def test_features_on_every_way_out(d, M, L, dtype, stab, past):
     assert ctx.status() == 0
     check(phi, ls, X, Om, pr, d, stab)
     assert bool((buf[:past + guard] == -7.0).all()) and bool((buf[past + guard + 3 * L * M:] == -7.0).all())
+
+
+@pytest.mark.parametrize("d,M,groups,dtype", [(16, 144, 3, "f32"), (32, 272, 3, "f32"), (64, 256, 3, "f32"), (64, 48, 90, "f32"), (128, 144, 3, "f32"),
+                                              (64, 256, 3, "bf16"), (64, 256, 90, "bf16")])
+def test_features_of_a_dense_quadratic_form(d, M, groups, dtype):
+    """All fits give a diagonal A; a blob may hold any.  bf16: the operand images of the tensor-core kernels."""
+    ctx = fb.Context(0)
+    gen = torch.Generator(device="cuda").manual_seed(d + M)
+    X = torch.randn(1, 3, 150, d, generator=gen, device="cuda").to(torch.bfloat16 if dtype == "bf16" else torch.float32) * d ** -0.25
+    Om = dev(wl.orthogonal_omega(M, d, 4))
+    _, pr = gpu_fit(ctx, X, X, d, "saderf")
+    S = torch.randn(3, d, d, generator=gen, device="cuda", dtype=torch.float64) * 0.02 / d ** 0.5
+    pr[:, :d * d] += (S + S.transpose(1, 2)).flatten(1)
+    n = groups // 3
+    for side in (1, 2):
+        phi, ls = ctx.fsharp_featurize(X.repeat(1, n, 1, 1), Om, pr.repeat(n, 1), side, stab=fb.STAB_ROW)
+        assert ctx.status() == 0 and torch.equal(phi, phi[:, :3].repeat(1, n, 1, 1))
+        for h in range(3):
+            e = log_features(X[0, h], Om, pr[h], side, d)
+            w, A = Om.double().abs(), pr[h, :d * d].view(d, d).abs()
+            # as above, and the same of the terms of w^T A w; tensor-core kernels: W rounded to 11 bits (the bound of their other tests)
+            tol = 2.0 ** -24 * float(e.abs().max() + (w @ A * w).sum(1).max()) * math.sqrt(d) + 1e-6 if dtype == "f32" else 1e-2
+            assert (ls[0, h].double() - e.amax(1)).abs().max() < tol * max(1.0, float(e.abs().max()))
+            assert (phi[0, h].double() - (e - ls[0, h].double()[:, None]).exp()).abs().max() < tol

@@ -490,8 +490,8 @@ def test_attend_strided_layout_per_head_omega_and_pooling(ctx):
 
 @pytest.mark.parametrize("chunk,M", [(128, 256), (256, 384), (64, 512)])
 def test_causal_d128_chain_of_tensor_core_kernels(ctx, chunk, M):
-    """bf16, d = dv = 128 has no fused kernel: exponents, in-chunk scores, per-chunk key-side sums and the query side
-    each run on the tensor cores (chunk 64 leaves the last three to the fp32 kernels).  [B, L, H, *] storage,
+    """bf16, d = dv = 128 has no fused kernel: feature maps, running key-side sums and the query side with its in-chunk scores
+    each run on the tensor cores (chunk 64 leaves the last two to the fp32 kernels).  [B, L, H, *] storage,
     per-head Omega, parameters pooled per head, several chunks, a query / key scale; against the definition, unit by
     unit, and against the fp32 kernels."""
     w = W["cfg5"].scaled(B=2, H=2, L=768, M=M, chunk=chunk, outlier_frac=0.05)
@@ -510,7 +510,7 @@ def test_causal_d128_chain_of_tensor_core_kernels(ctx, chunk, M):
         Y32 = ctx.fsharp_attend(tr(dQ), tr(dK), tr(dV), dev(OmH), pr, causal=True, chunk=chunk, pool=fb.POOL_PER_HEAD, qk_scale=s)
     finally:
         ctx.set_impl(fb.IMPL_AUTO)
-    assert ctx.status() == 0 and launches == 12        # prep; 4 + 3 feature kernels; sums, scan, scores, query side
+    assert ctx.status() == 0 and launches == 12        # prep; 4 + 3 feature kernels; totals, scan, running sums, query side
     Y, Y32 = host(Y), host(Y32)
     prh = pr.cpu().numpy()
     for b in range(w.B):
