@@ -148,7 +148,7 @@ int fsharp_read_timing(fsharp_ctx* ctx, int cap, float* total_ms, int* launches)
 const char* fsharp_kernel_name(int id) {
   switch (id) {
     case FS_K_STATS: return "stats_kernel";
-    case FS_K_FIT: return "fit_kernel";
+    case FS_K_FIT: return "fit_kernel";      // all kernels of a fit: this one, closed_fit_kernel, the chain of fit_wide.cu
     case FS_K_PREP: return "prep_kernel";
     case FS_K_ROWTERM: return "rowterm3_kernel";
     case FS_K_FEAT: return "feat3_kernel";

@@ -3,7 +3,8 @@
 //
 // One thread block accumulates the Gram matrix of a slice of tokens of one
 // (batch, head, side): products in fp32 over 64 tokens, then folded into fp64
-// registers; slices are combined with fp64 atomics.
+// registers; slices are combined with fp64 atomics.  Tokens are read in 16-byte pieces: base and strides are multiples of 16 bytes
+// (the entry points refuse others).
 #include "common.cuh"
 
 namespace {

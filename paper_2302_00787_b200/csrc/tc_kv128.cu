@@ -12,7 +12,10 @@
 // 265 us, moved 2.2 GB that never had to; the two launches take 139 and 292 us.)
 // Segments: as many as there are SMs for all (segment, block, (batch, head)); where there is more than one, a first launch
 // (EMIT = false) adds up the earlier ones, cut finer so that it fills the chip too, and the scan kernel turns the pieces' sums into
-// what precedes every piece.
+// what precedes every piece.  From half as many (block, (batch, head))s as SMs there is one segment each, also where that leaves SMs without
+// work or a second wave short: the totals would read everything once more.  (Steps before, with single chunks' sums and their scan, and now, us:
+// 25 x 4096 tokens, M = 512, 100 blocks, 481 and 334; 38 x 4096, M = 512, 152 blocks, 608 and 470; 75 x 2048, M = 256, 150, 438 and 349; 76 x 4096,
+// M = 128, 76, 521 and 385.)
 #include "common.cuh"
 #include "tc_common.cuh"
 #include "tc_layout.cuh"
