@@ -260,7 +260,6 @@ rowterm3_kernel(const __grid_constant__ Args a) {
   const int total = a.first[2];
   const int w0 = (int)((int64_t)total * blockIdx.x / gridDim.x), w1 = (int)((int64_t)total * (blockIdx.x + 1) / gridDim.x);
   for (size_t i = blockIdx.x * (size_t)RT_THREADS + tid; i < a.zero4; i += (size_t)gridDim.x * RT_THREADS) a.zero[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (w0 >= w1) return;                           // a block that only clears
   if (a.own_terms) {
     // nothing but the start values where all groups of this block have C = gamma I
     bool all = true;
