@@ -98,8 +98,12 @@ prep_kernel(const float* __restrict__ Omega, int64_t omega_head_stride, const do
   // are written as well, in the layouts of tc_layout.cuh
   constexpr int d = D, NW = 2 / SIDES;                                 // W roles
   static_assert(SIDES * D <= 128, "columns of one product");
-  extern __shared__ __align__(16) uint8_t raw[];
+  extern __shared__ __align__(1024) uint8_t raw[];
   const int g = blockIdx.x, role = blockIdx.y, tid = threadIdx.x;
+  if (reinterpret_cast<uintptr_t>(raw) & 1023) {                       // (there is no room to align the stages)
+    if (tid == 0) atomicExch(status, FSHARP_E_INTERNAL);
+    return;
+  }
   if (role == NW + 1) {
     if (blockIdx.z < 2) scalars_of<D>(g, blockIdx.z + 1, params, params_stride, M, half_log_m, prep, qk_scale, images, img_flags, alpha, raw);
     return;
@@ -237,14 +241,15 @@ int fs_run_prep_images(fsharp_ctx* ctx, const float* Omega, int64_t omega_head_s
   const int nz = nchunks > 2 ? nchunks : 2;
   const bool apart = d == 128 || (int64_t)G * 4 * nz <= (d == 64 ? 4 : 2) * ctx->sm_count;
   const dim3 grid(G, apart ? 4 : 3, nz);
-  // Where there are no more blocks than SMs, each takes more than half of an SM's shared memory: two on one SM, while others run the tail of the
-  // kernel before, take turns (attention of 1 x 17613 queries, 23266 keys: 65 us apart, 72 with room for two on the SMs that are free first).
-  constexpr size_t APART = 116 * 1024;
-  static_assert(mma3::SMEM <= APART, "one value for the attribute");
-  const size_t smem = (int64_t)grid.x * grid.y * grid.z <= ctx->sm_count ? APART : mma3::SMEM;
+  // Shared memory: one block on an SM while there are no more blocks than SMs, two beyond that; and never so much that an SM is set up with its
+  // largest share of it, as it is for the kernels around this one: with the same share the kernels that follow take longer (seen, not
+  // explained; launched one by one: step of 1 x 17613 queries and 23266 keys 84.5 to 89 us, 81 so; 2^20 pairs, 32 draws, 3960 and 3905).
+  constexpr size_t ONE = 116 * 1024, TWO = mma3::SMEM - 1024;          // 132 and 196 KB (1 KB more per block); the stages start at 0
+  static_assert(2 * (TWO + 1024) <= 196 * 1024 && 2 * (ONE + 1024) > 228 * 1024, "shares");
+  const size_t smem = (int64_t)grid.x * grid.y * grid.z <= ctx->sm_count ? ONE : TWO;
 #define FS_PREP(DD, SS)                                                                                              \
   do {                                                                                                               \
-    FS_CUDA_OK(cudaFuncSetAttribute(prep_kernel<DD, SS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)APART));    \
+    FS_CUDA_OK(cudaFuncSetAttribute(prep_kernel<DD, SS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ONE));    \
     FS_TIME_BEGIN(ctx, FS_K_PREP);                                                                                    \
     (void)fs_launch_chained(prep_kernel<DD, SS>, grid, dim3(PREP_THREADS), smem, ctx->stream, Omega, omega_head_stride, params, params_stride, H,   \
                                                                pool, M, prep, qk_scale, images, flags, 0.5 * log((double)M), alpha, ctx->d_status);  \
