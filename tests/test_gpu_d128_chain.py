@@ -44,16 +44,19 @@ def test_chain_against_fp32_kernels(B, H, L, M, chunk, variant):
     assert np.abs(Y[:, :, 0] - host(V)[:, :, 0]).max() < 1e-2 * np.abs(host(V)[:, :, 0]).max()
 
 
-@pytest.mark.parametrize("M,variant", [(512, "sderf"), (384, "aderf"), (256, "sderf")])
+@pytest.mark.parametrize("M,variant", [(512, "sderf"), (384, "aderf"), (256, "sderf"), (512, "mixed"), (256, "mixed")])
 def test_blocks_over_many_tiles(M, variant):
     """16 (batch, head)s of 40 token tiles.  Two blocks of features: a pair of blocks exchanges its rows' maxima over eight or nine
     tiles, four or five per warpgroup, so that every place and barrier of the exchange is used again.  C = gamma I: the epilogue's reads
-    of a tile are done before the next one is copied over it.  Always the same bits."""
+    of a tile are done before the next one is copied over it.  mixed: groups with C = gamma I between groups with a dense C.  Always the
+    same bits."""
     ctx = fb.Context(0)
-    w = wl.Workload("chain", 2, 8, 5120, 128, 128, M, "bf16", variant, True, 256, "orthogonal", outlier_frac=0.05, seed=3)
+    w = wl.Workload("chain", 2, 8, 5120, 128, 128, M, "bf16", "sderf", True, 256, "orthogonal", outlier_frac=0.05, seed=3)
     Q, K, V = (dev(t, "bf16") for t in wl.make_qkv(w))
     Om = dev(wl.make_omega(w))
-    _, pr = gpu_fit(ctx, Q, K, 128, variant)
+    st, pr = gpu_fit(ctx, Q, K, 128, "sderf" if variant == "mixed" else variant)
+    if variant == "mixed":
+        pr[1::3] = ctx.fsharp_fit_params(st, 128, "aderf")[1::3]
     at = dict(causal=True, chunk=256)
     Y = ctx.fsharp_attend(Q, K, V, Om, pr, **at)
     ref = host(ctx.fsharp_attend(Q.float(), K.float(), V.float(), Om, pr, **at))
