@@ -172,10 +172,11 @@ int launch_stats(fsharp_ctx* ctx, const void* Q, const void* K, const fsharp_dim
   const int BH = dm->B * dm->H;
   const int Lmax = dm->Lq > dm->Lk ? dm->Lq : dm->Lk;
   // The split with the least work on the fullest SM, over the blocks that have tokens.  A block's start, its fold and its atomics cost as much as
-  // some 64 + 4096 / d tokens; d = 128: one block on an SM at a time, else two, which together take 1.6 times as long as one.  (As many blocks as
+  // some 600 tokens at d = 16, 200, 100 and 70 at d = 32, 64 and 128; d = 128: one block on an SM at a time, else two, which together take
+  // one and a half times as long as one (chosen over 230 shapes and their splits).  (As many blocks as
   // are resident for two sequences of the longer length, rounded down: 75 x 1024 tokens, d = 64, 83.5 us, 71 for four blocks per SM's worth before the
   // tokens were shared out, 60 so; 2 x 512 queries and 8192 keys, d = 128, 49, 36 and 31; 40 x 4096, d = 128, 490, 597 and 313.)
-  const int64_t start = 64 + 4096 / dm->d;
+  const int64_t start = 64 + 140000 / (dm->d * dm->d);
   const int most = (Lmax + 127) / 128 < 4 * ctx->sm_count ? (Lmax + 127) / 128 : 4 * ctx->sm_count;
   int nsplit = 1, tps = 0;
   int64_t least = 0;
@@ -183,7 +184,7 @@ int launch_stats(fsharp_ctx* ctx, const void* Q, const void* K, const fsharp_dim
     const int t = ((Lmax + n - 1) / n + 31) / 32 * 32;
     if ((Lmax + t - 1) / t != n) continue;
     const int64_t blocks = (int64_t)BH * ((dm->Lq + t - 1) / t + (dm->Lk + t - 1) / t), per = (blocks + ctx->sm_count - 1) / ctx->sm_count;
-    const int64_t cost = (dm->d == 128 ? 5 * per : 8 * (per / 2) + 5 * (per % 2)) * (t + start);
+    const int64_t cost = (dm->d == 128 ? 2 * per : 3 * (per / 2) + 2 * (per % 2)) * (t + start);
     if (tps == 0 || cost < least) { least = cost; nsplit = n; tps = t; }
   }
   dim3 grid(nsplit, BH, 2);
