@@ -416,7 +416,7 @@ rowterm3_kernel(const __grid_constant__ Args a) {
 // leaves little room).  Bound of the writing pass: HBM (128 KB per tile of 128 x 256: 6.5 k cycles of this SM's share of the rate of writes)
 // against 3.4 k cycles of products;
 // 2 x 8 x 10007 fp32 tokens, d = 64, M = 256, both sides: 217.6 us with each lane storing its own row in 32-byte pieces (a store instruction
-// then touches 32 lines: 3.5 TB/s at best, whole lines 5.7), 212 us now.  Measured inside: 12 k cycles per tile, the two warpgroups' stores
+// then touches 32 lines: 3.5 TB/s at best, whole lines 5.7), 212 us so.  Measured inside: 12 k cycles per tile, the two warpgroups' stores
 // taking turns at some 15 bytes per cycle, and 3.5 k of each 23 k waiting for the next tile's products.
 constexpr int FT_AHEAD = 4;                                        // tiles pulled into L2 ahead of the two buffers (BP = 2)
 constexpr int FT_STAGE0 = 8, FT_MMA = 12, FT_THREADS = 416;
